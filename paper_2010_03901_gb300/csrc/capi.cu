@@ -130,6 +130,18 @@ RowArgs row_args(fc2d_plan_s* p, bool compact) {
   return a;
 }
 
+// 1/n, n < 2^62, as 2^exp (1 + m 2^-32 + r 2^-64) with 1/2 <= 1/n 2^-exp <= 1, from the
+// exact quotient (2^(k-1) - n) 2^64 / n, 2^(k-1) < n < 2^k
+static FxFactor fx_reciprocal(int64_t n) {
+  int k = 0;
+  while ((INT64_C(1) << k) < n) ++k;
+  if ((INT64_C(1) << k) == n) return {-k, 0, 0};
+  const __int128 num = ((__int128)(INT64_C(1) << (k - 1)) - n) << 64;
+  const __int128 q = -((-num + n / 2) / n);  // in (-2^63, 0)
+  const int32_t r = (int32_t)(int64_t)q;
+  return {1 - k, (int32_t)(((int64_t)q - r) >> 32), r};
+}
+
 FftArgs fft_args(fc2d_plan_s* p) {
   FftArgs a{};
   const bool f64 = p->prm.precision == FC2D_FP64;
@@ -145,6 +157,10 @@ FftArgs fft_args(fc2d_plan_s* p) {
   a.rtw = f64 ? (const void*)p->rtw64 : (const void*)p->rtw32;
   a.tsx = f64 ? (const void*)p->fx.tws64 : (const void*)p->fx.tws32;
   a.tsy = f64 ? (const void*)p->fy.tws64 : (const void*)p->fy.tws32;
+  a.fxx = reinterpret_cast<const int4*>(p->fx.fxs);
+  a.fxy = reinterpret_cast<const int4*>(p->fy.fxs);
+  a.fxr = reinterpret_cast<const int4*>(p->rfx);
+  a.fxs = fx_reciprocal((int64_t)p->grid.nx * p->grid.ny);
   a.scale = 1.0 / ((double)p->grid.nx * p->grid.ny);
   a.cc4k = p->tune_cc4k;
   a.cols_tma = p->tune_tma;

@@ -148,6 +148,12 @@ void launch_interp(const InterpArgs& a, int n_f, bool fp64, const void* F, void*
 void launch_assemble(const RowArgs& a, int n_f, bool fp64, const double* f_grid,
                      const void* vals, void* ext, cudaStream_t s);
 
+// 1/(nx ny) for the fixed-point DFT: 2^exp (1 + m 2^-32 + r 2^-64), m = r = 0 for a power
+// of two
+struct FxFactor {
+  int exp, m, r;
+};
+
 struct FftArgs {
   int nx, ny, pitch;          // pitch: complex elements per intermediate row
   int nrx, nry;               // number of radices
@@ -157,6 +163,10 @@ struct FftArgs {
   const void* rtw;            // exp(-2 pi i k/nx), k <= nx/2
   const void* tsx;            // per-stage twiddles of the row transform (power-of-two sizes)
   const void* tsy;            // per-stage twiddles of the column transform
+  // double plans (fx.cuh): twiddles w 2^60 in 32-bit limbs (re hi, lo, im hi, lo)
+  const int4 *fxx, *fxy;      // per stage of the row and column transforms (powers of two)
+  const int4* fxr;            // exp(-2 pi i k/nx), k <= nx/2
+  FxFactor fxs;               // 1/(nx ny)
   double scale;               // 1/(nx ny)
   int cc4k;                   // columns per block of the 4096-point FP32 column passes
   int cols_tma;               // 1: those passes in the TMA-pipelined persistent form

@@ -86,21 +86,25 @@ __global__ void __launch_bounds__(256) k_fft_cols(FftArgs fa, int cb,
   }
 }
 
-bool launch_fft_rows_p2(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
-                        const void* ext, const double* f_grid, const void* vals, void* inter,
-                        cudaStream_t s);
+bool launch_fft_rows_p2(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
+                        const double* f_grid, const void* vals, void* inter, cudaStream_t s);
 bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
                          const void* ext, const double* f_grid, const void* vals, void* inter,
                          cudaStream_t s);
-bool launch_fft_cols_p2(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
-                        cudaStream_t s);
+bool launch_fft_cols_p2(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
 bool launch_fft_cols_64n(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
                          cudaStream_t s);
+
+bool launch_fft_rows_fx(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
+                        const double* f_grid, const void* vals, void* inter, cudaStream_t s);
+bool launch_fft_cols_fx(const FftArgs& fa, int n_f, const void* inter, void* fhat, cudaStream_t s);
 
 void launch_fft_rows(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
                      const void* ext, const double* f_grid, const void* vals, void* inter,
                      cudaStream_t s) {
-  if (launch_fft_rows_p2(fa, ra, n_f, fp64, mode, ext, f_grid, vals, inter, s)) return;
+  if (fp64 ? launch_fft_rows_fx(fa, ra, n_f, mode, ext, f_grid, vals, inter, s)
+           : launch_fft_rows_p2(fa, ra, n_f, mode, ext, f_grid, vals, inter, s))
+    return;
   if (launch_fft_rows_64n(fa, ra, n_f, fp64, mode, ext, f_grid, vals, inter, s)) return;
   dim3 grid(fa.ny, n_f);
   if (fp64) {
@@ -127,7 +131,9 @@ static int pick_cb(int ny, size_t csize) {
 
 void launch_fft_cols(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
                      cudaStream_t s) {
-  if (launch_fft_cols_p2(fa, n_f, fp64, inter, fhat, s)) return;
+  if (fp64 ? launch_fft_cols_fx(fa, n_f, inter, fhat, s)
+           : launch_fft_cols_p2(fa, n_f, inter, fhat, s))
+    return;
   if (launch_fft_cols_64n(fa, n_f, fp64, inter, fhat, s)) return;
   const int ncol = fa.nx / 2 + 1;
   if (fp64) {

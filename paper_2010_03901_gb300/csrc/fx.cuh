@@ -1,0 +1,311 @@
+// Block fixed-point arithmetic for the double-precision transforms.
+//
+// GB300 issues 2 FP64 multiply-adds per clock and SM, but 128 32-bit integer additions
+// and 64 32 x 32 -> 64 bit integer multiply-adds (measured: 2.0, 122 and 58).  A DFT of
+// doubles therefore runs here on 64-bit integers: the values of a transform share one
+// exponent (a block exponent, chosen from their largest magnitude), additions are 64-bit
+// integer additions, and a product with a twiddle factor is formed from 32-bit limbs.
+// The doubles enter through their bit patterns and leave through them, rounded once; no
+// FP64 instruction is issued.
+//
+// Error: a stage keeps its values within 2^62 of a unit and rounds to that unit after each
+// twiddle product, whose result is at most 2^58.5: an error of 2^-58 of the block's
+// largest value per stage, where FP64 rounds every operation to 2^-53 of its own result.
+// Between stages the block is shifted left by the bits that its largest value leaves
+// unused, so the unit follows the data.  Twiddles carry 60 bits.  A transform with an
+// infinity or a NaN among its inputs returns NaN everywhere.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "fc2d_kernels.cuh"
+
+namespace fc2d {
+namespace fx {
+
+using i64 = long long;
+
+// a complex value in units of 2^e (e: the block's exponent); 16 bytes, as double2
+struct __align__(16) c64 {
+  i64 x, y;
+};
+
+constexpr int kScale = 60;          // twiddles are w 2^60, in balanced 32-bit limbs
+constexpr int kDrop = 64 - kScale;  // a product with a twiddle is scaled by 2^-kDrop
+constexpr int kNaN = 1 << 20;       // block exponent of a transform with non-finite input
+
+__device__ __forceinline__ c64 operator+(c64 a, c64 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ c64 operator-(c64 a, c64 b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ c64 mul_mi(c64 a) { return {a.y, -a.x}; }  // -i a
+
+// v = h 2^32 + l with l in [-2^31, 2^31)
+__device__ __forceinline__ int lo32(i64 v) { return (int)v; }
+__device__ __forceinline__ int hi32(i64 v) { return (int)((unsigned)(v >> 32) + ((unsigned)v >> 31)); }
+
+__device__ __forceinline__ i64 mad(int a, int b, i64 c) { return (i64)a * b + c; }
+
+// a w 2^-kDrop for |a.x|, |a.y| <= 2^62.5: the products of the high limbs, plus the mixed
+// products rounded at bit 32 (each sum of mixed products stays below 2^63); the products
+// of the low limbs are below half a unit and are left out.  w = (re hi, re lo, im hi, im lo)
+__device__ __forceinline__ c64 mulw(c64 a, int4 w) {
+  const int xh = hi32(a.x), xl = lo32(a.x), yh = hi32(a.y), yl = lo32(a.y);
+  const i64 half = i64(1) << 31;
+  const int nh = -w.z, nl = -w.w;  // limbs are never -2^31
+  const i64 mx = mad(xh, w.y, mad(xl, w.x, mad(yh, nl, mad(yl, nh, half))));
+  const i64 my = mad(xh, w.w, mad(xl, w.z, mad(yh, w.y, mad(yl, w.x, half))));
+  return {mad(xh, w.x, mad(yh, nh, mx >> 32)), mad(xh, w.z, mad(yh, w.x, my >> 32))};
+}
+
+// v c for a constant c in [1/2, 1) given as c - 1 = m 2^-32 + r 2^-64 (|v| < 2^62.5)
+__device__ __forceinline__ i64 mulc(i64 v, int m, int r) {
+  const int h = hi32(v), l = lo32(v);
+  const i64 t = mad(l, m, mad(h, r, i64(1) << 31));
+  return mad(h, m, v) + (t >> 32);
+}
+// sqrt(1/2) - 1 = kRtM 2^-32 + kRtR 2^-64
+constexpr int kRtM = -1257966796;
+constexpr int kRtR = -102865788;
+
+// bits that differ from their lower neighbour: the top one bounds |v| < 2^(32 + index)
+__device__ __forceinline__ unsigned spread(i64 v) {
+  const int h = (int)(v >> 32);
+  return (unsigned)(h ^ (h + h));
+}
+__device__ __forceinline__ unsigned spread(c64 v) { return spread(v.x) | spread(v.y); }
+// the left shift that brings a block with these spread bits to |v| <= 2^62
+__device__ __forceinline__ int headroom(unsigned h) { return min(__clz((int)h) - 1, 30); }
+
+// The magnitude bits of a double's high word (exponent in bits 20..30): the block maximum
+// of these gives the block exponent.
+__device__ __forceinline__ unsigned magnitude(double d) {
+  return (unsigned)__double2hiint(d) & 0x7FFFFFFFu;
+}
+// x in units of 2^(E - 1080), E the block's largest biased exponent (at least 1): the
+// 53-bit significand shifted to |v| < 2^58 for exponent E, right by E - e bits for others
+__device__ __forceinline__ i64 from_double(double d, int E) {
+  const unsigned hi = (unsigned)__double2hiint(d);
+  const int e = (int)(hi >> 20) & 0x7FF;
+  const unsigned mh = (hi & 0xFFFFFu) | (e ? 0x100000u : 0u);
+  const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
+  const int sh = E - max(e, 1);
+  const i64 v = sh < 63 ? m >> sh : 0;
+  const i64 s = (i64)((int)hi >> 31);
+  return (v ^ s) - s;
+}
+__device__ __forceinline__ c64 from_double(double2 d, int E) {
+  return {from_double(d.x, E), from_double(d.y, E)};
+}
+// block exponent of values converted with the block maximum mag of magnitude()
+__device__ __forceinline__ int block_exp(unsigned mag) { return max((int)(mag >> 20), 1); }
+
+// Whether every nonzero v with unit 2^e becomes a normal double (or overflows to infinity
+// by its exponent field): the same for a whole block.
+__device__ __forceinline__ bool plain_exp(int e) { return e + 1086 - 63 >= 1 && e + 1086 <= 2046; }
+// v 2^e as a double, rounded to nearest (ties away from zero): normalise, round at bit 11,
+// assemble
+__device__ __forceinline__ double plain_double(i64 v, int e) {
+  const i64 s = v >> 63;
+  const unsigned long long a = (unsigned long long)((v ^ s) - s);
+  const int n = __clzll((i64)a);
+  const unsigned long long m = a << (n & 63);
+  const unsigned long long q = (m >> 11) + ((m >> 10) & 1);
+  const unsigned long long b = q + ((unsigned long long)(unsigned)(e + 1085 - n) << 52);
+  const unsigned long long sg = (unsigned long long)s & 0x8000000000000000ull;
+  return a ? __longlong_as_double((i64)(b | sg)) : 0.0;
+}
+__device__ __forceinline__ double to_double(i64 v, int e, bool plain) {
+  if (plain) return plain_double(v, e);
+  return e > kNaN / 2 ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(plain_double(v, 0), e);
+}
+__device__ __forceinline__ double2 to_double(c64 v, int e, bool plain) {
+  return {to_double(v.x, e, plain), to_double(v.y, e, plain)};
+}
+
+// ------------------------------------------------------------------------- //
+// Small forward DFTs; inputs |z| <= 2^58.5 give outputs below 2^62
+// ------------------------------------------------------------------------- //
+__device__ __forceinline__ void dft4(c64& a0, c64& a1, c64& a2, c64& a3) {
+  const c64 t0 = a0 + a2, t1 = a0 - a2, t2 = a1 + a3, t3 = mul_mi(a1 - a3);
+  a0 = t0 + t2;
+  a2 = t0 - t2;
+  a1 = t1 + t3;
+  a3 = t1 - t3;
+}
+
+template <int R> __device__ __forceinline__ void dft(c64* v) {
+  if constexpr (R == 2) {
+    const c64 a = v[0], b = v[1];
+    v[0] = a + b;
+    v[1] = a - b;
+  } else if constexpr (R == 4) {
+    dft4(v[0], v[1], v[2], v[3]);
+  } else {
+    static_assert(R == 8, "radix 2, 4 or 8");
+    c64 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+    dft4(e0, e1, e2, e3);
+    dft4(o0, o1, o2, o3);
+    const c64 w1 = {mulc(o1.x + o1.y, kRtM, kRtR), mulc(o1.y - o1.x, kRtM, kRtR)};
+    const c64 w2 = mul_mi(o2);
+    const c64 w3 = {mulc(o3.y - o3.x, kRtM, kRtR), mulc(-o3.x - o3.y, kRtM, kRtR)};
+    v[0] = e0 + o0;
+    v[4] = e0 - o0;
+    v[1] = e1 + w1;
+    v[5] = e1 - w1;
+    v[2] = e2 + w2;
+    v[6] = e2 - w2;
+    v[3] = e3 + w3;
+    v[7] = e3 - w3;
+  }
+}
+
+// ------------------------------------------------------------------------- //
+// A transform of N = 2^LOGN points by NT = N/8 threads, eight values each, on one padded
+// shared buffer; Stockham stages of radix 8 (the last one N/NS).  Block statistics go
+// through `st`, kSlots shared words that are zero when the transform starts: st[0] the
+// largest magnitude of the inputs, st[k] the spread bits after stage k.  Every thread of
+// the block takes part in the barriers and reductions.
+// ------------------------------------------------------------------------- //
+constexpr int kSlots = 8;
+__device__ __forceinline__ int pad(int i) { return i + (i >> 3); }
+__host__ __device__ constexpr int padded(int n) { return n + (n >> 3); }
+// pad(i + r S) = pad(i) + r step(S) when S is a multiple of 8, or S = 1 and i of 8
+template <int S> __host__ __device__ constexpr int step() { return S % 8 == 0 ? S + S / 8 : S; }
+
+__device__ __forceinline__ void block_max(unsigned v, unsigned* slot) {
+  v = __reduce_max_sync(0xFFFFFFFFu, v);
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, v);
+}
+__device__ __forceinline__ void block_or(unsigned v, unsigned* slot) {
+  v = __reduce_or_sync(0xFFFFFFFFu, v);
+  if ((threadIdx.x & 31) == 0) atomicOr(slot, v);
+}
+
+// Offset of the stage with sub-length NS in the per-stage twiddle table
+__host__ __device__ constexpr int stage_off(int N, int NS) {
+  int off = 0, ns = 1;
+  while (ns < NS) {
+    const int R = (N / ns >= 8) ? 8 : N / ns;
+    if (ns > 1) off += R * ns;
+    ns *= R;
+  }
+  return off;
+}
+template <int LOGN> __host__ __device__ constexpr int last_ns() {
+  int ns = 1;
+  while (true) {
+    const int R = ((1 << LOGN) / ns >= 8) ? 8 : (1 << LOGN) / ns;
+    if (ns * R == (1 << LOGN)) return ns;
+    ns *= R;
+  }
+}
+
+// Rescale and twiddle the eight inputs of a stage after the first: the first value of each
+// butterfly by a shift, the others by their twiddles (tw[r NS + k]); radix-R DFTs.
+template <int R, int NS, int NT>
+__device__ __forceinline__ void butterflies(c64 (&v)[8], int t, const int4* __restrict__ tw, int L) {
+#pragma unroll
+  for (int m = 0; m < 8 / R; ++m) {
+    const int k = (t + m * NT) & (NS - 1);
+    c64* a = v + m * R;
+    const i64 rnd = 1 << (kDrop - 1);
+    a[0] = {((a[0].x << L) + rnd) >> kDrop, ((a[0].y << L) + rnd) >> kDrop};
+#pragma unroll
+    for (int r = 1; r < R; ++r) a[r] = mulw(c64{a[r].x << L, a[r].y << L}, __ldg(tw + r * NS + k));
+    dft<R>(a);
+  }
+}
+
+// All stages but the first.  buf holds the outputs of the stage before (sub-length NS),
+// st[SLOT] their spread.  On return v holds the thread's last-stage outputs (value r of
+// butterfly m belongs at index out_index<LOGN>(t, m, r)) and e their exponent.
+template <int LOGN, int NS, int SLOT>
+__device__ __forceinline__ void rest(c64 (&v)[8], c64* buf, int t, bool active, unsigned* st,
+                                     const int4* __restrict__ tw, int& e) {
+  constexpr int N = 1 << LOGN, NT = N / 8;
+  constexpr int R = N / NS >= 8 ? 8 : N / NS, NR = N / R, M = 8 / R;
+  const int L = headroom(st[SLOT]);
+  e += kDrop - L;
+  if (active) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      if constexpr (NR % 8 == 0) {
+        const c64* src = buf + pad(t + m * NT);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[m * R + r] = src[r * step<NR>()];
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[m * R + r] = buf[pad(t + m * NT + r * NR)];
+      }
+    }
+  }
+  if constexpr (NS * R < N) __syncthreads();
+  unsigned h = 0;
+  if (active) {
+    butterflies<R, NS, NT>(v, t, tw + stage_off(N, NS), L);
+    if constexpr (NS * R < N) {  // R = 8
+      const int k = t & (NS - 1);
+      const int base = (t / NS) * NS * R + k;
+      c64* dst = buf + pad(base);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        dst[r * step<NS>()] = v[r];
+        h |= spread(v[r]);
+      }
+    }
+  }
+  if constexpr (NS * R < N) {
+    block_or(h, st + SLOT + 1);
+    __syncthreads();
+    rest<LOGN, NS * R, SLOT + 1>(v, buf, t, active, st, tw, e);
+  }
+}
+
+// index of value r of the thread's last-stage butterfly m
+template <int LOGN> __device__ __forceinline__ int out_index(int t, int m, int r) {
+  constexpr int N = 1 << LOGN, NS = last_ns<LOGN>(), NT = N / 8;
+  return t + m * NT + r * NS;  // j = t + m NT < NS: (j / NS) NS R + (j mod NS) + r NS
+}
+template <int LOGN> __host__ __device__ constexpr int last_radix() { return (1 << LOGN) / last_ns<LOGN>(); }
+
+// The whole transform of the doubles u[r] = x[t + r N/8] (every thread's eight inputs are
+// in registers; `buf` may have held them).  v, e: as rest().
+template <int LOGN>
+__device__ __forceinline__ void transform(const double2 (&u)[8], c64 (&v)[8], c64* buf, int t,
+                                          bool active, unsigned* st, const int4* __restrict__ tw,
+                                          int& e) {
+  static_assert(LOGN >= 4, "at least two stages");
+  unsigned mag = 0;
+  if (active) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) mag = max(mag, max(magnitude(u[r].x), magnitude(u[r].y)));
+  }
+  block_max(mag, st);
+  __syncthreads();
+  const int E = block_exp(st[0]);
+  e = E >= 0x7FF ? kNaN : E - 1080;
+  unsigned h = 0;
+  if (active) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = from_double(u[r], E);
+    dft<8>(v);
+    c64* dst = buf + pad(8 * t);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      dst[r] = v[r];
+      h |= spread(v[r]);
+    }
+  }
+  block_or(h, st + 1);
+  __syncthreads();
+  rest<LOGN, 8, 1>(v, buf, t, active, st, tw, e);
+  if (E >= 0x7FF) e = kNaN;
+}
+
+// v times an FxFactor, its power of two left to the exponent
+__device__ __forceinline__ c64 scaled(c64 v, const FxFactor& f) {
+  return f.m ? c64{mulc(v.x, f.m, f.r), mulc(v.y, f.m, f.r)} : v;
+}
+
+}  // namespace fx
+}  // namespace fc2d

@@ -308,7 +308,18 @@ static void line_crossings(const Curve& c, int which, int nlines, double o, doub
 // ------------------------------------------------------------------------- //
 // FFT axis setup
 // ------------------------------------------------------------------------- //
-static bool fft_axis(int n, FftAxis& ax) {
+// x 2^60, |x| <= 1, rounded, as h 2^32 + l with -2^31 < l < 2^31 (a low limb of -2^31,
+// which has no negative, moves by one unit)
+static void fx_limbs(dd x, int32_t* out) {
+  const double a = std::ldexp(x.hi, 60), ai = std::floor(a);
+  int64_t v = (int64_t)ai + (int64_t)std::nearbyint((a - ai) + std::ldexp(x.lo, 60));
+  int32_t l = (int32_t)(uint32_t)(uint64_t)v;
+  if (l == INT32_MIN) l = (int32_t)(uint32_t)(uint64_t)++v;
+  out[0] = (int32_t)((v - l) >> 32);
+  out[1] = l;
+}
+
+static bool fft_axis(int n, bool fp64, FftAxis& ax) {
   ax.n = n;
   ax.n_radix = 0;
   int m = n;
@@ -319,11 +330,16 @@ static bool fft_axis(int n, FftAxis& ax) {
   while (m % 2 == 0) { ax.radix[ax.n_radix++] = 2; m /= 2; }
   if (m != 1 || ax.n_radix > kMaxRadices) return false;
   ax.tw_host.assign(2 * (size_t)n, 0.0);
+  ax.fx_host.assign(fp64 ? 4 * (size_t)n : 0, 0);
   for (int t = 0; t < n; ++t) {
     dd c, s;
     dd_cos_sin_turn(-(long long)t, n, c, s);
     ax.tw_host[2 * t] = to_double(c);
     ax.tw_host[2 * t + 1] = to_double(s);
+    if (fp64) {
+      fx_limbs(c, &ax.fx_host[4 * (size_t)t]);
+      fx_limbs(s, &ax.fx_host[4 * (size_t)t + 2]);
+    }
   }
   return true;
 }
@@ -331,9 +347,11 @@ static bool fft_axis(int n, FftAxis& ax) {
 // Twiddles of each Stockham stage after the first, for a power-of-two length N and
 // radices min(E, N/Ns): block s holds w^(r k N/(Ns R)), r < R, k < Ns, stored [r][k], so
 // that the lanes of a warp (consecutive k) read consecutive entries.
-static std::vector<double> stage_twiddles(const FftAxis& ax, int E) {
-  std::vector<double> out;
-  const int N = ax.n;
+// tab: w^t, t < N, of `words` words each.
+template <typename T>
+static std::vector<T> stage_twiddles(const FftAxis& ax, const std::vector<T>& tab, int words, int E) {
+  std::vector<T> out;
+  const int N = tab.empty() ? 0 : ax.n;
   if (N <= 0 || (N & (N - 1))) return out;
   for (int ns = 1; ns < N;) {
     const int R = (N / ns >= E) ? E : N / ns;
@@ -341,8 +359,7 @@ static std::vector<double> stage_twiddles(const FftAxis& ax, int E) {
       for (int r = 0; r < R; ++r)
         for (int k = 0; k < ns; ++k) {
           const long long t = ((long long)r * k * (N / (ns * R))) % N;
-          out.push_back(ax.tw_host[2 * t]);
-          out.push_back(ax.tw_host[2 * t + 1]);
+          out.insert(out.end(), tab.begin() + words * t, tab.begin() + words * (t + 1));
         }
     ns *= R;
   }
@@ -854,14 +871,20 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
   }
 
   // FFT axes
-  if (!fft_axis(nx / 2, p->fx) || !fft_axis(ny, p->fy))
+  const bool fp64 = P.precision == FC2D_FP64;
+  if (!fft_axis(nx / 2, fp64, p->fx) || !fft_axis(ny, fp64, p->fy))
     return fail(set_error(FC2D_ERR_UNSUPPORTED, "fc2d_plan: nx/2 and ny must be 2^a 3^b 5^c"));
   p->rtw_host.assign(2 * (size_t)(nx / 2 + 1), 0.0);
+  std::vector<int32_t> rfx(fp64 ? 4 * (size_t)(nx / 2 + 1) : 0);
   for (int t = 0; t <= nx / 2; ++t) {
     dd c, s;
     dd_cos_sin_turn(-(long long)t, nx, c, s);
     p->rtw_host[2 * t] = to_double(c);
     p->rtw_host[2 * t + 1] = to_double(s);
+    if (fp64) {
+      fx_limbs(c, &rfx[4 * (size_t)t]);
+      fx_limbs(s, &rfx[4 * (size_t)t + 2]);
+    }
   }
 
   // upload
@@ -880,8 +903,12 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
   // FP32: the table, then the same halved (exactly) for the row kernel's split
   std::vector<float> rtw32(p->rtw_host.begin(), p->rtw_host.end());
   for (size_t k = 0, n = p->rtw_host.size(); k < n; ++k) rtw32.push_back(0.5f * rtw32[k]);
-  std::vector<double> tsx64 = stage_twiddles(p->fx, 8), tsy64 = stage_twiddles(p->fy, 8);
-  std::vector<double> tsx16 = stage_twiddles(p->fx, 16), tsy16 = stage_twiddles(p->fy, 16);
+  std::vector<double> tsx64 = stage_twiddles(p->fx, p->fx.tw_host, 2, 8),
+                      tsy64 = stage_twiddles(p->fy, p->fy.tw_host, 2, 8);
+  std::vector<double> tsx16 = stage_twiddles(p->fx, p->fx.tw_host, 2, 16),
+                      tsy16 = stage_twiddles(p->fy, p->fy.tw_host, 2, 16);
+  std::vector<int32_t> fsx = stage_twiddles(p->fx, p->fx.fx_host, 4, 8),
+                       fsy = stage_twiddles(p->fy, p->fy.fx_host, 4, 8);
   std::vector<float> tsx32(tsx16.begin(), tsx16.end()), tsy32(tsy16.begin(), tsy16.end());
   std::vector<int> zero_status(1, 0);
   // the stencil taps as compact indices (every grid tap is an inside point); the
@@ -927,7 +954,10 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
       (st = upload(&p->fy.tw64, p->fy.tw_host)) || (st = upload(&p->fy.tw32, tw32y)) ||
       (st = upload(&p->rtw64, p->rtw_host)) || (st = upload(&p->rtw32, rtw32)) ||
       (st = upload(&p->fx.tws64, tsx64)) || (st = upload(&p->fy.tws64, tsy64)) ||
-      (st = upload(&p->fx.tws32, tsx32)) || (st = upload(&p->fy.tws32, tsy32)))
+      (st = upload(&p->fx.tws32, tsx32)) || (st = upload(&p->fy.tws32, tsy32)) ||
+      (st = upload(&p->fx.fx, p->fx.fx_host)) || (st = upload(&p->fy.fx, p->fy.fx_host)) ||
+      (st = upload(&p->fx.fxs, fsx)) || (st = upload(&p->fy.fxs, fsy)) ||
+      (st = upload(&p->rfx, rfx)))
     return fail(st);
   // interpolation weights (Section 3.4), computed once in FP64 on the GPU
   {
@@ -1003,7 +1033,8 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
                   p->dev.gidx_i, p->dev.gw_i, p->dev.wn_i, p->dev.gidx_ic,
                   p->dev.status, p->fx.tw64, p->fx.tw32,
                   p->fy.tw64, p->fy.tw32, p->rtw64, p->rtw32, p->ws.base,
-                  p->fx.tws64, p->fx.tws32, p->fy.tws64, p->fy.tws32};
+                  p->fx.tws64, p->fx.tws32, p->fy.tws64, p->fy.tws32, p->fx.fx,
+                  p->fx.fxs, p->fy.fx, p->fy.fxs, p->rfx};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (auto& r : p->prof) {

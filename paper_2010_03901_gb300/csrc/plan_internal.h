@@ -29,6 +29,9 @@ struct FftAxis {
   float* tw32 = nullptr;         // device, 2N floats
   // power-of-two lengths: per-stage twiddles [stage][r][k] for the radix-8 (double) and
   // radix-16 (float) Stockham sequences (see stage_twiddles in plan.cpp)
+  std::vector<int32_t> fx_host;  // double plans: w 2^60 in 32-bit limbs, 4 N words (fx.cuh)
+  int32_t* fx = nullptr;         // device, the same
+  int32_t* fxs = nullptr;        // device, per stage of the radix-8 Stockham sequence
   double* tws64 = nullptr;
   float* tws32 = nullptr;
 };
@@ -120,6 +123,7 @@ struct fc2d_plan_s {
   fc2d::FftAxis fx, fy;                      // nx/2 (complex) and ny
   std::vector<double> rtw_host;              // exp(-2 pi i k/nx), k <= nx/2 (R2C post-process)
   double* rtw64 = nullptr;
+  int32_t* rfx = nullptr;   // double plans: rtw 2^60 in 32-bit limbs
   float* rtw32 = nullptr;   // [2][nx/2 + 1] complex: exp(-2 pi i k/nx), then halved
   fc2d::DeviceTables dev;
   fc2d::Workspace ws;
