@@ -861,6 +861,30 @@ fc2d_status gi_work_fill(const GiPlanArgs& in, void* out, int* ldS) {
   return FC2D_OK;
 }
 
+// The records travel as kernel parameters (kWorkChunk at a time), so that a call needs no
+// host buffer that outlives it, captured or not.
+constexpr int kWorkChunk = 8;
+struct GiWorkChunk {
+  GiWork r[kWorkChunk];
+};
+__global__ void k_write_work(const __grid_constant__ GiWorkChunk c, int n, GiWork* dst,
+                             int* counter) {
+  if (threadIdx.x < (unsigned)n) dst[threadIdx.x] = c.r[threadIdx.x];
+  if (threadIdx.x == 0) *counter = 0;
+}
+
+fc2d_status launch_write_work(const void* records, int n, void* dst, int* counter,
+                              cudaStream_t s) {
+  const auto* r = static_cast<const GiWork*>(records);
+  for (int i = 0; i < n; i += kWorkChunk) {
+    GiWorkChunk c{};
+    const int m = std::min(kWorkChunk, n - i);
+    std::copy(r + i, r + i + m, c.r);
+    k_write_work<<<1, 32, 0, s>>>(c, m, static_cast<GiWork*>(dst) + i, counter);
+  }
+  return cuda_check(cudaGetLastError(), "work records launch");
+}
+
 fc2d_status launch_gather_interp_queue(const void* work, const int4* items, int n_items,
                                        int* counter, int nt, int max_ldS, int n_cta,
                                        cudaStream_t s) {

@@ -137,6 +137,9 @@ fc2d_status launch_gather_interp_tc(const GiPlanArgs& in, int nt, cudaStream_t s
 // gi_work_fill, which also returns the plan's staging row length); max_ldS: the largest.
 size_t gi_work_bytes();
 fc2d_status gi_work_fill(const GiPlanArgs& in, void* out, int* ldS);
+// writes n records to device memory and zeroes the counter, on the stream
+fc2d_status launch_write_work(const void* records, int n, void* dst, int* counter,
+                              cudaStream_t s);
 fc2d_status launch_gather_interp_queue(const void* work, const int4* items, int n_items,
                                        int* counter, int nt, int max_ldS, int n_cta,
                                        cudaStream_t s);

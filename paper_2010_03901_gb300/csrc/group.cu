@@ -1,15 +1,21 @@
-// Plan groups: several domains' extension + DFT pipelines (steps 5-7 of Section 3.5) as
-// one CUDA graph.  The strip-point values of every mixed-form member (the fused blend +
-// interpolation, steps 5-6) come from one persistent kernel over all members' work items
-// (plan, owner range, function), longest first; then each plan's row and column DFTs run
-// on their own branch (forked from the launching stream and joined back), so the
-// kernels of small domains run side by side.  FP64 members run their whole call on a
-// branch.  The graph is captured on the first call and replayed while the arguments
-// (function counts and pointers) and every plan's workspace (base and size) stay the
-// same, re-captured when any of them changes.  The workspace is part of the key because
-// the captured kernels hold its address: a later call on a member plan that needs more
-// workspace frees the old one and allocates another, and a replay of the old graph would
-// then read and write freed memory.
+// Plan groups: several domains' extension + DFT pipelines (steps 5-7 of Section 3.5) in
+// one call, every plan's work on its own stream forked from the caller's and joined back,
+// so that the kernels of small domains run side by side.  Two forms: "branches", each
+// plan's whole call on its stream; "persistent", the strip-point values of every
+// mixed-form member (the fused blend + interpolation, steps 5-6) from one persistent
+// kernel over all members' work items (plan, owner range, function), longest first, and
+// then each plan's row and column DFTs on its stream (FP64 members: their whole call).
+//
+// The form, and the persistent kernel's CTA shape, are timed once for a set of function
+// counts.  A call launches its kernels directly, whatever its buffers: capturing and
+// instantiating a graph for new buffers costs more host time (and, timed on them, more
+// device time) than the work itself: eight stars of 256^2 .. 2048^2 with 32 functions each
+// took 34.8 ms per call when every call came with other buffers, the kernels 2.6 ms of it.
+// A call with the arguments of the call before it is captured as a CUDA graph, which is
+// replayed while the arguments (function counts and pointers) and every plan's workspace
+// (base and size) stay the same.  The workspace is part of the key because the captured
+// kernels hold its address: a later call on a member plan that needs more workspace frees
+// the old one and allocates another, and a replay would then use freed memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,14 +46,15 @@ constexpr int64_t kItemFixed = 256;
 
 struct fc2d_group_s {
   std::vector<fc2d_plan_t> plans;
-  std::vector<cudaStream_t> branch;       // one capture stream per plan
-  cudaStream_t cap = nullptr;             // the capture origin
+  std::vector<cudaStream_t> branch;       // one stream per plan
+  cudaStream_t cap = nullptr;             // tuning runs, and the capture origin
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> join;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  std::vector<int> key_nf;                // arguments of the captured graph
-  std::vector<const void*> key_ptr;
+  std::vector<int> key_nf, graph_nf;      // arguments of the last call, of the graph
+  std::vector<const void*> key_ptr, graph_ptr;
+  std::vector<int> tuned_nf;              // function counts of the kept choice and items
   // the persistent blend + interpolation kernel: per-plan records, work items, counter
   cudaEvent_t fork_dft = nullptr;         // after the persistent kernel
   void* work = nullptr;
@@ -55,20 +62,27 @@ struct fc2d_group_s {
   int4* items = nullptr;
   size_t items_cap = 0;
   int* counter = nullptr;
-  int nt = 0;                             // its threads per CTA (autotuned at capture)
-  int persistent = 0;                     // the captured form (autotuned at capture)
+  int n_items = 0;
+  int nt = 0;                             // its threads per CTA (tuned)
+  int persistent = 0;                     // the kept form (tuned)
   int forced_form = -1, forced_nt = 0;    // fc2d_group_tuning_set (-1: tune)
-  // microseconds: queue kernel with 256 and 512 threads, graph with branches only,
-  // graph with the queue kernel
+  // microseconds: queue kernel with 256 and 512 threads, a call with branches only, a
+  // call with the queue kernel
   float tune_us[4] = {0.f, 0.f, 0.f, 0.f};
 };
 
 using namespace fc2d;
 
-static void group_free(fc2d_group_s* g) {
-  if (!g) return;
+static void drop_graph(fc2d_group_s* g) {
   if (g->exec) cudaGraphExecDestroy(g->exec);
   if (g->graph) cudaGraphDestroy(g->graph);
+  g->exec = nullptr;
+  g->graph = nullptr;
+}
+
+static void group_free(fc2d_group_s* g) {
+  if (!g) return;
+  drop_graph(g);
   for (cudaEvent_t e : g->join)
     if (e) cudaEventDestroy(e);
   if (g->fork) cudaEventDestroy(g->fork);
@@ -123,195 +137,164 @@ static fc2d_status grow(void** buf, size_t* cap, size_t bytes) {
   return FC2D_OK;
 }
 
-// Time the persistent kernel with 256 and 512 threads per CTA (two or one per SM) on the
-// call's own inputs (it recomputes the same strip values), three launches each after
-// one warm-up; keep the faster.
-static fc2d_status tune_queue(fc2d_group_s* g, int n_items, int max_ldS, int n_sm) {
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-    if (e0) cudaEventDestroy(e0);
-    return set_error(FC2D_ERR_CUDA, "fc2d_group: event creation failed");
-  }
-  fc2d_status st = FC2D_OK;
-  const int shapes[2] = {256, 512};
-  for (int k = 0; k < 2 && !st; ++k) {
-    const int nt = shapes[k], n_cta = std::min(n_items, n_sm * (512 / nt));
-    for (int r = 0; r < 4 && !st; ++r) {
-      if (r == 1) cudaEventRecord(e0, g->cap);
-      cudaMemsetAsync(g->counter, 0, sizeof(int), g->cap);
-      st = launch_gather_interp_queue(g->work, g->items, n_items, g->counter, nt, max_ldS, n_cta,
-                                      g->cap);
-    }
-    cudaEventRecord(e1, g->cap);
-    if (!st && cudaEventSynchronize(e1) != cudaSuccess)
-      st = set_error(FC2D_ERR_CUDA, "fc2d_group: tuning launch failed");
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    g->tune_us[k] = 1e3f * ms / 3;
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (!st) g->nt = g->tune_us[0] <= g->tune_us[1] ? 256 : 512;
-  return st;
-}
+// One call's arguments and what follows from them: the mixed-form members' records.
+struct Call {
+  const int* n_f;
+  const double* const* fg;
+  const double* const* fb;
+  void* const* fhat;
+  std::vector<char> fused;
+  std::vector<unsigned char> work;
+  std::vector<std::vector<int32_t>> points;  // strip points of each range, per record
+  int n_fused = 0, max_ldS = 0, n_sm = 1;
+  const double* bdry(int i) const { return fb ? fb[i] : nullptr; }
+};
 
-// Capture one form of the group call into *graph.  persistent: the queue kernel over
-// the mixed-form members' work items, then per plan the DFTs on its branch; otherwise
-// every plan's whole call on its branch (the domains' blends then overlap the other
-// domains' DFTs).  FP64 members run their whole call on a branch in both forms.
-static fc2d_status capture_form(fc2d_group_s* g, bool persistent, const std::vector<char>& fused,
-                                int n_items, int max_ldS, int n_sm, const int* n_f,
-                                const double* const* fg, const double* const* fb,
-                                void* const* fhat, cudaGraph_t* graph) {
+static fc2d_status describe(fc2d_group_s* g, Call& c) {
   const int n = (int)g->plans.size();
-  *graph = nullptr;
-  if (cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-    return set_error(FC2D_ERR_CUDA, "fc2d_group: stream capture failed to start");
-  fc2d_status st = FC2D_OK;
-  cudaEventRecord(g->fork, g->cap);
-  if (persistent) {
-    cudaMemsetAsync(g->counter, 0, sizeof(int), g->cap);
-    st = launch_gather_interp_queue(g->work, g->items, n_items, g->counter, g->nt, max_ldS,
-                                    std::min(n_items, n_sm * (512 / g->nt)), g->cap);
-    cudaEventRecord(g->fork_dft, g->cap);
-  }
-  for (int i = 0; i < n && !st; ++i) {
-    const bool q = persistent && fused[i];
-    cudaStreamWaitEvent(g->branch[i], q ? g->fork_dft : g->fork, 0);
-    st = q ? extend_coeffs_dft(g->plans[i], n_f[i], fg[i], fhat[i], g->branch[i])
-           : fc2d_extend_coeffs(g->plans[i], n_f[i], fg[i], fb ? fb[i] : nullptr, fhat[i],
-                                g->branch[i]);
-    cudaEventRecord(g->join[i], g->branch[i]);
-    cudaStreamWaitEvent(g->cap, g->join[i], 0);
-  }
-  const cudaError_t e = cudaStreamEndCapture(g->cap, graph);
-  if (st || e != cudaSuccess || !*graph) {
-    if (*graph) cudaGraphDestroy(*graph);
-    *graph = nullptr;
-    return st ? st : set_error(FC2D_ERR_CUDA, "fc2d_group: stream capture failed");
+  const size_t rec = gi_work_bytes();
+  c.fused.assign(n, 0);
+  for (int i = 0; i < n; ++i) {
+    fc2d_plan_s* p = g->plans[i];
+    fc2d_status st = extend_coeffs_check(p, c.n_f[i], c.fg[i], c.bdry(i), c.fhat[i]);
+    if (st) return st;
+    if (!group_fused(p)) continue;
+    c.points.emplace_back();
+    const GiPlanArgs a = group_fused_args(p, c.n_f[i], c.fg[i], c.bdry(i), &c.points.back());
+    c.work.resize((size_t)(c.n_fused + 1) * rec);
+    int ld = 0;
+    if ((st = gi_work_fill(a, c.work.data() + (size_t)c.n_fused * rec, &ld))) return st;
+    c.max_ldS = std::max(c.max_ldS, ld);
+    c.n_sm = std::max(c.n_sm, p->n_sm);
+    c.fused[i] = 1;
+    ++c.n_fused;
   }
   return FC2D_OK;
 }
 
-// Mean microseconds of three launches of `exec` after one warm-up.
-static float time_graph(fc2d_group_s* g, cudaGraphExec_t exec) {
+static fc2d_status queue(fc2d_group_s* g, const Call& c, int nt, cudaStream_t s) {
+  fc2d_status st = launch_write_work(c.work.data(), c.n_fused, g->work, g->counter, s);
+  if (st) return st;
+  return launch_gather_interp_queue(g->work, g->items, g->n_items, g->counter, nt, c.max_ldS,
+                                    std::min(g->n_items, c.n_sm * (512 / nt)), s);
+}
+
+// The whole call in one form on stream s.  Every branch that was forked is joined, also
+// after an error.
+static fc2d_status launch(fc2d_group_s* g, const Call& c, bool persistent, cudaStream_t s) {
+  const int n = (int)g->plans.size();
+  fc2d_status st = cuda_check(cudaEventRecord(g->fork, s), "fc2d_group: fork");
+  if (!st && persistent) {
+    st = queue(g, c, g->nt, s);
+    if (!st) st = cuda_check(cudaEventRecord(g->fork_dft, s), "fc2d_group: fork");
+  }
+  for (int i = 0; i < n && !st; ++i) {
+    const bool q = persistent && c.fused[i];
+    st = cuda_check(cudaStreamWaitEvent(g->branch[i], q ? g->fork_dft : g->fork, 0), "fc2d_group: fork");
+    if (st) break;
+    st = q ? extend_coeffs_dft(g->plans[i], c.n_f[i], c.fg[i], c.fhat[i], g->branch[i])
+           : fc2d_extend_coeffs(g->plans[i], c.n_f[i], c.fg[i], c.bdry(i), c.fhat[i], g->branch[i]);
+    const cudaError_t e0 = cudaEventRecord(g->join[i], g->branch[i]);
+    const cudaError_t e1 = cudaStreamWaitEvent(s, g->join[i], 0);
+    if (!st && (e0 != cudaSuccess || e1 != cudaSuccess))
+      st = set_error(FC2D_ERR_CUDA, "fc2d_group: join failed");
+  }
+  return st;
+}
+
+// Mean microseconds of `reps` runs of `run` on stream s after one warm-up.
+template <typename F>
+static fc2d_status time_runs(cudaStream_t s, int reps, float* us, F run) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   float ms = -1.f;
+  fc2d_status st = FC2D_OK;
   if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) {
-    cudaGraphLaunch(exec, g->cap);
-    cudaEventRecord(e0, g->cap);
-    for (int r = 0; r < 3; ++r) cudaGraphLaunch(exec, g->cap);
-    cudaEventRecord(e1, g->cap);
+    for (int r = 0; r <= reps && !st; ++r) {
+      if (r == 1) cudaEventRecord(e0, s);
+      st = run();
+    }
+    cudaEventRecord(e1, s);
     if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
-  return ms < 0.f ? -1.f : 1e3f * ms / 3;
+  *us = ms < 0.f ? 0.f : 1e3f * ms / reps;
+  return st || ms >= 0.f ? st : set_error(FC2D_ERR_CUDA, "fc2d_group: tuning launch failed");
 }
 
-// Capture the group call into g->graph / g->exec.  With mixed-form members both forms
-// are captured and timed on the call's inputs, and the faster is kept (the plan-group
-// autotuner; the persistent kernel's CTA shape is tuned first).
-static fc2d_status capture(fc2d_group_s* g, const int* n_f, const double* const* fg,
-                           const double* const* fb, void* const* fhat) {
+// For a new set of function counts: the work items of the mixed-form members, longest
+// first, and the choice of the form (with mixed-form members the persistent kernel's CTA
+// shape, 256 threads two per SM or 512 one per SM, then both forms, timed on the call's
+// inputs).
+static fc2d_status tune(fc2d_group_s* g, const Call& c) {
   const int n = (int)g->plans.size();
-  for (int i = 0; i < n; ++i) {
-    // workspace first: no allocation may happen while the graph is being captured
-    fc2d_status st = ensure_plan_workspace(g->plans[i], n_f[i]);
-    if (st) return st;
-    st = extend_coeffs_check(g->plans[i], n_f[i], fg[i], fb ? fb[i] : nullptr, fhat[i]);
-    if (st) return st;
-  }
-  // the work items of the mixed-form members, longest first
-  const size_t rec = gi_work_bytes();
-  std::vector<char> fused(n, 0);
-  std::vector<unsigned char> work;
+  g->tuned_nf.clear();
   std::vector<int4> items;
   std::vector<int64_t> cost;
-  int n_fused = 0, max_ldS = 0, n_sm = 1;
-  for (int i = 0; i < n; ++i) {
-    fc2d_plan_s* p = g->plans[i];
-    if (!group_fused(p)) continue;
-    std::vector<int32_t> pts;
-    const GiPlanArgs a = group_fused_args(p, n_f[i], fg[i], fb ? fb[i] : nullptr, &pts);
-    work.resize((size_t)(n_fused + 1) * rec);
-    int ld = 0;
-    fc2d_status st = gi_work_fill(a, work.data() + (size_t)n_fused * rec, &ld);
-    if (st) return st;
-    max_ldS = std::max(max_ldS, ld);
-    n_sm = std::max(n_sm, p->n_sm);
-    for (int c = 0; c < (int)pts.size(); ++c)
-      for (int f = 0; f < n_f[i]; ++f) {
-        items.push_back(make_int4(n_fused, c, f, 0));
-        cost.push_back(pts[c] + kItemFixed);
+  for (int i = 0, k = 0; i < n; ++i) {
+    if (!c.fused[i]) continue;
+    for (int r = 0; r < (int)c.points[k].size(); ++r)
+      for (int f = 0; f < c.n_f[i]; ++f) {
+        items.push_back(make_int4(k, r, f, 0));
+        cost.push_back(c.points[k][r] + kItemFixed);
       }
-    fused[i] = 1;
-    ++n_fused;
+    ++k;
   }
-  const int n_items = (int)items.size();
-  // a replay of the previous graph may still be reading the old records, and the
-  // tuning launches below write the plans' workspaces and outputs: let earlier work
-  // finish
-  cudaDeviceSynchronize();
-  if (g->exec) {
-    cudaGraphExecDestroy(g->exec);
-    g->exec = nullptr;
-  }
-  if (g->graph) {
-    cudaGraphDestroy(g->graph);
-    g->graph = nullptr;
-  }
+  // the previous call may still be reading the old items, and the tuning launches below
+  // write the plans' workspaces and outputs: let earlier work finish
+  fc2d_status st = cuda_check(cudaDeviceSynchronize(), "fc2d_group: synchronise");
+  if (st) return st;
+  g->n_items = (int)items.size();
   g->nt = 0;
   g->persistent = 0;
   for (float& u : g->tune_us) u = 0.f;
-  if (n_items) {
-    std::vector<int> order(n_items);
+  if (g->n_items) {
+    std::vector<int> order(items.size());
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
-    std::vector<int4> sorted(n_items);
-    for (int k = 0; k < n_items; ++k) sorted[k] = items[order[k]];
-    fc2d_status st = grow(&g->work, &g->work_cap, work.size());
-    if (!st) st = grow(reinterpret_cast<void**>(&g->items), &g->items_cap, sorted.size() * sizeof(int4));
-    if (st) return st;
-    if (cudaMemcpy(g->work, work.data(), work.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(g->items, sorted.data(), sorted.size() * sizeof(int4), cudaMemcpyHostToDevice) !=
-            cudaSuccess)
+    std::vector<int4> sorted(items.size());
+    for (size_t k = 0; k < items.size(); ++k) sorted[k] = items[order[k]];
+    if ((st = grow(&g->work, &g->work_cap, c.work.size())) ||
+        (st = grow(reinterpret_cast<void**>(&g->items), &g->items_cap, sorted.size() * sizeof(int4))))
+      return st;
+    if (cudaMemcpy(g->items, sorted.data(), sorted.size() * sizeof(int4), cudaMemcpyHostToDevice) !=
+        cudaSuccess)
       return set_error(FC2D_ERR_CUDA, "fc2d_group: work upload failed");
-    if (g->forced_form >= 0) g->nt = g->forced_nt;
-    else if ((st = tune_queue(g, n_items, max_ldS, n_sm))) return st;
-  }
-  cudaGraph_t graphs[2] = {nullptr, nullptr};
-  cudaGraphExec_t execs[2] = {nullptr, nullptr};
-  fc2d_status st = FC2D_OK;
-  // the forms to capture: both when tuning, the set one otherwise (branches only
-  // without mixed-form members)
-  const int first = (n_items && g->forced_form == 1) ? 1 : 0;
-  const int last = (n_items && g->forced_form != 0) ? 1 : 0;
-  for (int form = first; form <= last && !st; ++form) {
-    st = capture_form(g, form == 1, fused, n_items, max_ldS, n_sm, n_f, fg, fb, fhat, &graphs[form]);
-    if (!st && cudaGraphInstantiate(&execs[form], graphs[form], 0) != cudaSuccess) {
-      execs[form] = nullptr;
-      st = set_error(FC2D_ERR_CUDA, "fc2d_group: graph instantiation failed");
+    if (g->forced_form >= 0) {
+      g->nt = g->forced_nt;
+      g->persistent = g->forced_form;
+    } else {
+      for (int k = 0; k < 2 && !st; ++k)
+        st = time_runs(g->cap, 3, &g->tune_us[k], [&] { return queue(g, c, k ? 512 : 256, g->cap); });
+      g->nt = g->tune_us[0] <= g->tune_us[1] ? 256 : 512;
+      for (int k = 0; k < 2 && !st; ++k)
+        st = time_runs(g->cap, 3, &g->tune_us[2 + k], [&] { return launch(g, c, k == 1, g->cap); });
+      g->persistent = g->tune_us[3] < g->tune_us[2] ? 1 : 0;
+      if (st) return st;
     }
   }
-  int keep = first;
-  if (!st && first != last) {
-    g->tune_us[2] = time_graph(g, execs[0]);
-    g->tune_us[3] = time_graph(g, execs[1]);
-    if (g->tune_us[2] < 0.f || g->tune_us[3] < 0.f)
-      st = set_error(FC2D_ERR_CUDA, "fc2d_group: tuning launch failed");
-    keep = g->tune_us[3] < g->tune_us[2] ? 1 : 0;
-  }
-  for (int form = 0; form < 2; ++form) {
-    if (!st && form == keep) continue;
-    if (execs[form]) cudaGraphExecDestroy(execs[form]);
-    if (graphs[form]) cudaGraphDestroy(graphs[form]);
-  }
-  if (st) return st;
-  g->graph = graphs[keep];
-  g->exec = execs[keep];
-  g->persistent = keep;
+  g->tuned_nf.assign(c.n_f, c.n_f + n);
   return FC2D_OK;
+}
+
+// Capture the call into g->graph / g->exec.
+static fc2d_status capture(fc2d_group_s* g, const Call& c) {
+  // a replay of the previous graph may still be running
+  fc2d_status st = cuda_check(cudaDeviceSynchronize(), "fc2d_group: synchronise");
+  if (st) return st;
+  drop_graph(g);
+  if (cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+    return set_error(FC2D_ERR_CUDA, "fc2d_group: stream capture failed to start");
+  st = launch(g, c, g->persistent != 0, g->cap);
+  const cudaError_t e = cudaStreamEndCapture(g->cap, &g->graph);
+  if (!st && (e != cudaSuccess || !g->graph))
+    st = set_error(FC2D_ERR_CUDA, "fc2d_group: stream capture failed");
+  if (!st && cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess) {
+    g->exec = nullptr;
+    st = set_error(FC2D_ERR_CUDA, "fc2d_group: graph instantiation failed");
+  }
+  if (st) drop_graph(g);
+  return st;
 }
 
 extern "C" fc2d_status fc2d_group_extend_coeffs(fc2d_group_t g, const int* n_f,
@@ -338,13 +321,26 @@ extern "C" fc2d_status fc2d_group_extend_coeffs(fc2d_group_t g, const int* n_f,
     kptr.push_back(g->plans[i]->ws.base);
     kptr.push_back(reinterpret_cast<const void*>(g->plans[i]->ws.bytes));
   }
-  if (!g->exec || knf != g->key_nf || kptr != g->key_ptr) {
-    g->key_nf.clear();
-    g->key_ptr.clear();
-    fc2d_status st = capture(g, n_f, f_grid_dev, f_bdry_dev, fhat_dev);
+  if (!g->exec || knf != g->graph_nf || kptr != g->graph_ptr) {
+    Call c{n_f, f_grid_dev, f_bdry_dev, fhat_dev};
+    fc2d_status st = describe(g, c);
+    if (!st && knf != g->tuned_nf) st = tune(g, c);
     if (st) return st;
-    g->key_nf = knf;
-    g->key_ptr = kptr;
+    bool again = knf == g->key_nf && kptr == g->key_ptr;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (again && (cudaStreamIsCapturing((cudaStream_t)stream, &capturing) != cudaSuccess ||
+                  capturing != cudaStreamCaptureStatusNone)) {
+      cudaGetLastError();
+      again = false;  // the caller is capturing: its graph takes the kernels themselves
+    }
+    if (!again) {
+      g->key_nf = knf;
+      g->key_ptr = kptr;
+      return launch(g, c, g->persistent != 0, (cudaStream_t)stream);
+    }
+    if ((st = capture(g, c))) return st;
+    g->graph_nf = knf;
+    g->graph_ptr = kptr;
   }
   if (cudaGraphLaunch(g->exec, (cudaStream_t)stream) != cudaSuccess)
     return set_error(FC2D_ERR_CUDA, "fc2d_group: graph launch failed");
@@ -357,8 +353,9 @@ extern "C" fc2d_status fc2d_group_tuning_set(fc2d_group_t g, const int32_t* choi
     return set_error(FC2D_ERR_ARG, "fc2d_group_tuning_set: form 0 or 1, 256 or 512 threads");
   g->forced_form = choice ? choice[0] : -1;
   g->forced_nt = choice ? choice[1] : 0;
-  g->key_nf.clear();  // the next call captures anew
-  g->key_ptr.clear();
+  g->tuned_nf.clear();  // the next call tunes anew
+  g->key_nf.clear();
+  g->graph_nf.clear();
   return FC2D_OK;
 }
 

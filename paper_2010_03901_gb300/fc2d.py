@@ -336,8 +336,8 @@ def fc2d_plan(boundary, grid, params=None, precision=FC2D_FP64) -> Plan:
 
 
 class Group:
-    """A plan group: the extension + DFT of several domains as one CUDA graph, each plan
-    on its own branch (fc2d_group_create).  Keeps references to its plans."""
+    """A plan group: the extension + DFT of several domains in one call, each plan on a
+    stream of its own (fc2d_group_create).  Keeps references to its plans."""
 
     def __init__(self, plans):
         self.plans = list(plans)
@@ -366,8 +366,8 @@ class Group:
                 dict(zip(("queue256", "queue512", "branches", "persistent"), us)))
 
     def fc2d_group_tuning_set(self, form=None, threads=256):
-        """Fix the captured form ("persistent" or "branches") and the persistent kernel's
-        threads per CTA for later captures; form None: tune again."""
+        """Fix the form ("persistent" or "branches") and the persistent kernel's
+        threads per CTA for later calls; form None: tune again."""
         if form is None:
             _check(_lib.fc2d_group_tuning_set(self.handle, None))
         else:

@@ -1,0 +1,49 @@
+"""Plan-group calls with changing arguments: direct launches, the capture of a repeated
+call, replays of an older graph's arguments, changed function counts and boundary data, in
+both forms, equal to separate calls bit for bit."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("form", ["branches", "persistent"])
+def test_calls_in_any_order(form, precision):
+    torch = pytest.importorskip("torch")
+    from paper_2010_03901_gb300 import fc2d
+    prec = fc2d.FC2D_FP64 if precision == "fp64" else fc2d.FC2D_MIXED
+    out_t = torch.float64 if precision == "fp64" else torch.float32
+    names = ["disk64", "star200", "kite160x144"]
+    plans = []
+    for name in names * 3:  # nine records: more than one launch of the persistent form's
+        w = W.workload(name)
+        g, p = w.grid, w.params
+        plans.append(fc2d.fc2d_plan(w.boundary.arrays(), (g.a0, g.b0, g.h, g.nx, g.ny),
+                                    dict(B=p.B, k1=p.k1), precision=prec))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+
+    def fields(n_f):
+        rnd = lambda *s: torch.randn(s, dtype=torch.float64, device="cuda", generator=gen)  # noqa: E731
+        return (n_f, [rnd(n, p.ny, p.nx) for n, p in zip(n_f, plans)],
+                [rnd(n, p.n_bdry) for n, p in zip(n_f, plans)])
+
+    sets = [fields([1] * 9), fields([1] * 9), fields([1, 2, 3] * 3)]
+    outs = [[torch.zeros((n, p.ny, p.nx // 2 + 1, 2), dtype=out_t, device="cuda")
+             for n, p in zip(s[0], plans)] for s in sets]
+    grp = fc2d.fc2d_group_create(plans)
+    grp.fc2d_group_tuning_set(form, 256)
+    for k, bdry in [(0, True), (1, True), (0, True), (0, True), (0, True), (1, True), (0, True),
+                    (2, True), (2, False), (2, False), (0, True), (0, True)]:
+        n_f, f, b = sets[k]
+        b = b if bdry else None
+        for o in outs[k]:
+            o.fill_(7.0)
+        grp.fc2d_group_extend_coeffs(n_f, f, b, outs[k])
+        for i, p in enumerate(plans):
+            ref = torch.zeros_like(outs[k][i])
+            p.fc2d_extend_coeffs(n_f[i], f[i], b[i] if bdry else None, ref)
+            assert torch.equal(ref, outs[k][i]), (k, bdry, i)
+    grp.fc2d_group_destroy()
