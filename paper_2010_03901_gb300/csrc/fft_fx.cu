@@ -32,8 +32,14 @@ template <int LOGNH> __host__ __device__ constexpr int row_threads() {
   return (1 << LOGNH) / 8 < 32 ? 32 : (1 << LOGNH) / 8;
 }
 
+// resident blocks asked of the compiler: 64 registers per thread, within shared memory
+__host__ __device__ constexpr int blocks_for(int threads, int bytes) {
+  const int r = 1024 / threads, m = 220 * 1024 / (bytes + 1024);
+  return r < m ? (r < 1 ? 1 : r) : (m < 1 ? 1 : m);
+}
+
 template <int LOGNH>
-__global__ void __launch_bounds__(row_threads<LOGNH>())
+__global__ void __launch_bounds__(row_threads<LOGNH>(), blocks_for(row_threads<LOGNH>(), 16 * padded(1 << LOGNH)))
 k_rows_fx(FftArgs fa, RowArgs ra, int mode, const double* __restrict__ ext,
           const double* __restrict__ f_grid, const double* __restrict__ vals,
           double2* __restrict__ inter) {
@@ -75,7 +81,7 @@ k_rows_fx(FftArgs fa, RowArgs ra, int mode, const double* __restrict__ ext,
 }
 
 template <int LOGNY, int CB>
-__global__ void __launch_bounds__(CB * (1 << LOGNY) / 8)
+__global__ void __launch_bounds__(CB * (1 << LOGNY) / 8, blocks_for(CB * (1 << LOGNY) / 8, 16 * CB * padded(1 << LOGNY)))
 k_cols_fx(FftArgs fa, const double2* __restrict__ inter, double2* __restrict__ fhat) {
   constexpr int N = 1 << LOGNY, NT = N / 8, R = last_radix<LOGNY>();
   extern __shared__ __align__(16) unsigned char smem_raw[];

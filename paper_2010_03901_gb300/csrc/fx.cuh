@@ -43,7 +43,15 @@ __device__ __forceinline__ c64 mul_mi(c64 a) { return {a.y, -a.x}; }  // -i a
 __device__ __forceinline__ int lo32(i64 v) { return (int)v; }
 __device__ __forceinline__ int hi32(i64 v) { return (int)((unsigned)(v >> 32) + ((unsigned)v >> 31)); }
 
-__device__ __forceinline__ i64 mad(int a, int b, i64 c) { return (i64)a * b + c; }
+__device__ __forceinline__ i64 mad(int a, int b, i64 c) {  // one instruction
+  i64 d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+// c + (v >> 32) as one multiply-add by a 1 that the compiler cannot see (a shift, a sign
+// word and a 64-bit addition otherwise)
+__constant__ int kOne = 1;
+__device__ __forceinline__ i64 add_high(i64 v, i64 c) { return mad((int)(v >> 32), kOne, c); }
 
 // a w 2^-kDrop for |a.x|, |a.y| <= 2^62.5: the products of the high limbs, plus the mixed
 // products rounded at bit 32 (each sum of mixed products stays below 2^63); the products
@@ -54,14 +62,14 @@ __device__ __forceinline__ c64 mulw(c64 a, int4 w) {
   const int nh = -w.z, nl = -w.w;  // limbs are never -2^31
   const i64 mx = mad(xh, w.y, mad(xl, w.x, mad(yh, nl, mad(yl, nh, half))));
   const i64 my = mad(xh, w.w, mad(xl, w.z, mad(yh, w.y, mad(yl, w.x, half))));
-  return {mad(xh, w.x, mad(yh, nh, mx >> 32)), mad(xh, w.z, mad(yh, w.x, my >> 32))};
+  return {mad(xh, w.x, mad(yh, nh, add_high(mx, 0))), mad(xh, w.z, mad(yh, w.x, add_high(my, 0)))};
 }
 
 // v c for a constant c in [1/2, 1) given as c - 1 = m 2^-32 + r 2^-64 (|v| < 2^62.5)
 __device__ __forceinline__ i64 mulc(i64 v, int m, int r) {
   const int h = hi32(v), l = lo32(v);
   const i64 t = mad(l, m, mad(h, r, i64(1) << 31));
-  return mad(h, m, v) + (t >> 32);
+  return add_high(t, mad(h, m, v));
 }
 // sqrt(1/2) - 1 = kRtM 2^-32 + kRtR 2^-64
 constexpr int kRtM = -1257966796;
@@ -83,13 +91,24 @@ __device__ __forceinline__ unsigned magnitude(double d) {
 }
 // x in units of 2^(E - 1080), E the block's largest biased exponent (at least 1): the
 // 53-bit significand shifted to |v| < 2^58 for exponent E, right by E - e bits for others
+__device__ __forceinline__ i64 shift_right(i64 v, int n) {  // n >= 0; 0 from 64 on (v >= 0)
+  i64 r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
 __device__ __forceinline__ i64 from_double(double d, int E) {
   const unsigned hi = (unsigned)__double2hiint(d);
   const int e = (int)(hi >> 20) & 0x7FF;
+  if (E > 64) {  // a subnormal or zero (e = 0) shifts out
+    const unsigned mh = (hi & 0xFFFFFu) | 0x100000u;
+    const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
+    const i64 v = shift_right(m, E - e);
+    const i64 s = (i64)((int)hi >> 31);
+    return (v ^ s) - s;
+  }
   const unsigned mh = (hi & 0xFFFFFu) | (e ? 0x100000u : 0u);
   const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
-  const int sh = E - max(e, 1);
-  const i64 v = sh < 63 ? m >> sh : 0;
+  const i64 v = shift_right(m, E - max(e, 1));
   const i64 s = (i64)((int)hi >> 31);
   return (v ^ s) - s;
 }
@@ -102,21 +121,13 @@ __device__ __forceinline__ int block_exp(unsigned mag) { return max((int)(mag >>
 // Whether every nonzero v with unit 2^e becomes a normal double (or overflows to infinity
 // by its exponent field): the same for a whole block.
 __device__ __forceinline__ bool plain_exp(int e) { return e + 1086 - 63 >= 1 && e + 1086 <= 2046; }
-// v 2^e as a double, rounded to nearest (ties away from zero): normalise, round at bit 11,
-// assemble
-__device__ __forceinline__ double plain_double(i64 v, int e) {
-  const i64 s = v >> 63;
-  const unsigned long long a = (unsigned long long)((v ^ s) - s);
-  const int n = __clzll((i64)a);
-  const unsigned long long m = a << (n & 63);
-  const unsigned long long q = (m >> 11) + ((m >> 10) & 1);
-  const unsigned long long b = q + ((unsigned long long)(unsigned)(e + 1085 - n) << 52);
-  const unsigned long long sg = (unsigned long long)s & 0x8000000000000000ull;
-  return a ? __longlong_as_double((i64)(b | sg)) : 0.0;
-}
+// v 2^e as a double, rounded to nearest: the conversion instruction (2 per clock and SM, on
+// the FP64 pipe that is idle otherwise; the same in integer operations takes 24) and an
+// addition to the exponent field
 __device__ __forceinline__ double to_double(i64 v, int e, bool plain) {
-  if (plain) return plain_double(v, e);
-  return e > kNaN / 2 ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(plain_double(v, 0), e);
+  const double x = __ll2double_rn(v);
+  if (plain) return __hiloint2double(__double2hiint(x) + (v ? e << 20 : 0), __double2loint(x));
+  return e > kNaN / 2 ? __longlong_as_double(0x7FF8000000000000ll) : scalbn(x, e);
 }
 __device__ __forceinline__ double2 to_double(c64 v, int e, bool plain) {
   return {to_double(v.x, e, plain), to_double(v.y, e, plain)};
@@ -202,19 +213,28 @@ template <int LOGN> __host__ __device__ constexpr int last_ns() {
 
 // Rescale and twiddle the eight inputs of a stage after the first: the first value of each
 // butterfly by a shift, the others by their twiddles (tw[r NS + k]); radix-R DFTs.
-template <int R, int NS, int NT>
+template <int R, int NS, int NT, bool SHIFT>
 __device__ __forceinline__ void butterflies(c64 (&v)[8], int t, const int4* __restrict__ tw, int L) {
 #pragma unroll
   for (int m = 0; m < 8 / R; ++m) {
     const int k = (t + m * NT) & (NS - 1);
     c64* a = v + m * R;
     const i64 rnd = 1 << (kDrop - 1);
-    a[0] = {((a[0].x << L) + rnd) >> kDrop, ((a[0].y << L) + rnd) >> kDrop};
+    if constexpr (SHIFT) {
 #pragma unroll
-    for (int r = 1; r < R; ++r) a[r] = mulw(c64{a[r].x << L, a[r].y << L}, __ldg(tw + r * NS + k));
+      for (int r = 0; r < R; ++r) a[r] = {a[r].x << L, a[r].y << L};
+    }
+    a[0] = {(a[0].x + rnd) >> kDrop, (a[0].y + rnd) >> kDrop};
+#pragma unroll
+    for (int r = 1; r < R; ++r) a[r] = mulw(a[r], __ldg(tw + r * NS + k));
     dft<R>(a);
   }
 }
+
+// Whether the block is rescaled before stage k + 1 (k = 1, 2, ..): every other stage.  A
+// stage that is not preceded by a shift works on values that lost at most the 3.5 bits of
+// headroom of the stage before.
+__host__ __device__ constexpr bool shifts(int k) { return k % 2 == 0; }
 
 // All stages but the first.  buf holds the outputs of the stage before (sub-length NS),
 // st[SLOT] their spread.  On return v holds the thread's last-stage outputs (value r of
@@ -224,7 +244,7 @@ __device__ __forceinline__ void rest(c64 (&v)[8], c64* buf, int t, bool active, 
                                      const int4* __restrict__ tw, int& e) {
   constexpr int N = 1 << LOGN, NT = N / 8;
   constexpr int R = N / NS >= 8 ? 8 : N / NS, NR = N / R, M = 8 / R;
-  const int L = headroom(st[SLOT]);
+  const int L = shifts(SLOT) ? headroom(st[SLOT]) : 0;
   e += kDrop - L;
   if (active) {
 #pragma unroll
@@ -242,7 +262,7 @@ __device__ __forceinline__ void rest(c64 (&v)[8], c64* buf, int t, bool active, 
   if constexpr (NS * R < N) __syncthreads();
   unsigned h = 0;
   if (active) {
-    butterflies<R, NS, NT>(v, t, tw + stage_off(N, NS), L);
+    butterflies<R, NS, NT, shifts(SLOT)>(v, t, tw + stage_off(N, NS), L);
     if constexpr (NS * R < N) {  // R = 8
       const int k = t & (NS - 1);
       const int base = (t / NS) * NS * R + k;
@@ -250,12 +270,12 @@ __device__ __forceinline__ void rest(c64 (&v)[8], c64* buf, int t, bool active, 
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         dst[r * step<NS>()] = v[r];
-        h |= spread(v[r]);
+        if (shifts(SLOT + 1)) h |= spread(v[r]);
       }
     }
   }
   if constexpr (NS * R < N) {
-    block_or(h, st + SLOT + 1);
+    if constexpr (shifts(SLOT + 1)) block_or(h, st + SLOT + 1);
     __syncthreads();
     rest<LOGN, NS * R, SLOT + 1>(v, buf, t, active, st, tw, e);
   }
@@ -293,10 +313,10 @@ __device__ __forceinline__ void transform(const double2 (&u)[8], c64 (&v)[8], c6
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       dst[r] = v[r];
-      h |= spread(v[r]);
+      if (shifts(1)) h |= spread(v[r]);
     }
   }
-  block_or(h, st + 1);
+  if constexpr (shifts(1)) block_or(h, st + 1);
   __syncthreads();
   rest<LOGN, 8, 1>(v, buf, t, active, st, tw, e);
   if (E >= 0x7FF) e = kNaN;
