@@ -36,8 +36,8 @@ namespace {
 size_t al(size_t b) { return (b + 255) / 256 * 256; }
 
 struct Layout {
-  size_t F, vals, inter, coef, bvals, total;
-  size_t oF, ovals, ointer, ocoef, obvals;
+  size_t F, vals, inter, coef, bvals, exps, total;
+  size_t oF, ovals, ointer, ocoef, obvals, oexps;
 };
 
 // Row length of the strip values F in workspace: Cr + 1 for FP64; for the mixed form
@@ -60,7 +60,9 @@ Layout layout(const fc2d_plan_s* p, int n_f) {
   L.ointer = L.ovals + L.vals;
   L.ocoef = L.ointer + L.inter;
   L.obvals = L.ocoef + L.coef;
-  L.total = L.obvals + L.bvals;
+  L.oexps = L.obvals + L.bvals;
+  L.exps = p->prm.precision == FC2D_FP64 ? al(fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int)) : 0;
+  L.total = L.oexps + L.exps;
   return L;
 }
 
@@ -159,6 +161,8 @@ FftArgs fft_args(fc2d_plan_s* p) {
   a.tsy = f64 ? (const void*)p->fy.tws64 : (const void*)p->fy.tws32;
   a.fxx = reinterpret_cast<const int4*>(p->fx.fxs);
   a.fxy = reinterpret_cast<const int4*>(p->fy.fxs);
+  a.fxwx = reinterpret_cast<const int4*>(p->fx.fx);
+  a.fxwy = reinterpret_cast<const int4*>(p->fy.fx);
   a.fxr = reinterpret_cast<const int4*>(p->rfx);
   a.fxs = fx_reciprocal((int64_t)p->grid.nx * p->grid.ny);
   a.scale = 1.0 / ((double)p->grid.nx * p->grid.ny);
@@ -344,6 +348,7 @@ extern "C" fc2d_status fc2d_coeffs(fc2d_plan_t p, int n_f, const void* ext, void
   }
   {
     ProfScope ps(p, "fft_cols", s);
+    fa.exps = reinterpret_cast<int*>(ws(p, L.oexps));
     launch_fft_cols(fa, n_f, f64, ws(p, L.ointer), fhat, s);
   }
   return launched("fc2d_coeffs");
@@ -374,6 +379,7 @@ fc2d_status extend_coeffs_dft(fc2d_plan_s* p, int n_f, const double* fg, void* f
   }
   {
     ProfScope ps(p, "fft_cols", s);
+    fa.exps = reinterpret_cast<int*>(ws(p, L.oexps));
     launch_fft_cols(fa, n_f, f64, ws(p, L.ointer), fhat, s);
   }
   return launched("fc2d_extend_coeffs");
@@ -434,6 +440,7 @@ extern "C" fc2d_status fc2d_extend_coeffs_complex(fc2d_plan_t p, int n_f, const 
   }
   {
     ProfScope ps(p, "fft_cols", s);
+    fa.exps = reinterpret_cast<int*>(ws(p, L.oexps));
     launch_fft_cols(fa, n2, f64, ws(p, L.ointer), ws(p, ohalf), s);
   }
   {
@@ -477,6 +484,7 @@ extern "C" fc2d_status fc2d_extend_coeffs_compact(fc2d_plan_t p, int n_f, const 
   }
   {
     ProfScope ps(p, "fft_cols", s);
+    fa.exps = reinterpret_cast<int*>(ws(p, L.oexps));
     launch_fft_cols(fa, n_f, f64, ws(p, L.ointer), fhat, s);
   }
   return launched("fc2d_extend_coeffs_compact");
@@ -759,6 +767,7 @@ fc2d_status wave_spectra(fc2d_plan_s* p, int n_f, const double* u, const double*
   }
   {
     ProfScope ps(p, "fft_cols", s);
+    fa.exps = reinterpret_cast<int*>(ws(p, L.oexps));
     launch_fft_cols(fa, 2 * n_f, true, ws(p, L.ointer), spec, s);
   }
   return launched("wave spectra");

@@ -168,6 +168,8 @@ struct FftArgs {
   const void* tsy;            // per-stage twiddles of the column transform
   // double plans (fx.cuh): twiddles w 2^60 in 32-bit limbs (re hi, lo, im hi, lo)
   const int4 *fxx, *fxy;      // per stage of the row and column transforms (powers of two)
+  const int4 *fxwx, *fxwy;    // w^t of both lengths
+  int* exps;                  // two-pass columns: pass A's exponents (fx_exps ints)
   const int4* fxr;            // exp(-2 pi i k/nx), k <= nx/2
   FxFactor fxs;               // 1/(nx ny)
   double scale;               // 1/(nx ny)
@@ -175,6 +177,9 @@ struct FftArgs {
   int cols_tma;               // 1: those passes in the TMA-pipelined persistent form
   int* status;                // device status word (bounded waits record a timeout)
 };
+
+// ints of FftArgs::exps for n_f functions (one per 16 columns and residue of the rows)
+inline size_t fx_exps(int nx, int ny, int n_f) { return (size_t)n_f * (ny / 64 + 1) * (nx / 32 + 1); }
 
 // rows: mode 0 reads an extended grid (ext, type T); mode 1 assembles the extension
 // on the fly from f_grid + strip values; mode 2 likewise from f given at the inside

@@ -97,7 +97,7 @@ bool launch_fft_cols_64n(const FftArgs& fa, int n_f, bool fp64, void* inter, voi
 
 bool launch_fft_rows_fx(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
                         const double* f_grid, const void* vals, void* inter, cudaStream_t s);
-bool launch_fft_cols_fx(const FftArgs& fa, int n_f, const void* inter, void* fhat, cudaStream_t s);
+bool launch_fft_cols_fx(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
 
 void launch_fft_rows(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
                      const void* ext, const double* f_grid, const void* vals, void* inter,

@@ -17,12 +17,11 @@
 namespace fc2d {
 namespace fx {
 
-// X_k and X_{NH-k} (times 2^(kDrop+1), in the block's units) of a real row from its pairs'
-// transform: with zk = Z_k and zl = Z_{NH-k}, e = (zk + conj zl)/2, o = (zk - conj zl)/2,
+// X_k and X_{NH-k} (times 2^(1-kDrop), in the block's units) of a real row from its pairs'
+// transform (|z| <= 2^61.5): with zk = Z_k and zl = Z_{NH-k}, e = (zk + conj zl)/2, o = (zk - conj zl)/2,
 // X_k = e - i w^k o, X_{NH-k} = conj(e + i w^k o)
 __device__ __forceinline__ void split_pair(c64 zk, c64 zl, int4 w, c64& xk, c64& xl) {
-  const i64 rnd = 1 << (kDrop - 1);
-  const c64 e = {(zk.x + zl.x + rnd) >> kDrop, (zk.y - zl.y + rnd) >> kDrop};
+  const c64 e = drop(c64{zk.x + zl.x, zk.y - zl.y});
   const c64 wo = mulw(c64{zk.x - zl.x, zk.y + zl.y}, w);
   xk = {e.x + wo.y, e.y - wo.x};
   xl = {e.x - wo.y, -e.y - wo.x};
@@ -61,20 +60,27 @@ k_rows_fx(FftArgs fa, RowArgs ra, int mode, const double* __restrict__ ext,
   int e;
   transform<LOGNH>(u, v, buf, t, active, st, fa.fxx, e);
   __syncthreads();
+  unsigned h = 0;
   if (active) {
     constexpr int R = last_radix<LOGNH>();
 #pragma unroll
     for (int m = 0; m < 8 / R; ++m)
 #pragma unroll
-      for (int r = 0; r < R; ++r) buf[pad(out_index<LOGNH>(t, m, r))] = v[m * R + r];
+      for (int r = 0; r < R; ++r) {
+        buf[pad(out_index<LOGNH>(t, m, r))] = v[m * R + r];
+        h |= spread(v[m * R + r]);
+      }
   }
+  block_or(h, st + kSlots - 1);
   __syncthreads();
-  e += kDrop - 1;
+  const int L = max(headroom(st[kSlots - 1]) - 1, 0);  // |z| <= 2^61
+  e += kDrop - 1 - L;
   const bool plain = plain_exp(e);
   double2* out = inter + ((size_t)f * fa.ny + j) * fa.pitch;
   for (int k = t; k <= NH / 2; k += row_threads<LOGNH>()) {
     c64 xk, xl;
-    split_pair(buf[pad(k)], buf[pad(k ? NH - k : 0)], __ldg(fa.fxr + k), xk, xl);
+    const c64 zk = buf[pad(k)], zl = buf[pad(k ? NH - k : 0)];
+    split_pair(c64{zk.x << L, zk.y << L}, c64{zl.x << L, zl.y << L}, __ldg(fa.fxr + k), xk, xl);
     out[k] = to_double(xk, e, plain);
     if (k != NH - k) out[NH - k] = to_double(xl, e, plain);
   }
@@ -119,6 +125,66 @@ k_cols_fx(FftArgs fa, const double2* __restrict__ inter, double2* __restrict__ f
   }
 }
 
+// The two passes of columns of 64 N2 points from the row pass's intermediate (whose rows
+// pass A overwrites with its integers) to the spectrum.
+template <int N2>
+__global__ void __launch_bounds__(kColThreads, 8)
+k_cols2_a(FftArgs fa, double2* __restrict__ inter, int* __restrict__ exps) {
+  __shared__ c64 ex[64 * kCols];
+  __shared__ unsigned st[1];
+  if (threadIdx.x == 0) st[0] = 0;
+  const int ncol = fa.nx / 2 + 1, kx = blockIdx.x * kCols + (threadIdx.x & (kCols - 1));
+  const int j2 = blockIdx.y, f = blockIdx.z;
+  double2* slab = inter + (size_t)f * (64 * N2) * fa.pitch;
+  const unsigned pitch = fa.pitch;
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  cols_pass_a<N2>([&](int row, int k) { return slab[(unsigned)row * pitch + k]; },
+                  reinterpret_cast<c64*>(slab), pitch, j2, kx, kx < ncol, ex, st, fa.fxwy,
+                  exps + ((size_t)f * N2 + j2) * gridDim.x + blockIdx.x);
+}
+
+template <int N2>
+__global__ void __launch_bounds__(kColThreads, 8)
+k_cols2_b(FftArgs fa, const double2* __restrict__ inter, const int* __restrict__ exps,
+          double2* __restrict__ fhat) {
+  constexpr int R2 = N2 / 8, G = 8 / R2;  // G values of m1 per block
+  __shared__ c64 ex[64 * kCols];
+  __shared__ unsigned st[1];
+  if (threadIdx.x == 0) st[0] = 0;
+  const int ncol = fa.nx / 2 + 1, c = threadIdx.x & (kCols - 1), kx = blockIdx.x * kCols + c;
+  const int l = (threadIdx.x / kCols) % R2, g = threadIdx.x / (kCols * R2), f = blockIdx.z;
+  const int m1 = blockIdx.y * G + g;
+  const c64* slab = reinterpret_cast<const c64*>(inter) + (size_t)f * (64 * N2) * fa.pitch;
+  const bool live = kx < ncol;
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  c64 v[8];
+  int e = cols_pass_b<N2>(v, slab, fa.pitch, m1, l, kx, live, ex + g * 8 * R2 * kCols, st, fa.fxwy,
+                          exps + (size_t)f * N2 * gridDim.x + blockIdx.x, gridDim.x);
+  e += fa.fxs.exp;
+  const bool plain = plain_exp(e);
+  if (live) {
+    double2* dst = fhat + (size_t)f * (64 * N2) * ncol + kx;
+#pragma unroll
+    for (int mm = 0; mm < 8 / R2; ++mm)
+#pragma unroll
+      for (int q = 0; q < R2; ++q)
+        dst[(unsigned)(m1 + 64 * (l * (8 / R2) + mm + 8 * q)) * (unsigned)ncol] =
+            to_double(scaled(v[mm * R2 + q], fa.fxs), e, plain);
+  }
+}
+
+template <int N2>
+static void cols2_launch(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s) {
+  const int groups = (fa.nx / 2 + kCols) / kCols;
+  launch_pdl(k_cols2_a<N2>, dim3(groups, N2, n_f), dim3(kColThreads), 0, s, fa, (double2*)inter, fa.exps);
+  launch_pdl(k_cols2_b<N2>, dim3(groups, N2, n_f), dim3(kColThreads), 0, s, fa, (const double2*)inter,
+             (const int*)fa.exps, (double2*)fhat);
+}
+
 template <int L>
 static void rows_launch(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
                         const double* fg, const void* vals, void* inter, cudaStream_t s) {
@@ -160,15 +226,15 @@ bool launch_fft_rows_fx(const FftArgs& fa, const RowArgs& ra, int n_f, int mode,
 #undef FC2D_ROWS
 }
 
-bool launch_fft_cols_fx(const FftArgs& fa, int n_f, const void* inter, void* fhat, cudaStream_t s) {
+bool launch_fft_cols_fx(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s) {
   switch (fx::ilog2_exact(fa.ny)) {
     case 6: fx::cols_launch<6, 8>(fa, n_f, inter, fhat, s); return true;
     case 7: fx::cols_launch<7, 8>(fa, n_f, inter, fhat, s); return true;
     case 8: fx::cols_launch<8, 4>(fa, n_f, inter, fhat, s); return true;
     case 9: fx::cols_launch<9, 4>(fa, n_f, inter, fhat, s); return true;
     case 10: fx::cols_launch<10, 2>(fa, n_f, inter, fhat, s); return true;
-    case 11: fx::cols_launch<11, 2>(fa, n_f, inter, fhat, s); return true;
-    case 12: fx::cols_launch<12, 1>(fa, n_f, inter, fhat, s); return true;
+    case 11: fx::cols2_launch<32>(fa, n_f, inter, fhat, s); return true;
+    case 12: fx::cols2_launch<64>(fa, n_f, inter, fhat, s); return true;
     default: return false;
   }
 }

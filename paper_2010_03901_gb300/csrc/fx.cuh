@@ -75,6 +75,14 @@ __device__ __forceinline__ i64 mulc(i64 v, int m, int r) {
 constexpr int kRtM = -1257966796;
 constexpr int kRtR = -102865788;
 
+// v 2^-kDrop, rounded to nearest, ties toward zero.  (Ties are frequent here; rounding them
+// upward would shift a whole block by 1/32 of a unit, which the transform adds up in its
+// zero frequency.  For the same reason the twiddle 1 is stored as 1 - 2^-60.)
+__device__ __forceinline__ i64 drop(i64 v) {
+  return (v + ((1 << (kDrop - 1)) - 1) + (i64)((unsigned long long)v >> 63)) >> kDrop;
+}
+__device__ __forceinline__ c64 drop(c64 v) { return {drop(v.x), drop(v.y)}; }
+
 // bits that differ from their lower neighbour: the top one bounds |v| < 2^(32 + index)
 __device__ __forceinline__ unsigned spread(i64 v) {
   const int h = (int)(v >> 32);
@@ -219,12 +227,11 @@ __device__ __forceinline__ void butterflies(c64 (&v)[8], int t, const int4* __re
   for (int m = 0; m < 8 / R; ++m) {
     const int k = (t + m * NT) & (NS - 1);
     c64* a = v + m * R;
-    const i64 rnd = 1 << (kDrop - 1);
     if constexpr (SHIFT) {
 #pragma unroll
       for (int r = 0; r < R; ++r) a[r] = {a[r].x << L, a[r].y << L};
     }
-    a[0] = {(a[0].x + rnd) >> kDrop, (a[0].y + rnd) >> kDrop};
+    a[0] = drop(a[0]);
 #pragma unroll
     for (int r = 1; r < R; ++r) a[r] = mulw(a[r], __ldg(tw + r * NS + k));
     dft<R>(a);
@@ -320,6 +327,99 @@ __device__ __forceinline__ void transform(const double2 (&u)[8], c64 (&v)[8], c6
   __syncthreads();
   rest<LOGN, 8, 1>(v, buf, t, active, st, tw, e);
   if (E >= 0x7FF) e = kNaN;
+}
+
+// ------------------------------------------------------------------------- //
+// Column transforms of N = 64 N2 points in two passes (the four-step form): with
+// j = N2 j1 + j2 and m = m1 + 64 m2,
+//   pass A: Y[m1][j2] = sum_j1 x[N2 j1 + j2] w_64^(j1 m1), in place of the rows N2 j1 + j2;
+//   pass B: X[m1 + 64 m2] = sum_j2 (Y[m1][j2] w_N^(j2 m1)) w_N2^(j2 m2).
+// A block serves kCols adjacent columns, so a row of a block is a contiguous 256 bytes and
+// the lanes of a warp share their twiddles; eight values per thread.  Pass A leaves
+// integers with one exponent per block (exps[f][j2][column group]); pass B brings its
+// rows to a common exponent, fitted to its own largest value, as it reads them.
+// ------------------------------------------------------------------------- //
+constexpr int kCols = 16;
+constexpr int kColThreads = 128;
+
+// 8 R2-point DFT of v[i] = x[l + R2 i] held by the threads l < R2 of a column; on return
+// v[mm R2 + q] = X[m + 8 q] with m = l (8/R2) + mm.  ex: the group's [8][R2][kCols] exchange
+// buffer; w: w[ws t] = w_{8 R2}^t.  One barrier (none for R2 = 1); adds kDrop to the
+// exponent unless R2 = 1.
+template <int R2>
+__device__ __forceinline__ void dft_group(c64 (&v)[8], int c, int l, c64* ex,
+                                          const int4* __restrict__ w, int ws) {
+  dft<8>(v);
+  if constexpr (R2 > 1) {
+    v[0] = drop(v[0]);
+#pragma unroll
+    for (int m = 1; m < 8; ++m) v[m] = mulw(v[m], __ldg(w + ws * (l * m)));
+#pragma unroll
+    for (int m = 0; m < 8; ++m) ex[(m * R2 + l) * kCols + c] = v[m];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = ex[(l * 8 + k) * kCols + c];
+#pragma unroll
+    for (int mm = 0; mm < 8 / R2; ++mm) dft<R2>(v + mm * R2);
+  }
+}
+
+// Pass A for rows N2 j1 + j2 of the columns from kx0 on.  load(row, kx): the doubles;
+// live: whether this thread's column exists.  st: two zeroed shared words.
+template <int N2, typename Load>
+__device__ __forceinline__ void cols_pass_a(Load load, c64* __restrict__ mid, unsigned pitch, int j2,
+                                            int kx, bool live, c64* ex, unsigned* st,
+                                            const int4* __restrict__ w, int* exp_out) {
+  const int c = threadIdx.x & (kCols - 1), l = threadIdx.x / kCols;
+  double2 u[8];
+  c64 v[8];
+  unsigned mag = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    u[i] = live ? load(N2 * (l + 8 * i) + j2, kx) : double2{0.0, 0.0};
+    mag = max(mag, max(magnitude(u[i].x), magnitude(u[i].y)));
+  }
+  block_max(mag, st);
+  __syncthreads();
+  const int E = block_exp(st[0]);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = from_double(u[i], E);
+  dft_group<8>(v, c, l, ex, w, N2);
+  if (live) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mid[(unsigned)(N2 * (l + 8 * q) + j2) * pitch + kx] = v[q];
+  }
+  if (threadIdx.x == 0) *exp_out = E >= 0x7FF ? kNaN : E - 1080 + kDrop;
+}
+
+// Pass B for m1: v[mm R2 + q] = X[m1 + 64 (m + 8 q)], m = l (8/R2) + mm, and their exponent.
+// exps: exponents of the rows j2, at stride estride.
+template <int N2>
+__device__ __forceinline__ int cols_pass_b(c64 (&v)[8], const c64* __restrict__ mid, unsigned pitch,
+                                           int m1, int l, int kx, bool live, c64* ex, unsigned* st,
+                                           const int4* __restrict__ w, const int* __restrict__ exps,
+                                           int estride) {
+  constexpr int R2 = N2 / 8;
+  const int c = threadIdx.x & (kCols - 1);
+  int er[8], top = -2048;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    er[i] = exps[(l + R2 * i) * estride];
+    v[i] = live ? mid[(unsigned)(N2 * m1 + l + R2 * i) * pitch + kx] : c64{0, 0};
+    top = max(top, er[i] + 63 - __clz((int)(spread(v[i]) | 1u)));
+  }
+  block_max((unsigned)(top + 4096), st);
+  __syncthreads();
+  const int e0 = (int)st[0] - 4096 - 62;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int s = er[i] - e0, up = max(s, 0), dn = min(max(-s, 0), 63);
+    const i64 rnd = (i64)((1ull << dn) >> 1);
+    const c64 a = {((v[i].x << up) + rnd) >> dn, ((v[i].y << up) + rnd) >> dn};
+    v[i] = mulw(a, __ldg(w + (l + R2 * i) * m1));
+  }
+  dft_group<R2>(v, c, l, ex, w, 64);
+  return e0 + kDrop + (R2 > 1 ? kDrop : 0);
 }
 
 // v times an FxFactor, its power of two left to the exponent

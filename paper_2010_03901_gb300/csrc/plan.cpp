@@ -309,10 +309,12 @@ static void line_crossings(const Curve& c, int which, int nlines, double o, doub
 // FFT axis setup
 // ------------------------------------------------------------------------- //
 // x 2^60, |x| <= 1, rounded, as h 2^32 + l with -2^31 < l < 2^31 (a low limb of -2^31,
-// which has no negative, moves by one unit)
+// which has no negative, moves by one unit), +-1 as +-(1 - 2^-60) (see drop() in fx.cuh)
 static void fx_limbs(dd x, int32_t* out) {
   const double a = std::ldexp(x.hi, 60), ai = std::floor(a);
   int64_t v = (int64_t)ai + (int64_t)std::nearbyint((a - ai) + std::ldexp(x.lo, 60));
+  const int64_t one = INT64_C(1) << 60;
+  v = std::min(std::max(v, 1 - one), one - 1);
   int32_t l = (int32_t)(uint32_t)(uint64_t)v;
   if (l == INT32_MIN) l = (int32_t)(uint32_t)(uint64_t)++v;
   out[0] = (int32_t)((v - l) >> 32);

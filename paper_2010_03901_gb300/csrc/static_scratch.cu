@@ -24,9 +24,12 @@
 namespace fc2d {
 
 constexpr size_t kStaticScratchBytes = size_t(64) << 20;
+// behind it: the exponents of the two-pass double columns, at most 9/8 per 1024 complex
+// values of the scratch
+constexpr size_t kStaticExpBytes = size_t(32) << 10;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_scratch[kStaticScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[kStaticScratchBytes + kStaticExpBytes];
 
 static std::mutex g_scratch_mu;
 static void* g_scratch_addr[kMaxDevices] = {nullptr};
@@ -73,7 +76,8 @@ extern "C" fc2d_status fc2d_coeffs_static(fc2d_plan_t p, int n_f, const void* ex
   // The row pass writes every intermediate element the column pass reads, so nothing
   // needs clearing between calls.  The argument blocks are the plan's own, as in
   // fc2d_coeffs.
-  const FftArgs fa = fft_args(p);
+  FftArgs fa = fft_args(p);
+  fa.exps = reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + kStaticScratchBytes);
   const RowArgs ra = row_args(p);
   cudaStream_t s = (cudaStream_t)stream;
   launch_fft_rows(fa, ra, n_f, f64, 0, ext, nullptr, nullptr, scratch, s);
