@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -792,8 +793,24 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
     return set_error(FC2D_ERR_UNSUPPORTED, "fc2d_wave_interior: ny <= 4736");
   cudaSetDevice(p->device);
   Layout L = layout(p, 2 * n_f);
-  if ((st = ensure_workspace(p, L.total))) return st;
   cudaStream_t s = (cudaStream_t)stream;
+  if (wave_fx_sizes(p->grid.nx, p->grid.ny)) {  // fixed point (fx_wave.cu)
+    const size_t spec = al((size_t)2 * n_f * p->grid.ny * (p->grid.nx / 2 + 1) * 16);
+    const size_t nexp = al(wave_fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int));
+    if ((st = ensure_workspace(p, L.total + spec + nexp)) || (st = wave_fx_prepare(p))) return st;
+    void* S = ws(p, L.total);
+    int* exps = reinterpret_cast<int*>(ws(p, L.total + spec));
+    if ((st = wave_spectra(p, n_f, u0, u0_bdry, ut0, ut0_bdry, S, s))) return st;
+    const FftArgs fa = fft_args(p);
+    const int eT = wave_fx_time(t, p->grid.h, c);
+    wave_fx_spectra(fa, n_f, eT, S, exps, s);
+    for (int k = 0; k < 2; ++k)
+      if ((st = wave_fx_eval(p, fa, n_f, k == 1, c, t, c * t / p->grid.h, eT, S, exps,
+                             ws(p, L.ointer), k ? ut_out : u_out, nullptr, nullptr, s)))
+        return st;
+    return launched("fc2d_wave_interior");
+  }
+  if ((st = ensure_workspace(p, L.total))) return st;
   const size_t pitch = row_pitch(p);
   FftArgs fa = fft_args(p);
   for (int half = 0; half < 2; ++half) {

@@ -199,6 +199,18 @@ void launch_complex_spectrum(int nx, int ny, int n_f, bool fp64, const void* hal
 // Fourier Forwarding: modal advance of [2 n_f] row spectra (u's then u_t's), in place.
 void launch_wave_cols(const FftArgs& fa, int n_f, void* inter, double c, double t, double Lx,
                       double Ly, cudaStream_t s);
+// Fourier Forwarding in fixed point (fx_wave.cu) for ny = 512 .. 4096 and nx/2 = 2^5 .. 2^12:
+// the spectra [2 n_f][ny][nx/2+1] (u's, then u_t's) to integers in place for times up to
+// 2^eT (exps: wave_fx_exps ints), then u or (deriv) u_t at t = cells h / c, on the grid or at
+// listed points (off[ny + 1], linear indices ascending); inter: 2 n_f ny pitch complex values.
+bool wave_fx_sizes(int nx, int ny);
+int wave_fx_time(double t, double h, double c);  // eT for times up to t
+size_t wave_fx_exps(int nx, int ny, int n_f);
+fc2d_status wave_fx_prepare(fc2d_plan_s* p);
+void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, cudaStream_t s);
+fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
+                         double cells, int eT, const void* spec, int* exps, void* inter, double* out,
+                         const int32_t* off, const int32_t* points, cudaStream_t s);
 // FP64 inverse real row DFT of an [n_f][ny][pitch] half spectrum already inverted along
 // the columns; c00 (NULL allowed) adds c00[f] (x^2 + y^2)/4.
 void launch_inverse_rows(const FftArgs& fa, int n_f, const void* inter, const double* c00,

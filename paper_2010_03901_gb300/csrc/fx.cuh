@@ -65,6 +65,21 @@ __device__ __forceinline__ c64 mulw(c64 a, int4 w) {
   return {mad(xh, w.x, mad(yh, nh, add_high(mx, 0))), mad(xh, w.z, mad(yh, w.x, add_high(my, 0)))};
 }
 
+// a conj(w) 2^-kDrop
+__device__ __forceinline__ c64 mulw_conj(c64 a, int4 w) { return mulw(a, int4{w.x, w.y, -w.z, -w.w}); }
+
+// (a p + b q) 2^-kDrop for real factors p, q (limbs of p 2^60, q 2^60), |a|, |b| <= 2^62
+__device__ __forceinline__ i64 dot(i64 a, i64 b, int4 pq) {
+  const int ah = hi32(a), al = lo32(a), bh = hi32(b), bl = lo32(b);
+  const i64 m = mad(ah, pq.y, mad(al, pq.x, mad(bh, pq.w, mad(bl, pq.z, i64(1) << 31))));
+  return mad(ah, pq.x, mad(bh, pq.z, add_high(m, 0)));
+}
+// a b 2^-64, |a|, |b| <= 2^62
+__device__ __forceinline__ i64 mulh(i64 a, i64 b) {
+  const int ah = hi32(a), al = lo32(a), bh = hi32(b), bl = lo32(b);
+  return mad(ah, bh, add_high(mad(ah, bl, mad(al, bh, i64(1) << 31)), 0));
+}
+
 // v c for a constant c in [1/2, 1) given as c - 1 = m 2^-32 + r 2^-64 (|v| < 2^62.5)
 __device__ __forceinline__ i64 mulc(i64 v, int m, int r) {
   const int h = hi32(v), l = lo32(v);
@@ -97,31 +112,31 @@ __device__ __forceinline__ int headroom(unsigned h) { return min(__clz((int)h) -
 __device__ __forceinline__ unsigned magnitude(double d) {
   return (unsigned)__double2hiint(d) & 0x7FFFFFFFu;
 }
-// x in units of 2^(E - 1080), E the block's largest biased exponent (at least 1): the
-// 53-bit significand shifted to |v| < 2^58 for exponent E, right by E - e bits for others
+// x in units of 2^(E - 1075 - UP), E at least x's biased exponent: the 53-bit significand
+// shifted to |v| < 2^(53 + UP) for exponent E, right by E - e bits for others
 __device__ __forceinline__ i64 shift_right(i64 v, int n) {  // n >= 0; 0 from 64 on (v >= 0)
   i64 r;
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
   return r;
 }
+template <int UP = 5>
 __device__ __forceinline__ i64 from_double(double d, int E) {
   const unsigned hi = (unsigned)__double2hiint(d);
   const int e = (int)(hi >> 20) & 0x7FF;
-  if (E > 64) {  // a subnormal or zero (e = 0) shifts out
-    const unsigned mh = (hi & 0xFFFFFu) | 0x100000u;
-    const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
-    const i64 v = shift_right(m, E - e);
-    const i64 s = (i64)((int)hi >> 31);
-    return (v ^ s) - s;
+  unsigned mh = (hi & 0xFFFFFu) | 0x100000u;
+  int sh = E - e;
+  if (E <= 64 && e == 0) {  // for a larger block exponent a subnormal or zero shifts out
+    mh = hi & 0xFFFFFu;
+    sh = E - 1;
   }
-  const unsigned mh = (hi & 0xFFFFFu) | (e ? 0x100000u : 0u);
-  const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << 5;
-  const i64 v = shift_right(m, E - max(e, 1));
+  const i64 m = (i64)(((unsigned long long)mh << 32) | (unsigned)__double2loint(d)) << UP;
+  const i64 v = shift_right(m, sh);
   const i64 s = (i64)((int)hi >> 31);
   return (v ^ s) - s;
 }
+template <int UP = 5>
 __device__ __forceinline__ c64 from_double(double2 d, int E) {
-  return {from_double(d.x, E), from_double(d.y, E)};
+  return {from_double<UP>(d.x, E), from_double<UP>(d.y, E)};
 }
 // block exponent of values converted with the block maximum mag of magnitude()
 __device__ __forceinline__ int block_exp(unsigned mag) { return max((int)(mag >> 20), 1); }
@@ -327,6 +342,24 @@ __device__ __forceinline__ void transform(const double2 (&u)[8], c64 (&v)[8], c6
   __syncthreads();
   rest<LOGN, 8, 1>(v, buf, t, active, st, tw, e);
   if (E >= 0x7FF) e = kNaN;
+}
+
+// The whole transform of the integers v[r] = x[t + r N/8], |z| <= 2^58.5 (read from `buf` by
+// the caller), in units of 2^e.
+template <int LOGN>
+__device__ __forceinline__ void transform(c64 (&v)[8], c64* buf, int t, bool active, unsigned* st,
+                                          const int4* __restrict__ tw, int& e) {
+  static_assert(LOGN >= 4, "at least two stages");
+  __syncthreads();
+  if (active) {
+    dft<8>(v);
+    c64* dst = buf + pad(8 * t);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) dst[r] = v[r];
+  }
+  __syncthreads();
+  static_assert(!shifts(1), "no statistics after the first stage");
+  rest<LOGN, 8, 1>(v, buf, t, active, st, tw, e);
 }
 
 // ------------------------------------------------------------------------- //

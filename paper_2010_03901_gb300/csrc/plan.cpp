@@ -321,6 +321,19 @@ static void fx_limbs(dd x, int32_t* out) {
   out[1] = l;
 }
 
+std::vector<int64_t> fx_turn_table(int n) {
+  std::vector<int64_t> out;
+  for (int t = 0; t < n; ++t) {
+    dd c, s;
+    dd_cos_sin_turn(t, n, c, s);
+    for (dd x : {c, s}) {
+      const double a = std::ldexp(x.hi, 62), ai = std::floor(a);
+      out.push_back((int64_t)ai + (int64_t)std::nearbyint((a - ai) + std::ldexp(x.lo, 62)));
+    }
+  }
+  return out;
+}
+
 static bool fft_axis(int n, bool fp64, FftAxis& ax) {
   ax.n = n;
   ax.n_radix = 0;
@@ -1025,6 +1038,7 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
   if (!p) return;
   poisson_destroy(p);
   wave_destroy(p);
+  wave_modes_destroy(p);
   void* ptrs[] = {p->dev.Q, p->dev.Ar, p->dev.Ar_hi, p->dev.Ar_lo, p->dev.gidx, p->dev.gw,
                   p->dev.wn, p->dev.s_lin, p->dev.s_theta, p->dev.s_eta, p->dev.s_w,
                   p->dev.s_pb, p->dev.s_sb, p->dev.own[0].off, p->dev.own[0].k,

@@ -133,6 +133,7 @@ struct fc2d_plan_s {
   std::vector<void*> event_pool;               // reusable cudaEvent_t
   void* poisson = nullptr;                     // Poisson tables (poisson.cu)
   void* wave = nullptr;                        // Fourier Forwarding state (ff.cu)
+  void* modes = nullptr;                       // its mode table (fx_wave.cu)
   // autotuned launch shapes (tune_plan): columns per block of the 4096-point FP32
   // column passes, their form (0 a block per tile, direct loads; 1 persistent blocks,
   // TMA-pipelined loads) and the candidates' times (microseconds per call, direct 16,
@@ -174,6 +175,10 @@ void poisson_stats(const fc2d_plan_s* p, int* iters, double* resid, int64_t* n_n
 
 // Fourier Forwarding state (ff.cu)
 void wave_destroy(fc2d_plan_s* p);
+void wave_modes_destroy(fc2d_plan_s* p);
+
+// (cos, sin)(2 pi i/n) 2^62, i < n, rounded (plan.cpp)
+std::vector<int64_t> fx_turn_table(int n);
 
 // Plan-time autotuning of launch shapes that change no result (capi.cu).
 fc2d_status tune_plan(fc2d_plan_s* p);

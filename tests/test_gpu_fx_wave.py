@@ -1,0 +1,62 @@
+"""The fixed-point modal solutions of Fourier Forwarding (csrc/fx_wave.cu) against the same
+formulas in long double, from the plan's own extensions of u and u_t.
+
+The bar: forward transforms, time factors and inverse transforms each within 3 2^-53 (see
+test_gpu_fx.py; the factors are 60-bit) of operators of norm 1 and t (for u), or w_max and
+1 (for u_t): 10 2^-53 (|F| + t |G|) and 10 2^-53 (w_max |F| + |G|) in the 2-norm.  The phase
+w t is exact to 2^-64 of a turn per cell travelled, so long times keep the bar.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_fx import plan_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 512), (64, 512), (1024, 512), (512, 1024), (128, 2048),
+                                   (64, 4096)])
+@pytest.mark.parametrize("cells", [0.0, 1e-7, 0.01, 0.5, 8.0, 1000.25])
+def test_modal_solutions(nx, ny, cells):
+    torch = pytest.importorskip("torch")
+    fft = pytest.importorskip("scipy.fft")
+    plan = plan_of(nx, ny)
+    n = min(nx, ny)
+    h, c = 2.0 / (0.45 * n), 1.7
+    t = cells * h / c
+    rng = np.random.default_rng(nx + ny)
+    x = (np.arange(nx) - 0.5 * nx) * h
+    y = (np.arange(ny) - 0.5 * ny) * h
+    xy = plan.fc2d_boundary_points().T
+    fields = []
+    for amp in (1.0, 1.0 / max(t, h)):
+        k, s = rng.uniform(2, 8, 4), rng.uniform(0, 6, 4)
+        fn = lambda X, Y: amp * sum(np.cos(kk * (X * np.cos(ss) + Y * np.sin(ss)) + ss) for kk, ss in zip(k, s))  # noqa: E731,B023
+        fields.append((fn(x[None, :], y[:, None]), fn(xy[0], xy[1])))
+    T = lambda a: torch.tensor(a[None], dtype=torch.float64, device="cuda")  # noqa: E731
+    (u, ub), (v, vb) = [(T(a), T(b)) for a, b in fields]
+    ext = []
+    for a, b in ((u, ub), (v, vb)):
+        e = torch.zeros_like(a)
+        plan.fc2d_extend(1, a, b, e)
+        ext.append(e.cpu().numpy()[0].astype(np.longdouble))
+    got, got_t = torch.zeros_like(u), torch.zeros_like(u)
+    plan.fc2d_wave_interior(1, c, t, u, ub, v, vb, got, got_t)
+    plan.fc2d_sync_status()
+    F, G = fft.rfft2(ext[0]), fft.rfft2(ext[1])
+    L = np.longdouble
+    l = np.arange(nx // 2 + 1, dtype=L) / nx
+    m = np.abs(np.fft.fftfreq(ny) * ny).astype(L) / ny
+    two_pi = 2 * L("3.14159265358979323846264338327950288")
+    w = two_pi * L(c) * np.sqrt(l[None, :] ** 2 + m[:, None] ** 2) / L(h)
+    wt = two_pi * ((w / two_pi * L(t)) % 1)
+    sw = np.where(w > 0, np.sin(wt) / np.where(w > 0, w, 1), L(t))
+    ref = fft.irfft2(F * np.cos(wt) + G * sw, s=(ny, nx))
+    ref_t = fft.irfft2(G * np.cos(wt) - F * w * np.sin(wt), s=(ny, nx))
+    norm = lambda a: float(np.sqrt((np.abs(a) ** 2).sum()))  # noqa: E731
+    f, g = norm(ext[0]), norm(ext[1])
+    # wt itself, in the reference, from the doubles h, c and t: c t/h is rounded once
+    slack = float(w.max()) * t * 2.0 ** -52
+    eps = 10 * 2.0 ** -53 + slack
+    assert norm(got.cpu().numpy()[0] - ref) < eps * (f + t * g)
+    assert norm(got_t.cpu().numpy()[0] - ref_t) < eps * (float(w.max()) * f + g)
