@@ -31,6 +31,7 @@
 
 #include "fc2d_kernels.cuh"
 #include "fft_generic.cuh"
+#include "fx_squares.h"
 #include "plan_internal.h"
 #include "wave_band.h"
 
@@ -58,10 +59,12 @@ struct DevSquares {
   int32_t* served_local = nullptr;
   double* A = nullptr;              // [C][d]
   double* Q = nullptr;              // [d][d]
-  double2* tw = nullptr;            // exp(-2 pi i t / P), t < P
-  float4* tw_df = nullptr;          // the same as double-float pairs (re hi, lo, im hi, lo)
+  int32_t* tw = nullptr;            // exp(-2 pi i t / P) 2^60 in limbs, t < P (fx.cuh)
   int32_t* rows = nullptr;          // [n_sq][2]: first and last box row holding served points
-  int n = 0;
+  int n = 0, max_rows = 0;          // squares; the most rows any of them needs
+  SquareArgs args() const {
+    return {n, origin, A, Q, reinterpret_cast<const int4*>(tw), served_off, served_lin, served_local, rows};
+  }
 };
 
 struct DevBand {
@@ -143,19 +146,12 @@ fc2d_status upload_squares(const fc2d_plan_s* p, DevBand& b, int n_c) {
     }
     rows[2 * k] = lo;
     rows[2 * k + 1] = hi;
-  }
-  std::vector<double2> tw(h.P);
-  std::vector<float4> tw_df(h.P);
-  for (int t = 0; t < h.P; ++t) {
-    const double ang = -2.0 * M_PI * double(t) / double(h.P);
-    tw[t] = double2{std::cos(ang), std::sin(ang)};
-    const float ch = (float)tw[t].x, sh = (float)tw[t].y;
-    tw_df[t] = float4{ch, (float)(tw[t].x - (double)ch), sh, (float)(tw[t].y - (double)sh)};
+    q->max_rows = std::max(q->max_rows, hi - lo + 1);
   }
   if ((st = upload(&q->origin, origin)) || (st = upload(&q->served_off, h.served_off)) ||
       (st = upload(&q->served_lin, h.served_lin)) || (st = upload(&q->served_local, h.served_local)) ||
-      (st = upload(&q->A, h.A)) || (st = upload(&q->Q, h.Q)) || (st = upload(&q->tw, tw)) ||
-      (st = upload(&q->tw_df, tw_df)) || (st = upload(&q->rows, rows)))
+      (st = upload(&q->A, h.A)) || (st = upload(&q->Q, h.Q)) || (st = upload(&q->tw, fx_twiddle_table(h.P))) ||
+      (st = upload(&q->rows, rows)))
     return st;
   b.sq = std::move(q);
   return FC2D_OK;
@@ -362,407 +358,6 @@ __global__ void __launch_bounds__(256) k_ff_cols(FftArgs fa, int n_f, const doub
   }
 }
 
-// ------------------------------------------------------------------------- //
-// The small-square procedure (Section 4.2; wave_band.cpp builds the squares)
-// ------------------------------------------------------------------------- //
-constexpr int kSqThreads = 256;
-
-// 1D-FC continuation (eq. (2.7)) of the length-n sequence x[at(0)], ..., x[at(n-1)]
-// (complex values: two real functions at once) into x[at(n)] .. x[at(n + C - 1)]:
-// the C values (A Q^T r)_k + (A Q^T l)_{C-1-k}, r the last d values, l the first d in
-// reverse order.  One thread per continuation point.
-template <typename At>
-__device__ __forceinline__ void fc1d_continue(double2* x, At at, int n, int C, int d,
-                                              const double* __restrict__ A,
-                                              const double* __restrict__ Q, int k) {
-  double2 cr[kMaxD], cl[kMaxD];
-  for (int i = 0; i < d; ++i) {  // Gram coefficients c = Q^T f
-    double2 r = {0.0, 0.0}, l = {0.0, 0.0};
-    for (int m = 0; m < d; ++m) {
-      const double qm = __ldg(Q + m * d + i);
-      const double2 fr = x[at(n - d + m)], fl = x[at(d - 1 - m)];
-      r.x += qm * fr.x;
-      r.y += qm * fr.y;
-      l.x += qm * fl.x;
-      l.y += qm * fl.y;
-    }
-    cr[i] = r;
-    cl[i] = l;
-  }
-  double2 vr = {0.0, 0.0}, vl = {0.0, 0.0};
-  for (int i = 0; i < d; ++i) {
-    const double ar = __ldg(A + k * d + i), al = __ldg(A + (C - 1 - k) * d + i);
-    vr.x += ar * cr[i].x;
-    vr.y += ar * cr[i].y;
-    vl.x += al * cl[i].x;
-    vl.y += al * cl[i].y;
-  }
-  x[at(n + k)] = double2{vl.x + vr.x, vl.y + vr.y};
-}
-
-// 64-point DFT of the padded sequence x[pad(e) ST], e < 64 (pad(e) = e + e/8), by the 8
-// threads q = 0..7 of a group, as 8 x 8: X[k1 + 8 k2] = sum_q w8^(q k2) w64^(q k1)
-// sum_r x[q + 8 r] w8^(r k1); the result replaces x in natural order.  Every thread of
-// the block calls it (three barriers, the last after the result is stored); `active`
-// false: a group with nothing to transform.
-__device__ __forceinline__ int sq_pad(int e) { return e + (e >> 3); }
-
-// Forward 8-point DFT in registers (radix 2 x 4: two 4-point DFTs of the even and odd
-// entries, the twiddles exp(-2 pi i k/8), one butterfly).
-__device__ __forceinline__ void dft8_regs(double2 (&v)[8]) {
-  const double s = 0.70710678118654752440;
-  auto d4 = [](double2& a0, double2& a1, double2& a2, double2& a3) {
-    const double2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3);
-    const double2 t3 = mul_mi(csub(a1, a3));
-    a0 = cadd(t0, t2);
-    a2 = csub(t0, t2);
-    a1 = cadd(t1, t3);
-    a3 = csub(t1, t3);
-  };
-  double2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  d4(e0, e1, e2, e3);
-  d4(o0, o1, o2, o3);
-  const double2 w1 = {s * (o1.x + o1.y), s * (o1.y - o1.x)};
-  const double2 w2 = mul_mi(o2);
-  const double2 w3 = {s * (o3.y - o3.x), -s * (o3.x + o3.y)};
-  v[0] = cadd(e0, o0);
-  v[4] = csub(e0, o0);
-  v[1] = cadd(e1, w1);
-  v[5] = csub(e1, w1);
-  v[2] = cadd(e2, w2);
-  v[6] = csub(e2, w2);
-  v[3] = cadd(e3, w3);
-  v[7] = csub(e3, w3);
-}
-
-template <int ST = 1>
-__device__ __forceinline__ void fft64(double2* x, int q, bool active,
-                                      const double2* __restrict__ tw) {
-  double2 v[8];
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = x[sq_pad(q + 8 * r) * ST];
-    dft8_regs(v);
-#pragma unroll
-    for (int k = 1; k < 8; ++k) v[k] = cmul(v[k], __ldg(tw + q * k));  // w64^(q k1)
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[sq_pad(q + 8 * k) * ST] = v[k];
-  }
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = x[sq_pad(8 * q + r) * ST];  // thread q is k1 here
-    dft8_regs(v);
-  }
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[sq_pad(q + 8 * k) * ST] = v[k];
-  }
-  __syncthreads();
-}
-
-// A complex double as double-float pairs: hi = RN(x), lo = RN(x - hi).
-__device__ __forceinline__ float4 split_df(double2 v) {
-  const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-  return float4{rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih)};
-}
-
-// Once per large step: each square's expansion.  Block (square, function): the square's
-// u and u_t as one complex field z = u + i u_t, continued along rows, then columns, to
-// P x P; its 2D DFT, normalised, stored transposed: Z[l][m] (l: x frequency).
-// DF: Z as double-float pairs (float4 re hi, re lo, im hi, im lo) for k_sq_eval_df.
-// One padded buffer holds the field and both transforms in place: value (y, x) at
-// sq_pad(y) kSqRow + sq_pad(x).  The 64-point DFTs (fft64, 8 threads each) run along x at
-// unit stride and along y at stride kSqRow; kSqRow is odd in 16-byte units, so both
-// access patterns of fft64 (consecutive and every 8th element) spread over all banks in
-// either direction.  83 KB of shared memory allow two blocks per SM.
-constexpr int kSqRow = 73;                       // row stride (complex values)
-constexpr int kSqRows = 64 + 64 / 8 - 1;         // sq_pad(63) + 1 rows
-constexpr size_t kSqForwardSmem = (size_t)kSqRows * kSqRow * sizeof(double2);
-
-template <bool DF>
-__global__ void __launch_bounds__(kSqThreads, 2) k_sq_forward(
-    int n_side, int C, int d, int nx, int64_t grid_stride, int n_f,
-    const int32_t* __restrict__ origin, const double* __restrict__ A,
-    const double* __restrict__ Q, const double2* __restrict__ tw, const double* __restrict__ u,
-    const double* __restrict__ ut, double2* __restrict__ Z) {
-  constexpr int P = kSqP;  // n_side + C = P (the host checks)
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* buf = reinterpret_cast<double2*>(smem_raw);
-  const int sq = blockIdx.x, f = blockIdx.y;
-  const int j0 = __ldg(origin + 2 * sq), i0 = __ldg(origin + 2 * sq + 1);
-  const double* uf = u + (size_t)f * grid_stride;
-  const double* tf = ut + (size_t)f * grid_stride;
-  for (int t = threadIdx.x; t < n_side * n_side; t += blockDim.x) {
-    const int y = t / n_side, x = t - y * n_side;
-    const size_t g = (size_t)(j0 + y) * nx + (i0 + x);
-    buf[sq_pad(y) * kSqRow + sq_pad(x)] = double2{uf[g], tf[g]};
-  }
-  __syncthreads();
-  const auto along_x = [](int i) { return sq_pad(i); };
-  const auto along_y = [](int i) { return sq_pad(i) * kSqRow; };
-  for (int t = threadIdx.x; t < n_side * C; t += blockDim.x) {  // rows
-    const int y = t / C, k = t - y * C;
-    fc1d_continue(buf + sq_pad(y) * kSqRow, along_x, n_side, C, d, A, Q, k);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < P * C; t += blockDim.x) {  // columns
-    const int x = t / C, k = t - x * C;
-    fc1d_continue(buf + sq_pad(x), along_y, n_side, C, d, A, Q, k);
-  }
-  __syncthreads();
-  const int g = threadIdx.x >> 3, q = threadIdx.x & 7;
-  constexpr int G = kSqThreads / 8;  // transforms per call
-#pragma unroll 1
-  for (int y0 = 0; y0 < P; y0 += G)  // along x: (y, l)
-    fft64<1>(buf + sq_pad(y0 + g) * kSqRow, q, y0 + g < P, tw);
-#pragma unroll 1
-  for (int l0 = 0; l0 < P; l0 += G)  // along y: (m, l)
-    fft64<kSqRow>(buf + sq_pad(l0 + g), q, l0 + g < P, tw);
-  const double sc = 1.0 / ((double)P * P);
-  double2* dst = Z + ((size_t)sq * n_f + f) * P * P;
-  for (int t = threadIdx.x; t < P * P; t += blockDim.x) {
-    const int l = t / P, m = t - l * P;
-    const double2 w = buf[sq_pad(m) * kSqRow + sq_pad(l)];
-    const double2 v = double2{w.x * sc, w.y * sc};
-    if constexpr (DF) reinterpret_cast<float4*>(dst)[t] = split_df(v);
-    else dst[t] = v;
-  }
-}
-
-constexpr int kSqPad = 72;        // padded length of a 64-point sequence
-constexpr int kSqEvalThreads = 512;
-
-// Every small step: U at the served interface points at time tau = s dt after the
-// expansion.  Block (square, function pair) of 512 threads (64 groups of 8): for functions
-// f0 = 2 blockIdx.y and f0 + 1 the spectra of u and u_t are separated from Z (hat f =
-// (Z_k + conj Z_-k)/2, hat g = (Z_k - conj Z_-k)/(2i)), advanced with the time factors
-// (cos w tau, sin(w tau)/w) of the P-periodic box (table tab[l][m]) and packed as
-// conj(a_f0 + i a_f1); the inverse 2D DFT runs as forward 64-point DFTs along m for every
-// l, a transpose of the rows the served points need (rows r0..r1 of the square), and
-// forward DFTs along l for those rows; the real part of the conjugated result is f0's
-// field, the imaginary part with its sign changed f1's.
-__global__ void __launch_bounds__(kSqEvalThreads, 2) k_sq_eval(
-    int n_f, const double2* __restrict__ Z, const double2* __restrict__ tab,
-    const double2* __restrict__ tw, const int32_t* __restrict__ served_off,
-    const int32_t* __restrict__ served_lin, const int32_t* __restrict__ served_local,
-    const int32_t* __restrict__ rows, int64_t grid_stride, double* __restrict__ out) {
-  constexpr int P = kSqP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* T1 = reinterpret_cast<double2*>(smem_raw);  // [64][72]: transform l along m
-  double2* T2 = T1 + P * kSqPad;                        // [rows][72]: transform y along l
-  const int sq = blockIdx.x, f0 = 2 * blockIdx.y;
-  const bool two = f0 + 1 < n_f;
-  const double2* Z0 = Z + ((size_t)sq * n_f + f0) * P * P;
-  const double2* Z1 = Z0 + (size_t)P * P;
-  const int g = threadIdx.x >> 3, q = threadIdx.x & 7;
-  for (int t = threadIdx.x; t < P * P; t += blockDim.x) {
-    const int l = t / P, m = t - l * P;
-    const int tn = ((P - l) & (P - 1)) * P + ((P - m) & (P - 1));  // the index of -k
-    const double2 tt = __ldg(tab + t);
-    auto adv = [&](const double2* Zf) {
-      const double2 zk = Zf[t], zn = Zf[tn];
-      const double2 F = {0.5 * (zk.x + zn.x), 0.5 * (zk.y - zn.y)};   // (Z_k + conj Z_-k)/2
-      const double2 G = {0.5 * (zk.y + zn.y), -0.5 * (zk.x - zn.x)};  // (Z_k - conj Z_-k)/(2i)
-      return double2{F.x * tt.x + G.x * tt.y, F.y * tt.x + G.y * tt.y};
-    };
-    const double2 a0 = adv(Z0);
-    const double2 a1 = two ? adv(Z1) : double2{0.0, 0.0};
-    T1[l * kSqPad + sq_pad(m)] = double2{a0.x - a1.y, -(a0.y + a1.x)};  // conj(a0 + i a1)
-  }
-  __syncthreads();
-  fft64(T1 + g * kSqPad, q, true, tw);  // T1[l][y]
-  const int r0 = __ldg(rows + 2 * sq), nr = __ldg(rows + 2 * sq + 1) - r0 + 1;
-  for (int t = threadIdx.x; t < nr * P; t += blockDim.x) {
-    const int yr = t / P, l = t - yr * P;
-    T2[yr * kSqPad + sq_pad(l)] = T1[l * kSqPad + sq_pad(r0 + yr)];
-  }
-  __syncthreads();
-  fft64(T2 + g * kSqPad, q, g < nr, tw);  // T2[y - r0][x]
-  const int s0 = __ldg(served_off + sq), s1 = __ldg(served_off + sq + 1);
-  for (int k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
-    const int loc = __ldg(served_local + k), y = loc / P, x = loc - y * P;
-    const double2 v = T2[(y - r0) * kSqPad + sq_pad(x)];
-    const int32_t lin = __ldg(served_lin + k);
-    out[(size_t)f0 * grid_stride + lin] = v.x;
-    if (two) out[(size_t)(f0 + 1) * grid_stride + lin] = -v.y;
-  }
-}
-
-// ------------------------------------------------------------------------- //
-// The same evaluation in double-float arithmetic (interface mode 2).  A real number is
-// the unevaluated sum hi + lo of two floats; sums use Knuth's TwoSum with the low parts
-// added after it and Dekker's FastTwoSum to renormalise, products the FMA form of
-// Dekker's TwoProduct (Dekker 1971; Knuth, TAOCP vol. 2, 4.2.2).  Each operation is
-// accurate to about 2^-44 of its operands' size, on the FP32 pipe, which on this part
-// issues 64 times as many operations as the FP64 pipe.
-// ------------------------------------------------------------------------- //
-struct df2 {
-  float hi, lo;
-};
-struct dfc {
-  df2 re, im;
-};
-__device__ __forceinline__ df2 df_fast(float a, float b) {  // |a| >= |b| or a = 0
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ df2 df_add(df2 a, df2 b) {
-  const float s = __fadd_rn(a.hi, b.hi), bb = __fsub_rn(s, a.hi);
-  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-  return df_fast(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
-}
-__device__ __forceinline__ df2 df_neg(df2 a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ df2 df_sub(df2 a, df2 b) { return df_add(a, df_neg(b)); }
-__device__ __forceinline__ df2 df_mul(df2 a, df2 b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  float e = fmaf(a.hi, b.hi, -p);
-  e = fmaf(a.hi, b.lo, e);
-  e = fmaf(a.lo, b.hi, e);
-  return df_fast(p, e);
-}
-__device__ __forceinline__ df2 df_half(df2 a) { return {0.5f * a.hi, 0.5f * a.lo}; }
-__device__ __forceinline__ dfc dfc_load(float4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
-__device__ __forceinline__ float4 dfc_store(dfc a) { return float4{a.re.hi, a.re.lo, a.im.hi, a.im.lo}; }
-__device__ __forceinline__ dfc dfc_add(dfc a, dfc b) { return {df_add(a.re, b.re), df_add(a.im, b.im)}; }
-__device__ __forceinline__ dfc dfc_sub(dfc a, dfc b) { return {df_sub(a.re, b.re), df_sub(a.im, b.im)}; }
-__device__ __forceinline__ dfc dfc_mul_mi(dfc a) { return {a.im, df_neg(a.re)}; }  // -i a
-__device__ __forceinline__ dfc dfc_mul(dfc a, dfc b) {
-  return {df_sub(df_mul(a.re, b.re), df_mul(a.im, b.im)),
-          df_add(df_mul(a.re, b.im), df_mul(a.im, b.re))};
-}
-__device__ __forceinline__ double df_to_double(df2 a) { return (double)a.hi + (double)a.lo; }
-
-// Forward 8-point DFT in registers (as dft8_regs)
-__device__ __forceinline__ void dft8_df(dfc (&v)[8]) {
-  constexpr double kS = 0.70710678118654752440;
-  const df2 s = {(float)kS, (float)(kS - (double)(float)kS)};
-  auto d4 = [](dfc& a0, dfc& a1, dfc& a2, dfc& a3) {
-    const dfc t0 = dfc_add(a0, a2), t1 = dfc_sub(a0, a2), t2 = dfc_add(a1, a3);
-    const dfc t3 = dfc_mul_mi(dfc_sub(a1, a3));
-    a0 = dfc_add(t0, t2);
-    a2 = dfc_sub(t0, t2);
-    a1 = dfc_add(t1, t3);
-    a3 = dfc_sub(t1, t3);
-  };
-  dfc e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  d4(e0, e1, e2, e3);
-  d4(o0, o1, o2, o3);
-  const dfc w1 = {df_mul(s, df_add(o1.re, o1.im)), df_mul(s, df_sub(o1.im, o1.re))};
-  const dfc w2 = dfc_mul_mi(o2);
-  const dfc w3 = {df_mul(s, df_sub(o3.im, o3.re)), df_neg(df_mul(s, df_add(o3.re, o3.im)))};
-  v[0] = dfc_add(e0, o0);
-  v[4] = dfc_sub(e0, o0);
-  v[1] = dfc_add(e1, w1);
-  v[5] = dfc_sub(e1, w1);
-  v[2] = dfc_add(e2, w2);
-  v[6] = dfc_sub(e2, w2);
-  v[3] = dfc_add(e3, w3);
-  v[7] = dfc_sub(e3, w3);
-}
-
-// 64-point DFT of the padded sequence x[pad(e)] (as fft64)
-__device__ __forceinline__ void fft64_df(float4* x, int q, bool active,
-                                         const float4* __restrict__ tw) {
-  dfc v[8];
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = dfc_load(x[sq_pad(q + 8 * r)]);
-    dft8_df(v);
-#pragma unroll
-    for (int k = 1; k < 8; ++k) v[k] = dfc_mul(v[k], dfc_load(__ldg(tw + q * k)));
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[sq_pad(q + 8 * k)] = dfc_store(v[k]);
-  }
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = dfc_load(x[sq_pad(8 * q + r)]);
-    dft8_df(v);
-  }
-  __syncthreads();
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[sq_pad(q + 8 * k)] = dfc_store(v[k]);
-  }
-  __syncthreads();
-}
-
-// k_sq_eval in double-float: Z and tab hold double-float pairs (float4), tw_df the box's
-// twiddles; the served values are converted to double on output.
-__global__ void __launch_bounds__(kSqEvalThreads, 2) k_sq_eval_df(
-    int n_f, const float4* __restrict__ Z, const float4* __restrict__ tab,
-    const float4* __restrict__ tw, const int32_t* __restrict__ served_off,
-    const int32_t* __restrict__ served_lin, const int32_t* __restrict__ served_local,
-    const int32_t* __restrict__ rows, int64_t grid_stride, double* __restrict__ out) {
-  constexpr int P = kSqP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* T1 = reinterpret_cast<float4*>(smem_raw);  // [64][72]: transform l along m
-  float4* T2 = T1 + P * kSqPad;                       // [rows][72]: transform y along l
-  const int sq = blockIdx.x, f0 = 2 * blockIdx.y;
-  const bool two = f0 + 1 < n_f;
-  const float4* Z0 = Z + ((size_t)sq * n_f + f0) * P * P;
-  const float4* Z1 = Z0 + (size_t)P * P;
-  const int g = threadIdx.x >> 3, q = threadIdx.x & 7;
-  for (int t = threadIdx.x; t < P * P; t += blockDim.x) {
-    const int l = t / P, m = t - l * P;
-    const int tn = ((P - l) & (P - 1)) * P + ((P - m) & (P - 1));  // the index of -k
-    const dfc tt = dfc_load(__ldg(tab + t));                        // (cos w tau, sin(w tau)/w)
-    auto adv = [&](const float4* Zf) {
-      const dfc zk = dfc_load(Zf[t]), zn = dfc_load(Zf[tn]);
-      const dfc F = {df_half(df_add(zk.re, zn.re)), df_half(df_sub(zk.im, zn.im))};
-      const dfc G = {df_half(df_add(zk.im, zn.im)), df_neg(df_half(df_sub(zk.re, zn.re)))};
-      return dfc{df_add(df_mul(F.re, tt.re), df_mul(G.re, tt.im)),
-                 df_add(df_mul(F.im, tt.re), df_mul(G.im, tt.im))};
-    };
-    const dfc a0 = adv(Z0);
-    const dfc a1 = two ? adv(Z1) : dfc{{0.f, 0.f}, {0.f, 0.f}};
-    T1[l * kSqPad + sq_pad(m)] = dfc_store(dfc{df_sub(a0.re, a1.im), df_neg(df_add(a0.im, a1.re))});
-  }
-  __syncthreads();
-  fft64_df(T1 + g * kSqPad, q, true, tw);  // T1[l][y]
-  const int r0 = __ldg(rows + 2 * sq), nr = __ldg(rows + 2 * sq + 1) - r0 + 1;
-  for (int t = threadIdx.x; t < nr * P; t += blockDim.x) {
-    const int yr = t / P, l = t - yr * P;
-    T2[yr * kSqPad + sq_pad(l)] = T1[l * kSqPad + sq_pad(r0 + yr)];
-  }
-  __syncthreads();
-  fft64_df(T2 + g * kSqPad, q, g < nr, tw);  // T2[y - r0][x]
-  const int s0 = __ldg(served_off + sq), s1 = __ldg(served_off + sq + 1);
-  for (int k = s0 + threadIdx.x; k < s1; k += blockDim.x) {
-    const int loc = __ldg(served_local + k), y = loc / P, x = loc - y * P;
-    const dfc v = dfc_load(T2[(y - r0) * kSqPad + sq_pad(x)]);
-    const int32_t lin = __ldg(served_lin + k);
-    out[(size_t)f0 * grid_stride + lin] = df_to_double(v.re);
-    if (two) out[(size_t)(f0 + 1) * grid_stride + lin] = -df_to_double(v.im);
-  }
-}
-
-// The box's time factors for the small steps s = 0..S-1: tab[s][l][m] =
-// (cos w tau, sin(w tau)/w) at tau = s dt ((1, tau) at w = 0), w = 2 pi c |k| / (P h).
-template <bool DF>
-__global__ void k_sq_table(int P, int S, double c, double h, double dt, double2* __restrict__ tab) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)S * P * P) return;
-  const int s = (int)(t / (P * P)), lm = (int)(t - (int64_t)s * P * P);
-  const int l = lm / P, m = lm - l * P;
-  const int ls = l <= P / 2 ? l : l - P, ms = m <= P / 2 ? m : m - P;
-  const double L = P * h, tau = s * dt;
-  const double fl = ls / L, fm = ms / L;
-  const double w = 6.283185307179586476925286766559 * c * sqrt(fl * fl + fm * fm);
-  double2 v;
-  if (w == 0.0) {
-    v = double2{1.0, tau};
-  } else {
-    double sn, co;
-    sincos(w * tau, &sn, &co);
-    v = double2{co, sn / w};
-  }
-  if constexpr (DF) reinterpret_cast<float4*>(tab)[t] = split_df(v);
-  else tab[t] = v;
-}
-
 unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -783,8 +378,7 @@ void wave_destroy(fc2d_plan_s* p) {
     if (b.sq) {
       DevSquares& q = *b.sq;
       for (void* ptr : {(void*)q.origin, (void*)q.served_off, (void*)q.served_lin,
-                        (void*)q.served_local, (void*)q.A, (void*)q.Q, (void*)q.tw, (void*)q.tw_df,
-                        (void*)q.rows})
+                        (void*)q.served_local, (void*)q.A, (void*)q.Q, (void*)q.tw, (void*)q.rows})
         cudaFree(ptr);
     }
   }
@@ -890,8 +484,8 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   cudaSetDevice(p->device);
   cudaStream_t s = (cudaStream_t)stream;
   DevBand* b;
-  // mode 2: the squares of mode 1, evaluated in double-float arithmetic
-  const bool df = interface_mode == 2;
+  // mode 2 (once the squares in double-float arithmetic) runs the fixed-point squares of
+  // mode 1, which are both faster and more accurate
   if ((st = get_band(p, n_c, interface_mode ? 1 : 0, &b))) return st;
   const int nx = p->grid.nx, ny = p->grid.ny, nxh = nx / 2 + 1;
   const int64_t NN = (int64_t)nx * ny, nb = p->n_bdry, Nu = b->L.rows;
@@ -905,10 +499,11 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
                b_grid = al((size_t)n_f * NN * 8), b_ub = al((size_t)std::max<int64_t>(1, Nu) * n_f * 8),
                b_zero = al((size_t)n_f * nb * 8);
   const DevSquares* sq = b->sq.get();
-  const int P = sq ? sq->host.P : 0, n_sq = sq ? sq->n : 0;
-  const size_t b_sqz = al((size_t)n_sq * n_f * P * P * 16), b_sqt = al((size_t)S * P * P * 16);
+  const int n_sq = sq ? sq->n : 0;
+  const size_t b_sqz = al(squares_spectrum_bytes(n_sq, n_f)), b_sqt = sq ? al(squares_factor_bytes(S)) : 0;
+  const size_t b_sqe = al((size_t)n_sq * n_f * sizeof(int));
   const size_t b_exps = al(wave_fx_exps(nx, ny, n_f) * sizeof(int));
-  const size_t need = b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero + b_sqz + b_sqt + b_exps;
+  const size_t need = b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero + b_sqz + b_sqt + b_sqe + b_exps;
   WaveState* W = state(p);
   if (W->scr.bytes < need) {
     cudaDeviceSynchronize();
@@ -927,30 +522,14 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   for (int k = 0; k < 4; ++k)
     ub[k] = reinterpret_cast<double*>(base + b_spec + b_inter + 2 * b_grid + k * b_ub);
   double* zero = reinterpret_cast<double*>(base + b_spec + b_inter + 2 * b_grid + 4 * b_ub);
-  double2* sqZ = reinterpret_cast<double2*>(base + b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero);
-  double2* sqT = reinterpret_cast<double2*>(base + b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero + b_sqz);
+  char* sqZ = base + b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero;
+  char* sqT = sqZ + b_sqz;
+  int* sqE = reinterpret_cast<int*>(sqT + b_sqt);
   int* exps = reinterpret_cast<int*>(base + need - b_exps);
   cudaMemsetAsync(zero, 0, (size_t)n_f * nb * 8, s);
-  const size_t sm_sq = kSqForwardSmem;
-  int max_rows = 0;
-  if (sq)
-    for (int k = 0; k < n_sq; ++k) {
-      int lo = P, hi = -1;
-      for (int i = sq->host.served_off[k]; i < sq->host.served_off[k + 1]; ++i) {
-        lo = std::min(lo, sq->host.served_local[i] / P);
-        hi = std::max(hi, sq->host.served_local[i] / P);
-      }
-      max_rows = std::max(max_rows, hi - lo + 1);
-    }
-  const size_t sm_ev = (size_t)(P + max_rows) * kSqPad * sizeof(double2);
-  if (sq) {
-    cudaFuncSetAttribute(k_sq_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sq);
-    cudaFuncSetAttribute(k_sq_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sq);
-    cudaFuncSetAttribute(k_sq_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ev);
-    cudaFuncSetAttribute(k_sq_eval_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_ev);
-    if (df) k_sq_table<true><<<blocks((int64_t)S * P * P, 256), 256, 0, s>>>(P, S, c, h, dt, sqT);
-    else k_sq_table<false><<<blocks((int64_t)S * P * P, 256), 256, 0, s>>>(P, S, c, h, dt, sqT);
-  }
+  // the spectra of u_t are scaled by 2^eT >= dT in the fixed-point solutions
+  const int eT = wave_fx_time(dT, h, c);
+  if (sq) squares_factors(S, c, h, dt, eT, sqT, s);
   auto gat = [&](int64_t m) { return g_dir ? g_dir + (size_t)m * n_f * nb : nullptr; };
   auto gtat = [&](int64_t j) { return gt_dir ? gt_dir + (size_t)j * n_f * nb : nullptr; };
   FftArgs fa = fft_args(p);
@@ -959,7 +538,6 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   cudaFuncSetAttribute(k_ff_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc);
   // fixed-point modal solutions (fx_wave.cu) where the sizes allow; FP64 kernels otherwise
   const bool fxw = wave_fx_sizes(nx, ny);
-  const int eT = wave_fx_time(dT, h, c);
   if (fxw && (st = wave_fx_prepare(p))) return st;
   // U_FC at tau = cells h / c: u and, with out_ut, its time derivative on the grid; with
   // `points` only u at the interface points
@@ -1005,9 +583,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
     if (sq) {  // the squares' expansions of u(T_j), u_t(T_j), before u and ut change
       ProfScope ps(p, "sq_forward", s);
       const SquareSet& H = sq->host;
-      auto kf = df ? k_sq_forward<true> : k_sq_forward<false>;
-      kf<<<dim3(n_sq, n_f), kSqThreads, sm_sq, s>>>(2 * H.a + 1, H.C, H.d, nx, NN, n_f,
-                                                     sq->origin, sq->A, sq->Q, sq->tw, u, ut, sqZ);
+      squares_expand(sq->args(), 2 * H.a + 1, H.C, H.d, nx, NN, n_f, eT, u, ut, sqZ, sqE, s);
     }
     if ((st = wave_spectra(p, n_f, u, g_dir ? gat(m0) : zero, ut, gt_dir ? gtat(j) : zero, spec, s)))
       return st;
@@ -1016,15 +592,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
       const int64_t m = m0 + sidx;
       if (sq) {
         ProfScope ps(p, "sq_eval", s);
-        if (df)
-          k_sq_eval_df<<<dim3(n_sq, (n_f + 1) / 2), kSqEvalThreads, sm_ev, s>>>(
-              n_f, reinterpret_cast<const float4*>(sqZ),
-              reinterpret_cast<const float4*>(sqT) + (size_t)sidx * P * P, sq->tw_df,
-              sq->served_off, sq->served_lin, sq->served_local, sq->rows, NN, ufc[f_cur]);
-        else
-          k_sq_eval<<<dim3(n_sq, (n_f + 1) / 2), kSqEvalThreads, sm_ev, s>>>(
-              n_f, sqZ, sqT + (size_t)sidx * P * P, sq->tw, sq->served_off, sq->served_lin,
-              sq->served_local, sq->rows, NN, ufc[f_cur]);
+        squares_solve(sq->args(), sq->max_rows, NN, n_f, sqZ, sqE, sqT, sidx, ufc[f_cur], s);
       } else {
         if ((st = eval_ufc(sidx * dt, sidx * kUbCfl, ufc[f_cur], nullptr, true))) return st;
       }

@@ -321,6 +321,17 @@ static void fx_limbs(dd x, int32_t* out) {
   out[1] = l;
 }
 
+std::vector<int32_t> fx_twiddle_table(int n) {
+  std::vector<int32_t> out(4 * (size_t)n);
+  for (int t = 0; t < n; ++t) {
+    dd c, s;
+    dd_cos_sin_turn(-(long long)t, n, c, s);
+    fx_limbs(c, &out[4 * (size_t)t]);
+    fx_limbs(s, &out[4 * (size_t)t + 2]);
+  }
+  return out;
+}
+
 std::vector<int64_t> fx_turn_table(int n) {
   std::vector<int64_t> out;
   for (int t = 0; t < n; ++t) {

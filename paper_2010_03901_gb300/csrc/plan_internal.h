@@ -179,6 +179,8 @@ void wave_modes_destroy(fc2d_plan_s* p);
 
 // (cos, sin)(2 pi i/n) 2^62, i < n, rounded (plan.cpp)
 std::vector<int64_t> fx_turn_table(int n);
+// exp(-2 pi i t/n) 2^60 in limbs (re hi, lo, im hi, lo), t < n
+std::vector<int32_t> fx_twiddle_table(int n);
 
 // Plan-time autotuning of launch shapes that change no result (capi.cu).
 fc2d_status tune_plan(fc2d_plan_s* p);
