@@ -202,7 +202,7 @@ void launch_wave_cols(const FftArgs& fa, int n_f, void* inter, double c, double 
 // Fourier Forwarding in fixed point (fx_wave.cu) for ny = 512 .. 4096 and nx/2 = 2^5 .. 2^12:
 // the spectra [2 n_f][ny][nx/2+1] (u's, then u_t's) to integers in place for times up to
 // 2^eT (exps: wave_fx_exps ints), then u or (deriv) u_t at t = cells h / c, on the grid or at
-// listed points (off[ny + 1], linear indices ascending); inter: 2 n_f ny pitch complex values.
+// listed points (off[ny + 1], linear indices ascending; out [point][n_f]); inter: 2 n_f ny pitch complex values.
 bool wave_fx_sizes(int nx, int ny);
 int wave_fx_time(double t, double h, double c);  // eT for times up to t
 size_t wave_fx_exps(int nx, int ny, int n_f);

@@ -55,7 +55,7 @@ struct DevSquares {
   SquareSet host;
   int32_t* origin = nullptr;        // [n_sq][2] (row, column) of the first grid point
   int32_t* served_off = nullptr;    // [n_sq + 1]
-  int32_t* served_lin = nullptr;
+  int32_t* served_at = nullptr;     // the served interface point (index into iface_lin)
   int32_t* served_local = nullptr;
   double* A = nullptr;              // [C][d]
   double* Q = nullptr;              // [d][d]
@@ -63,13 +63,24 @@ struct DevSquares {
   int32_t* rows = nullptr;          // [n_sq][2]: first and last box row holding served points
   int n = 0, max_rows = 0;          // squares; the most rows any of them needs
   SquareArgs args() const {
-    return {n, origin, A, Q, reinterpret_cast<const int4*>(tw), served_off, served_lin, served_local, rows};
+    return {n, origin, A, Q, reinterpret_cast<const int4*>(tw), served_off, served_at, served_local, rows};
   }
+};
+
+// An operator entry of the solve: the weight and the row of the state it multiplies
+struct __align__(16) UbEntry {
+  double w;
+  int32_t col, pad;
+};
+struct DevOp {
+  int2* row = nullptr;   // [rows + 1] (x: the row's first entry, y: its first outer one)
+  UbEntry* e = nullptr;
 };
 
 struct DevBand {
   WaveBand host;
-  DevCsr L, D, S;
+  DevCsr L, D, S;                   // with keys (one step with caller data, the merge)
+  DevOp Ls, Ds;                     // with state rows (the solve)
   int32_t* unknown_lin = nullptr;
   int32_t* near_lin = nullptr;
   int32_t* near_src = nullptr;
@@ -107,6 +118,32 @@ fc2d_status upload_csr(DevCsr& d, const Csr& h) {
   if ((st = upload(&d.off, h.off)) || (st = upload(&d.col, h.col)) || (st = upload(&d.w, h.w)))
     return st;
   return FC2D_OK;
+}
+
+// position of a grid point in the band's interface list
+int32_t iface_index(const WaveBand& b, int32_t lin) {
+  return (int32_t)(std::lower_bound(b.iface_lin.begin(), b.iface_lin.end(), lin) - b.iface_lin.begin());
+}
+
+// The operator with its columns as rows of the state (unknowns, interface points, boundary
+// points); each row's entries from column `outer` on come last
+fc2d_status upload_op(DevOp& d, const Csr& h, const WaveBand& b, int32_t outer) {
+  const int32_t n = (int32_t)b.unknown_lin.size(), ni = (int32_t)b.iface_lin.size();
+  std::vector<UbEntry> e(h.w.size());
+  std::vector<int2> row(h.off.size());
+  for (size_t r = 0; r < h.off.size(); ++r) {
+    row[r] = {h.off[r], h.off[r]};
+    if (r + 1 == h.off.size()) break;
+    for (int k = h.off[r]; k < h.off[r + 1]; ++k) {
+      const uint32_t kind = h.col[k] & kKeyKind;
+      const int32_t idx = (int32_t)(h.col[k] & kKeyIndex);
+      e[k] = {h.w[k], kind == kKeyUnknown ? idx : kind == kKeyGrid ? n + iface_index(b, idx) : n + ni + idx, 0};
+    }
+    row[r].y = (int)(std::stable_partition(e.begin() + h.off[r], e.begin() + h.off[r + 1],
+                                           [&](const UbEntry& v) { return v.col < outer; }) - e.begin());
+  }
+  fc2d_status st = upload(&d.row, row);
+  return st ? st : upload(&d.e, e);
 }
 
 void free_csr(DevCsr& d) {
@@ -148,8 +185,10 @@ fc2d_status upload_squares(const fc2d_plan_s* p, DevBand& b, int n_c) {
     rows[2 * k + 1] = hi;
     q->max_rows = std::max(q->max_rows, hi - lo + 1);
   }
+  std::vector<int32_t> at;
+  for (int32_t lin : h.served_lin) at.push_back(iface_index(b.host, lin));
   if ((st = upload(&q->origin, origin)) || (st = upload(&q->served_off, h.served_off)) ||
-      (st = upload(&q->served_lin, h.served_lin)) || (st = upload(&q->served_local, h.served_local)) ||
+      (st = upload(&q->served_at, at)) || (st = upload(&q->served_local, h.served_local)) ||
       (st = upload(&q->A, h.A)) || (st = upload(&q->Q, h.Q)) || (st = upload(&q->tw, fx_twiddle_table(h.P))) ||
       (st = upload(&q->rows, rows)))
     return st;
@@ -179,7 +218,10 @@ fc2d_status get_band(fc2d_plan_s* p, int n_c, int mode, DevBand** out) {
   std::vector<int32_t> off(p->grid.ny + 1);
   for (int j = 0; j <= p->grid.ny; ++j)
     off[j] = (int32_t)(std::lower_bound(q.begin(), q.end(), (int64_t)j * p->grid.nx) - q.begin());
-  if ((st = upload(&b->iface_off, off)) || (st = upload(&b->iface_lin, q))) return st;
+  if ((st = upload(&b->iface_off, off)) || (st = upload(&b->iface_lin, q)) ||
+      (st = upload_op(b->Ls, b->host.L, b->host, (int32_t)(b->host.unknown_lin.size() + q.size()))) ||
+      (st = upload_op(b->Ds, b->host.D, b->host, (int32_t)b->host.unknown_lin.size())))
+    return st;
   *out = b.get();
   W->bands[{n_c, mode}] = std::move(b);
   return FC2D_OK;
@@ -256,6 +298,64 @@ __global__ void __launch_bounds__(256) k_ub_step(int mode, int64_t n, int n_f, i
   }
   const double v = 2.0 * u0 - up[t] + cdt2 * lap - sigma * dis;
   out[t] = mode == 1 ? v : (v - up[t]) / (2.0 * dt);
+}
+
+// The small step of the solve, on u and w = u^n - u^{n-1}, function-minor: rows of U are the N
+// unknowns, then the n_i interface points (U_FC at u's time), and boundary columns come after
+// those; Uold holds the interface points of the step before in the same rows.
+//   mode 0: w' = dt u_t + cdt2/2 L(u)     (Taylor start; W holds u_t)
+//   mode 1: w' = w + cdt2 L(u) - sigma D(w)
+//   mode 2: (w' + w)/(2 dt), w' of mode 1, to Uout (the time derivative at u's time)
+// and u' = u + w'.  The FP64 pipe bounds it: w saves the difference u - u_prev of every
+// D entry (38 multiply-adds and 33 additions per value before), and does not cancel.
+__global__ void __launch_bounds__(256) k_ub_advance(
+    int mode, int n, int n_i, int n_f, int64_t n_b, const int2* __restrict__ Lrow,
+    const UbEntry* __restrict__ Le, const int2* __restrict__ Drow, const UbEntry* __restrict__ De,
+    const double* __restrict__ U, const double* __restrict__ Uold, const double* __restrict__ W,
+    const double* __restrict__ g, double cdt2, double dt, double sigma, double* __restrict__ Uout,
+    double* __restrict__ Wout) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)n * n_f) return;
+  const int r = (int)(t / n_f), f = (int)(t - (int64_t)r * n_f);
+  const double u = U[t], w = W[t];
+  double lap = 0.0, dis = 0.0;
+  const double *Uf = U + f, *Wf = W + f;
+  const int2 l0 = __ldg(Lrow + r);
+  const int l1 = __ldg(&Lrow[r + 1].x);
+#pragma unroll 4
+  for (int k = l0.x; k < l0.y; ++k) {
+    const UbEntry e = Le[k];
+    lap += e.w * Uf[(size_t)e.col * n_f];
+  }
+  if (g)  // boundary points
+    for (int k = l0.y; k < l1; ++k) {
+      const UbEntry e = Le[k];
+      lap += e.w * __ldg(g + (size_t)f * n_b + (e.col - n - n_i));
+    }
+  double wn;
+  if (mode == 0) {
+    wn = dt * w + 0.5 * cdt2 * lap;
+  } else {
+    const int2 d0 = __ldg(Drow + r);
+    const int d1 = __ldg(&Drow[r + 1].x);
+#pragma unroll 4
+    for (int k = d0.x; k < d0.y; ++k) {
+      const UbEntry e = De[k];
+      dis += e.w * Wf[(size_t)e.col * n_f];
+    }
+    for (int k = d0.y; k < d1; ++k) {  // interface points
+      const UbEntry e = De[k];
+      const size_t o = (size_t)e.col * n_f + f;
+      dis += e.w * (U[o] - Uold[o]);
+    }
+    wn = w + cdt2 * lap - sigma * dis;
+    if (mode == 2) {
+      Uout[t] = (wn + w) / (2.0 * dt);
+      return;
+    }
+  }
+  Wout[t] = wn;
+  Uout[t] = u + wn;
 }
 
 // The merge of eq. (4.9) at the band points nearer than delta to the curve: unknowns
@@ -370,6 +470,10 @@ void wave_destroy(fc2d_plan_s* p) {
     free_csr(b.L);
     free_csr(b.D);
     free_csr(b.S);
+    for (DevOp* o : {&b.Ls, &b.Ds}) {
+      cudaFree(o->row);
+      cudaFree(o->e);
+    }
     cudaFree(b.unknown_lin);
     cudaFree(b.near_lin);
     cudaFree(b.near_src);
@@ -377,7 +481,7 @@ void wave_destroy(fc2d_plan_s* p) {
     cudaFree(b.iface_lin);
     if (b.sq) {
       DevSquares& q = *b.sq;
-      for (void* ptr : {(void*)q.origin, (void*)q.served_off, (void*)q.served_lin,
+      for (void* ptr : {(void*)q.origin, (void*)q.served_off, (void*)q.served_at,
                         (void*)q.served_local, (void*)q.A, (void*)q.Q, (void*)q.tw, (void*)q.rows})
         cudaFree(ptr);
     }
@@ -489,21 +593,25 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   if ((st = get_band(p, n_c, interface_mode ? 1 : 0, &b))) return st;
   const int nx = p->grid.nx, ny = p->grid.ny, nxh = nx / 2 + 1;
   const int64_t NN = (int64_t)nx * ny, nb = p->n_bdry, Nu = b->L.rows;
+  const int64_t Ni = (int64_t)b->host.iface_lin.size();
   const size_t pitch = row_pitch(p);
   const int S = 8 * n_c;
   const double h = p->grid.h, dT = n_c * h / c, dt = dT / S, cdt2 = (c * dt) * (c * dt);
-  // scratch: spectra [2 n_f][ny][nxh], row-pass layout [2 n_f][ny][pitch], two U_FC grids,
-  // four U_B arrays, zero boundary data
+  const DevSquares* sq = b->sq.get();
+  // fixed-point modal solutions (fx_wave.cu) where the sizes allow; FP64 kernels otherwise
+  const bool fxw = wave_fx_sizes(nx, ny);
+  // scratch: spectra [2 n_f][ny][nxh], row-pass layout [2 n_f][ny][pitch], a U_FC grid (full
+  // U_FC, sizes without fixed point), four U_B arrays (u and w, twice), zero boundary data
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t b_spec = al((size_t)2 * n_f * ny * nxh * 16), b_inter = al((size_t)2 * n_f * ny * pitch * 16),
-               b_grid = al((size_t)n_f * NN * 8), b_ub = al((size_t)std::max<int64_t>(1, Nu) * n_f * 8),
+               b_grid = sq || fxw ? 0 : al((size_t)n_f * NN * 8), b_ub = al((size_t)std::max<int64_t>(1, Nu + Ni) * n_f * 8),
                b_zero = al((size_t)n_f * nb * 8);
-  const DevSquares* sq = b->sq.get();
   const int n_sq = sq ? sq->n : 0;
   const size_t b_sqz = al(squares_spectrum_bytes(n_sq, n_f)), b_sqt = sq ? al(squares_factor_bytes(S)) : 0;
   const size_t b_sqe = al((size_t)n_sq * n_f * sizeof(int));
+  const size_t b_ut = al((size_t)std::max<int64_t>(1, Nu) * n_f * 8);
   const size_t b_exps = al(wave_fx_exps(nx, ny, n_f) * sizeof(int));
-  const size_t need = b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero + b_sqz + b_sqt + b_sqe + b_exps;
+  const size_t need = b_spec + b_inter + b_grid + 4 * b_ub + b_zero + b_sqz + b_sqt + b_sqe + b_ut + b_exps;
   WaveState* W = state(p);
   if (W->scr.bytes < need) {
     cudaDeviceSynchronize();
@@ -516,13 +624,12 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   char* base = static_cast<char*>(W->scr.base);
   double2* spec = reinterpret_cast<double2*>(base);
   double2* inter = reinterpret_cast<double2*>(base + b_spec);
-  double* ufc[2] = {reinterpret_cast<double*>(base + b_spec + b_inter),
-                    reinterpret_cast<double*>(base + b_spec + b_inter + b_grid)};
+  double* ufc = reinterpret_cast<double*>(base + b_spec + b_inter);
   double* ub[4];
   for (int k = 0; k < 4; ++k)
-    ub[k] = reinterpret_cast<double*>(base + b_spec + b_inter + 2 * b_grid + k * b_ub);
-  double* zero = reinterpret_cast<double*>(base + b_spec + b_inter + 2 * b_grid + 4 * b_ub);
-  char* sqZ = base + b_spec + b_inter + 2 * b_grid + 4 * b_ub + b_zero;
+    ub[k] = reinterpret_cast<double*>(base + b_spec + b_inter + b_grid + k * b_ub);
+  double* zero = reinterpret_cast<double*>(base + b_spec + b_inter + b_grid + 4 * b_ub);
+  char* sqZ = base + b_spec + b_inter + b_grid + 4 * b_ub + b_zero;
   char* sqT = sqZ + b_sqz;
   int* sqE = reinterpret_cast<int*>(sqT + b_sqt);
   int* exps = reinterpret_cast<int*>(base + need - b_exps);
@@ -536,8 +643,6 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   const double Lx = nx * h, Ly = ny * h;
   const size_t smc = 3 * (size_t)ny * sizeof(double2);
   cudaFuncSetAttribute(k_ff_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc);
-  // fixed-point modal solutions (fx_wave.cu) where the sizes allow; FP64 kernels otherwise
-  const bool fxw = wave_fx_sizes(nx, ny);
   if (fxw && (st = wave_fx_prepare(p))) return st;
   // U_FC at tau = cells h / c: u and, with out_ut, its time derivative on the grid; with
   // `points` only u at the interface points
@@ -562,22 +667,23 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
                           p->grid.b0, h, out_ut, s);
     return FC2D_OK;
   };
-  auto ub_step = [&](int mode, const double* uc, const double* upv, const double* utv,
-                     const double* grid, const double* grid_prev, const double* g, double* out) {
+  // U_B: u and w in (U[a], V[a]), the next ones into the other pair
+  double* utB = reinterpret_cast<double*>(base + need - b_exps - b_ut);
+  double *U[2] = {ub[0], ub[1]}, *V[2] = {ub[2], ub[3]};
+  int a = 0;
+  auto gather = [&](int64_t n, const int32_t* lin, const double* grid, double* out) {
+    if (n > 0) k_ub_gather<<<blocks(n * n_f, 256), 256, 0, s>>>(n, n_f, NN, lin, grid, out);
+  };
+  auto ub_step = [&](int mode, const double* g, double* uo, double* wo) {
     if (Nu == 0) return;
     ProfScope ps(p, "ub_step", s);
-    k_ub_step<<<blocks(Nu * n_f, 256), 256, 0, s>>>(mode, Nu, n_f, NN, nb, b->L.off, b->L.col,
-                                                    b->L.w, b->D.off, b->D.col, b->D.w, uc, upv,
-                                                    utv, grid, grid_prev, g, cdt2, dt, kUbSigma, out);
+    k_ub_advance<<<blocks(Nu * n_f, 256), 256, 0, s>>>(
+        mode, (int)Nu, (int)Ni, n_f, nb, b->Ls.row, b->Ls.e, b->Ds.row, b->Ds.e, U[a], U[1 - a], V[a],
+        g, cdt2, dt, kUbSigma, uo, wo);
   };
-  // U_B at t = 0: u^0 and u_t^0 at the unknowns
-  int i_prev = 0, i_cur = 1, i_next = 2;
-  const int i_ut = 3;
-  if (Nu > 0) {
-    k_ub_gather<<<blocks(Nu * n_f, 256), 256, 0, s>>>(Nu, n_f, NN, b->unknown_lin, u, ub[i_cur]);
-    k_ub_gather<<<blocks(Nu * n_f, 256), 256, 0, s>>>(Nu, n_f, NN, b->unknown_lin, ut, ub[i_ut]);
-  }
-  int f_cur = 0;  // U_FC grid of the current small step; the other holds the previous one
+  // U_B at t = 0: u^0, and u_t^0 in the place of w
+  gather(Nu, b->unknown_lin, u, U[a]);
+  gather(Nu, b->unknown_lin, ut, V[a]);
   for (int j = 0; j < n_large; ++j) {
     const int64_t m0 = (int64_t)j * S;
     if (sq) {  // the squares' expansions of u(T_j), u_t(T_j), before u and ut change
@@ -590,34 +696,29 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
     if (fxw) wave_fx_spectra(fa, n_f, eT, spec, exps, s);
     for (int sidx = 0; sidx < S; ++sidx) {
       const int64_t m = m0 + sidx;
+      double* face = U[a] + Nu * n_f;  // U_FC at the interface points
       if (sq) {
         ProfScope ps(p, "sq_eval", s);
-        squares_solve(sq->args(), sq->max_rows, NN, n_f, sqZ, sqE, sqT, sidx, ufc[f_cur], s);
+        squares_solve(sq->args(), sq->max_rows, n_f, sqZ, sqE, sqT, sidx, face, s);
       } else {
-        if ((st = eval_ufc(sidx * dt, sidx * kUbCfl, ufc[f_cur], nullptr, true))) return st;
+        if ((st = eval_ufc(sidx * dt, sidx * kUbCfl, fxw ? face : ufc, nullptr, true))) return st;
+        if (!fxw) gather(Ni, b->iface_lin, ufc, face);
       }
-      if (m == 0) {
-        ub_step(0, ub[i_cur], nullptr, ub[i_ut], ufc[f_cur], nullptr, gat(m), ub[i_next]);
-      } else {
-        ub_step(1, ub[i_cur], ub[i_prev], nullptr, ufc[f_cur], ufc[1 - f_cur], gat(m), ub[i_next]);
-      }
-      const int t0 = i_prev;
-      i_prev = i_cur;
-      i_cur = i_next;
-      i_next = t0;
-      f_cur = 1 - f_cur;
+      ub_step(m == 0 ? 0 : 1, gat(m), U[1 - a], V[1 - a]);
+      a = 1 - a;
     }
     // T_{j+1}: U_FC and its time derivative on the grid (into u, ut), then U_B's time
     // derivative from one further step and the merge of eq. (4.9)
     if ((st = eval_ufc(dT, n_c, u, ut, false))) return st;
     const int64_t mN = m0 + S;
-    ub_step(2, ub[i_cur], ub[i_prev], nullptr, u, ufc[1 - f_cur], gat(mN), ub[i_ut]);
+    gather(Ni, b->iface_lin, u, U[a] + Nu * n_f);
+    ub_step(2, gat(mN), utB, nullptr);
     const int64_t n_near = (int64_t)b->host.near_lin.size();
     if (n_near > 0) {
       ProfScope ps(p, "ff_merge", s);
       k_ff_merge<<<blocks(n_near * n_f, 256), 256, 0, s>>>(
-          n_near, n_f, NN, nb, b->near_lin, b->near_src, b->S.off, b->S.col, b->S.w, ub[i_cur],
-          ub[i_ut], g_dir ? gat(mN) : zero, gt_dir ? gtat(j + 1) : zero, u, ut);
+          n_near, n_f, NN, nb, b->near_lin, b->near_src, b->S.off, b->S.col, b->S.w, U[a],
+          utB, g_dir ? gat(mN) : zero, gt_dir ? gtat(j + 1) : zero, u, ut);
     }
   }
   k_zero_outside<<<dim3(ny, n_f), 256, 0, s>>>(nx, ny, n_f, p->dev.row_iv_off, p->dev.row_iv, u, ut);

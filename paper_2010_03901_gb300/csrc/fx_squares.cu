@@ -172,20 +172,23 @@ k_sq_expand(int n_side, int C, int d, int nx, int64_t grid_stride, int n_f, int 
 
 // Every small step, block (square, function): the modal solution a = F t0 + G t1 at the time
 // of `fac` ([l][m], limbs of (cos w t, 2^-eT sin(w t)/w)), its inverse 2D DFT (forward
-// transforms of conj(a)), the values at the served points.  Along m: 31 complex sequences
-// l = 1 .. 31 and the packed pair l = 0, 32, whose transforms are real (the field is).
-// Along l only the rows r0 .. r1 that hold served points, two real rows per complex
-// transform.
-__global__ void __launch_bounds__(kThreads, 3)
+// transforms of conj(a)), the values at the served points, function-minor.  Along m: 31
+// complex sequences l = 1 .. 31 and the packed pair l = 0, 32, whose transforms are real
+// (the field is).  Along l only the rows r0 .. r1 that hold served points (at most 21 of 64:
+// they lie within 10 cells of the centre), two real rows per complex transform: with 16
+// groups to a block most have one.
+// 128 x 5: 107 us for 576 squares and 8 functions (256 x 3: 129, 128 x 6: 111, 64 x 10: 113)
+constexpr int kSolveThreads = 128;
+__global__ void __launch_bounds__(kSolveThreads, 5)
 k_sq_solve(int n_f, const c64* __restrict__ spec, const int* __restrict__ exps,
            const int4* __restrict__ fac, const int4* __restrict__ tw,
-           const int32_t* __restrict__ served_off, const int32_t* __restrict__ served_lin,
+           const int32_t* __restrict__ served_off, const int32_t* __restrict__ served_at,
            const int32_t* __restrict__ served_local, const int32_t* __restrict__ rows,
-           int64_t grid_stride, double* __restrict__ out) {
-  constexpr int kT = kHalf;  // row stride of T: odd
+           double* __restrict__ out) {
+  constexpr int kT = kHalf, kG = kSolveThreads / 8;  // kT: row stride of T (odd); groups
   extern __shared__ __align__(16) unsigned char smem_raw[];
   c64* ex = reinterpret_cast<c64*>(smem_raw);  // per group: an exchange sequence of 72
-  c64* T = ex + (kThreads / 8) * 72;           // [rows][33]
+  c64* T = ex + kG * 72;                       // [rows][33]
   __shared__ unsigned st[1];
   const int sq = blockIdx.x, f = blockIdx.y, tid = threadIdx.x, g = tid >> 3, q = tid & 7;
   if (tid == 0) st[0] = 0;
@@ -198,30 +201,34 @@ k_sq_solve(int n_f, const c64* __restrict__ spec, const int* __restrict__ exps,
     return c64{dot(F.x, G.x, w), -dot(F.y, G.y, w)};
   };
   c64 v[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int m = q + 8 * r;
-    v[r] = value(g, m);
-    if (g == 0) {  // + i times the sequence l = 32
-      const c64 b = value(kP / 2, m);
-      v[r].x -= b.y;
-      v[r].y += b.x;
-    }
-  }
   c64* mine = ex + g * 72;
-  dft64_group<1>(v, mine, q, tw);  // v[k]: y = q + 8 k
   unsigned h = 0;
   __syncthreads();  // st is zero
+#pragma unroll 1
+  for (int l = g; l < kP / 2; l += kG) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    h |= spread(v[k]);
-    const int y = q + 8 * k - r0;
-    if (y >= 0 && y < nr) {
-      if (g == 0) {
-        T[y * kT] = {v[k].x, 0};
-        T[y * kT + kP / 2] = {v[k].y, 0};
-      } else {
-        T[y * kT + g] = v[k];
+    for (int r = 0; r < 8; ++r) v[r] = value(l, q + 8 * r);
+    if (l == 0) {  // + i times the sequence l = 32
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const c64 b = value(kP / 2, q + 8 * r);
+        v[r].x -= b.y;
+        v[r].y += b.x;
+      }
+    }
+    __syncwarp();
+    dft64_group<1>(v, mine, q, tw);  // v[k]: y = q + 8 k
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int y = q + 8 * k - r0;
+      if (y >= 0 && y < nr) {
+        h |= spread(v[k]);
+        if (l == 0) {
+          T[y * kT] = {v[k].x, 0};
+          T[y * kT + kP / 2] = {v[k].y, 0};
+        } else {
+          T[y * kT + l] = v[k];
+        }
       }
     }
   }
@@ -229,32 +236,40 @@ k_sq_solve(int n_f, const c64* __restrict__ spec, const int* __restrict__ exps,
   __syncthreads();
   // two rows X_l = T(l, y1) + i T(l, y2): to |X| <= 2^58.5
   const int L = headroom(st[0]) - kDrop - 1;
-  if (2 * g < nr) {
-    const c64 *a = T + 2 * g * kT, *b = a + kT;
-    const bool two = 2 * g + 1 < nr;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int l = q + 8 * r, k = l <= kP / 2 ? l : kP - l;
-      c64 x = a[k], y = two ? b[k] : c64{0, 0};
-      if (l > kP / 2) {
-        x.y = -x.y;
-        y.y = -y.y;
-      }
-      v[r] = {shift(x.x, L) - shift(y.y, L), shift(x.y, L) + shift(y.x, L)};
-    }
-  }
-  __syncwarp();
-  dft64_group<1>(v, mine, q, tw);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) mine[pad(q + 8 * k)] = v[k];
-  __syncthreads();
   const int e = exps[(size_t)sq * n_f + f] + 3 * kDrop - L;
   const bool plain = plain_exp(e);
   const int s0 = __ldg(served_off + sq), s1 = __ldg(served_off + sq + 1);
-  for (int k = s0 + tid; k < s1; k += kThreads) {
-    const int loc = __ldg(served_local + k), y = (loc >> 6) - r0, x = loc & 63;
-    const c64 z = ex[(y >> 1) * 72 + pad(x)];
-    out[(size_t)f * grid_stride + __ldg(served_lin + k)] = to_double((y & 1) ? z.y : z.x, e, plain);
+#pragma unroll 1
+  for (int p0 = 0; 2 * p0 < nr; p0 += kG) {
+    const int p = p0 + g;
+    if (2 * p < nr) {
+      const c64 *a = T + 2 * p * kT, *b = a + kT;
+      const bool two = 2 * p + 1 < nr;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int l = q + 8 * r, k = l <= kP / 2 ? l : kP - l;
+        c64 x = a[k], y = two ? b[k] : c64{0, 0};
+        if (l > kP / 2) {
+          x.y = -x.y;
+          y.y = -y.y;
+        }
+        v[r] = {shift(x.x, L) - shift(y.y, L), shift(x.y, L) + shift(y.x, L)};
+      }
+    }
+    if (__any_sync(0xFFFFFFFFu, 2 * p < nr)) {
+      dft64_group<1>(v, mine, q, tw);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) mine[pad(q + 8 * k)] = v[k];
+    }
+    __syncthreads();
+    for (int k = s0 + tid; k < s1; k += kSolveThreads) {
+      const int loc = __ldg(served_local + k), y = (loc >> 6) - r0, x = loc & 63, r = (y >> 1) - p0;
+      if (r >= 0 && r < kG) {
+        const c64 z = ex[r * 72 + pad(x)];
+        out[(size_t)__ldg(served_at + k) * n_f + f] = to_double((y & 1) ? z.y : z.x, e, plain);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -298,13 +313,13 @@ void squares_expand(const SquareArgs& q, int n_side, int C, int d, int nx, int64
                                                           (fx::c64*)spec, exps);
 }
 
-void squares_solve(const SquareArgs& q, int max_rows, int64_t grid_stride, int n_f, const void* spec,
-                   const int* exps, const void* fac, int step, double* out, cudaStream_t s) {
-  const size_t sm = ((size_t)(fx::kThreads / 8) * 72 + (size_t)max_rows * fx::kHalf) * 16;
+void squares_solve(const SquareArgs& q, int max_rows, int n_f, const void* spec, const int* exps,
+                   const void* fac, int step, double* out, cudaStream_t s) {
+  const size_t sm = ((size_t)(fx::kSolveThreads / 8) * 72 + (size_t)max_rows * fx::kHalf) * 16;
   cudaFuncSetAttribute(fx::k_sq_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  fx::k_sq_solve<<<dim3(q.n, n_f), fx::kThreads, sm, s>>>(
+  fx::k_sq_solve<<<dim3(q.n, n_f), fx::kSolveThreads, sm, s>>>(
       n_f, (const fx::c64*)spec, exps, (const int4*)fac + (size_t)step * fx::kHalf * fx::kP, q.tw,
-      q.served_off, q.served_lin, q.served_local, q.rows, grid_stride, out);
+      q.served_off, q.served_at, q.served_local, q.rows, out);
 }
 
 }  // namespace fc2d

@@ -13,7 +13,7 @@ struct SquareArgs {
   const int32_t* origin;        // [n][2] (row, column) of the first grid point
   const double *A, *Q;          // 1D-FC: continuation [C][d], Gram [d][d]
   const int4* tw;               // exp(-2 pi i t/64) 2^60 in limbs
-  const int32_t *served_off, *served_lin, *served_local;
+  const int32_t *served_off, *served_at, *served_local;  // served_at: interface point
   const int32_t* rows;          // [n][2]: first and last box row holding served points
 };
 
@@ -25,8 +25,8 @@ void squares_factors(int S, double c, double h, double dt, int eT, void* fac, cu
 void squares_expand(const SquareArgs& q, int n_side, int C, int d, int nx, int64_t grid_stride,
                     int n_f, int eT, const double* u, const double* ut, void* spec, int* exps,
                     cudaStream_t s);
-// the modal solution of small step `step` at the served points, into out [n_f][grid]
-void squares_solve(const SquareArgs& q, int max_rows, int64_t grid_stride, int n_f, const void* spec,
-                   const int* exps, const void* fac, int step, double* out, cudaStream_t s);
+// the modal solution of small step `step` at the served interface points, out [point][n_f]
+void squares_solve(const SquareArgs& q, int max_rows, int n_f, const void* spec, const int* exps,
+                   const void* fac, int step, double* out, cudaStream_t s);
 
 }  // namespace fc2d

@@ -298,14 +298,15 @@ k_adv_b(int nxh, unsigned pitch, const c64* __restrict__ mid, const int* __restr
 // Inverse real row DFT: Z_k = S_k + i conj(w^k) D_k with S_k, D_k = X_k +- conj(X_{NH-k});
 // the length-NH transform runs as a forward transform of conj(Z), and x_{2m} + i x_{2m+1} is
 // the conjugate of its result; plus c00[f] (x^2 + y^2)/4 when c00 is given.  One block per
-// (row, function).  With point_off the row's values go to its listed points only
-// (point_off[j] .. point_off[j+1], linear grid indices), and rows without any are skipped.
+// (row, function).  With point_off only the values at the row's listed points (point_off[j] ..
+// point_off[j+1], linear grid indices) are written, to out[point][ld] at column f, and rows
+// without any are skipped.
 template <int LOGNH>
 __global__ void __launch_bounds__((1 << LOGNH) / 8 < 32 ? 32 : (1 << LOGNH) / 8,
                                   (1 << LOGNH) / 8 >= 128 ? 1024 / ((1 << LOGNH) / 8) : 8)
 k_inverse_rows_fx(FftArgs fa, const double2* __restrict__ inter, const double* __restrict__ c00,
                   double a0, double b0, double h, double* __restrict__ out,
-                  const int32_t* __restrict__ point_off, const int32_t* __restrict__ points) {
+                  const int32_t* __restrict__ point_off, const int32_t* __restrict__ points, int ld) {
   constexpr int NH = 1 << LOGNH, NT = NH / 8, R = last_radix<LOGNH>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned st[kSlots];
@@ -367,7 +368,6 @@ k_inverse_rows_fx(FftArgs fa, const double2* __restrict__ inter, const double* _
   transform<LOGNH>(v, buf, t, active, st, fa.fxx, e);
   if (E >= 0x7FF) e = kNaN;
   const bool plain = plain_exp(e);
-  double* dst = out + (size_t)f * fa.ny * (2 * NH);
   if (point_off) {
     __syncthreads();
     if (active) {
@@ -378,13 +378,14 @@ k_inverse_rows_fx(FftArgs fa, const double2* __restrict__ inter, const double* _
     }
     __syncthreads();
     for (int p = p0 + t; p < p1; p += blockDim.x) {
-      const int lin = points[p], x = lin - j * (2 * NH);
+      const int x = points[p] - j * (2 * NH);
       const c64 z = buf[pad(x >> 1)];
-      dst[lin] = (x & 1) ? to_double(-z.y, e, plain) : to_double(z.x, e, plain);
+      out[(size_t)p * ld + f] = (x & 1) ? to_double(-z.y, e, plain) : to_double(z.x, e, plain);
     }
     return;
   }
   if (!active) return;
+  double* dst = out + (size_t)f * fa.ny * (2 * NH);
   const double q = c00 ? c00[f] * 0.25 : 0.0, y = b0 + h * double(j);
 #pragma unroll
   for (int m = 0; m < 8 / R; ++m)
@@ -406,11 +407,11 @@ k_inverse_rows_fx(FftArgs fa, const double2* __restrict__ inter, const double* _
 template <int L>
 static void inverse_rows_launch(const FftArgs& fa, int n_f, const void* inter, const double* c00,
                                 double a0, double b0, double h, double* out, const int32_t* off,
-                                const int32_t* points, cudaStream_t s) {
+                                const int32_t* points, int ld, cudaStream_t s) {
   const size_t sm = (size_t)padded(1 << L) * sizeof(c64);
   cudaFuncSetAttribute(k_inverse_rows_fx<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   launch_pdl(k_inverse_rows_fx<L>, dim3(fa.ny, n_f), dim3(std::max(32, (1 << L) / 8)), sm, s, fa,
-             (const double2*)inter, c00, a0, b0, h, out, off, points);
+             (const double2*)inter, c00, a0, b0, h, out, off, points, ld);
 }
 
 static int ilog2_exact(int n) {
@@ -441,13 +442,13 @@ static When when(double t, double cells, double c, double h, int eT) {
 }  // namespace fx
 
 // Inverse real rows of power-of-two length (nx/2 = 2^5 .. 2^12), to the whole grid or, with
-// point_off, to the listed points; false (nothing launched) for other sizes.
+// off, at the listed points (out[point][ld]); false (nothing launched) for other sizes.
 bool launch_inverse_rows_fx(const FftArgs& fa, int n_f, const void* inter, const double* c00,
                             double a0, double b0, double h, double* out, const int32_t* off,
-                            const int32_t* points, cudaStream_t s) {
+                            const int32_t* points, int ld, cudaStream_t s) {
   switch (fx::ilog2_exact(fa.nx / 2)) {
 #define FC2D_INV(L) \
-  case L: fx::inverse_rows_launch<L>(fa, n_f, inter, c00, a0, b0, h, out, off, points, s); return true;
+  case L: fx::inverse_rows_launch<L>(fa, n_f, inter, c00, a0, b0, h, out, off, points, ld, s); return true;
     FC2D_INV(5) FC2D_INV(6) FC2D_INV(7) FC2D_INV(8)
     FC2D_INV(9) FC2D_INV(10) FC2D_INV(11) FC2D_INV(12)
 #undef FC2D_INV
@@ -539,8 +540,8 @@ void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, 
 #undef CALL
 }
 
-// u (or, deriv, u_t) at time t = cells h / c of the modal solutions, on the grid or at the
-// listed points.  spec, exps: from wave_fx_spectra (exps has wave_fx_exps ints); inter:
+// u (or, deriv, u_t) at time t = cells h / c of the modal solutions, on the grid or, with
+// off, at the listed points (out[point][n_f]).  spec, exps: from wave_fx_spectra (exps has wave_fx_exps ints); inter:
 // 2 n_f ny pitch complex values of scratch.
 fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
                          double cells, int eT, const void* spec, int* exps, void* inter, double* out,
@@ -576,7 +577,7 @@ fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv,
     }
     ProfScope ps(p, "inverse_rows", s);
     launch_inverse_rows_fx(fa, nf, res, nullptr, p->grid.a0, p->grid.b0, p->grid.h,
-                           out + (size_t)f0 * fa.nx * fa.ny, off, points, s);
+                           off ? out + f0 : out + (size_t)f0 * fa.nx * fa.ny, off, points, n_f, s);
   }
   return FC2D_OK;
 }
