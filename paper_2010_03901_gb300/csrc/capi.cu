@@ -157,9 +157,10 @@ FftArgs fft_args(fc2d_plan_s* p) {
   for (int i = 0; i < a.nry; ++i) a.ry[i] = p->fy.radix[i];
   a.twx = f64 ? (const void*)p->fx.tw64 : (const void*)p->fx.tw32;
   a.twy = f64 ? (const void*)p->fy.tw64 : (const void*)p->fy.tw32;
-  a.rtw = f64 ? (const void*)p->rtw64 : (const void*)p->rtw32;
-  a.tsx = f64 ? (const void*)p->fx.tws64 : (const void*)p->fx.tws32;
-  a.tsy = f64 ? (const void*)p->fy.tws64 : (const void*)p->fy.tws32;
+  a.rtw = p->rtw32;
+  a.tsx = p->fx.tws32;
+  a.tsy = p->fy.tws32;
+  a.mix = p->mix;
   a.fxx = reinterpret_cast<const int4*>(p->fx.fxs);
   a.fxy = reinterpret_cast<const int4*>(p->fy.fxs);
   a.fxwx = reinterpret_cast<const int4*>(p->fx.fx);
@@ -794,55 +795,18 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
   cudaSetDevice(p->device);
   Layout L = layout(p, 2 * n_f);
   cudaStream_t s = (cudaStream_t)stream;
-  if (wave_fx_sizes(p->grid.nx, p->grid.ny)) {  // fixed point (fx_wave.cu)
-    const size_t spec = al((size_t)2 * n_f * p->grid.ny * (p->grid.nx / 2 + 1) * 16);
-    const size_t nexp = al(wave_fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int));
-    if ((st = ensure_workspace(p, L.total + spec + nexp)) || (st = wave_fx_prepare(p))) return st;
-    void* S = ws(p, L.total);
-    int* exps = reinterpret_cast<int*>(ws(p, L.total + spec));
-    if ((st = wave_spectra(p, n_f, u0, u0_bdry, ut0, ut0_bdry, S, s))) return st;
-    const FftArgs fa = fft_args(p);
-    const int eT = wave_fx_time(t, p->grid.h, c);
-    wave_fx_spectra(fa, n_f, eT, S, exps, s);
-    for (int k = 0; k < 2; ++k)
-      if ((st = wave_fx_eval(p, fa, n_f, k == 1, c, t, c * t / p->grid.h, eT, S, exps,
-                             ws(p, L.ointer), k ? ut_out : u_out, nullptr, nullptr, s)))
-        return st;
-    return launched("fc2d_wave_interior");
-  }
-  if ((st = ensure_workspace(p, L.total))) return st;
-  const size_t pitch = row_pitch(p);
-  FftArgs fa = fft_args(p);
-  for (int half = 0; half < 2; ++half) {
-    const double* fg = half ? ut0 : u0;
-    const double* fb = half ? ut0_bdry : u0_bdry;
-    double* F = reinterpret_cast<double*>(ws(p, L.oF)) + (size_t)half * n_f * p->prm.B * (p->Cr + 1);
-    double* vals = reinterpret_cast<double*>(ws(p, L.ovals)) + (size_t)half * n_f * p->strip_lin.size();
-    double2* inter = reinterpret_cast<double2*>(ws(p, L.ointer)) + (size_t)half * n_f * p->grid.ny * pitch;
-    {
-      ProfScope ps(p, "gather_blend", s);
-      launch_gather_blend(gather_args(p, fg, fb, F, nullptr, nullptr), n_f, true, s);
-    }
-    {
-      ProfScope ps(p, "interp", s);
-      launch_interp(interp_args(p, p->Cr + 1), n_f, true, F, vals, s);
-    }
-    {
-      ProfScope ps(p, "fft_rows_fused", s);
-      launch_fft_rows(fa, row_args(p), n_f, true, 1, nullptr, fg, vals, inter, s);
-    }
-  }
-  {
-    ProfScope ps(p, "wave_cols", s);
-    launch_wave_cols(fa, n_f, ws(p, L.ointer), c, t, p->grid.nx * p->grid.h,
-                     p->grid.ny * p->grid.h, s);
-  }
-  {
-    ProfScope ps(p, "inverse_rows", s);
-    double2* inter = reinterpret_cast<double2*>(ws(p, L.ointer));
-    launch_inverse_rows(fa, n_f, inter, nullptr, p->grid.a0, p->grid.b0, p->grid.h, u_out, s);
-    launch_inverse_rows(fa, n_f, inter + (size_t)n_f * p->grid.ny * pitch, nullptr, p->grid.a0,
-                        p->grid.b0, p->grid.h, ut_out, s);
-  }
+  const size_t spec = al((size_t)2 * n_f * p->grid.ny * (p->grid.nx / 2 + 1) * 16);
+  const size_t nexp = al(wave_fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int));
+  if ((st = ensure_workspace(p, L.total + spec + nexp)) || (st = wave_fx_prepare(p))) return st;
+  void* S = ws(p, L.total);
+  int* exps = reinterpret_cast<int*>(ws(p, L.total + spec));
+  if ((st = wave_spectra(p, n_f, u0, u0_bdry, ut0, ut0_bdry, S, s))) return st;
+  const FftArgs fa = fft_args(p);
+  const int eT = wave_fx_time(t, p->grid.h, c);
+  wave_fx_spectra(fa, n_f, eT, S, exps, s);
+  for (int k = 0; k < 2; ++k)
+    if ((st = wave_fx_eval(p, fa, n_f, k == 1, c, t, c * t / p->grid.h, eT, S, exps,
+                           ws(p, L.ointer), k ? ut_out : u_out, nullptr, nullptr, s)))
+      return st;
   return launched("fc2d_wave_interior");
 }

@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "../../include/fc2d.h"
+#include "fx_types.h"
 
 struct fc2d_plan_s;
 
@@ -151,12 +152,6 @@ void launch_interp(const InterpArgs& a, int n_f, bool fp64, const void* F, void*
 void launch_assemble(const RowArgs& a, int n_f, bool fp64, const double* f_grid,
                      const void* vals, void* ext, cudaStream_t s);
 
-// 1/(nx ny) for the fixed-point DFT: 2^exp (1 + m 2^-32 + r 2^-64), m = r = 0 for a power
-// of two
-struct FxFactor {
-  int exp, m, r;
-};
-
 struct FftArgs {
   int nx, ny, pitch;          // pitch: complex elements per intermediate row
   int nrx, nry;               // number of radices
@@ -164,13 +159,14 @@ struct FftArgs {
   const void* twx;            // exp(-2 pi i t/(nx/2)) table for the row transform
   const void* twy;            // exp(-2 pi i t/ny)
   const void* rtw;            // exp(-2 pi i k/nx), k <= nx/2
-  const void* tsx;            // per-stage twiddles of the row transform (power-of-two sizes)
-  const void* tsy;            // per-stage twiddles of the column transform
+  const void* tsx;            // FP32: per-stage twiddles of the row transform (power-of-two sizes)
+  const void* tsy;            // of the column transform
   // double plans (fx.cuh): twiddles w 2^60 in 32-bit limbs (re hi, lo, im hi, lo)
   const int4 *fxx, *fxy;      // per stage of the row and column transforms (powers of two)
   const int4 *fxwx, *fxwy;    // w^t of both lengths
   int* exps;                  // two-pass columns: pass A's exponents (fx_exps ints)
   const int4* fxr;            // exp(-2 pi i k/nx), k <= nx/2
+  FxMixed mix;                // sizes that are not powers of two
   FxFactor fxs;               // 1/(nx ny)
   double scale;               // 1/(nx ny)
   int cc4k;                   // columns per block of the 4096-point FP32 column passes
@@ -178,8 +174,13 @@ struct FftArgs {
   int* status;                // device status word (bounded waits record a timeout)
 };
 
-// ints of FftArgs::exps for n_f functions (one per 16 columns and residue of the rows)
-inline size_t fx_exps(int nx, int ny, int n_f) { return (size_t)n_f * (ny / 64 + 1) * (nx / 32 + 1); }
+// ints of FftArgs::exps for n_f functions: one per 16 columns and residue of the rows, of which
+// there are ny/64 (512 .. 4096 rows) or up to sqrt(ny)
+inline size_t fx_exps(int nx, int ny, int n_f) {
+  size_t k = 1;
+  while ((k + 1) * (k + 1) <= (size_t)ny) ++k;
+  return (size_t)n_f * (k > (size_t)ny / 64 || ny > 4096 ? k : ny / 64) * (nx / 32 + 1);
+}
 
 // rows: mode 0 reads an extended grid (ext, type T); mode 1 assembles the extension
 // on the fly from f_grid + strip values; mode 2 likewise from f given at the inside
@@ -196,14 +197,9 @@ void launch_fft_cols(const FftArgs& fa, int n_f, bool fp64, void* inter, void* f
 // imaginary parts, stored as functions 2f and 2f + 1 of `half`
 void launch_complex_spectrum(int nx, int ny, int n_f, bool fp64, const void* half, void* out,
                              cudaStream_t s);
-// Fourier Forwarding: modal advance of [2 n_f] row spectra (u's then u_t's), in place.
-void launch_wave_cols(const FftArgs& fa, int n_f, void* inter, double c, double t, double Lx,
-                      double Ly, cudaStream_t s);
-// Fourier Forwarding in fixed point (fx_wave.cu) for ny = 512 .. 4096 and nx/2 = 2^5 .. 2^12:
-// the spectra [2 n_f][ny][nx/2+1] (u's, then u_t's) to integers in place for times up to
+// Fourier Forwarding in fixed point (fx_wave.cu): the spectra [2 n_f][ny][nx/2+1] (u's, then u_t's) to integers in place for times up to
 // 2^eT (exps: wave_fx_exps ints), then u or (deriv) u_t at t = cells h / c, on the grid or at
 // listed points (off[ny + 1], linear indices ascending; out [point][n_f]); inter: 2 n_f ny pitch complex values.
-bool wave_fx_sizes(int nx, int ny);
 int wave_fx_time(double t, double h, double c);  // eT for times up to t
 size_t wave_fx_exps(int nx, int ny, int n_f);
 fc2d_status wave_fx_prepare(fc2d_plan_s* p);
@@ -211,7 +207,7 @@ void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, 
 fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
                          double cells, int eT, const void* spec, int* exps, void* inter, double* out,
                          const int32_t* off, const int32_t* points, cudaStream_t s);
-// FP64 inverse real row DFT of an [n_f][ny][pitch] half spectrum already inverted along
+// Inverse real row DFT of an [n_f][ny][pitch] half spectrum (double) already inverted along
 // the columns; c00 (NULL allowed) adds c00[f] (x^2 + y^2)/4.
 void launch_inverse_rows(const FftArgs& fa, int n_f, const void* inter, const double* c00,
                          double a0, double b0, double h, double* out, cudaStream_t s);

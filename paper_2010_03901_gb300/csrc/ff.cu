@@ -30,7 +30,6 @@
 #include <string>
 
 #include "fc2d_kernels.cuh"
-#include "fft_generic.cuh"
 #include "fx_squares.h"
 #include "plan_internal.h"
 #include "wave_band.h"
@@ -39,9 +38,6 @@ namespace fc2d {
 
 fc2d_status wave_spectra(fc2d_plan_s* p, int n_f, const double* u, const double* ub,
                          const double* ut, const double* utb, void* spec, cudaStream_t s);
-bool launch_ff_cols_p2(const FftArgs& fa, int n_f, int n_out, const void* spec, void* out,
-                       double c, double tau, double Lx, double Ly, cudaStream_t s);
-
 namespace {
 
 struct DevCsr {
@@ -409,60 +405,12 @@ __global__ void k_zero_outside(int nx, int ny, int n_f, const int32_t* __restric
   }
 }
 
-// Modal advance of the normalised half spectra (F: spec[f], G: spec[n_f + f]) to time
-// tau and the inverse column DFT (a forward transform of the conjugate), into the
-// row-pass layout [n_out][ny][pitch] for the inverse real row DFT: blockIdx.y = 0: a(tau)
-// into out[f]; 1: a'(tau) into out[n_f + f].  One block per (column, output) loops over
-// the functions, so the column's time factors (t0, t1) are computed once: a = F t0 + G t1
-// with (cos w tau, sin(w tau)/w), or (-w sin w tau, cos w tau) for a'; (1, tau) and (0, 1)
-// at w = 0.  Mixed-radix sizes; power-of-two columns take k_ff_cols_p2 (fft_pow2.cu).
-__global__ void __launch_bounds__(256) k_ff_cols(FftArgs fa, int n_f, const double2* __restrict__ spec,
-                                                 double2* __restrict__ out, double c, double tau,
-                                                 double Lx, double Ly) {
-  using C = double2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ny = fa.ny, nxh = fa.nx / 2 + 1, kx = blockIdx.x, which = blockIdx.y;
-  double2* tab = reinterpret_cast<double2*>(smem_raw);
-  C* A = tab + ny;
-  C* S = A + ny;
-  const double two_pi = 6.283185307179586476925286766559;
-  for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
-    const int m = ky <= ny / 2 ? ky : ky - ny;
-    const double fl = kx / Lx, fm = m / Ly;
-    const double w = two_pi * c * sqrt(fl * fl + fm * fm);
-    double t0, t1;
-    if (w == 0.0) {
-      t0 = which ? 0.0 : 1.0;
-      t1 = which ? 1.0 : tau;
-    } else {
-      double sn, co;
-      sincos(w * tau, &sn, &co);
-      t0 = which ? -w * sn : co;
-      t1 = which ? co : sn / w;
-    }
-    tab[ky] = double2{t0, t1};
-  }
-  for (int f = 0; f < n_f; ++f) {
-    const C* colF = spec + (size_t)f * ny * nxh + kx;
-    const C* colG = spec + (size_t)(n_f + f) * ny * nxh + kx;
-    __syncthreads();
-    for (int ky = threadIdx.x; ky < ny; ky += blockDim.x) {
-      const double2 t = tab[ky];
-      const C F = colF[(size_t)ky * nxh], G = colG[(size_t)ky * nxh];
-      A[ky] = C{F.x * t.x + G.x * t.y, -(F.y * t.x + G.y * t.y)};
-    }
-    __syncthreads();
-    const C* r = stockham<double>(A, S, ny, 1, fa.ry, fa.nry, reinterpret_cast<const C*>(fa.twy), 1);
-    C* dst = out + ((size_t)which * n_f + f) * ny * fa.pitch + kx;
-    for (int y = threadIdx.x; y < ny; y += blockDim.x) dst[(size_t)y * fa.pitch] = C{r[y].x, -r[y].y};
-  }
-}
-
 unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
 void wave_destroy(fc2d_plan_s* p) {
+  wave_modes_destroy(p);
   if (!p->wave) return;
   auto* W = static_cast<WaveState*>(p->wave);
   for (auto& kv : W->bands) {
@@ -598,20 +546,17 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   const int S = 8 * n_c;
   const double h = p->grid.h, dT = n_c * h / c, dt = dT / S, cdt2 = (c * dt) * (c * dt);
   const DevSquares* sq = b->sq.get();
-  // fixed-point modal solutions (fx_wave.cu) where the sizes allow; FP64 kernels otherwise
-  const bool fxw = wave_fx_sizes(nx, ny);
-  // scratch: spectra [2 n_f][ny][nxh], row-pass layout [2 n_f][ny][pitch], a U_FC grid (full
-  // U_FC, sizes without fixed point), four U_B arrays (u and w, twice), zero boundary data
+  // scratch: spectra [2 n_f][ny][nxh], row-pass layout [2 n_f][ny][pitch], four U_B arrays (u and w, twice), zero boundary data
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t b_spec = al((size_t)2 * n_f * ny * nxh * 16), b_inter = al((size_t)2 * n_f * ny * pitch * 16),
-               b_grid = sq || fxw ? 0 : al((size_t)n_f * NN * 8), b_ub = al((size_t)std::max<int64_t>(1, Nu + Ni) * n_f * 8),
+               b_ub = al((size_t)std::max<int64_t>(1, Nu + Ni) * n_f * 8),
                b_zero = al((size_t)n_f * nb * 8);
   const int n_sq = sq ? sq->n : 0;
   const size_t b_sqz = al(squares_spectrum_bytes(n_sq, n_f)), b_sqt = sq ? al(squares_factor_bytes(S)) : 0;
   const size_t b_sqe = al((size_t)n_sq * n_f * sizeof(int));
   const size_t b_ut = al((size_t)std::max<int64_t>(1, Nu) * n_f * 8);
   const size_t b_exps = al(wave_fx_exps(nx, ny, n_f) * sizeof(int));
-  const size_t need = b_spec + b_inter + b_grid + 4 * b_ub + b_zero + b_sqz + b_sqt + b_sqe + b_ut + b_exps;
+  const size_t need = b_spec + b_inter + 4 * b_ub + b_zero + b_sqz + b_sqt + b_sqe + b_ut + b_exps;
   WaveState* W = state(p);
   if (W->scr.bytes < need) {
     cudaDeviceSynchronize();
@@ -624,12 +569,11 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   char* base = static_cast<char*>(W->scr.base);
   double2* spec = reinterpret_cast<double2*>(base);
   double2* inter = reinterpret_cast<double2*>(base + b_spec);
-  double* ufc = reinterpret_cast<double*>(base + b_spec + b_inter);
   double* ub[4];
   for (int k = 0; k < 4; ++k)
-    ub[k] = reinterpret_cast<double*>(base + b_spec + b_inter + b_grid + k * b_ub);
-  double* zero = reinterpret_cast<double*>(base + b_spec + b_inter + b_grid + 4 * b_ub);
-  char* sqZ = base + b_spec + b_inter + b_grid + 4 * b_ub + b_zero;
+    ub[k] = reinterpret_cast<double*>(base + b_spec + b_inter + k * b_ub);
+  double* zero = reinterpret_cast<double*>(base + b_spec + b_inter + 4 * b_ub);
+  char* sqZ = base + b_spec + b_inter + 4 * b_ub + b_zero;
   char* sqT = sqZ + b_sqz;
   int* sqE = reinterpret_cast<int*>(sqT + b_sqt);
   int* exps = reinterpret_cast<int*>(base + need - b_exps);
@@ -640,32 +584,12 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   auto gat = [&](int64_t m) { return g_dir ? g_dir + (size_t)m * n_f * nb : nullptr; };
   auto gtat = [&](int64_t j) { return gt_dir ? gt_dir + (size_t)j * n_f * nb : nullptr; };
   FftArgs fa = fft_args(p);
-  const double Lx = nx * h, Ly = ny * h;
-  const size_t smc = 3 * (size_t)ny * sizeof(double2);
-  cudaFuncSetAttribute(k_ff_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc);
-  if (fxw && (st = wave_fx_prepare(p))) return st;
-  // U_FC at tau = cells h / c: u and, with out_ut, its time derivative on the grid; with
-  // `points` only u at the interface points
-  auto eval_ufc = [&](double tau, double cells, double* out_u, double* out_ut, bool points) {
-    const int n_out = out_ut ? 2 : 1;
-    if (fxw) {
-      fc2d_status e = FC2D_OK;
-      for (int k = 0; k < n_out && !e; ++k)
-        e = wave_fx_eval(p, fa, n_f, k == 1, c, tau, cells, eT, spec, exps, inter, k ? out_ut : out_u,
-                         points ? b->iface_off : nullptr, points ? b->iface_lin : nullptr, s);
-      return e;
-    }
-    {
-      ProfScope ps(p, "ff_cols", s);
-      if (!launch_ff_cols_p2(fa, n_f, n_out, spec, inter, c, tau, Lx, Ly, s))
-        k_ff_cols<<<dim3(nxh, n_out), 256, smc, s>>>(fa, n_f, spec, inter, c, tau, Lx, Ly);
-    }
-    ProfScope ps(p, "inverse_rows", s);
-    launch_inverse_rows(fa, n_f, inter, nullptr, p->grid.a0, p->grid.b0, h, out_u, s);
-    if (n_out == 2)
-      launch_inverse_rows(fa, n_f, inter + (size_t)n_f * ny * pitch, nullptr, p->grid.a0,
-                          p->grid.b0, h, out_ut, s);
-    return FC2D_OK;
+  if ((st = wave_fx_prepare(p))) return st;
+  // U_FC at tau = cells h / c: u, or (deriv) its time derivative, on the grid or at the
+  // interface points
+  auto eval_ufc = [&](double tau, double cells, bool deriv, double* out, bool points) {
+    return wave_fx_eval(p, fa, n_f, deriv, c, tau, cells, eT, spec, exps, inter, out,
+                        points ? b->iface_off : nullptr, points ? b->iface_lin : nullptr, s);
   };
   // U_B: u and w in (U[a], V[a]), the next ones into the other pair
   double* utB = reinterpret_cast<double*>(base + need - b_exps - b_ut);
@@ -693,7 +617,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
     }
     if ((st = wave_spectra(p, n_f, u, g_dir ? gat(m0) : zero, ut, gt_dir ? gtat(j) : zero, spec, s)))
       return st;
-    if (fxw) wave_fx_spectra(fa, n_f, eT, spec, exps, s);
+    wave_fx_spectra(fa, n_f, eT, spec, exps, s);
     for (int sidx = 0; sidx < S; ++sidx) {
       const int64_t m = m0 + sidx;
       double* face = U[a] + Nu * n_f;  // U_FC at the interface points
@@ -701,15 +625,14 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
         ProfScope ps(p, "sq_eval", s);
         squares_solve(sq->args(), sq->max_rows, n_f, sqZ, sqE, sqT, sidx, face, s);
       } else {
-        if ((st = eval_ufc(sidx * dt, sidx * kUbCfl, fxw ? face : ufc, nullptr, true))) return st;
-        if (!fxw) gather(Ni, b->iface_lin, ufc, face);
+        if ((st = eval_ufc(sidx * dt, sidx * kUbCfl, false, face, true))) return st;
       }
       ub_step(m == 0 ? 0 : 1, gat(m), U[1 - a], V[1 - a]);
       a = 1 - a;
     }
     // T_{j+1}: U_FC and its time derivative on the grid (into u, ut), then U_B's time
     // derivative from one further step and the merge of eq. (4.9)
-    if ((st = eval_ufc(dT, n_c, u, ut, false))) return st;
+    if ((st = eval_ufc(dT, n_c, false, u, false)) || (st = eval_ufc(dT, n_c, true, ut, false))) return st;
     const int64_t mN = m0 + S;
     gather(Ni, b->iface_lin, u, U[a] + Nu * n_f);
     ub_step(2, gat(mN), utB, nullptr);

@@ -1,5 +1,5 @@
 // Hand-written 2D real-to-complex DFT of the extended grid (eq. (3.1), Section 3.5
-// step 7) for sizes 2^a 3^b 5^c.
+// step 7) for sizes 2^a 3^b 5^c: the dispatch, and the general FP32 kernels.
 //
 // Pass 1 (k_fft_rows): one block per (row, function).  The row of nx reals is loaded
 // into shared memory as nx/2 complex pairs z_n = x_{2n} + i x_{2n+1} -- either from an
@@ -88,38 +88,36 @@ __global__ void __launch_bounds__(256) k_fft_cols(FftArgs fa, int cb,
 
 bool launch_fft_rows_p2(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
                         const double* f_grid, const void* vals, void* inter, cudaStream_t s);
-bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
+bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, int mode,
                          const void* ext, const double* f_grid, const void* vals, void* inter,
                          cudaStream_t s);
 bool launch_fft_cols_p2(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
-bool launch_fft_cols_64n(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
-                         cudaStream_t s);
+bool launch_fft_cols_64n(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
 
+// double plans, in fixed point: power-of-two sizes (fft_fx.cu), others (fft_fx_mixed.cu)
 bool launch_fft_rows_fx(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
                         const double* f_grid, const void* vals, void* inter, cudaStream_t s);
 bool launch_fft_cols_fx(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
+void launch_fft_rows_mixed(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
+                           const double* f_grid, const void* vals, void* inter, cudaStream_t s);
+void launch_fft_cols_mixed(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s);
 
 void launch_fft_rows(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
                      const void* ext, const double* f_grid, const void* vals, void* inter,
                      cudaStream_t s) {
-  if (fp64 ? launch_fft_rows_fx(fa, ra, n_f, mode, ext, f_grid, vals, inter, s)
-           : launch_fft_rows_p2(fa, ra, n_f, mode, ext, f_grid, vals, inter, s))
-    return;
-  if (launch_fft_rows_64n(fa, ra, n_f, fp64, mode, ext, f_grid, vals, inter, s)) return;
-  dim3 grid(fa.ny, n_f);
   if (fp64) {
-    size_t sm = (size_t)fa.nx * sizeof(double2);  // two buffers of nx/2 complex
-    auto k = k_fft_rows<double, double>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<grid, 256, sm, s>>>(fa, ra, mode, (const double*)ext, f_grid, (const double*)vals,
-                            (double2*)inter);
-  } else {
-    size_t sm = (size_t)fa.nx * sizeof(float2);
-    auto k = k_fft_rows<float, float>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<grid, 256, sm, s>>>(fa, ra, mode, (const float*)ext, f_grid, (const float*)vals,
-                            (float2*)inter);
+    if (!launch_fft_rows_fx(fa, ra, n_f, mode, ext, f_grid, vals, inter, s))
+      launch_fft_rows_mixed(fa, ra, n_f, mode, ext, f_grid, vals, inter, s);
+    return;
   }
+  if (launch_fft_rows_p2(fa, ra, n_f, mode, ext, f_grid, vals, inter, s) ||
+      launch_fft_rows_64n(fa, ra, n_f, mode, ext, f_grid, vals, inter, s))
+    return;
+  const size_t sm = (size_t)fa.nx * sizeof(float2);  // two buffers of nx/2 complex
+  auto k = k_fft_rows<float, float>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k<<<dim3(fa.ny, n_f), 256, sm, s>>>(fa, ra, mode, (const float*)ext, f_grid, (const float*)vals,
+                                      (float2*)inter);
 }
 
 static int pick_cb(int ny, size_t csize) {
@@ -131,26 +129,17 @@ static int pick_cb(int ny, size_t csize) {
 
 void launch_fft_cols(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
                      cudaStream_t s) {
-  if (fp64 ? launch_fft_cols_fx(fa, n_f, inter, fhat, s)
-           : launch_fft_cols_p2(fa, n_f, inter, fhat, s))
-    return;
-  if (launch_fft_cols_64n(fa, n_f, fp64, inter, fhat, s)) return;
-  const int ncol = fa.nx / 2 + 1;
   if (fp64) {
-    int cb = pick_cb(fa.ny, sizeof(double2));
-    size_t sm = 2 * (size_t)cb * fa.ny * sizeof(double2);
-    auto k = k_fft_cols<double>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<dim3((ncol + cb - 1) / cb, n_f), 256, sm, s>>>(fa, cb, (const double2*)inter,
-                                                       (double2*)fhat);
-  } else {
-    int cb = pick_cb(fa.ny, sizeof(float2));
-    size_t sm = 2 * (size_t)cb * fa.ny * sizeof(float2);
-    auto k = k_fft_cols<float>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k<<<dim3((ncol + cb - 1) / cb, n_f), 256, sm, s>>>(fa, cb, (const float2*)inter,
-                                                       (float2*)fhat);
+    if (!launch_fft_cols_fx(fa, n_f, inter, fhat, s)) launch_fft_cols_mixed(fa, n_f, inter, fhat, s);
+    return;
   }
+  if (launch_fft_cols_p2(fa, n_f, inter, fhat, s) || launch_fft_cols_64n(fa, n_f, inter, fhat, s)) return;
+  const int ncol = fa.nx / 2 + 1;
+  const int cb = pick_cb(fa.ny, sizeof(float2));
+  const size_t sm = 2 * (size_t)cb * fa.ny * sizeof(float2);
+  auto k = k_fft_cols<float>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k<<<dim3((ncol + cb - 1) / cb, n_f), 256, sm, s>>>(fa, cb, (const float2*)inter, (float2*)fhat);
 }
 
 // Full spectrum of a complex function u + i v from the half spectra A of u and B of v

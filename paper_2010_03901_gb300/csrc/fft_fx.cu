@@ -17,16 +17,6 @@
 namespace fc2d {
 namespace fx {
 
-// X_k and X_{NH-k} (times 2^(1-kDrop), in the block's units) of a real row from its pairs'
-// transform (|z| <= 2^61.5): with zk = Z_k and zl = Z_{NH-k}, e = (zk + conj zl)/2, o = (zk - conj zl)/2,
-// X_k = e - i w^k o, X_{NH-k} = conj(e + i w^k o)
-__device__ __forceinline__ void split_pair(c64 zk, c64 zl, int4 w, c64& xk, c64& xl) {
-  const c64 e = drop(c64{zk.x + zl.x, zk.y - zl.y});
-  const c64 wo = mulw(c64{zk.x - zl.x, zk.y + zl.y}, w);
-  xk = {e.x + wo.y, e.y - wo.x};
-  xl = {e.x - wo.y, -e.y - wo.x};
-}
-
 template <int LOGNH> __host__ __device__ constexpr int row_threads() {
   return (1 << LOGNH) / 8 < 32 ? 32 : (1 << LOGNH) / 8;
 }

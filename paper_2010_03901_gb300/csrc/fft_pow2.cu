@@ -1123,193 +1123,6 @@ static void cols4k_launch(const FftArgs& fa, int n_f, void* inter, void* fhat, c
   }
 }
 
-// ------------------------------------------------------------------------- //
-// Inverse real row DFT (FP64) of rows whose half length NH = 2^LOGNH is a power of
-// two: the inverse of the even/odd split gives Z_k = S_k + i conj(w^k) D_k from X_k and
-// conj(X_{NH-k}), the length-NH transform runs as a forward transform of conj(Z) on the
-// compile-time Stockham stages, and x_{2m} + i x_{2m+1} = conj of its result; plus the
-// quadratic term c00[f] (x^2 + y^2)/4 when c00 is given.  One block per (row, function).
-// ------------------------------------------------------------------------- //
-template <int LOGNH>
-__global__ void __launch_bounds__((1 << LOGNH) / 8)
-    k_inverse_rows_p2(FftArgs fa, const double2* __restrict__ inter,
-                      const double* __restrict__ c00, double a0, double b0, double h,
-                      double* __restrict__ up) {
-  using C = double2;
-  constexpr int NH = 1 << LOGNH, E = 8;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  const int j = blockIdx.x, f = blockIdx.y, t = threadIdx.x;
-  const C* row = inter + ((size_t)f * fa.ny + j) * fa.pitch;
-  const C* rtw = reinterpret_cast<const C*>(fa.rtw);
-  pdl_wait();
-  pdl_trigger();
-  for (int k = t; k < NH; k += blockDim.x) {
-    const C bk = row[k];
-    C bc = row[NH - k];
-    bc.y = -bc.y;  // conj X_{NH-k}
-    const C sm = {bk.x + bc.x, bk.y + bc.y}, d = {bk.x - bc.x, bk.y - bc.y};
-    C w = __ldg(rtw + k);
-    w.y = -w.y;  // conj(w^k)
-    const C dw = {d.x * w.x - d.y * w.y, d.x * w.y + d.y * w.x};
-    buf[pad<double>(k)] = C{sm.x - dw.y, -(sm.y + dw.x)};  // conj(s + i dw)
-  }
-  __syncthreads();
-  block_fft<double, LOGNH, E>(buf, t, true, reinterpret_cast<const C*>(fa.tsx), 1);
-  const double q = c00 ? c00[f] * 0.25 : 0.0;
-  const double y = b0 + h * double(j);
-  double* out = up + ((size_t)f * fa.ny + j) * (2 * NH);
-  for (int m = t; m < NH; m += blockDim.x) {
-    const C z = buf[pad<double>(m)];
-    const double x0 = a0 + h * double(2 * m), x1 = a0 + h * double(2 * m + 1);
-    out[2 * m] = z.x + q * (x0 * x0 + y * y);
-    out[2 * m + 1] = -z.y + q * (x1 * x1 + y * y);
-  }
-}
-
-template <int LOGNH>
-static void inverse_rows_p2_launch(const FftArgs& fa, int n_f, const void* inter,
-                                   const double* c00, double a0, double b0, double h,
-                                   double* out, cudaStream_t s) {
-  const size_t sm = (size_t)padded<double>(1 << LOGNH) * sizeof(double2);
-  cudaFuncSetAttribute(k_inverse_rows_p2<LOGNH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sm);
-  launch_pdl(k_inverse_rows_p2<LOGNH>, dim3(fa.ny, n_f), dim3((1 << LOGNH) / 8), sm, s, fa,
-             (const double2*)inter, c00, a0, b0, h, out);
-}
-
-// ------------------------------------------------------------------------- //
-// Fourier Forwarding modal advance on power-of-two columns (FP64; see wave.cu for the
-// formulas): one block per (column, pair), both columns in place in padded shared
-// memory, the compile-time Stockham stages of block_fft for the forward transforms, the
-// advance, and the inverse transforms as forward transforms of the conjugates.
-// ------------------------------------------------------------------------- //
-template <int LOGNY>
-__global__ void __launch_bounds__((1 << LOGNY) / 8, LOGNY == 11 ? 2 : 1)
-    k_wave_cols_p2(FftArgs fa, int n_f, double2* __restrict__ inter, double c, double t,
-                   double Lx, double Ly) {
-  using C = double2;
-  constexpr int N = 1 << LOGNY, E = 8;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* A = reinterpret_cast<C*>(smem_raw);
-  C* Bv = A + padded<double>(N);
-  const int kx = blockIdx.x, f = blockIdx.y, tid = threadIdx.x;
-  C* colu = inter + (size_t)f * N * fa.pitch + kx;
-  C* colt = inter + (size_t)(n_f + f) * N * fa.pitch + kx;
-  const C* tw = reinterpret_cast<const C*>(fa.tsy);
-  for (int y = tid; y < N; y += blockDim.x) {
-    A[pad<double>(y)] = colu[(size_t)y * fa.pitch];
-    Bv[pad<double>(y)] = colt[(size_t)y * fa.pitch];
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int h = 0; h < 2; ++h) block_fft<double, LOGNY, E>(h ? Bv : A, tid, true, tw, 1);
-  const double two_pi = 6.283185307179586476925286766559;
-  for (int ky = tid; ky < N; ky += blockDim.x) {
-    const int m = ky <= N / 2 ? ky : ky - N;
-    const double fl = kx / Lx, fm = m / Ly;
-    const double w = two_pi * c * sqrt(fl * fl + fm * fm);
-    const C a0 = A[pad<double>(ky)], b0 = Bv[pad<double>(ky)];
-    const C F = C{a0.x * fa.scale, a0.y * fa.scale};
-    const C G = C{b0.x * fa.scale, b0.y * fa.scale};
-    C a, at;
-    if (w == 0.0) {
-      a = C{F.x + t * G.x, F.y + t * G.y};
-      at = G;
-    } else {
-      double sn, co;
-      sincos(w * t, &sn, &co);
-      const double sw = sn / w;
-      a = C{F.x * co + G.x * sw, F.y * co + G.y * sw};
-      at = C{-F.x * w * sn + G.x * co, -F.y * w * sn + G.y * co};
-    }
-    A[pad<double>(ky)] = C{a.x, -a.y};  // conj: inverse by a forward transform
-    Bv[pad<double>(ky)] = C{at.x, -at.y};
-  }
-  __syncthreads();
-#pragma unroll 1
-  for (int h = 0; h < 2; ++h) block_fft<double, LOGNY, E>(h ? Bv : A, tid, true, tw, 1);
-  for (int y = tid; y < N; y += blockDim.x) {
-    const C u = A[pad<double>(y)], v = Bv[pad<double>(y)];
-    colu[(size_t)y * fa.pitch] = C{u.x, -u.y};
-    colt[(size_t)y * fa.pitch] = C{v.x, -v.y};
-  }
-}
-
-template <int LOGNY>
-static void wave_cols_p2_launch(const FftArgs& fa, int n_f, void* inter, double c, double t,
-                                double Lx, double Ly, cudaStream_t s) {
-  const size_t sm = 2 * (size_t)padded<double>(1 << LOGNY) * sizeof(double2);
-  cudaFuncSetAttribute(k_wave_cols_p2<LOGNY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_wave_cols_p2<LOGNY><<<dim3(fa.nx / 2 + 1, n_f), (1 << LOGNY) / 8, sm, s>>>(
-      fa, n_f, (double2*)inter, c, t, Lx, Ly);
-}
-
-// ------------------------------------------------------------------------- //
-// Fourier Forwarding solve, per small step (FP64, ff.cu): the modal advance of the
-// normalised half spectra to time tau (a = F t0 + G t1 with (t0, t1) = (cos w tau,
-// sin(w tau)/w), or for the time derivative (-w sin w tau, cos w tau); (1, tau) and
-// (0, 1) at w = 0) and the inverse column DFT as a forward transform of the conjugate.
-// One block per (column, output) loops over the n_f functions, so the 2 ny time
-// factors of its column are computed once (in shared memory) for all of them; the
-// transform runs on the compile-time Stockham stages in padded shared memory.
-// ------------------------------------------------------------------------- //
-template <int LOGNY>
-__global__ void __launch_bounds__((1 << LOGNY) / 8)
-    k_ff_cols_p2(FftArgs fa, int n_f, const double2* __restrict__ spec, double2* __restrict__ out,
-                 double c, double tau, double Lx, double Ly) {
-  using C = double2;
-  constexpr int N = 1 << LOGNY, E = 8;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* tab = reinterpret_cast<double2*>(smem_raw);
-  C* buf = tab + N;
-  const int nxh = fa.nx / 2 + 1, kx = blockIdx.x, which = blockIdx.y, tid = threadIdx.x;
-  const double two_pi = 6.283185307179586476925286766559;
-  for (int ky = tid; ky < N; ky += blockDim.x) {
-    const int m = ky <= N / 2 ? ky : ky - N;
-    const double fl = kx / Lx, fm = m / Ly;
-    const double w = two_pi * c * sqrt(fl * fl + fm * fm);
-    double t0, t1;
-    if (w == 0.0) {
-      t0 = which ? 0.0 : 1.0;
-      t1 = which ? 1.0 : tau;
-    } else {
-      double sn, co;
-      sincos(w * tau, &sn, &co);
-      t0 = which ? -w * sn : co;
-      t1 = which ? co : sn / w;
-    }
-    tab[ky] = double2{t0, t1};
-  }
-  const C* tw = reinterpret_cast<const C*>(fa.tsy);
-  for (int f = 0; f < n_f; ++f) {
-    const C* colF = spec + (size_t)f * N * nxh + kx;
-    const C* colG = spec + (size_t)(n_f + f) * N * nxh + kx;
-    __syncthreads();  // the table is ready; the previous function's stores are done
-    for (int ky = tid; ky < N; ky += blockDim.x) {
-      const double2 t = tab[ky];
-      const C F = colF[(size_t)ky * nxh], G = colG[(size_t)ky * nxh];
-      buf[pad<double>(ky)] = C{F.x * t.x + G.x * t.y, -(F.y * t.x + G.y * t.y)};
-    }
-    __syncthreads();
-    block_fft<double, LOGNY, E>(buf, tid, true, tw, 1);
-    C* dst = out + ((size_t)which * n_f + f) * N * fa.pitch + kx;
-    for (int y = tid; y < N; y += blockDim.x) {
-      const C r = buf[pad<double>(y)];
-      dst[(size_t)y * fa.pitch] = C{r.x, -r.y};
-    }
-  }
-}
-
-template <int LOGNY>
-static void ff_cols_p2_launch(const FftArgs& fa, int n_f, int n_out, const void* spec, void* out,
-                              double c, double tau, double Lx, double Ly, cudaStream_t s) {
-  const size_t sm = ((size_t)(1 << LOGNY) + padded<double>(1 << LOGNY)) * sizeof(double2);
-  cudaFuncSetAttribute(k_ff_cols_p2<LOGNY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_ff_cols_p2<LOGNY><<<dim3(fa.nx / 2 + 1, n_out), (1 << LOGNY) / 8, sm, s>>>(
-      fa, n_f, (const double2*)spec, (double2*)out, c, tau, Lx, Ly);
-}
-
 template <typename T, typename TV, int L>
 static void rows_launch(const FftArgs& fa, const RowArgs& ra, int n_f, int mode, const void* ext,
                         const double* fg, const void* vals, void* inter, cudaStream_t s) {
@@ -1367,10 +1180,10 @@ bool launch_fft_rows_p2(const FftArgs& fa, const RowArgs& ra, int n_f, int mode,
 
 // FP32 rows of 2 x 64 N2 reals for N2 = 3, 5, 6, 10, 12.  Returns false (nothing launched)
 // for other sizes.
-bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp64, int mode,
+bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, int mode,
                          const void* ext, const double* f_grid, const void* vals, void* inter,
                          cudaStream_t s) {
-  if (fp64 || fa.nx % 128) return false;
+  if (fa.nx % 128) return false;
   switch (fa.nx / 128) {
     case 3: p2::rows64n_launch<3>(fa, ra, n_f, mode, ext, f_grid, vals, inter, s); return true;
     case 5: p2::rows64n_launch<5>(fa, ra, n_f, mode, ext, f_grid, vals, inter, s); return true;
@@ -1383,9 +1196,8 @@ bool launch_fft_rows_64n(const FftArgs& fa, const RowArgs& ra, int n_f, bool fp6
 
 // FP32 columns of 64 N2 points for N2 = 6, 10, 12, 24 (two passes).  Returns false
 // (nothing launched) for other sizes.
-bool launch_fft_cols_64n(const FftArgs& fa, int n_f, bool fp64, void* inter, void* fhat,
-                         cudaStream_t s) {
-  if (fp64 || fa.ny % 64) return false;
+bool launch_fft_cols_64n(const FftArgs& fa, int n_f, void* inter, void* fhat, cudaStream_t s) {
+  if (fa.ny % 64) return false;
   switch (fa.ny / 64) {
     case 6: p2::cols64_launch<2, 3>(fa, n_f, inter, fhat, s); return true;
     case 10: p2::cols64_launch<2, 5>(fa, n_f, inter, fhat, s); return true;
@@ -1422,30 +1234,6 @@ bool launch_fft_cols_p2(const FftArgs& fa, int n_f, void* inter, void* fhat, cud
 #undef FC2D_COLS
 }
 
-// FP64 inverse real rows with nx/2 = 2^8 .. 2^11; false (nothing launched) otherwise.
-bool launch_inverse_rows_p2(const FftArgs& fa, int n_f, const void* inter, const double* c00,
-                            double a0, double b0, double h, double* out, cudaStream_t s) {
-  if (!fa.tsx || !fa.rtw) return false;  // needs the per-stage twiddle table
-  switch (ilog2_exact(fa.nx / 2)) {
-    case 8: p2::inverse_rows_p2_launch<8>(fa, n_f, inter, c00, a0, b0, h, out, s); return true;
-    case 9: p2::inverse_rows_p2_launch<9>(fa, n_f, inter, c00, a0, b0, h, out, s); return true;
-    case 10: p2::inverse_rows_p2_launch<10>(fa, n_f, inter, c00, a0, b0, h, out, s); return true;
-    case 11: p2::inverse_rows_p2_launch<11>(fa, n_f, inter, c00, a0, b0, h, out, s); return true;
-    default: return false;
-  }
-}
-
-// Fourier Forwarding columns of 2048 or 4096 points; false (nothing launched) otherwise.
-bool launch_wave_cols_p2(const FftArgs& fa, int n_f, void* inter, double c, double t,
-                         double Lx, double Ly, cudaStream_t s) {
-  if (!fa.tsy) return false;  // needs the per-stage twiddle table
-  switch (ilog2_exact(fa.ny)) {
-    case 11: p2::wave_cols_p2_launch<11>(fa, n_f, inter, c, t, Lx, Ly, s); return true;
-    case 12: p2::wave_cols_p2_launch<12>(fa, n_f, inter, c, t, Lx, Ly, s); return true;
-    default: return false;
-  }
-}
-
 // One-time host setup of the 4096-point passes' TMA form on the current device (the
 // shared-memory limit, the occupancy query, the tensor-map encoder), at plan time,
 // outside any stream capture a later call may run under.
@@ -1473,20 +1261,6 @@ bool cols4k_tma_usable(const FftArgs& fa, int cc, int n_f, void* inter) {
   CUtensorMap t;
   return nb > 0 && nsm > 0 && p2::cols_tma_map(0, cc, fa, n_f, inter, &t) &&
          p2::cols_tma_map(1, cc, fa, n_f, inter, &t);
-}
-
-// Fourier Forwarding solve columns of 512 .. 4096 points; false (nothing launched)
-// otherwise.
-bool launch_ff_cols_p2(const FftArgs& fa, int n_f, int n_out, const void* spec, void* out,
-                       double c, double tau, double Lx, double Ly, cudaStream_t s) {
-  if (!fa.tsy) return false;  // needs the per-stage twiddle table
-  switch (ilog2_exact(fa.ny)) {
-    case 9: p2::ff_cols_p2_launch<9>(fa, n_f, n_out, spec, out, c, tau, Lx, Ly, s); return true;
-    case 10: p2::ff_cols_p2_launch<10>(fa, n_f, n_out, spec, out, c, tau, Lx, Ly, s); return true;
-    case 11: p2::ff_cols_p2_launch<11>(fa, n_f, n_out, spec, out, c, tau, Lx, Ly, s); return true;
-    case 12: p2::ff_cols_p2_launch<12>(fa, n_f, n_out, spec, out, c, tau, Lx, Ly, s); return true;
-    default: return false;
-  }
 }
 
 }  // namespace fc2d

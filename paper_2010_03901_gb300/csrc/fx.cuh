@@ -74,6 +74,17 @@ __device__ __forceinline__ i64 dot(i64 a, i64 b, int4 pq) {
   const i64 m = mad(ah, pq.y, mad(al, pq.x, mad(bh, pq.w, mad(bl, pq.z, i64(1) << 31))));
   return mad(ah, pq.x, mad(bh, pq.z, add_high(m, 0)));
 }
+// a p + b q = (hi + mid 2^-32) 2^64 up to 2^-32 (dot() rounds it to hi + (mid >> 32))
+struct Wide {
+  i64 hi, mid;
+};
+__device__ __forceinline__ Wide dot_wide(i64 a, i64 b, int4 pq) {
+  const int ah = hi32(a), al = lo32(a), bh = hi32(b), bl = lo32(b);
+  const i64 low = mad(al, pq.y, mad(bl, pq.w, 0));
+  const i64 m = mad(ah, pq.y, mad(al, pq.x, mad(bh, pq.w, mad(bl, pq.z, low >> 32))));
+  return {mad(ah, pq.x, mad(bh, pq.z, 0)), m};
+}
+
 // a b 2^-64, |a|, |b| <= 2^62
 __device__ __forceinline__ i64 mulh(i64 a, i64 b) {
   const int ah = hi32(a), al = lo32(a), bh = hi32(b), bl = lo32(b);
@@ -97,6 +108,16 @@ __device__ __forceinline__ i64 drop(i64 v) {
   return (v + ((1 << (kDrop - 1)) - 1) + (i64)((unsigned long long)v >> 63)) >> kDrop;
 }
 __device__ __forceinline__ c64 drop(c64 v) { return {drop(v.x), drop(v.y)}; }
+
+// X_k and X_{NH-k} (times 2^(1-kDrop), in the block's units) of a real row from its pairs'
+// transform (|z| <= 2^61.5): with zk = Z_k and zl = Z_{NH-k}, e = (zk + conj zl)/2, o = (zk - conj zl)/2,
+// X_k = e - i w^k o, X_{NH-k} = conj(e + i w^k o)
+__device__ __forceinline__ void split_pair(c64 zk, c64 zl, int4 w, c64& xk, c64& xl) {
+  const c64 e = drop(c64{zk.x + zl.x, zk.y - zl.y});
+  const c64 wo = mulw(c64{zk.x - zl.x, zk.y + zl.y}, w);
+  xk = {e.x + wo.y, e.y - wo.x};
+  xl = {e.x - wo.y, -e.y - wo.x};
+}
 
 // bits that differ from their lower neighbour: the top one bounds |v| < 2^(32 + index)
 __device__ __forceinline__ unsigned spread(i64 v) {

@@ -180,17 +180,6 @@ k_factors(int nxh, bool deriv, When w, const Mode* __restrict__ modes,
   if (l < nxh) fac[at] = v;
 }
 
-// a p + b q = (hi + mid 2^-32) 2^64 up to 2^-32 (dot() rounds it to hi + (mid >> 32))
-struct Wide {
-  i64 hi, mid;
-};
-__device__ __forceinline__ Wide dot_wide(i64 a, i64 b, int4 pq) {
-  const int ah = hi32(a), al = lo32(a), bh = hi32(b), bl = lo32(b);
-  const i64 low = mad(al, pq.y, mad(bl, pq.w, 0));
-  const i64 m = mad(ah, pq.y, mad(al, pq.x, mad(bh, pq.w, mad(bl, pq.z, low >> 32))));
-  return {mad(ah, pq.x, mad(bh, pq.z, 0)), m};
-}
-
 // Modal advance and pass A of the inverse column transform (a forward transform of the
 // conjugate) for the functions f0 <= f < f0 + gridDim.z: spec, exps as k_spec_fix leaves
 // them; mid [nf][ny][pitch] integers with exponents mexps[nf][N2][column group].
@@ -456,10 +445,15 @@ bool launch_inverse_rows_fx(const FftArgs& fa, int n_f, const void* inter, const
   }
 }
 
-bool wave_fx_sizes(int nx, int ny) {
-  const int L = fx::ilog2_exact(nx / 2);
-  return (ny == 512 || ny == 1024 || ny == 2048 || ny == 4096) && L >= 5 && L <= 12;
-}
+void launch_inverse_rows_mixed(const FftArgs& fa, int n_f, const void* inter, const double* c00,
+                               double a0, double b0, double h, double* out, const int32_t* off,
+                               const int32_t* points, int ld, cudaStream_t s);
+void launch_spec_fix_mixed(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, cudaStream_t s);
+void launch_adv_mixed(const FftArgs& fa, int n_f, int f0, int nf, bool deriv, int eS, const int4* fac,
+                      const void* spec, const int* exps, void* mid, int* mexps, void* res, cudaStream_t s);
+
+// columns of 64 x 8, 16, 32 or 64 points
+static bool wave_cols64(int ny) { return ny == 512 || ny == 1024 || ny == 2048 || ny == 4096; }
 
 // The exponent eT of the times up to t: 2^eT >= t, and at least the time h/(8 c) in which a
 // wave crosses an eighth of a cell (u_t is of the size of w u, w up to 4.4 c/h)
@@ -533,6 +527,7 @@ fc2d_status wave_fx_prepare(fc2d_plan_s* p) {
 
 // Spectra [2 n_f][ny][nx/2+1] (F's, then G's) to integers for times up to 2^eT.
 void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, cudaStream_t s) {
+  if (!wave_cols64(fa.ny)) return launch_spec_fix_mixed(fa, n_f, eT, spec, exps, s);
   const dim3 grid(fa.nx / 32 + 1, fa.ny / 64, n_f);
 #define CALL(N2) \
   launch_pdl(fx::k_spec_fix<N2>, grid, dim3(fx::kColThreads), 0, s, fa.nx / 2 + 1, n_f, eT, (double2*)spec, exps)
@@ -566,18 +561,24 @@ fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv,
     const int nf = std::min(chunk, n_f - f0);
     {
       ProfScope ps(p, "ff_cols", s);
+      if (!wave_cols64(fa.ny)) {
+        launch_adv_mixed(fa, n_f, f0, nf, deriv, deriv ? w.eS : 0, m->fac, spec, exps, mid, mexps, res, s);
+      } else {
 #define CALL(N)                                                                                   \
   launch_pdl(deriv ? fx::k_adv_a<N, true> : fx::k_adv_a<N, false>, dim3(groups, N2, nf),           \
              dim3(fx::kColThreads), 0, s, nxh, pitch, n_f, f0, deriv ? w.eS : 0, m->fac,             \
              (const fx::c64*)spec, exps, fa.fxwy, mid, mexps);                                       \
   launch_pdl(fx::k_adv_b<N>, dim3(groups, N2, nf), dim3(fx::kColThreads), 0, s, nxh, pitch,          \
              (const fx::c64*)mid, (const int*)mexps, fa.fxwy, res)
-      FC2D_N2(fa.ny, CALL)
+        FC2D_N2(fa.ny, CALL)
 #undef CALL
+      }
     }
     ProfScope ps(p, "inverse_rows", s);
-    launch_inverse_rows_fx(fa, nf, res, nullptr, p->grid.a0, p->grid.b0, p->grid.h,
-                           off ? out + f0 : out + (size_t)f0 * fa.nx * fa.ny, off, points, n_f, s);
+    double* dst = off ? out + f0 : out + (size_t)f0 * fa.nx * fa.ny;
+    const fc2d_grid& gr = p->grid;
+    if (!launch_inverse_rows_fx(fa, nf, res, nullptr, gr.a0, gr.b0, gr.h, dst, off, points, n_f, s))
+      launch_inverse_rows_mixed(fa, nf, res, nullptr, gr.a0, gr.b0, gr.h, dst, off, points, n_f, s);
   }
   return FC2D_OK;
 }

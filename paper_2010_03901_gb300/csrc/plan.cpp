@@ -345,6 +345,60 @@ std::vector<int64_t> fx_turn_table(int n) {
   return out;
 }
 
+// Stages of a length 2^a 3^b 5^c: the fewest, odd radices first (their writes spread over the
+// shared-memory banks)
+static FxRadices fx_radices(int n) {
+  static const int cand[8] = {9, 5, 3, 10, 6, 8, 4, 2};
+  FxRadices best{};
+  best.n = 100;
+  FxRadices cur{};
+  auto go = [&](auto&& self, int m, int from) -> void {
+    if (m == 1) {
+      if (cur.n < best.n) best = cur;
+      return;
+    }
+    if (cur.n + 1 >= best.n || cur.n >= kFxMaxRadices) return;
+    for (int i = from; i < 8; ++i)
+      if (m % cand[i] == 0) {
+        cur.r[cur.n++] = (signed char)cand[i];
+        self(self, m / cand[i], i);
+        --cur.n;
+      }
+  };
+  go(go, n, 0);
+  return best;
+}
+
+// threads per column: the even number of 4 .. 10 with the fewest thread-rounds over the stages
+static int fx_col_threads(const FxRadices& r, int n) {
+  int best = 4;
+  long cost = 1L << 60;
+  for (int t = 4; t <= 10; t += 2) {
+    long c = 0;
+    for (int s = 0; s < r.n; ++s) c += (long)((n / r.r[s] + t - 1) / t) * r.r[s] * (t + 2);
+    if (c < cost) {
+      cost = c;
+      best = t;
+    }
+  }
+  return best;
+}
+
+FxMixed fx_mixed(int nx, int ny) {
+  FxMixed m{};
+  m.row = fx_radices(nx / 2);
+  int n2 = 1;
+  for (int k = 1; k * k <= ny; ++k)
+    if (ny % k == 0) n2 = k;
+  m.n2 = n2;
+  m.n1 = ny / n2;
+  m.a = fx_radices(m.n1);
+  m.b = fx_radices(m.n2);
+  m.ta = fx_col_threads(m.a, m.n1);
+  m.tb = fx_col_threads(m.b, m.n2);
+  return m;
+}
+
 static bool fft_axis(int n, bool fp64, FftAxis& ax) {
   ax.n = n;
   ax.n_radix = 0;
@@ -900,6 +954,7 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
   const bool fp64 = P.precision == FC2D_FP64;
   if (!fft_axis(nx / 2, fp64, p->fx) || !fft_axis(ny, fp64, p->fy))
     return fail(set_error(FC2D_ERR_UNSUPPORTED, "fc2d_plan: nx/2 and ny must be 2^a 3^b 5^c"));
+  p->mix = fx_mixed(nx, ny);
   p->rtw_host.assign(2 * (size_t)(nx / 2 + 1), 0.0);
   std::vector<int32_t> rfx(fp64 ? 4 * (size_t)(nx / 2 + 1) : 0);
   for (int t = 0; t <= nx / 2; ++t) {
@@ -929,8 +984,6 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
   // FP32: the table, then the same halved (exactly) for the row kernel's split
   std::vector<float> rtw32(p->rtw_host.begin(), p->rtw_host.end());
   for (size_t k = 0, n = p->rtw_host.size(); k < n; ++k) rtw32.push_back(0.5f * rtw32[k]);
-  std::vector<double> tsx64 = stage_twiddles(p->fx, p->fx.tw_host, 2, 8),
-                      tsy64 = stage_twiddles(p->fy, p->fy.tw_host, 2, 8);
   std::vector<double> tsx16 = stage_twiddles(p->fx, p->fx.tw_host, 2, 16),
                       tsy16 = stage_twiddles(p->fy, p->fy.tw_host, 2, 16);
   std::vector<int32_t> fsx = stage_twiddles(p->fx, p->fx.fx_host, 4, 8),
@@ -978,8 +1031,7 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
       (st = upload(&p->dev.status, zero_status)) ||
       (st = upload(&p->fx.tw64, p->fx.tw_host)) || (st = upload(&p->fx.tw32, tw32x)) ||
       (st = upload(&p->fy.tw64, p->fy.tw_host)) || (st = upload(&p->fy.tw32, tw32y)) ||
-      (st = upload(&p->rtw64, p->rtw_host)) || (st = upload(&p->rtw32, rtw32)) ||
-      (st = upload(&p->fx.tws64, tsx64)) || (st = upload(&p->fy.tws64, tsy64)) ||
+      (st = upload(&p->rtw32, rtw32)) ||
       (st = upload(&p->fx.tws32, tsx32)) || (st = upload(&p->fy.tws32, tsy32)) ||
       (st = upload(&p->fx.fx, p->fx.fx_host)) || (st = upload(&p->fy.fx, p->fy.fx_host)) ||
       (st = upload(&p->fx.fxs, fsx)) || (st = upload(&p->fy.fxs, fsy)) ||
@@ -1049,7 +1101,6 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
   if (!p) return;
   poisson_destroy(p);
   wave_destroy(p);
-  wave_modes_destroy(p);
   void* ptrs[] = {p->dev.Q, p->dev.Ar, p->dev.Ar_hi, p->dev.Ar_lo, p->dev.gidx, p->dev.gw,
                   p->dev.wn, p->dev.s_lin, p->dev.s_theta, p->dev.s_eta, p->dev.s_w,
                   p->dev.s_pb, p->dev.s_sb, p->dev.own[0].off, p->dev.own[0].k,
@@ -1059,8 +1110,8 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
                   p->dev.row_iv, p->dev.row_strip_off, p->dev.row_iv_coff, p->dev.gidx_c,
                   p->dev.gidx_i, p->dev.gw_i, p->dev.wn_i, p->dev.gidx_ic,
                   p->dev.status, p->fx.tw64, p->fx.tw32,
-                  p->fy.tw64, p->fy.tw32, p->rtw64, p->rtw32, p->ws.base,
-                  p->fx.tws64, p->fx.tws32, p->fy.tws64, p->fy.tws32, p->fx.fx,
+                  p->fy.tw64, p->fy.tw32, p->rtw32, p->ws.base,
+                  p->fx.tws32, p->fy.tws32, p->fx.fx,
                   p->fx.fxs, p->fy.fx, p->fy.fxs, p->rfx};
   for (void* q : ptrs)
     if (q) cudaFree(q);

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fc2d.h"
+#include "fx_types.h"
 
 namespace fc2d {
 
@@ -27,12 +28,11 @@ struct FftAxis {
   std::vector<double> tw_host;   // interleaved re, im (2N doubles)
   double* tw64 = nullptr;        // device, 2N doubles
   float* tw32 = nullptr;         // device, 2N floats
-  // power-of-two lengths: per-stage twiddles [stage][r][k] for the radix-8 (double) and
+  // power-of-two lengths: per-stage twiddles [stage][r][k] for the radix-8 (fxs) and
   // radix-16 (float) Stockham sequences (see stage_twiddles in plan.cpp)
   std::vector<int32_t> fx_host;  // double plans: w 2^60 in 32-bit limbs, 4 N words (fx.cuh)
   int32_t* fx = nullptr;         // device, the same
   int32_t* fxs = nullptr;        // device, per stage of the radix-8 Stockham sequence
-  double* tws64 = nullptr;
   float* tws32 = nullptr;
 };
 
@@ -121,8 +121,8 @@ struct fc2d_plan_s {
   bool interior_ok = true;  // every red star has a grid node (interior-only form usable)
   int n_sm = 0;             // SMs of the plan's device
   fc2d::FftAxis fx, fy;                      // nx/2 (complex) and ny
+  fc2d::FxMixed mix;                               // stages of sizes that are not powers of two
   std::vector<double> rtw_host;              // exp(-2 pi i k/nx), k <= nx/2 (R2C post-process)
-  double* rtw64 = nullptr;
   int32_t* rfx = nullptr;   // double plans: rtw 2^60 in 32-bit limbs
   float* rtw32 = nullptr;   // [2][nx/2 + 1] complex: exp(-2 pi i k/nx), then halved
   fc2d::DeviceTables dev;
@@ -174,7 +174,7 @@ const double* poisson_nodes(const fc2d_plan_s* p);
 void poisson_stats(const fc2d_plan_s* p, int* iters, double* resid, int64_t* n_near);
 
 // Fourier Forwarding state (ff.cu)
-void wave_destroy(fc2d_plan_s* p);
+void wave_destroy(fc2d_plan_s* p);  // with its mode table
 void wave_modes_destroy(fc2d_plan_s* p);
 
 // (cos, sin)(2 pi i/n) 2^62, i < n, rounded (plan.cpp)

@@ -13,7 +13,7 @@
 //   value (trigonometric interpolation of g - u_p) and refined sums at 5s/R..(M_P+3)s/R.
 //
 // Kernels: k_poisson_cols (forward column DFT, multiplier, inverse column DFT in
-// shared memory), k_poisson_rows (inverse real row DFT + quadratic term), k_up_nodes,
+// shared memory), the inverse real rows + quadratic term (fx_wave.cu), k_up_nodes,
 // GMRES kernels, k_density_dft / k_density_refine, k_dlp (trapezoidal sums over a point
 // list), k_dlp_close (one block per close point), k_zero_outside.
 #include <cuda_runtime.h>
@@ -127,46 +127,6 @@ __global__ void __launch_bounds__(256) k_poisson_cols(FftArgs fa, int cb, double
       C v = Z[(size_t)c * ny + y];
       col[(size_t)y * fa.pitch + c] = C{v.x, -v.y};
     }
-  }
-}
-
-// Inverse real row DFT: from B_k (k = 0..nx/2) the real row x_n = sum B_k e^{2 pi i k n/nx}
-// (full Hermitian sum), via z = length-nx/2 inverse DFT of
-// Z'_k = (B_k + conj B_{nx/2-k}) + i (B_k - conj B_{nx/2-k}) conj(w^k), w = e^{-2 pi i/nx},
-// x_{2m} = Re z_m, x_{2m+1} = Im z_m; plus c00 (x^2 + y^2)/4.
-__global__ void __launch_bounds__(256) k_poisson_rows(FftArgs fa, const double2* inter,
-                                                      const double* c00, double a0, double b0,
-                                                      double h, double* up) {
-  using C = double2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nx = fa.nx, Nh = nx / 2, j = blockIdx.x, f = blockIdx.y;
-  C* A = reinterpret_cast<C*>(smem_raw);
-  C* Bf = A + Nh;
-  const C* row = inter + ((size_t)f * fa.ny + j) * fa.pitch;
-  const C* rtw = reinterpret_cast<const C*>(fa.rtw);
-  for (int k = threadIdx.x; k < Nh; k += blockDim.x) {
-    C bk = row[k];
-    C bc = row[Nh - k];
-    bc.y = -bc.y;  // conj B_{Nh-k}
-    C s = C{bk.x + bc.x, bk.y + bc.y};
-    C d = C{bk.x - bc.x, bk.y - bc.y};
-    C w = rtw[k];
-    w.y = -w.y;  // conj(w^k)
-    C dw = C{d.x * w.x - d.y * w.y, d.x * w.y + d.y * w.x};
-    C z = C{s.x - dw.y, s.y + dw.x};  // s + i dw
-    A[k] = C{z.x, -z.y};              // conj for the inverse
-  }
-  __syncthreads();
-  const C* tw = reinterpret_cast<const C*>(fa.twx);
-  C* Z = stockham<double>(A, Bf, Nh, 1, fa.rx, fa.nrx, tw, 1);
-  const double q = c00 ? c00[f] * 0.25 : 0.0;
-  const double y = b0 + h * double(j);
-  double* out = up + ((size_t)f * fa.ny + j) * nx;
-  for (int m = threadIdx.x; m < Nh; m += blockDim.x) {
-    C z = Z[m];
-    double x0 = a0 + h * double(2 * m), x1 = a0 + h * double(2 * m + 1);
-    out[2 * m] = z.x + q * (x0 * x0 + y * y);
-    out[2 * m + 1] = -z.y + q * (x1 * x1 + y * y);
   }
 }
 
@@ -871,20 +831,7 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
   const double a0 = p->grid.a0, b0 = p->grid.b0, h = p->grid.h;
   if (n_f > 1024) return set_error(FC2D_ERR_ARG, "fc2d_poisson: n_f <= 1024");
   // u_p (forward rows already in `inter` from the caller): multiplier + inverse
-  FftArgs fa{};
-  fa.nx = nx;
-  fa.ny = ny;
-  fa.pitch = (int)row_pitch(p);
-  fa.nrx = p->fx.n_radix;
-  fa.nry = p->fy.n_radix;
-  for (int i = 0; i < fa.nrx; ++i) fa.rx[i] = p->fx.radix[i];
-  for (int i = 0; i < fa.nry; ++i) fa.ry[i] = p->fy.radix[i];
-  fa.twx = p->fx.tw64;
-  fa.twy = p->fy.tw64;
-  fa.tsx = p->fx.tws64;  // per-stage tables of the power-of-two inverse rows
-  fa.tsy = p->fy.tws64;
-  fa.rtw = p->rtw64;
-  fa.scale = 1.0 / ((double)nx * ny);
+  const FftArgs fa = fft_args(p);
   {
     ProfScope ps(p, "poisson_cols", s);
     const int ncol = nx / 2 + 1;
@@ -957,16 +904,18 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
   return cuda_check(cudaGetLastError(), "Poisson solve");
 }
 
-// inverse real 2D-DFT rows (after an inverse column pass) for callers outside this file
-bool launch_inverse_rows_p2(const FftArgs& fa, int n_f, const void* inter, const double* c00,
-                            double a0, double b0, double h, double* out, cudaStream_t s);
+// inverse real 2D-DFT rows (after an inverse column pass)
+bool launch_inverse_rows_fx(const FftArgs& fa, int n_f, const void* inter, const double* c00,
+                            double a0, double b0, double h, double* out, const int32_t* off,
+                            const int32_t* points, int ld, cudaStream_t s);
+void launch_inverse_rows_mixed(const FftArgs& fa, int n_f, const void* inter, const double* c00,
+                               double a0, double b0, double h, double* out, const int32_t* off,
+                               const int32_t* points, int ld, cudaStream_t s);
 
 void launch_inverse_rows(const FftArgs& fa, int n_f, const void* inter, const double* c00,
                          double a0, double b0, double h, double* out, cudaStream_t s) {
-  if (launch_inverse_rows_p2(fa, n_f, inter, c00, a0, b0, h, out, s)) return;
-  size_t sm = (size_t)fa.nx * sizeof(double2);
-  cudaFuncSetAttribute(k_poisson_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_poisson_rows<<<dim3(fa.ny, n_f), 256, sm, s>>>(fa, (const double2*)inter, c00, a0, b0, h, out);
+  if (!launch_inverse_rows_fx(fa, n_f, inter, c00, a0, b0, h, out, nullptr, nullptr, 0, s))
+    launch_inverse_rows_mixed(fa, n_f, inter, c00, a0, b0, h, out, nullptr, nullptr, 0, s);
 }
 
 int poisson_nb(const fc2d_plan_s* p) {

@@ -24,9 +24,9 @@
 namespace fc2d {
 
 constexpr size_t kStaticScratchBytes = size_t(64) << 20;
-// behind it: the exponents of the two-pass double columns, at most 9/8 per 1024 complex
-// values of the scratch
-constexpr size_t kStaticExpBytes = size_t(32) << 10;
+// behind it: the exponents of the two-pass double columns (fx_exps, at most one per 16 of the
+// scratch's 2^22 complex values, for ny = 2)
+constexpr size_t kStaticExpBytes = size_t(1) << 20;
 constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_scratch[kStaticScratchBytes + kStaticExpBytes];

@@ -41,7 +41,11 @@ def spectrum(plan, f):
 
 
 @pytest.mark.parametrize("nx,ny", [(64, 64), (128, 1024), (256, 128), (512, 256), (1024, 512),
-                                   (2048, 64), (4096, 128), (128, 2048), (128, 4096), (8192, 64)])
+                                   (2048, 64), (4096, 128), (128, 2048), (128, 4096), (8192, 64),
+                                   # every radix of the other sizes, first and last; one, two
+                                   # and many stages; one power-of-two side
+                                   (60, 90), (96, 72), (100, 50), (162, 486), (250, 750), (128, 1200),
+                                   (1728, 64), (2160, 80), (4374, 54), (540, 2048), (72, 3750)])
 def test_against_long_double(nx, ny):
     fft = pytest.importorskip("scipy.fft")
     plan = plan_of(nx, ny)

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny", [(512, 512), (64, 512), (1024, 512), (512, 1024), (128, 2048),
-                                   (64, 4096)])
+                                   (64, 4096), (90, 100), (162, 250), (360, 72), (1200, 512), (128, 720)])
 @pytest.mark.parametrize("cells", [0.0, 1e-7, 0.01, 0.5, 8.0, 1000.25])
 def test_modal_solutions(nx, ny, cells):
     torch = pytest.importorskip("torch")
