@@ -37,8 +37,8 @@ namespace {
 size_t al(size_t b) { return (b + 255) / 256 * 256; }
 
 struct Layout {
-  size_t F, vals, inter, coef, bvals, exps, total;
-  size_t oF, ovals, ointer, ocoef, obvals, oexps;
+  size_t F, vals, inter, coef, bvals, exps, fexp, total;
+  size_t oF, ovals, ointer, ocoef, obvals, oexps, ofexp;
 };
 
 // Row length of the strip values F in workspace: Cr + 1 for FP64; for the mixed form
@@ -63,7 +63,9 @@ Layout layout(const fc2d_plan_s* p, int n_f) {
   L.obvals = L.ocoef + L.coef;
   L.oexps = L.obvals + L.bvals;
   L.exps = p->prm.precision == FC2D_FP64 ? al(fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int)) : 0;
-  L.total = L.oexps + L.exps;
+  L.ofexp = L.oexps + L.exps;
+  L.fexp = p->prm.precision == FC2D_FP64 ? al((size_t)n_f * p->prm.B * sizeof(int)) : 0;
+  L.total = L.ofexp + L.fexp;
   return L;
 }
 
@@ -211,13 +213,16 @@ fc2d_status mixed_blend(fc2d_plan_s* p, int n_f, const double* fg, const double*
 
 // The fused blend + interpolation call (mixed form, M = 8) for n_f functions: one
 // function on CTAs of 512 threads, one per SM (own[0]); several on CTAs of 256 threads,
-// two per SM, one function each, over the balanced ranges while the call's CTAs fit in
-// about one wave, else over the fewest CTAs (own[1]).
+// two per SM, one function each, over the partition of the most CTAs that run at once
+// (2 per SM), else over the one of the fewest (two functions at 1024^2: 41.5 us with 42 CTAs
+// each, 32.9 with 152; four: 45.3 with 42, 43.0 with 76, 47.3 with 36).
 GiPlanArgs gi_call(fc2d_plan_s* p, int n_f, const double* fg, const double* fb,
                    const Layout& L, bool compact, int* nt, const DeviceTables::Owners** own) {
-  const auto& o = (n_f > 1 && p->dev.own[1].n && n_f * (int64_t)p->dev.own[0].n > 3 * (int64_t)p->n_sm)
-                      ? p->dev.own[1]
-                      : p->dev.own[0];
+  int set = 0;
+  while (n_f > 1 && set + 1 < kOwnerSets && p->dev.own[set + 1].n &&
+         n_f * (int64_t)p->dev.own[set].n > 2 * (int64_t)p->n_sm)
+    ++set;
+  const auto& o = p->dev.own[set];
   GiPlanArgs a{};
   a.g = gather_args(p, fg, fb, nullptr, nullptr, nullptr, compact);
   a.n_f = n_f;
@@ -238,28 +243,40 @@ GiPlanArgs gi_call(fc2d_plan_s* p, int n_f, const double* fg, const double* fb,
   return a;
 }
 
+// Double plans: strip values of n_f functions into F and their strip-point values, from
+// function f0 of the workspace on.
+fc2d_status strip_values_fx(fc2d_plan_s* p, int n_f, int f0, const double* fg, const double* fb,
+                            const Layout& L, cudaStream_t s, bool compact = false) {
+  StripFx x{p->dev.fx_Ar, p->dev.fx_Aexp, p->dev.fx_w,
+            reinterpret_cast<long long*>(ws(p, L.oF)) + (size_t)f0 * p->prm.B * (p->Cr + 1),
+            reinterpret_cast<int*>(ws(p, L.ofexp)) + (size_t)f0 * p->prm.B};
+  {
+    ProfScope ps(p, "gather_blend", s);
+    launch_gather_blend_fx(gather_args(p, fg, fb, nullptr, nullptr, nullptr, compact), x, n_f, s);
+  }
+  ProfScope ps(p, "interp", s);
+  launch_interp_fx(interp_args(p, p->Cr + 1), x, n_f,
+                   reinterpret_cast<double*>(ws(p, L.ovals)) + (size_t)f0 * p->strip_lin.size(), s);
+  return launched("strip values");
+}
+
 // Steps 5 and 6 into workspace: strip values F, then the strip-point values.
 fc2d_status strip_values(fc2d_plan_s* p, int n_f, const double* fg, const double* fb,
                          const Layout& L, cudaStream_t s, bool compact = false) {
-  const bool f64 = p->prm.precision == FC2D_FP64;
+  if (p->prm.precision == FC2D_FP64) return strip_values_fx(p, n_f, 0, fg, fb, L, s, compact);
   void* F = ws(p, L.oF);
-  if (!f64 && p->dev.own[0].off) {
+  if (p->dev.own[0].off) {
     // mixed form, M = 8: blend and interpolation in one kernel, F stays on chip
     int nt = 0;
     const GiPlanArgs a = gi_call(p, n_f, fg, fb, L, compact, &nt, nullptr);
     ProfScope ps(p, "gather_blend_interp_tc", s);
     return launch_gather_interp_tc(a, nt, s);
   }
-  if (f64) {
-    ProfScope ps(p, "gather_blend", s);
-    launch_gather_blend(gather_args(p, fg, fb, F, nullptr, nullptr, compact), n_f, true, s);
-  } else {
-    fc2d_status st = mixed_blend(p, n_f, fg, fb, F, ws_ldF(p), L, s, compact);
-    if (st) return st;
-  }
+  fc2d_status st = mixed_blend(p, n_f, fg, fb, F, ws_ldF(p), L, s, compact);
+  if (st) return st;
   {
     ProfScope ps(p, "interp", s);
-    launch_interp(interp_args(p, ws_ldF(p)), n_f, f64, F, ws(p, L.ovals), s);
+    launch_interp(interp_args(p, ws_ldF(p)), n_f, false, F, ws(p, L.ovals), s);
   }
   return launched("strip values");
 }
@@ -648,7 +665,9 @@ bool cols4k_tma_usable(const FftArgs& fa, int cc, int n_f, void* inter);
 // on a private stream.  The fastest step is kept.  The passes timed on their own do not
 // predict the step, where their blocks also overlap the previous and the next kernel.
 // Without the memory for the inputs the plan keeps the untuned shape {16, direct}.
+// Double plans take their integer strip tables here, the last step of a plan.
 fc2d_status tune_plan(fc2d_plan_s* p) {
+  if (p->prm.precision == FC2D_FP64) return strip_fx_plan(p);
   if (p->prm.precision != FC2D_MIXED || p->grid.ny != 4096) return FC2D_OK;
   cols4k_prepare();
   const size_t ng = (size_t)p->grid.nx * p->grid.ny;
@@ -751,17 +770,9 @@ fc2d_status wave_spectra(fc2d_plan_s* p, int n_f, const double* u, const double*
   for (int half = 0; half < 2; ++half) {
     const double* fg = half ? ut : u;
     const double* fb = half ? utb : ub;
-    double* F = reinterpret_cast<double*>(ws(p, L.oF)) + (size_t)half * n_f * p->prm.B * (p->Cr + 1);
     double* vals = reinterpret_cast<double*>(ws(p, L.ovals)) + (size_t)half * n_f * p->strip_lin.size();
     double2* inter = reinterpret_cast<double2*>(ws(p, L.ointer)) + (size_t)half * n_f * p->grid.ny * pitch;
-    {
-      ProfScope ps(p, "gather_blend", s);
-      launch_gather_blend(gather_args(p, fg, fb, F, nullptr, nullptr), n_f, true, s);
-    }
-    {
-      ProfScope ps(p, "interp", s);
-      launch_interp(interp_args(p, p->Cr + 1), n_f, true, F, vals, s);
-    }
+    if ((st = strip_values_fx(p, n_f, half * n_f, fg, fb, L, s))) return st;
     {
       ProfScope ps(p, "fft_rows_fused", s);
       launch_fft_rows(fa, row_args(p), n_f, true, 1, nullptr, fg, vals, inter, s);

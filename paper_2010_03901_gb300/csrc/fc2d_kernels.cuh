@@ -30,6 +30,17 @@ struct GatherArgs {
   double* bvals;          // mixed form: boundary datum per normal [n_f][B]
 };
 
+// Double plans: strip values as integers with one exponent per normal (fx_strip.cu)
+struct StripFx {
+  const int2* Ar;           // [d][Cr] A_r[q][j] 2^(60 - Aexp[j]) in limbs (hi, lo)
+  const int* Aexp;          // [d]: |A_r[.][j]| <= 2^Aexp[j]
+  const int2* w;            // [2M][n_strip] weights in limbs: theta 2^60, eta 2^(60 - strip_gain(M))
+  long long* F;             // [n_f][B][Cr + 1]
+  int* exps;                // [n_f][B]
+};
+// |Lagrange weights| of M equispaced nodes over their interval sum to less than 2^gain
+__host__ __device__ constexpr int strip_gain(int M) { return M <= 8 ? 4 : M <= 11 ? 5 : M <= 13 ? 7 : 9; }
+
 struct InterpArgs {
   int n_strip, M, B, Cr;
   int ldF;               // row length of F (>= Cr + 1)
@@ -147,6 +158,9 @@ fc2d_status launch_gather_interp_queue(const void* work, const int4* items, int 
 // The tensor-core kernels' bounded mbarrier wait on a barrier nothing arrives on: after
 // 2 x limit polls FC2D_ERR_TIMEOUT is latched in *status and the kernel returns.
 fc2d_status launch_wait_probe(int* status, uint32_t limit, cudaStream_t s);
+// the same two steps on integers: strip values of the normals, values at the strip points
+void launch_gather_blend_fx(const GatherArgs& a, const StripFx& x, int n_f, cudaStream_t s);
+void launch_interp_fx(const InterpArgs& a, const StripFx& x, int n_f, double* vals, cudaStream_t s);
 void launch_interp(const InterpArgs& a, int n_f, bool fp64, const void* F, void* vals,
                    cudaStream_t s);
 void launch_assemble(const RowArgs& a, int n_f, bool fp64, const double* f_grid,

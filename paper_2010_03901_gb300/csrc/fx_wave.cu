@@ -503,11 +503,12 @@ void wave_modes_destroy(fc2d_plan_s* p) {
   p->modes = nullptr;
 }
 
-// Functions per launch: their intermediate (written by one pass, read by the next) within
-// half of L2
+// Functions per launch: 160 MB of intermediate.  Smaller launches would keep it in L2, but
+// their last waves cost more (8 solutions at 1024^2, one large step: 12.0 ms with 40 MB, 11.2
+// with 80 MB or more)
 static int wave_chunk(const FftArgs& fa, int n_f) {
   const size_t one = (size_t)fa.ny * fa.pitch * 16;
-  return (int)std::min<size_t>(n_f, std::max<size_t>(1, (size_t(40) << 20) / one));
+  return (int)std::min<size_t>(n_f, std::max<size_t>(1, (size_t(160) << 20) / one));
 }
 
 size_t wave_fx_exps(int nx, int ny, int n_f) { return 2 * fx_exps(nx, ny, n_f); }

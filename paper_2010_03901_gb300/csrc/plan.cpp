@@ -527,11 +527,13 @@ static std::vector<int32_t> partition_owners(const std::vector<int64_t>& cnt, in
 // Strip points grouped by the blend CTA that interpolates them (mixed form, M = 8):
 // CTA c of a function computes the kTcComputed normals from start_c on (mod B) and owns
 // the strip points whose first normal pb lies in [start_c, start_{c+1}), at most
-// kTcOwned normals, so that pb .. pb + M - 1 are among its normals.  Two partitions:
-// one CTA per SM where B allows ~48 normals each (a call of few functions then fills
-// the SMs once, with the ranges balanced by their numbers of points), and the fewest
-// CTAs, ceil(B / kTcOwned) (for calls of many functions, whose CTAs fill the SMs anyway
-// and where extra CTAs only repeat gathers).  Within a CTA the points are ordered by
+// kTcOwned normals, so that pb .. pb + M - 1 are among its normals.  Up to four
+// partitions: one CTA per SM where B leaves 8 normals to each (the phases of a CTA follow
+// one another, so that a call of one function takes as long as its largest CTA: a star at
+// 512^2 took 23.2 us with 48 normals to a CTA, 16.2 with 14), half as many, ~48 normals to
+// a CTA, and the fewest CTAs, ceil(B / kTcOwned) (for calls of many functions, whose CTAs fill the SMs
+// anyway and where extra CTAs only repeat gathers); gi_call in capi.cu chooses.  The ranges
+// are balanced by their numbers of points.  Within a CTA the points are ordered by
 // first normal, then fine node; the weights are reordered to match.
 static fc2d_status owner_set(fc2d_plan_s* p, const std::vector<int32_t>& pb,
                              const std::vector<int32_t>& sb, const std::vector<float>& w,
@@ -587,7 +589,7 @@ static fc2d_status owner_tables(fc2d_plan_s* p, int ns, int M) {
     n_sm = 0;
   p->n_sm = n_sm;
   const int n_min = (B + kTcOwned - 1) / kTcOwned;
-  const int n_wide = std::max(n_min, std::min(n_sm, B / 48));
+  const int n_wide = std::max(n_min, std::min(n_sm, B / 8));
   std::vector<int32_t> pb(ns), sb(ns);
   std::vector<float> w((size_t)2 * M * ns);
   if (cudaMemcpy(pb.data(), p->dev.s_pb, (size_t)ns * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
@@ -601,9 +603,14 @@ static fc2d_status owner_tables(fc2d_plan_s* p, int ns, int M) {
       return set_error(FC2D_ERR_GEOMETRY, "interpolation node index out of range");
     ++cnt[pb[k]];
   }
-  fc2d_status st = owner_set(p, pb, sb, w, cnt, n_wide, M, p->dev.own[0]);
-  if (!st && n_wide > n_min) st = owner_set(p, pb, sb, w, cnt, n_min, M, p->dev.own[1]);
-  return st;
+  const int n_mid = std::max(n_min, std::min(n_sm, B / 48));
+  std::vector<int> sizes = {n_wide, std::max(n_wide / 2, n_mid), n_mid, n_min};
+  sizes.erase(std::unique(sizes.begin(), sizes.end()), sizes.end());
+  for (size_t k = 0; k < sizes.size(); ++k) {
+    const fc2d_status st = owner_set(p, pb, sb, w, cnt, sizes[k], M, p->dev.own[k]);
+    if (st) return st;
+  }
+  return FC2D_OK;
 }
 
 extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid* grid,
@@ -1102,11 +1109,8 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
   poisson_destroy(p);
   wave_destroy(p);
   void* ptrs[] = {p->dev.Q, p->dev.Ar, p->dev.Ar_hi, p->dev.Ar_lo, p->dev.gidx, p->dev.gw,
-                  p->dev.wn, p->dev.s_lin, p->dev.s_theta, p->dev.s_eta, p->dev.s_w,
-                  p->dev.s_pb, p->dev.s_sb, p->dev.own[0].off, p->dev.own[0].k,
-                  p->dev.own[0].pack, p->dev.own[0].w, p->dev.own[0].start,
-                  p->dev.own[1].off, p->dev.own[1].k, p->dev.own[1].pack, p->dev.own[1].w,
-                  p->dev.own[1].start, p->dev.row_iv_off,
+                  p->dev.wn, p->dev.s_lin, p->dev.s_theta, p->dev.s_eta, p->dev.s_w, p->dev.fx_Ar, p->dev.fx_Aexp, p->dev.fx_w,
+                  p->dev.s_pb, p->dev.s_sb, p->dev.row_iv_off,
                   p->dev.row_iv, p->dev.row_strip_off, p->dev.row_iv_coff, p->dev.gidx_c,
                   p->dev.gidx_i, p->dev.gw_i, p->dev.wn_i, p->dev.gidx_ic,
                   p->dev.status, p->fx.tw64, p->fx.tw32,
@@ -1115,6 +1119,9 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
                   p->fx.fxs, p->fy.fx, p->fy.fxs, p->rfx};
   for (void* q : ptrs)
     if (q) cudaFree(q);
+  for (auto& o : p->dev.own)
+    for (void* q : {(void*)o.off, (void*)o.k, (void*)o.pack, (void*)o.w, (void*)o.start})
+      if (q) cudaFree(q);
   for (auto& r : p->prof) {
     p->event_pool.push_back(r.start);
     p->event_pool.push_back(r.stop);

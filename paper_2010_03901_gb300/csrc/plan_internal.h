@@ -19,6 +19,7 @@ constexpr int kMaxM = 16;
 // M-normal stencils then lie within the CTA's normals.
 constexpr int kTcComputed = 64;
 constexpr int kTcOwned = 57;
+constexpr int kOwnerSets = 4;   // partitions of the normals over the CTAs (plan.cpp)
 
 // One 1D FFT length: its radix sequence and twiddle tables exp(-2 pi i t/N), t < N.
 struct FftAxis {
@@ -57,11 +58,15 @@ struct DeviceTables {
   double* s_theta = nullptr; // [n_strip]
   double* s_eta = nullptr;   // [n_strip]
   void* s_w = nullptr;       // [2M][n_strip] interpolation weights (double or float)
+  // double plans: A_r and the weights as limbs of fixed-point numbers (fx_strip.cu)
+  int2* fx_Ar = nullptr;     // [d][Cr]
+  int* fx_Aexp = nullptr;    // [d]
+  int2* fx_w = nullptr;      // [2M][n_strip]
   int32_t* s_pb = nullptr;   // [n_strip] first normal index
   int32_t* s_sb = nullptr;   // [n_strip] first fine index
   // strip points grouped by owning blend CTA (mixed form, M = 8; else null)
   // ownership of the strip points by the blend + interpolation CTAs (mixed, M = 8):
-  // own[0] one CTA per SM (balanced ranges), own[1] the fewest CTAs (n = 0: same as 0)
+  // partitions from one CTA per SM (own[0]) down to the fewest CTAs (n = 0: not built)
   struct Owners {
     int32_t* off = nullptr;    // [n + 1] offsets of each CTA's points
     int32_t* k = nullptr;      // [n_strip] strip index of each grouped point
@@ -70,7 +75,7 @@ struct DeviceTables {
     int32_t* start = nullptr;  // [n + 1] first normal owned by each CTA, then B
     int n = 0;                 // CTAs per function (ownership ranges)
     std::vector<int32_t> off_host;  // host copy of off (work costs of plan groups)
-  } own[2];
+  } own[kOwnerSets];
   // per-row tables
   int32_t* row_iv_off = nullptr;    // [ny+1] offsets into row_iv
   int32_t* row_iv = nullptr;        // pairs (i_lo, i_hi), inclusive
@@ -182,7 +187,11 @@ std::vector<int64_t> fx_turn_table(int n);
 // exp(-2 pi i t/n) 2^60 in limbs (re hi, lo, im hi, lo), t < n
 std::vector<int32_t> fx_twiddle_table(int n);
 
-// Plan-time autotuning of launch shapes that change no result (capi.cu).
+// plan-time tables of the integer strip values (fx_strip.cu)
+fc2d_status strip_fx_plan(fc2d_plan_s* p);
+
+// The last step of a plan (capi.cu): autotuning of launch shapes that change no result, the
+// integer strip tables of double plans.
 fc2d_status tune_plan(fc2d_plan_s* p);
 
 // kernel timing: bracket one launch with events when the plan is profiling
