@@ -1,0 +1,244 @@
+// Trapezoidal sums of the double-layer potential over the partition of dlp_tree.h.
+//
+// k_node_coef: the nodes' coefficients q_k and their largest magnitude.  k_dlp_expand: one
+// warp per (box, up to 128 nodes): A_j = sum_k q_k w_k^(j+1), w_k = R0/(z_k - c), in 64-bit
+// fixed point; the warps of a box add up by integer atomics (exact in any order).
+// k_dlp_eval: one block per (leaf, up to 64 points): Horner's rule for each expansion of
+// the leaf's chain, then the near nodes term by term in double-float arithmetic.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "dfl.cuh"
+#include "dlp_sum.h"
+#include "fx.cuh"
+
+namespace fc2d {
+
+using namespace fx;
+
+namespace {
+
+constexpr int P = kDlpOrder;
+static_assert(P == 32, "one coefficient per lane");
+constexpr int kUp = 8;    // q in units of 2^(E - 1075 - kUp): |Re|, |Im| < 2^61
+constexpr int kFac = 61;  // factors w, t (at most 1) times 2^kFac
+
+// factor limbs; the lowest bit is set so that no low limb is -2^31 (it is negated below)
+__device__ __forceinline__ int4 limbs(c64 w) {
+  w.x |= 1;
+  w.y |= 1;
+  return {hi32(w.x), lo32(w.x), hi32(w.y), lo32(w.y)};
+}
+// a w for |a| <= 2^61.5, |w| <= 1, w given as the limbs of w 2^kFac (products of the low
+// limbs, at most 2 units, are left out)
+__device__ __forceinline__ c64 mulf(c64 a, int4 w) {
+  constexpr int D = 64 - kFac;
+  const int xh = hi32(a.x), xl = lo32(a.x), yh = hi32(a.y), yl = lo32(a.y);
+  const i64 half = i64(1) << (31 - D);
+  const int nh = -w.z, nl = -w.w;
+  const i64 mx = mad(xh, w.y, mad(xl, w.x, mad(yh, nl, mad(yl, nh, half))));
+  const i64 my = mad(xh, w.w, mad(xl, w.z, mad(yh, w.y, mad(yl, w.x, half))));
+  const i64 hx = mad(xh, w.x, mad(yh, nh, 0)), hy = mad(xh, w.z, mad(yh, w.x, 0));
+  return {(i64)((unsigned long long)hx << D) + (mx >> (32 - D)),
+          (i64)((unsigned long long)hy << D) + (my >> (32 - D))};
+}
+
+// R0/d 2^kFac for d = x 2^-shift: the float reciprocal (about 2^-20), two Newton steps
+__device__ __forceinline__ int4 inverse(c64 x, int lr, int shift) {
+  const float dx = (float)(int)(x.x >> 32), dy = (float)(int)(x.y >> 32);
+  // x 2^-32 = d 2^(shift - 32)
+  const float s = __frcp_rn(fmaf(dx, dx, dy * dy)) * exp2f((float)(lr + shift - 32 + kFac - 30));
+  c64 w = {(i64)__float2int_rn(dx * s) << 30, -((i64)__float2int_rn(dy * s) << 30)};
+  const i64 one = i64(1) << (lr + shift);  // R0 in the unit of x
+  const int up = kFac - lr - shift;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int4 l = limbs(w);
+    const c64 p = mulf(x, l);                           // R0 (1 - e)
+    const c64 c = mulf(c64{one - p.x, -p.y}, l);        // e w, in units of 2^(kFac - up)
+    w = {w.x + (c.x << up), w.y + (c.y << up)};
+  }
+  return limbs(w);
+}
+
+__global__ void __launch_bounds__(256) k_node_coef(int N, const double* x1, const double* y1,
+                                                   const double* phi, double2* q, float4* ab,
+                                                   unsigned* mag) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned m = 0;
+  if (k < N) {
+    const double a = y1[k] * phi[k] / N, b = x1[k] * phi[k] / N;
+    q[k] = double2{b, a};
+    float4 c;
+    split_df(a, c.x, c.y);
+    split_df(b, c.z, c.w);
+    ab[k] = c;
+    m = max(magnitude(a), magnitude(b));
+  }
+  block_max(m, mag);
+}
+
+// sums of a[0 .. 2 H) over the lanes, halving the number of values in each step: lane j of 32
+// ends with the sums 2 j and 2 j + 1 in a[0], a[1]
+template <int H> __device__ __forceinline__ void fold(i64* a, int lane) {
+  const bool up = lane & (H / 2);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const i64 send = up ? a[i] : a[i + H], keep = up ? a[i + H] : a[i];
+    a[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, H / 2);
+  }
+  if constexpr (H > 2) fold<H / 2>(a, lane);
+}
+
+__global__ void __launch_bounds__(128) k_dlp_expand(int n_spans, const DlpSpan* spans,
+                                                    const DlpBox* boxes, const c64* pos, int shift,
+                                                    const double2* q, const unsigned* mag,
+                                                    unsigned long long* coef) {
+  const int item = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (item >= n_spans) return;  // a whole warp
+  const DlpSpan sp = spans[item];
+  const DlpBox b = boxes[sp.box];
+  const int E = block_exp(*mag);
+  const i64 half = b.hb ? i64(1) << (b.hb - 1) : 0;
+  i64 a[2 * P];
+#pragma unroll
+  for (int j = 0; j < 2 * P; ++j) a[j] = 0;
+  for (int k = sp.k0 + lane; k < sp.k0 + sp.n; k += 32) {
+    const c64 z = pos[k];
+    const int4 w = inverse(c64{z.x - b.cx, z.y - b.cy}, b.lr, shift);
+    c64 g = mulf(from_double<kUp>(q[k], E), w);
+    g = {(g.x + half) >> b.hb, (g.y + half) >> b.hb};
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      a[2 * j] += g.x;
+      a[2 * j + 1] += g.y;
+      if (j + 1 < P) g = mulf(g, w);
+    }
+  }
+  fold<P>(a, lane);  // lane j holds A_j
+  unsigned long long* dst = coef + (size_t)sp.box * 2 * P + 2 * lane;
+  atomicAdd(dst, (unsigned long long)a[0]);
+  atomicAdd(dst + 1, (unsigned long long)a[1]);
+}
+
+// fixed-point coordinate -> integer part and fraction
+__device__ __forceinline__ void cell(i64 X, int shift, float& n, float& fh, float& fl) {
+  n = (float)(int)(X >> shift);
+  split_df(scalbn((double)(X & ((i64(1) << shift) - 1)), -shift), fh, fl);
+}
+
+// GRID: the points are grid points lin[] and u[lin] += v/h; otherwise the points pts[] and
+// out[p] = v/h
+template <bool GRID>
+__global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
+    const DlpItem* items, const DlpLeaf* leaves, const int32_t* chain, const DlpSpan* near,
+    const DlpBox* boxes, const c64* coef, int shift, const unsigned* mag, const int32_t* lin,
+    int nx, const c64* pts, const int32_t* idx, double inv_h, const float4* pos, const float4* ab,
+    double* out) {
+  constexpr int T = kDlpPoints;
+  __shared__ c64 A[P];
+  __shared__ float4 s0[T], sc[T];
+  __shared__ float2 s1[T];
+  const DlpItem it = items[blockIdx.x];
+  const DlpLeaf lf = leaves[it.leaf];
+  const int t = threadIdx.x, p = it.p0 + min(t, it.n - 1);
+  c64 X;
+  int l;
+  if (GRID) {
+    l = lin[p];
+    X = {(i64)(l % nx) << shift, (i64)(l / nx) << shift};
+  } else {
+    l = idx[p];
+    X = pts[p];
+  }
+  const unsigned m = *mag;
+  const int e0 = m >= 0x7FF00000u ? kNaN : block_exp(m) - 1075 - kUp;
+  double v = 0.0;
+  for (int c = 0; c < lf.nc; ++c) {
+    const int box = chain[lf.c0 + c];
+    if (c) __syncthreads();
+    if (t < P) A[t] = coef[(size_t)box * P + t];
+    const DlpBox b = boxes[box];
+    __syncthreads();
+    const int up = kFac - shift - b.lr;
+    const int4 z = limbs(c64{(i64)((unsigned long long)(X.x - b.cx) << up),
+                             (i64)((unsigned long long)(X.y - b.cy) << up)});
+    c64 s = A[P - 1];
+#pragma unroll 8
+    for (int j = P - 2; j >= 0; --j) s = A[j] + mulf(s, z);
+    const int e = e0 + b.hb - b.lr;
+    v -= to_double(s.y, e, plain_exp(e));
+  }
+  float px, pfh, pfl, py, qfh, qfl;
+  if (GRID) {
+    px = (float)(l % nx);
+    py = (float)(l / nx);
+  } else {
+    cell(X.x, shift, px, pfh, pfl);
+    cell(X.y, shift, py, qfh, qfl);
+  }
+  dfl acc = {0.f, 0.f};
+  for (int d = 0; d < lf.nd; ++d) {
+    const DlpSpan sp = near[lf.d0 + d];
+    for (int k0 = sp.k0; k0 < sp.k0 + sp.n; k0 += T) {
+      const int cnt = min(T, sp.k0 + sp.n - k0);
+      __syncthreads();
+      if (t < cnt) {
+        s0[t] = pos[2 * (k0 + t)];
+        const float4 y = pos[2 * (k0 + t) + 1];
+        s1[t] = float2{y.x, y.y};
+        sc[t] = ab[k0 + t];
+      }
+      __syncthreads();
+      for (int k = 0; k < cnt; ++k) {
+        const float4 a = s0[k], c = sc[k];
+        const float2 b = s1[k];
+        // (point - node) = (i_p - i_n) + (f_p - f_n)
+        dfl dx = int_minus(px - a.x, a.z, a.w), dy = int_minus(py - a.y, b.x, b.y);
+        if (!GRID) {
+          dx = df_add(dx, {pfh, pfl});
+          dy = df_add(dy, {qfh, qfl});
+        }
+        const dfl term = dl_term(dx, dy, c.x, c.y, c.z, c.w);
+        const dfl s = two_sum(acc.hi, term.hi);
+        acc = fast_two_sum(s.hi, s.lo + (acc.lo + term.lo));
+      }
+    }
+  }
+  if (t >= it.n) return;
+  v += (double)acc.hi + (double)acc.lo;
+  if (GRID) out[l] += v * inv_h;
+  else out[l] = v * inv_h;
+}
+
+}  // namespace
+
+void launch_node_coef(int N, const double* x1, const double* y1, const double* phi, double2* q,
+                      float4* ab, unsigned* mag, cudaStream_t s) {
+  k_node_coef<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, x1, y1, phi, q, ab, mag);
+}
+
+void launch_dlp_expand(const DlpDev& d, const double2* q, cudaStream_t s) {
+  if (d.n_expand)
+    k_dlp_expand<<<(unsigned)((d.n_expand + 3) / 4), 128, 0, s>>>(
+        d.n_expand, d.expand, d.box, (const c64*)d.nodes, d.shift, q, d.mag, d.coef);
+}
+
+void launch_dlp_grid(const DlpDev& d, const int32_t* lin, int nx, double h, const float4* pos,
+                     const float4* ab, double* u, cudaStream_t s) {
+  if (d.n_grid)
+    k_dlp_eval<true><<<(unsigned)d.n_grid, kDlpPoints, 0, s>>>(
+        d.grid_items, d.leaf, d.chain, d.near, d.box, (const c64*)d.coef, d.shift, d.mag, lin, nx,
+        nullptr, nullptr, 1.0 / h, pos, ab, u);
+}
+
+void launch_dlp_free(const DlpDev& d, double h, const float4* pos, const float4* ab, double* out,
+                     cudaStream_t s) {
+  if (d.n_free)
+    k_dlp_eval<false><<<(unsigned)d.n_free, kDlpPoints, 0, s>>>(
+        d.free_items, d.leaf, d.chain, d.near, d.box, (const c64*)d.coef, d.shift, d.mag, nullptr,
+        0, (const c64*)d.points, d.points_idx, 1.0 / h, pos, ab, out);
+}
+
+}  // namespace fc2d

@@ -14,8 +14,8 @@
 //
 // Kernels: k_poisson_cols (forward column DFT, multiplier, inverse column DFT in
 // shared memory), the inverse real rows + quadratic term (fx_wave.cu), k_up_nodes,
-// GMRES kernels, k_density_dft / k_density_refine, k_dlp (trapezoidal sums over a point
-// list), k_dlp_close (one block per close point), k_zero_outside.
+// GMRES kernels, k_density_dft / k_density_refine, the sums (dlp_sum.cu), k_close (one block
+// per close point), k_zero_outside.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "dd.h"
+#include "dlp_sum.h"
 #include "fc2d_kernels.cuh"
 #include "fft_generic.cuh"
 #include "plan_internal.h"
@@ -46,14 +47,14 @@ struct PoissonState {
   int32_t *ui0 = nullptr, *uj0 = nullptr;                               // [Nb]
   double *uwx = nullptr, *uwy = nullptr;                                // [Nb][MP]
   int64_t n_far = 0, n_mid = 0, n_close = 0;
-  int n_sm = 0;                 // SMs of the plan's device
-  int s_far = 1, s_mid = 1;     // node splits of the far and mid point sums (dlp_splits)
-  double* part = nullptr;       // [S][n] partial sums of a split launch
+  DlpDev far, near;             // partitions of the far and the refined sums
+  size_t sum_bytes = 0;         // their coefficients and magnitudes, zeroed per solution
+  double2 *qB = nullptr, *qR = nullptr;  // node coefficients [Nb], [R Nb]
+  double* close_v = nullptr;    // [n_close][MP - 1] refined sums along the normals
   int32_t *far_lin = nullptr, *mid_lin = nullptr, *close_lin = nullptr;
   double* close_geo = nullptr;  // [n_close][5]: foot x, y, normal x, y, theta
   double* close_w = nullptr;    // [n_close][MP]
   std::vector<double> close_nodes;  // [MP] distances along the normal
-  double* dnodes = nullptr;         // device copy
   // per-solve workspace
   double *V = nullptr, *w = nullptr, *h = nullptr, *g = nullptr, *phi = nullptr;
   struct GmresDev* gm = nullptr;  // GMRES's Hessenberg part and state (device)
@@ -307,216 +308,39 @@ __global__ void k_density_refine(int Nb, int NR, const double2* ghat, const doub
   out[m] = s;
 }
 
-// node coefficients of the trapezoidal sum: a_k = y'_k phi_k / N, b_k = x'_k phi_k / N
-// ------------------------------------------------------------------------- //
-// Double-layer sums in double-float arithmetic on the FP32 units.  A value is the
-// unevaluated sum hi + lo of two floats (about 48 significant bits), built from Knuth's
-// TwoSum, the FMA form of Dekker's TwoProduct and the sums and products of Dekker
-// (1971).  The narrow FP64 pipe would need ~12 operations per (point, node) term.
-// Coordinates are in grid units: a grid point is an exact integer pair, a node or an
-// off-grid point an integer cell index plus a double-float fraction, so every
-// coordinate difference is an integer minus a fraction, accurate to ~2^-48 of a cell.
-// With d' = d/h, r2' = r2/h^2 the term (a dx - b dy)/r2 = (a dx' - b dy')/(h r2').
-// ------------------------------------------------------------------------- //
-struct dfl {
-  float hi, lo;
-};
-__device__ __forceinline__ dfl two_sum(float a, float b) {
-  const float s = a + b, bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ dfl fast_two_sum(float a, float b) {  // |a| >= |b|
-  const float s = a + b;
-  return {s, b - (s - a)};
-}
-__device__ __forceinline__ dfl df_add(dfl x, dfl y) {
-  dfl s = two_sum(x.hi, y.hi);
-  const dfl t = two_sum(x.lo, y.lo);
-  s = fast_two_sum(s.hi, s.lo + t.hi);
-  return fast_two_sum(s.hi, s.lo + t.lo);
-}
-__device__ __forceinline__ dfl df_mul(dfl x, dfl y) {
-  const float p = __fmul_rn(x.hi, y.hi);  // never fused into the sum below
-  float e = fmaf(x.hi, y.hi, -p);
-  e = fmaf(x.hi, y.lo, e);
-  e = fmaf(x.lo, y.hi, e);
-  return fast_two_sum(p, e);
-}
-// integer n minus the fraction (fh, fl)
-__device__ __forceinline__ dfl int_minus(float n, float fh, float fl) {
-  const dfl s = two_sum(n, -fh);
-  return fast_two_sum(s.hi, s.lo - fl);
-}
-// (a dx - b dy) / (dx^2 + dy^2) with a = (ah, al), b = (bh, bl)
-__device__ __forceinline__ dfl dl_term(dfl dx, dfl dy, float ah, float al, float bh, float bl) {
-  const dfl xx = df_mul(dx, dx), yy = df_mul(dy, dy);
-  const dfl r2 = df_add(xx, yy);
-  const dfl num = df_add(df_mul({ah, al}, dx), df_mul({-bh, -bl}, dy));
-  // 1/r2: the correctly rounded float reciprocal and one Newton step (relative error
-  // about the square of the seed's, 2^-46)
-  const float y0 = __frcp_rn(r2.hi);
-  float t = fmaf(-r2.hi, y0, 1.0f);
-  t = fmaf(-r2.lo, y0, t);
-  return df_mul(num, fast_two_sum(y0, y0 * t));
-}
-__device__ __forceinline__ void split_df(double v, float& hi, float& lo) {
-  hi = (float)v;
-  lo = (float)(v - (double)hi);
-}
-
-// per-solve node coefficients (y' phi/N, x' phi/N) as double-float pairs (ah, al, bh, bl)
-__global__ void k_node_coef(int N, const double* x1, const double* y1, const double* phi,
-                            float4* ab) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= N) return;
-  float4 c;
-  split_df(y1[k] * phi[k] / N, c.x, c.y);
-  split_df(x1[k] * phi[k] / N, c.z, c.w);
-  ab[k] = c;
-}
-
-// v at listed grid points by the trapezoidal sum over N nodes; u = u_p + v there.
-// Blocks of 256 points, tiles of 256 nodes.  SPLIT: blockIdx.y picks one of gridDim.y
-// node ranges and the partial sums go to part[blockIdx.y][n] (k_dlp_combine adds them).
-// pos: per node (ix, iy, fx_hi, fx_lo), (fy_hi, fy_lo, -, -) in grid units.
-template <bool SPLIT>
-__global__ void __launch_bounds__(256) k_dlp(int n_pts, const int32_t* lin, int nx, double inv_h,
-                                             int N, const float4* pos, const float4* ab,
-                                             double* u, double* part) {
-  __shared__ float4 s0[256], s1[256], sc[256];
-  int n = blockIdx.x * blockDim.x + threadIdx.x;
-  bool act = n < n_pts;
-  int l = act ? lin[n] : 0;
-  const float pi = (float)(l % nx), pj = (float)(l / nx);
-  // node range of this block row (the whole set when the launch is not split)
-  const int k0 = SPLIT ? (int)((int64_t)N * blockIdx.y / gridDim.y) : 0;
-  const int k1 = SPLIT ? (int)((int64_t)N * (blockIdx.y + 1) / gridDim.y) : N;
-  dfl acc = {0.f, 0.f};
-  for (int t0 = k0; t0 < k1; t0 += 256) {
-    __syncthreads();
-    for (int q = threadIdx.x; q < 256 && t0 + q < k1; q += blockDim.x) {
-      s0[q] = pos[2 * (t0 + q)];
-      s1[q] = pos[2 * (t0 + q) + 1];
-      sc[q] = ab[t0 + q];
-    }
-    __syncthreads();
-    const int cnt = min(256, k1 - t0);
-    for (int k = 0; k < cnt; ++k) {
-      const float4 a = s0[k], b = s1[k], c = sc[k];
-      const dfl dx = int_minus(pi - a.x, a.z, a.w), dy = int_minus(pj - a.y, b.x, b.y);
-      const dfl term = dl_term(dx, dy, c.x, c.y, c.z, c.w);
-      const dfl s = two_sum(acc.hi, term.hi);
-      acc = fast_two_sum(s.hi, s.lo + (acc.lo + term.lo));
-    }
-  }
-  if (!act) return;
-  const double v = (double)acc.hi + (double)acc.lo;
-  if (SPLIT) part[(size_t)blockIdx.y * n_pts + n] = v;
-  else u[l] += v * inv_h;
-}
-
-// A split k_dlp launch's S partial sums per point, added in node-range order: u += sum / h.
-__global__ void __launch_bounds__(256) k_dlp_combine(int n_pts, const int32_t* lin, int S,
-                                                     const double* part, double inv_h, double* u) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= n_pts) return;
-  double v = 0.0;
-  for (int y = 0; y < S; ++y) v += part[(size_t)y * n_pts + n];
-  u[lin[n]] += v * inv_h;
-}
-
-// close points: one block per point; the MP - 1 refined sums along the normal (each
-// thread takes a node once for all of them), the boundary value by trigonometric
-// interpolation of g - u_p, and the Lagrange combination.
-template <int KMP>  // compile-time M_P (0: any M_P <= kMaxM)
-__global__ void __launch_bounds__(256) k_dlp_close(int n_close, const int32_t* lin,
-                                                   const double* cgeo, const double* cw,
-                                                   const double* nodes, int MP, int NR,
-                                                   double a0, double b0, double h,
-                                                   const float4* posR, const float4* abR,
-                                                   int Nb, const double2* ghat_g, double* u) {
-  constexpr int NP = KMP > 0 ? KMP : kMaxM;
-  if (KMP > 0) MP = KMP;
-  __shared__ double red[256];
-  __shared__ float pt[NP][6];  // per point: ix, iy, fx_hi, fx_lo, fy_hi, fy_lo
+// close points: one block per point; the boundary value by trigonometric interpolation of
+// g - u_p and the Lagrange combination with the MP - 1 refined sums along the normal,
+// vals[n][MP - 1].  The block has one thread per 8 frequencies or so: a thread's first
+// e^{i k theta} costs a sincos, the next ones a complex product each.
+__global__ void __launch_bounds__(256) k_close(int n_close, const int32_t* lin, const double* cgeo,
+                                               const double* cw, int MP, const double* vals, int Nb,
+                                               const double2* ghat, double* u) {
+  __shared__ double red[8];
   const int n = blockIdx.x;
-  if (n >= n_close) return;
-  const double fx = cgeo[5 * n], fy = cgeo[5 * n + 1], nxv = cgeo[5 * n + 2],
-               nyv = cgeo[5 * n + 3], th = cgeo[5 * n + 4];
-  const double inv_h = 1.0 / h;
-  if (threadIdx.x < MP - 1) {
-    const int j = threadIdx.x + 1;
-    const double ux = (fx - nodes[j] * nxv - a0) * inv_h, uy = (fy - nodes[j] * nyv - b0) * inv_h;
-    const double ix = floor(ux), iy = floor(uy);
-    pt[j][0] = (float)ix;
-    pt[j][1] = (float)iy;
-    split_df(ux - ix, pt[j][2], pt[j][3]);
-    split_df(uy - iy, pt[j][4], pt[j][5]);
+  const double th = cgeo[5 * n + 4];
+  double acc = 0.0;
+  // sum_k c_k e^{i k theta} over the Hermitian half (Nyquist halved)
+  const int half = Nb / 2;
+  double s, c, ss, cs;
+  sincos(double(threadIdx.x) * th, &s, &c);
+  sincos(double(blockDim.x) * th, &ss, &cs);
+  for (int k = threadIdx.x; k <= half; k += blockDim.x) {
+    const double re = ghat[k].x * c - ghat[k].y * s;
+    const double fac = (k == 0 || 2 * k == Nb) ? 1.0 : 2.0;
+    acc = fma(fac, re, acc);
+    const double c2 = c * cs - s * ss, s2 = s * cs + c * ss;
+    c = c2;
+    s = s2;
   }
+  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  dfl acc[NP];
-#pragma unroll
-  for (int j = 0; j < NP; ++j) acc[j] = {0.f, 0.f};
-  for (int k = threadIdx.x; k < NR; k += blockDim.x) {
-    const float4 a = posR[2 * k], b = posR[2 * k + 1], c = abR[k];
-#pragma unroll
-    for (int j = 1; j < NP; ++j) {
-      if (KMP == 0 && j >= MP) break;
-      // (point - node) = (i_p - i_n) + (f_p - f_n)
-      const dfl dx = df_add(int_minus(pt[j][0] - a.x, a.z, a.w), {pt[j][2], pt[j][3]});
-      const dfl dy = df_add(int_minus(pt[j][1] - a.y, b.x, b.y), {pt[j][4], pt[j][5]});
-      const dfl term = dl_term(dx, dy, c.x, c.y, c.z, c.w);
-      const dfl s = two_sum(acc[j].hi, term.hi);
-      acc[j] = fast_two_sum(s.hi, s.lo + (acc[j].lo + term.lo));
-    }
-  }
-  double vals[NP];
-#pragma unroll
-  for (int j = 1; j < NP; ++j) {
-    if (KMP == 0 && j >= MP) break;
-    red[threadIdx.x] = (double)acc[j].hi + (double)acc[j].lo;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    vals[j] = red[0] * inv_h;
-    __syncthreads();
-  }
-  // boundary value: sum_k c_k e^{i k theta} over the Hermitian half (Nyquist halved)
-  {
-    double acc0 = 0.0;
-    const int half = Nb / 2;
-    // e^{i k theta} for k = tid, tid + blockDim, ...: one sincos each for the first k and
-    // the stride, then complex products (at most a few steps: Nb/2 <= a few blockDim)
-    double s, c, ss, cs;
-    sincos(double(threadIdx.x) * th, &s, &c);
-    sincos(double(blockDim.x) * th, &ss, &cs);
-    for (int k = threadIdx.x; k <= half; k += blockDim.x) {
-      double re = ghat_g[k].x * c - ghat_g[k].y * s;
-      double fac = (k == 0 || 2 * k == Nb) ? 1.0 : 2.0;
-      acc0 = fma(fac, re, acc0);
-      const double c2 = c * cs - s * ss, s2 = s * cs + c * ss;
-      c = c2;
-      s = s2;
-    }
-    red[threadIdx.x] = acc0;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-      if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    vals[0] = red[0];
-  }
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      if (KMP == 0 && j >= MP) break;
-      v = fma(cw[(size_t)n * MP + j], vals[j], v);
-    }
-    u[lin[n]] += v;
-  }
+  if (threadIdx.x) return;
+  for (unsigned k = 1; k < blockDim.x / 32; ++k) acc += red[k];
+  double v = cw[(size_t)n * MP] * acc;
+  for (int j = 1; j < MP; ++j)
+    v = fma(cw[(size_t)n * MP + j], vals[(size_t)n * (MP - 1) + j - 1], v);
+  u[lin[n]] += v;
 }
 
 __global__ void k_zero_outside(int nx, const int32_t* row_iv_off, const int32_t* row_iv,
@@ -578,18 +402,34 @@ static void lagr(const double* nodes, int n, double t, double* w) {
   }
 }
 
-// Node splits of a k_dlp launch over n points and N nodes: each point's sum over the
-// nodes is cut into S consecutive node ranges, one row of blocks each (partial sums
-// combined by k_dlp_combine in range order), so that a launch over few points still
-// has about 48 warps per SM; below that the sums are bound by each warp's dependent
-// double-float chain rather than by issue.  At most 8 ranges of at least 1024 nodes.
-static int dlp_splits(int64_t n, int N, int n_sm) {
-  if (n_sm <= 0 || n <= 0) return 1;
-  const int64_t warps = (n + 255) / 256 * 8;
-  int64_t S = (48LL * n_sm + warps - 1) / warps;
-  S = std::min<int64_t>(S, 8);
-  S = std::min<int64_t>(S, std::max(1, N / 1024));
-  return (int)std::max<int64_t>(S, 1);
+// A partition's arrays on the device (coefficients and magnitude word are placed by the
+// caller).  pts: the free points.
+static fc2d_status up_tree(PoissonState* P, DlpDev* d, const DlpTree& t,
+                           const std::vector<double>& px, const std::vector<double>& py) {
+  std::vector<long long> pts(2 * px.size());
+  for (size_t k = 0; k < px.size(); ++k) {
+    pts[2 * k] = std::llrint(std::ldexp(px[t.free_order[k]], t.shift));
+    pts[2 * k + 1] = std::llrint(std::ldexp(py[t.free_order[k]], t.shift));
+  }
+  auto put = [&](auto** dst, const auto& v) {
+    typename std::remove_const<typename std::remove_reference<decltype(**dst)>::type>::type* q =
+        nullptr;
+    const fc2d_status st = up(P, &q, v);
+    *dst = q;
+    return st;
+  };
+  d->shift = t.shift;
+  d->n_expand = (int)t.expand.size();
+  d->n_grid = (int)t.grid_items.size();
+  d->n_free = (int)t.free_items.size();
+  fc2d_status st;
+  if ((st = put(&d->nodes, t.nodes)) || (st = put(&d->box, t.box)) ||
+      (st = put(&d->expand, t.expand)) || (st = put(&d->near, t.near)) ||
+      (st = put(&d->chain, t.chain)) || (st = put(&d->leaf, t.leaf)) ||
+      (st = put(&d->grid_items, t.grid_items)) || (st = put(&d->free_items, t.free_items)) ||
+      (st = put(&d->points, pts)) || (st = put(&d->points_idx, t.free_order)))
+    return st;
+  return FC2D_OK;
 }
 
 fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
@@ -602,8 +442,6 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
   auto* P = new PoissonState();
   P->Nb = Nb;
   P->MP = MP;
-  if (cudaDeviceGetAttribute(&P->n_sm, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess)
-    P->n_sm = 0;
   const Curve& cv = p->curve;
   const double a0 = p->grid.a0, b0 = p->grid.b0, h = p->grid.h;
   const double two_pi = 2.0 * M_PI;
@@ -743,6 +581,30 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
   std::vector<int32_t> far;
   for (size_t l = 0; l < inside.size(); ++l)
     if (inside[l] && !near[l]) far.push_back((int32_t)l);
+  // partitions of the sums, in grid units; the point lists in their leaves' order
+  auto grid = [&](const std::vector<double>& v, double o) {
+    std::vector<double> r(v.size());
+    for (size_t k = 0; k < v.size(); ++k) r[k] = (v[k] - o) / h;
+    return r;
+  };
+  std::vector<double> px, py;
+  for (size_t n = 0; n < close.size(); ++n)
+    for (int j = 1; j < MP; ++j) {
+      px.push_back((cgeo[5 * n] - P->close_nodes[j] * cgeo[5 * n + 2] - a0) / h);
+      py.push_back((cgeo[5 * n + 1] - P->close_nodes[j] * cgeo[5 * n + 3] - b0) / h);
+    }
+  auto partition = [&](std::vector<int32_t>& lin, const std::vector<double>& X,
+                       const std::vector<double>& Y, const std::vector<double>& fx,
+                       const std::vector<double>& fy) {
+    std::vector<int32_t> gi(lin.size()), gj(lin.size()), ord(lin.size());
+    for (size_t k = 0; k < lin.size(); ++k) gi[k] = lin[k] % nx, gj[k] = lin[k] / nx;
+    DlpTree t = dlp_tree(grid(X, a0), grid(Y, b0), gi, gj, fx, fy, std::max(nx, ny));
+    for (size_t k = 0; k < lin.size(); ++k) ord[k] = lin[t.grid_order[k]];
+    lin.swap(ord);
+    return t;
+  };
+  const DlpTree tf = partition(far, x, y, {}, {});
+  const DlpTree tn = partition(mid, rx, ry, px, py);
   P->n_far = (int64_t)far.size();
   P->n_mid = (int64_t)mid.size();
   P->n_close = (int64_t)close.size();
@@ -753,7 +615,9 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       (st = up(P, &P->uwx, uwx)) || (st = up(P, &P->uwy, uwy)) ||
       (st = up(P, &P->far_lin, far)) || (st = up(P, &P->mid_lin, mid)) ||
       (st = up(P, &P->close_lin, close)) || (st = up(P, &P->close_geo, cgeo)) ||
-      (st = up(P, &P->close_w, cw)) || (st = up(P, &P->dnodes, P->close_nodes)) ||
+      (st = up(P, &P->close_w, cw)) || (st = up_tree(P, &P->far, tf, {}, {})) ||
+      (st = up_tree(P, &P->near, tn, px, py)) || (st = alloc(P, &P->close_v, px.size())) ||
+      (st = alloc(P, &P->qB, Nb)) || (st = alloc(P, &P->qR, NR)) ||
       (st = up(P, &P->posB, grid_units(x, y, a0, b0, h))) ||
       (st = up(P, &P->posR, grid_units(rx, ry, a0, b0, h))))
     return fail(st);
@@ -766,11 +630,14 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       (st = alloc(P, &P->phiR, NR)) || (st = alloc(P, &P->ab, (size_t)Nb)) ||
       (st = alloc(P, &P->abR, (size_t)NR)) || (st = alloc(P, &P->c00, 1024)))
     return fail(st);
-  P->s_far = dlp_splits(P->n_far, Nb, P->n_sm);
-  P->s_mid = dlp_splits(P->n_mid, NR, P->n_sm);
-  const size_t n_part = std::max(P->s_far > 1 ? (size_t)P->s_far * P->n_far : 0,
-                                 P->s_mid > 1 ? (size_t)P->s_mid * P->n_mid : 0);
-  if (n_part && (st = alloc(P, &P->part, n_part))) return fail(st);
+  const size_t cf = tf.box.size() * 2 * kDlpOrder, cn = tn.box.size() * 2 * kDlpOrder;
+  unsigned long long* sums = nullptr;
+  if ((st = alloc(P, &sums, cf + cn + 2))) return fail(st);
+  P->sum_bytes = (cf + cn + 2) * sizeof(*sums);
+  P->far.coef = sums;
+  P->near.coef = sums + cf;
+  P->far.mag = reinterpret_cast<unsigned*>(sums + cf + cn);
+  P->near.mag = reinterpret_cast<unsigned*>(sums + cf + cn + 1);
   k_bie_matrix<<<dim3((Nb + 255) / 256, Nb), 256>>>(Nb, P->bx, P->by, P->bx1, P->by1, ddiag,
                                                     P->A);
   if ((st = cuda_check(cudaDeviceSynchronize(), "BIE matrix"))) return fail(st);
@@ -864,39 +731,31 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
                                                                      (double2*)P->ghat);
     k_density_refine<<<(unsigned)((NR + 255) / 256), 256, 0, s>>>(Nb, NR, (const double2*)P->ghat,
                                                                  (const double2*)P->twr, P->phiR);
-    k_node_coef<<<gb, 256, 0, s>>>(Nb, P->bx1, P->by1, P->phi, P->ab);
-    k_node_coef<<<(unsigned)((NR + 255) / 256), 256, 0, s>>>(NR, P->rx1, P->ry1, P->phiR,
-                                                            P->abR);
-    // the trapezoidal sums at n listed points over N nodes, split into S node ranges
-    auto dlp = [&](int64_t n, const int32_t* lin, int N, int S, const float4* pos,
-                   const float4* ab) {
-      const unsigned nb = (unsigned)((n + 255) / 256);
-      if (S == 1) {
-        k_dlp<false><<<nb, 256, 0, s>>>((int)n, lin, nx, 1.0 / h, N, pos, ab, uf, nullptr);
-        return;
-      }
-      k_dlp<true><<<dim3(nb, (unsigned)S), 256, 0, s>>>((int)n, lin, nx, 1.0 / h, N, pos, ab, uf,
-                                                       P->part);
-      k_dlp_combine<<<nb, 256, 0, s>>>((int)n, lin, S, P->part, 1.0 / h, uf);
-    };
+    cudaMemsetAsync(P->far.coef, 0, P->sum_bytes, s);
+    launch_node_coef(Nb, P->bx1, P->by1, P->phi, P->qB, P->ab, P->far.mag, s);
+    launch_node_coef(NR, P->rx1, P->ry1, P->phiR, P->qR, P->abR, P->near.mag, s);
     {
       ProfScope ps(p, "dlp_far", s);
-      if (P->n_far) dlp(P->n_far, P->far_lin, Nb, P->s_far, P->posB, P->ab);
+      if (P->n_far) {
+        launch_dlp_expand(P->far, P->qB, s);
+        launch_dlp_grid(P->far, P->far_lin, nx, h, P->posB, P->ab, uf, s);
+      }
     }
     {
       ProfScope ps(p, "dlp_near", s);
-      if (P->n_mid) dlp(P->n_mid, P->mid_lin, NR, P->s_mid, P->posR, P->abR);
+      if (P->n_mid || P->n_close) {
+        launch_dlp_expand(P->near, P->qR, s);
+        launch_dlp_grid(P->near, P->mid_lin, nx, h, P->posR, P->abR, uf, s);
+      }
       if (P->n_close) {
+        launch_dlp_free(P->near, h, P->posR, P->abR, P->close_v, s);
         // boundary values g - u_p: reuse ghat for their coefficients
         k_density_dft<<<(unsigned)((Nb / 2 + 1 + 127) / 128), 128, 0, s>>>(
             Nb, P->g, (const double2*)P->twb, (double2*)P->ghat);
-        auto kc = MP == 8    ? k_dlp_close<8>
-                  : MP == 13 ? k_dlp_close<13>
-                  : MP == 15 ? k_dlp_close<15>
-                             : k_dlp_close<0>;
-        kc<<<(unsigned)P->n_close, 256, 0, s>>>(
-            (int)P->n_close, P->close_lin, P->close_geo, P->close_w, P->dnodes, MP, NR, a0, b0,
-            h, P->posR, P->abR, Nb, (const double2*)P->ghat, uf);
+        const int threads = std::min(256, std::max(32, Nb / 16 / 32 * 32));
+        k_close<<<(unsigned)P->n_close, threads, 0, s>>>((int)P->n_close, P->close_lin,
+                                                         P->close_geo, P->close_w, MP, P->close_v,
+                                                         Nb, (const double2*)P->ghat, uf);
       }
     }
     k_zero_outside<<<ny, 256, 0, s>>>(nx, p->dev.row_iv_off, p->dev.row_iv, uf);
