@@ -30,4 +30,11 @@ void launch_dlp_grid(const DlpDev& d, const int32_t* lin, int nx, double h, cons
 void launch_dlp_free(const DlpDev& d, double h, const float4* pos, const float4* ab, double* out,
                      cudaStream_t s);
 
+// u[lin] += Lagrange combination (weights w[n][MP]) of the trigonometric interpolant with
+// coefficients ghat[0 .. Nb/2] (largest magnitude *mag) at the angles with e^{i theta} = z and
+// vals[n][MP - 1]
+void launch_close(int n, const int32_t* lin, const double2* z, const double* w, int MP,
+                  const double* vals, int Nb, const double2* ghat, const unsigned* mag, double* u,
+                  cudaStream_t s);
+
 }  // namespace fc2d

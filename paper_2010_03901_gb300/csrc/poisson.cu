@@ -14,8 +14,8 @@
 //
 // Kernels: k_poisson_cols (forward column DFT, multiplier, inverse column DFT in
 // shared memory), the inverse real rows + quadratic term (fx_wave.cu), k_up_nodes,
-// GMRES kernels, k_density_dft / k_density_refine, the sums (dlp_sum.cu), k_close (one block
-// per close point), k_zero_outside.
+// GMRES (gmres.cu), k_density_dft / k_density_refine, the sums and the close points'
+// values (dlp_sum.cu), k_zero_outside.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -29,11 +29,12 @@
 #include "dlp_sum.h"
 #include "fc2d_kernels.cuh"
 #include "fft_generic.cuh"
+#include "fx.cuh"
+#include "gmres.h"
 #include "plan_internal.h"
 
 namespace fc2d {
 
-constexpr int kGmresMax = 200;
 constexpr int kRefine = 8;
 
 struct PoissonState {
@@ -49,15 +50,16 @@ struct PoissonState {
   int64_t n_far = 0, n_mid = 0, n_close = 0;
   DlpDev far, near;             // partitions of the far and the refined sums
   size_t sum_bytes = 0;         // their coefficients and magnitudes, zeroed per solution
+  unsigned* mags = nullptr;     // magnitudes of the boundary values' and density's coefficients
   double2 *qB = nullptr, *qR = nullptr;  // node coefficients [Nb], [R Nb]
   double* close_v = nullptr;    // [n_close][MP - 1] refined sums along the normals
   int32_t *far_lin = nullptr, *mid_lin = nullptr, *close_lin = nullptr;
-  double* close_geo = nullptr;  // [n_close][5]: foot x, y, normal x, y, theta
+  double* close_z = nullptr;    // [n_close][2]: cos, sin of the foot's parameter
   double* close_w = nullptr;    // [n_close][MP]
   std::vector<double> close_nodes;  // [MP] distances along the normal
   // per-solve workspace
-  double *V = nullptr, *w = nullptr, *h = nullptr, *g = nullptr, *phi = nullptr;
-  struct GmresDev* gm = nullptr;  // GMRES's Hessenberg part and state (device)
+  double *g = nullptr, *phi = nullptr;
+  Gmres gm;
   double *ghat = nullptr, *phiR = nullptr, *c00 = nullptr;
   float4 *ab = nullptr, *abR = nullptr;        // double-float node coefficients [Nb], [R Nb]
   float4 *posB = nullptr, *posR = nullptr;     // nodes in grid units [Nb][2], [R Nb][2]
@@ -162,185 +164,56 @@ __global__ void k_bie_matrix(int Nb, const double* x, const double* y, const dou
   A[(size_t)i * Nb + k] = v;
 }
 
-// y = A x, one warp per row
-// The GMRES vector kernels return at once when *stop is set (a batch of iterations
-// launched ahead of the host's convergence check ran past the converged one).
-__global__ void k_gemv(int n, const double* A, const double* x, double* y, const int* stop) {
-  if (*stop) return;
-  int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const double* a = A + (size_t)row * n;
-  double s = 0.0;
-  for (int k = lane; k < n; k += 32) s = fma(a[k], x[k], s);
-  for (int o = 16; o; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if (lane == 0) y[row] = s;
-}
-
-// h[i] = <V_i, w>, i < m (one block per i)
-__global__ void k_dots(int n, int m, const double* V, const double* w, double* h, const int* stop) {
-  __shared__ double red[256];
-  int i = blockIdx.x;
-  if (i >= m || *stop) return;
-  double s = 0.0;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) s = fma(V[(size_t)i * n + k], w[k], s);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) h[i] = red[0];
-}
-
-// w -= sum_{i<m} h[i] V_i
-__global__ void k_sub_proj(int n, int m, const double* V, const double* h, double* w,
-                           const int* stop) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n || *stop) return;
-  double s = w[k];
-  for (int i = 0; i < m; ++i) s = fma(-h[i], V[(size_t)i * n + k], s);
-  w[k] = s;
-}
-
-__global__ void k_scale_to(int n, const double* w, const double* nrm, double* v, const int* stop) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n && !*stop) v[k] = w[k] / *nrm;
-}
-
-// x = sum_{i<m} y[i] V_i
-__global__ void k_combine(int n, int m, const double* V, const double* y, double* x) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  double s = 0.0;
-  for (int i = 0; i < m; ++i) s = fma(y[i], V[(size_t)i * n + k], s);
-  x[k] = s;
-}
-
-// GMRES's small dense part on the device (one thread): the Hessenberg matrix H, the
-// Givens rotations (cs, sn), the rotated right-hand side e and the state, so that the
-// host reads the state once per batch of iterations instead of after every dot product.
-struct GmresDev {
-  double H[(kGmresMax + 1) * kGmresMax];  // H[i][j] at i kGmresMax + j
-  double cs[kGmresMax], sn[kGmresMax], e[kGmresMax + 1], y[kGmresMax];
-  double h1[kGmresMax + 1], h2[kGmresMax + 1];  // the two Gram-Schmidt passes' projections
-  double nn, hn, beta, resid;                   // ||w||^2, ||w||, ||g||, |e_m| / beta
-  int stop, done, m, pad;                       // stop: no further vector work
-};
-
-// beta = ||g|| (nn holds <g, g>); V_0 = g / beta follows with hn = beta
-__global__ void k_gmres_init(GmresDev* G) {
-  const double beta = sqrt(G->nn);
-  G->beta = beta;
-  G->hn = beta;
-  G->e[0] = beta;
-  G->m = 0;
-  G->resid = 0.0;
-  G->done = beta == 0.0 ? 1 : 0;
-  G->stop = G->done;
-}
-
-// Iteration j after the two projections (h1, h2) and <w, w> (nn): column j of H, the
-// earlier rotations applied to it, its own rotation, the residual estimate |e_{j+1}|.
-__global__ void k_gmres_step(GmresDev* G, int j, double tol) {
-  if (G->done) return;
-  double* H = G->H;
-  for (int i = 0; i <= j; ++i) H[i * kGmresMax + j] = G->h1[i] + G->h2[i];
-  const double hn = sqrt(G->nn);
-  G->hn = hn;
-  H[(j + 1) * kGmresMax + j] = hn;
-  for (int i = 0; i < j; ++i) {
-    const double a = H[i * kGmresMax + j], b = H[(i + 1) * kGmresMax + j];
-    H[i * kGmresMax + j] = G->cs[i] * a + G->sn[i] * b;
-    H[(i + 1) * kGmresMax + j] = -G->sn[i] * a + G->cs[i] * b;
-  }
-  const double a = H[j * kGmresMax + j], b = H[(j + 1) * kGmresMax + j];
-  const double r = hypot(a, b);
-  G->cs[j] = r == 0 ? 1.0 : a / r;
-  G->sn[j] = r == 0 ? 0.0 : b / r;
-  H[j * kGmresMax + j] = r;
-  H[(j + 1) * kGmresMax + j] = 0.0;
-  G->e[j + 1] = -G->sn[j] * G->e[j];
-  G->e[j] = G->cs[j] * G->e[j];
-  G->m = j + 1;
-  G->resid = fabs(G->e[j + 1]) / G->beta;
-  if (fabs(G->e[j + 1]) <= tol * G->beta || hn == 0.0 || j + 1 == kGmresMax) {
-    G->done = 1;
-    G->stop = 1;
-  }
-}
-
-// y from the triangular system R y = e over the first m columns
-__global__ void k_gmres_solve(GmresDev* G) {
-  const int m = G->m;
-  for (int i = m - 1; i >= 0; --i) {
-    double sacc = G->e[i];
-    for (int k = i + 1; k < m; ++k) sacc -= G->H[i * kGmresMax + k] * G->y[k];
-    G->y[i] = sacc / G->H[i * kGmresMax + i];
-  }
-}
-
-// hat phi_k = (1/Nb) sum_j phi_j e^{-2 pi i jk/Nb}, k = 0..Nb/2
-__global__ void k_density_dft(int Nb, const double* phi, const double2* twb, double2* ghat) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
+// hat phi_k = (1/Nb) sum_j phi_j e^{-2 pi i jk/Nb}, k = 0..Nb/2: a warp per k; mag: the
+// largest magnitude
+__global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, const double2* twb,
+                                                     double2* ghat, unsigned* mag) {
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (k > Nb / 2) return;
   double re = 0.0, im = 0.0;
-  for (int j = 0; j < Nb; ++j) {
-    double2 w = twb[(int)(((int64_t)j * k) % Nb)];
+  int at = (int)(((int64_t)lane * k) % Nb);  // j k mod Nb
+  const int step = (int)((32 * (int64_t)k) % Nb);
+  for (int j = lane; j < Nb; j += 32) {
+    const double2 w = twb[at];
     re = fma(phi[j], w.x, re);
     im = fma(phi[j], w.y, im);
+    at += step;
+    at -= at >= Nb ? Nb : 0;
   }
+  for (int o = 16; o; o >>= 1) {
+    re += __shfl_xor_sync(0xFFFFFFFFu, re, o);
+    im += __shfl_xor_sync(0xFFFFFFFFu, im, o);
+  }
+  if (lane) return;
   ghat[k] = double2{re / Nb, im / Nb};
+  atomicMax(mag, max(fx::magnitude(re / Nb), fx::magnitude(im / Nb)));
 }
 
-// trigonometric interpolant of the density at the R Nb refined parameters
-__global__ void k_density_refine(int Nb, int NR, const double2* ghat, const double2* twr,
-                                 double* out) {
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= NR) return;
-  const int half = Nb / 2;
-  double s = ghat[0].x;
-  for (int k = 1; k <= half; ++k) {
-    double2 e = twr[(int)(((int64_t)k * m) % NR)];  // e^{+2 pi i k m/NR}
-    double re = ghat[k].x * e.x - ghat[k].y * e.y;
-    double fac = (2 * k == Nb) ? 1.0 : 2.0;
-    s = fma(fac, re, s);
+// Trigonometric interpolant of the density at the NR = R Nb refined parameters: a warp per
+// pair of parameters m and NR - m, whose sums are C - S and C + S with C = sum a_k cos,
+// S = sum b_k sin (a_k + i b_k: the coefficients, doubled but for the constant and Nyquist).
+__global__ void __launch_bounds__(128) k_density_refine(int Nb, int NR, const double2* ghat,
+                                                        const double2* twr, double* out) {
+  const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (m > NR / 2) return;
+  double C = 0.0, S = 0.0;
+  int at = (int)(((int64_t)lane * m) % NR);  // k m mod NR
+  const int step = (int)((32 * (int64_t)m) % NR);
+  for (int k = lane; k <= Nb / 2; k += 32) {
+    const double2 e = twr[at], g = ghat[k];
+    const double fac = k == 0 || 2 * k == Nb ? 1.0 : 2.0;
+    C = fma(fac * g.x, e.x, C);
+    S = fma(fac * g.y, e.y, S);
+    at += step;
+    at -= at >= NR ? NR : 0;
   }
-  out[m] = s;
-}
-
-// close points: one block per point; the boundary value by trigonometric interpolation of
-// g - u_p and the Lagrange combination with the MP - 1 refined sums along the normal,
-// vals[n][MP - 1].  The block has one thread per 8 frequencies or so: a thread's first
-// e^{i k theta} costs a sincos, the next ones a complex product each.
-__global__ void __launch_bounds__(256) k_close(int n_close, const int32_t* lin, const double* cgeo,
-                                               const double* cw, int MP, const double* vals, int Nb,
-                                               const double2* ghat, double* u) {
-  __shared__ double red[8];
-  const int n = blockIdx.x;
-  const double th = cgeo[5 * n + 4];
-  double acc = 0.0;
-  // sum_k c_k e^{i k theta} over the Hermitian half (Nyquist halved)
-  const int half = Nb / 2;
-  double s, c, ss, cs;
-  sincos(double(threadIdx.x) * th, &s, &c);
-  sincos(double(blockDim.x) * th, &ss, &cs);
-  for (int k = threadIdx.x; k <= half; k += blockDim.x) {
-    const double re = ghat[k].x * c - ghat[k].y * s;
-    const double fac = (k == 0 || 2 * k == Nb) ? 1.0 : 2.0;
-    acc = fma(fac, re, acc);
-    const double c2 = c * cs - s * ss, s2 = s * cs + c * ss;
-    c = c2;
-    s = s2;
+  for (int o = 16; o; o >>= 1) {
+    C += __shfl_xor_sync(0xFFFFFFFFu, C, o);
+    S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
   }
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x) return;
-  for (unsigned k = 1; k < blockDim.x / 32; ++k) acc += red[k];
-  double v = cw[(size_t)n * MP] * acc;
-  for (int j = 1; j < MP; ++j)
-    v = fma(cw[(size_t)n * MP + j], vals[(size_t)n * (MP - 1) + j - 1], v);
-  u[lin[n]] += v;
+  if (lane) return;
+  out[m] = C - S;
+  if (m > 0 && m < NR - m) out[NR - m] = C + S;
 }
 
 __global__ void k_zero_outside(int nx, const int32_t* row_iv_off, const int32_t* row_iv,
@@ -553,7 +426,7 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
   if (st) return fail(st);
   std::vector<uint8_t> near((size_t)nx * ny, 0);
   std::vector<int32_t> mid, close;
-  std::vector<double> cgeo, cw;
+  std::vector<double> cgeo, cz, cw;  // foot and normal, e^{i theta}, Lagrange weights
   P->close_nodes.assign(MP, 0.0);
   for (int j = 1; j < MP; ++j) P->close_nodes[j] = (P->delta + P->s * (j - 1)) / R;
   for (size_t n = 0; n < cl.size(); ++n) {
@@ -572,7 +445,8 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       cv.eval_d(t, 1, xd, yd);
       double sp = std::hypot(xd, yd);
       close.push_back(cl[n]);
-      cgeo.insert(cgeo.end(), {fx, fy, yd / sp, -xd / sp, t});
+      cgeo.insert(cgeo.end(), {fx, fy, yd / sp, -xd / sp});
+      cz.insert(cz.end(), {std::cos(t), std::sin(t)});
       double w[kMaxM];
       lagr(P->close_nodes.data(), MP, eta, w);
       cw.insert(cw.end(), w, w + MP);
@@ -590,8 +464,8 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
   std::vector<double> px, py;
   for (size_t n = 0; n < close.size(); ++n)
     for (int j = 1; j < MP; ++j) {
-      px.push_back((cgeo[5 * n] - P->close_nodes[j] * cgeo[5 * n + 2] - a0) / h);
-      py.push_back((cgeo[5 * n + 1] - P->close_nodes[j] * cgeo[5 * n + 3] - b0) / h);
+      px.push_back((cgeo[4 * n] - P->close_nodes[j] * cgeo[4 * n + 2] - a0) / h);
+      py.push_back((cgeo[4 * n + 1] - P->close_nodes[j] * cgeo[4 * n + 3] - b0) / h);
     }
   auto partition = [&](std::vector<int32_t>& lin, const std::vector<double>& X,
                        const std::vector<double>& Y, const std::vector<double>& fx,
@@ -614,7 +488,7 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       (st = up(P, &P->twr, twr)) || (st = up(P, &P->ui0, ui0)) || (st = up(P, &P->uj0, uj0)) ||
       (st = up(P, &P->uwx, uwx)) || (st = up(P, &P->uwy, uwy)) ||
       (st = up(P, &P->far_lin, far)) || (st = up(P, &P->mid_lin, mid)) ||
-      (st = up(P, &P->close_lin, close)) || (st = up(P, &P->close_geo, cgeo)) ||
+      (st = up(P, &P->close_lin, close)) || (st = up(P, &P->close_z, cz)) ||
       (st = up(P, &P->close_w, cw)) || (st = up_tree(P, &P->far, tf, {}, {})) ||
       (st = up_tree(P, &P->near, tn, px, py)) || (st = alloc(P, &P->close_v, px.size())) ||
       (st = alloc(P, &P->qB, Nb)) || (st = alloc(P, &P->qR, NR)) ||
@@ -622,9 +496,17 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       (st = up(P, &P->posR, grid_units(rx, ry, a0, b0, h))))
     return fail(st);
   double* ddiag = nullptr;
+  int n_sm = 1;
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, p->device);
+  P->gm.n = Nb;
+  P->gm.rows = gmres_rows(Nb, n_sm);
+  P->gm.n_blk = (Nb + P->gm.rows - 1) / P->gm.rows;
+  const size_t n_blk = P->gm.n_blk;
   if ((st = up(P, &ddiag, diag)) || (st = alloc(P, &P->A, (size_t)Nb * Nb)) ||
-      (st = alloc(P, &P->V, (size_t)(kGmresMax + 1) * Nb)) || (st = alloc(P, &P->w, Nb)) ||
-      (st = alloc(P, &P->h, kGmresMax + 2)) || (st = alloc(P, &P->gm, 1)) ||
+      (st = alloc(P, &P->gm.V, (size_t)(kGmresMax + 1) * Nb)) ||
+      (st = alloc(P, &P->gm.w, Nb)) || (st = alloc(P, &P->gm.dev, 1)) || (st = alloc(P, &P->gm.norm, n_blk)) ||
+      (st = alloc(P, &P->gm.part[0], n_blk * (kGmresMax + 1))) ||
+      (st = alloc(P, &P->gm.part[1], n_blk * (kGmresMax + 1))) ||
       (st = alloc(P, &P->g, Nb)) ||
       (st = alloc(P, &P->phi, Nb)) || (st = alloc(P, &P->ghat, 2 * (Nb / 2 + 1))) ||
       (st = alloc(P, &P->phiR, NR)) || (st = alloc(P, &P->ab, (size_t)Nb)) ||
@@ -632,62 +514,19 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
     return fail(st);
   const size_t cf = tf.box.size() * 2 * kDlpOrder, cn = tn.box.size() * 2 * kDlpOrder;
   unsigned long long* sums = nullptr;
-  if ((st = alloc(P, &sums, cf + cn + 2))) return fail(st);
-  P->sum_bytes = (cf + cn + 2) * sizeof(*sums);
+  if ((st = alloc(P, &sums, cf + cn + 4))) return fail(st);
+  P->sum_bytes = (cf + cn + 4) * sizeof(*sums);
   P->far.coef = sums;
   P->near.coef = sums + cf;
   P->far.mag = reinterpret_cast<unsigned*>(sums + cf + cn);
   P->near.mag = reinterpret_cast<unsigned*>(sums + cf + cn + 1);
+  P->mags = reinterpret_cast<unsigned*>(sums + cf + cn + 2);
   k_bie_matrix<<<dim3((Nb + 255) / 256, Nb), 256>>>(Nb, P->bx, P->by, P->bx1, P->by1, ddiag,
                                                     P->A);
+  P->gm.A = P->A;
   if ((st = cuda_check(cudaDeviceSynchronize(), "BIE matrix"))) return fail(st);
   p->poisson = P;
   return FC2D_OK;
-}
-
-// GMRES (no restart) for A phi = g: Arnoldi with classical Gram-Schmidt twice on device
-// vectors, the Hessenberg least squares by Givens rotations on the device
-// (k_gmres_step); iterations are launched in batches of kGmresBatch and the host reads
-// the state once per batch (the vector kernels of iterations past convergence return
-// at once).
-constexpr int kGmresBatch = 8;
-static fc2d_status gmres(PoissonState* P, cudaStream_t s, double tol) {
-  const int n = P->Nb;
-  const unsigned gb = (unsigned)((n + 255) / 256);
-  GmresDev* G = P->gm;
-  int* stop = &G->stop;
-  cudaMemsetAsync(stop, 0, sizeof(int), s);
-  // beta = ||g||, V_0 = g / beta
-  k_dots<<<1, 256, 0, s>>>(n, 1, P->g, P->g, &G->nn, stop);
-  k_gmres_init<<<1, 1, 0, s>>>(G);
-  k_scale_to<<<gb, 256, 0, s>>>(n, P->g, &G->hn, P->V, stop);
-  int state[4] = {0, 0, 0, 0};  // stop, done, m, pad
-  for (int j0 = 0; j0 < kGmresMax && !state[1]; j0 += kGmresBatch) {
-    for (int j = j0; j < std::min(j0 + kGmresBatch, kGmresMax); ++j) {
-      const double* vj = P->V + (size_t)j * n;
-      k_gemv<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(n, P->A, vj, P->w, stop);
-      k_dots<<<j + 1, 256, 0, s>>>(n, j + 1, P->V, P->w, G->h1, stop);
-      k_sub_proj<<<gb, 256, 0, s>>>(n, j + 1, P->V, G->h1, P->w, stop);
-      k_dots<<<j + 1, 256, 0, s>>>(n, j + 1, P->V, P->w, G->h2, stop);
-      k_sub_proj<<<gb, 256, 0, s>>>(n, j + 1, P->V, G->h2, P->w, stop);
-      k_dots<<<1, 256, 0, s>>>(n, 1, P->w, P->w, &G->nn, stop);
-      k_gmres_step<<<1, 1, 0, s>>>(G, j, tol);
-      k_scale_to<<<gb, 256, 0, s>>>(n, P->w, &G->hn, P->V + (size_t)(j + 1) * n, stop);
-    }
-    cudaMemcpyAsync(state, stop, sizeof(state), cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "GMRES");
-  }
-  const int m = state[2];
-  double resid = 0.0;
-  cudaMemcpyAsync(&resid, &G->resid, sizeof(double), cudaMemcpyDeviceToHost, s);
-  k_gmres_solve<<<1, 1, 0, s>>>(G);
-  k_combine<<<gb, 256, 0, s>>>(n, m, P->V, G->y, P->phi);
-  if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "GMRES");
-  P->last_iters = m;
-  P->last_resid = resid;
-  if (resid > 1e3 * tol)
-    return set_error(FC2D_ERR_NOT_CONVERGED, "GMRES did not reach its tolerance");
-  return cuda_check(cudaGetLastError(), "GMRES");
 }
 
 fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const double* fb,
@@ -722,16 +561,19 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
                                   gn + (size_t)f * Nb, P->g);
     {
       ProfScope ps(p, "bie_gmres", s);
-      if ((st = gmres(P, s, 1e-14))) return st;
+      if ((st = gmres_solve(P->gm, P->g, P->phi, 1e-14, &P->last_iters, &P->last_resid, s)))
+        return st;
     }
     if (phi_out) cudaMemcpyAsync(phi_out + (size_t)f * Nb, P->phi, Nb * 8, cudaMemcpyDeviceToDevice, s);
     // density refinement and node coefficients
-    k_density_dft<<<(unsigned)((Nb / 2 + 1 + 127) / 128), 128, 0, s>>>(Nb, P->phi,
-                                                                     (const double2*)P->twb,
-                                                                     (double2*)P->ghat);
-    k_density_refine<<<(unsigned)((NR + 255) / 256), 256, 0, s>>>(Nb, NR, (const double2*)P->ghat,
-                                                                 (const double2*)P->twr, P->phiR);
     cudaMemsetAsync(P->far.coef, 0, P->sum_bytes, s);
+    auto dft = [&](const double* v, unsigned* mag) {
+      k_density_dft<<<(unsigned)((Nb / 2 + 4) / 4), 128, 0, s>>>(Nb, v, (const double2*)P->twb,
+                                                                 (double2*)P->ghat, mag);
+    };
+    dft(P->phi, P->mags + 1);
+    k_density_refine<<<(unsigned)((NR / 2 + 4) / 4), 128, 0, s>>>(
+        Nb, NR, (const double2*)P->ghat, (const double2*)P->twr, P->phiR);
     launch_node_coef(Nb, P->bx1, P->by1, P->phi, P->qB, P->ab, P->far.mag, s);
     launch_node_coef(NR, P->rx1, P->ry1, P->phiR, P->qR, P->abR, P->near.mag, s);
     {
@@ -750,12 +592,9 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
       if (P->n_close) {
         launch_dlp_free(P->near, h, P->posR, P->abR, P->close_v, s);
         // boundary values g - u_p: reuse ghat for their coefficients
-        k_density_dft<<<(unsigned)((Nb / 2 + 1 + 127) / 128), 128, 0, s>>>(
-            Nb, P->g, (const double2*)P->twb, (double2*)P->ghat);
-        const int threads = std::min(256, std::max(32, Nb / 16 / 32 * 32));
-        k_close<<<(unsigned)P->n_close, threads, 0, s>>>((int)P->n_close, P->close_lin,
-                                                         P->close_geo, P->close_w, MP, P->close_v,
-                                                         Nb, (const double2*)P->ghat, uf);
+        dft(P->g, P->mags);
+        launch_close((int)P->n_close, P->close_lin, (const double2*)P->close_z, P->close_w, MP,
+                     P->close_v, Nb, (const double2*)P->ghat, P->mags, uf, s);
       }
     }
     k_zero_outside<<<ny, 256, 0, s>>>(nx, p->dev.row_iv_off, p->dev.row_iv, uf);

@@ -89,3 +89,36 @@ def test_double_layer_sums(name, nb):
         err = np.abs(got - v)
         print(name, nb, int(pick.sum()), float((err / bound).max()), float((err / a).max()))
         assert (err <= bound).all()
+
+
+@pytest.mark.parametrize("name,nb", [("disk128", 40), ("star200", 200), ("star200", 333),
+                                     ("kite160x144", 1201), ("star200", 3000)])
+def test_boundary_density(name, nb):
+    """The density solves the Nystrom system: node counts below, at and above one row per warp
+    and block, odd ones among them."""
+    torch = pytest.importorskip("torch")
+    from oracle import geometry as OG
+    from oracle import poisson as OP
+    from paper_2010_03901_gb300 import fc2d
+    w = W.workload(name)
+    g, p = w.grid, w.params
+    plan = fc2d.fc2d_plan(w.boundary.arrays(), (g.a0, g.b0, g.h, g.nx, g.ny),
+                          dict(B=p.B, k1=p.k1))
+    plan.fc2d_poisson_plan(nb)
+    dev = torch.device("cuda:0")
+    n = len(plan.fc2d_poisson_nodes())
+    fg = torch.zeros((2, g.ny, g.nx), dtype=torch.float64, device=dev)
+    fb = torch.zeros((2, len(plan.fc2d_boundary_points())), dtype=torch.float64, device=dev)
+    th = 2 * np.pi * np.arange(n) / n
+    gn = np.stack([np.cos(2 * th) + 0.3 * np.sin(3 * th) + 1.0, np.zeros(n)])
+    u, phi = torch.zeros_like(fg), torch.ones((2, n), dtype=torch.float64, device=dev)
+    plan.fc2d_poisson(2, fg, fb, torch.tensor(gn, device=dev), u, phi)
+    plan.fc2d_sync_status()
+    phi = phi.cpu().numpy()
+    assert (phi[1] == 0).all() and float(u[1].abs().max()) == 0.0
+    A = OP.bie_matrix(OG.build_geometry(w).curve, n)
+    res = np.linalg.norm(A @ phi[0] - gn[0])
+    # the stopping rule, and n products and sums per row in either program
+    bound = 1e-14 * np.linalg.norm(gn[0]) + n * 2.0 ** -52 * np.linalg.norm(np.abs(A) @ np.abs(phi[0]))
+    print(name, n, res / bound)
+    assert res <= bound
