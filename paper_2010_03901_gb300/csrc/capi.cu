@@ -153,12 +153,13 @@ FftArgs fft_args(fc2d_plan_s* p) {
   a.nx = p->grid.nx;
   a.ny = p->grid.ny;
   a.pitch = (int)row_pitch(p);
+  a.opitch = a.nx / 2 + 1;
   a.nrx = p->fx.n_radix;
   a.nry = p->fy.n_radix;
   for (int i = 0; i < a.nrx; ++i) a.rx[i] = p->fx.radix[i];
   for (int i = 0; i < a.nry; ++i) a.ry[i] = p->fy.radix[i];
-  a.twx = f64 ? (const void*)p->fx.tw64 : (const void*)p->fx.tw32;
-  a.twy = f64 ? (const void*)p->fy.tw64 : (const void*)p->fy.tw32;
+  a.twx = p->fx.tw32;
+  a.twy = p->fy.tw32;
   a.rtw = p->rtw32;
   a.tsx = p->fx.tws32;
   a.tsy = p->fy.tws32;

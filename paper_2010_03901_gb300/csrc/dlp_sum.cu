@@ -212,8 +212,7 @@ __global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
   else out[l] = v * inv_h;
 }
 
-// Close points, a warp each: sum_k c_k z^k over the Hermitian half of the coefficients
-// (doubled but for the constant and Nyquist), lane l taking k = l, l + 32, .. by Horner's
+// Close points, a warp each: Re sum_k c_k z^k over the Hermitian half of the coefficients, lane l taking k = l, l + 32, .. by Horner's
 // rule in z^32 and a last factor z^l; then the Lagrange combination along the normal.  In
 // fixed point (45 instructions per term and no sincos per lane: with FP64 and one sincos per
 // thread the 7500 points of a star at 1024^2 took 190 us).
@@ -225,9 +224,9 @@ __global__ void __launch_bounds__(128) k_close(int n_pts, const int32_t* lin, co
   if (n >= n_pts) return;
   const int half = Nb / 2, terms = half / 32 + 1;
   const unsigned m = *mag;
-  // |c| < 2^59 in the unit of UP = 5: doubled, complex and summed below 2^61
+  // a lane's sum, of up to 2^(E' - E) terms below 2^60.5, stays below that
   const int E = block_exp(m) + (32 - __clz(terms - 1));
-  const int e = m >= 0x7FF00000u ? kNaN : E - 1075 - kUp + 2;
+  const int e = m >= 0x7FF00000u ? kNaN : E - 1075 - kUp + 1;
   const double2 zd = z[n];
   const double one = scalbn(1.0, kFac);
   c64 p = {__double2ll_rn(zd.x * one), __double2ll_rn(zd.y * one)}, zl = {i64(1) << kFac, 0};
@@ -244,9 +243,8 @@ __global__ void __launch_bounds__(128) k_close(int n_pts, const int32_t* lin, co
     const int k = lane + 32 * i;
     s = mulf(s, zp);
     if (k <= half) {
-      const c64 c = from_double<kUp - 2>(ghat[k], E);
-      const int sh = k == 0 || 2 * k == Nb ? 0 : 1;
-      s = {s.x + (c.x << sh), s.y + (c.y << sh)};
+      const c64 c = from_double<kUp - 1>(ghat[k], E);
+      s = s + c;
     }
   }
   s = mulf(s, limbs(zl));

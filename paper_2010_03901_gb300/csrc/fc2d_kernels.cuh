@@ -168,6 +168,7 @@ void launch_assemble(const RowArgs& a, int n_f, bool fp64, const double* f_grid,
 
 struct FftArgs {
   int nx, ny, pitch;          // pitch: complex elements per intermediate row
+  int opitch;                 // of the double spectrum's rows (nx/2 + 1)
   int nrx, nry;               // number of radices
   int rx[24], ry[24];
   const void* twx;            // exp(-2 pi i t/(nx/2)) table for the row transform

@@ -105,13 +105,13 @@ k_cols_fx(FftArgs fa, const double2* __restrict__ inter, double2* __restrict__ f
   transform<LOGNY>(u, v, col, t, true, st, fa.fxy, e);
   e += fa.fxs.exp;
   const bool plain = plain_exp(e);
-  double2* dst = fhat + (size_t)f * N * ncol + kx;
+  double2* dst = fhat + (size_t)f * N * fa.opitch + kx;
   if (live) {
 #pragma unroll
     for (int m = 0; m < 8 / R; ++m)
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        dst[(size_t)out_index<LOGNY>(t, m, r) * ncol] = to_double(scaled(v[m * R + r], fa.fxs), e, plain);
+        dst[(size_t)out_index<LOGNY>(t, m, r) * fa.opitch] = to_double(scaled(v[m * R + r], fa.fxs), e, plain);
   }
 }
 
@@ -157,12 +157,13 @@ k_cols2_b(FftArgs fa, const double2* __restrict__ inter, const int* __restrict__
   e += fa.fxs.exp;
   const bool plain = plain_exp(e);
   if (live) {
-    double2* dst = fhat + (size_t)f * (64 * N2) * ncol + kx;
+    const unsigned opitch = fa.opitch;
+    double2* dst = fhat + (size_t)f * (64 * N2) * opitch + kx;
 #pragma unroll
     for (int mm = 0; mm < 8 / R2; ++mm)
 #pragma unroll
       for (int q = 0; q < R2; ++q)
-        dst[(unsigned)(m1 + 64 * (l * (8 / R2) + mm + 8 * q)) * (unsigned)ncol] =
+        dst[(unsigned)(m1 + 64 * (l * (8 / R2) + mm + 8 * q)) * opitch] =
             to_double(scaled(v[mm * R2 + q], fa.fxs), e, plain);
   }
 }

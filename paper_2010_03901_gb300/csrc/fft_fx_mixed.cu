@@ -220,14 +220,14 @@ k_cols_mixed_b(FftArgs fa, const double2* __restrict__ inter, const int* __restr
   if (threadIdx.x < kMixedSlots) st[threadIdx.x] = 0;
   const int ncol = fa.nx / 2 + 1, kx = blockIdx.x * kCols + (threadIdx.x & (kCols - 1)), f = blockIdx.z;
   const c64* slab = reinterpret_cast<const c64*>(inter) + (size_t)f * fa.ny * fa.pitch;
-  double2* dst = fhat + (size_t)f * fa.ny * ncol + kx;
+  double2* dst = fhat + (size_t)f * fa.ny * fa.opitch + kx;
   __syncthreads();
   pdl_wait();
   pdl_trigger();
   mixed_pass_b(fa.mix, smem_raw, st, slab, fa.pitch, blockIdx.y, kx, kx < ncol, fa.fxwy,
                exps + (size_t)f * fa.mix.n2 * gridDim.x + blockIdx.x, gridDim.x, fa.fxs.exp,
                [&](int row, c64 v, int e, bool plain) {
-                 dst[(unsigned)row * (unsigned)ncol] = to_double(scaled(v, fa.fxs), e, plain);
+                 dst[(unsigned)row * (unsigned)fa.opitch] = to_double(scaled(v, fa.fxs), e, plain);
                });
 }
 

@@ -1036,8 +1036,8 @@ extern "C" fc2d_status fc2d_plan(const fc2d_boundary* boundary, const fc2d_grid*
       (compact && (st = upload(&p->dev.gidx_c, gidx_c))) ||
       (compact && (st = upload(&p->dev.gidx_ic, gidx_ic))) ||
       (st = upload(&p->dev.status, zero_status)) ||
-      (st = upload(&p->fx.tw64, p->fx.tw_host)) || (st = upload(&p->fx.tw32, tw32x)) ||
-      (st = upload(&p->fy.tw64, p->fy.tw_host)) || (st = upload(&p->fy.tw32, tw32y)) ||
+      (st = upload(&p->fx.tw32, tw32x)) ||
+      (st = upload(&p->fy.tw32, tw32y)) ||
       (st = upload(&p->rtw32, rtw32)) ||
       (st = upload(&p->fx.tws32, tsx32)) || (st = upload(&p->fy.tws32, tsy32)) ||
       (st = upload(&p->fx.fx, p->fx.fx_host)) || (st = upload(&p->fy.fx, p->fy.fx_host)) ||
@@ -1113,8 +1113,8 @@ extern "C" void fc2d_destroy(fc2d_plan_t p) {
                   p->dev.s_pb, p->dev.s_sb, p->dev.row_iv_off,
                   p->dev.row_iv, p->dev.row_strip_off, p->dev.row_iv_coff, p->dev.gidx_c,
                   p->dev.gidx_i, p->dev.gw_i, p->dev.wn_i, p->dev.gidx_ic,
-                  p->dev.status, p->fx.tw64, p->fx.tw32,
-                  p->fy.tw64, p->fy.tw32, p->rtw32, p->ws.base,
+                  p->dev.status, p->fx.tw32,
+                  p->fy.tw32, p->rtw32, p->ws.base,
                   p->fx.tws32, p->fy.tws32, p->fx.fx,
                   p->fx.fxs, p->fy.fx, p->fy.fxs, p->rfx};
   for (void* q : ptrs)

@@ -27,7 +27,6 @@ struct FftAxis {
   int n_radix = 0;
   int radix[kMaxRadices] = {0};
   std::vector<double> tw_host;   // interleaved re, im (2N doubles)
-  double* tw64 = nullptr;        // device, 2N doubles
   float* tw32 = nullptr;         // device, 2N floats
   // power-of-two lengths: per-stage twiddles [stage][r][k] for the radix-8 (fxs) and
   // radix-16 (float) Stockham sequences (see stage_twiddles in plan.cpp)

@@ -12,8 +12,8 @@
 //   the degree M_P - 1 Lagrange interpolant along the normal through the boundary
 //   value (trigonometric interpolation of g - u_p) and refined sums at 5s/R..(M_P+3)s/R.
 //
-// Kernels: k_poisson_cols (forward column DFT, multiplier, inverse column DFT in
-// shared memory), the inverse real rows + quadratic term (fx_wave.cu), k_up_nodes,
+// Kernels: the forward column DFT, k_symbol (multiplier), the same DFT on reversed rows as the
+// inverse one, the inverse real rows + quadratic term (fx_wave.cu), k_up_nodes,
 // GMRES (gmres.cu), k_density_dft / k_density_refine, the sums and the close points'
 // values (dlp_sum.cu), k_zero_outside.
 #include <cuda_runtime.h>
@@ -28,7 +28,6 @@
 #include "dd.h"
 #include "dlp_sum.h"
 #include "fc2d_kernels.cuh"
-#include "fft_generic.cuh"
 #include "fx.cuh"
 #include "gmres.h"
 #include "plan_internal.h"
@@ -51,6 +50,8 @@ struct PoissonState {
   DlpDev far, near;             // partitions of the far and the refined sums
   size_t sum_bytes = 0;         // their coefficients and magnitudes, zeroed per solution
   unsigned* mags = nullptr;     // magnitudes of the boundary values' and density's coefficients
+  double2* spec = nullptr;      // [ny][pitch]: a function's spectrum, then its inverse columns
+  int* exps = nullptr;          // of its two-pass columns
   double2 *qB = nullptr, *qR = nullptr;  // node coefficients [Nb], [R Nb]
   double* close_v = nullptr;    // [n_close][MP - 1] refined sums along the normals
   int32_t *far_lin = nullptr, *mid_lin = nullptr, *close_lin = nullptr;
@@ -83,70 +84,49 @@ void poisson_destroy(fc2d_plan_s* p) {
 // ------------------------------------------------------------------------- //
 // Kernels
 // ------------------------------------------------------------------------- //
-// Forward column DFT, hat f = scale * DFT, record hat f_00, multiply by the inverse
-// Laplacian symbol, inverse (unnormalised) column DFT by conj(DFT(conj)), in place.
-__global__ void __launch_bounds__(256) k_poisson_cols(FftArgs fa, int cb, double2* inter,
-                                                      double* c00, double Lx, double Ly) {
-  using C = double2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ny = fa.ny, ncol = fa.nx / 2 + 1;
-  const int c0 = blockIdx.x * cb, f = blockIdx.y;
-  const int nc = min(cb, ncol - c0);
-  C* A = reinterpret_cast<C*>(smem_raw);
-  C* Bf = A + (size_t)cb * ny;
-  C* col = inter + (size_t)f * ny * fa.pitch + c0;
-  for (int idx = threadIdx.x; idx < ny * cb; idx += blockDim.x) {
-    int y = idx / cb, c = idx - y * cb;
-    A[(size_t)c * ny + y] = c < nc ? col[(size_t)y * fa.pitch + c] : C{0, 0};
-  }
-  __syncthreads();
-  const C* tw = reinterpret_cast<const C*>(fa.twy);
-  C* Y = stockham<double>(A, Bf, ny, cb, fa.ry, fa.nry, tw, 1);
-  C* other = (Y == A) ? Bf : A;
-  const double two_pi = 6.283185307179586476925286766559;
-  for (int idx = threadIdx.x; idx < ny * cb; idx += blockDim.x) {
-    int c = idx / ny, ky = idx - c * ny;
-    int kx = c0 + c;
-    C v = Y[idx];
-    v.x *= fa.scale;
-    v.y *= fa.scale;
-    int m = ky <= ny / 2 ? ky : ky - ny;
-    double kxx = two_pi * kx / Lx, kyy = two_pi * m / Ly;
-    double k2 = kxx * kxx + kyy * kyy;
-    C b;
+// hat f times the inverse Laplacian symbol; hat f_00 goes to c00.  The rows are written in
+// reversed order, ky at (ny - ky) mod ny: the forward column DFT of that is the inverse one of
+// the spectrum.
+constexpr int kSymbolRows = 8;
+__global__ void __launch_bounds__(128) k_symbol(int nxh, int ny, int pitch, const double2* spec,
+                                                double2* out, double* c00, double wx, double wy) {
+  const int kx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (kx >= nxh) return;
+  const double kxx = wx * kx, kx2 = kxx * kxx;
+#pragma unroll
+  for (int r = 0; r < kSymbolRows; ++r) {
+    const int ky = blockIdx.y * kSymbolRows + r;
+    if (ky >= ny) return;
+    const double kyy = wy * (ky <= ny / 2 ? ky : ky - ny);
+    const double2 v = spec[(size_t)ky * pitch + kx];
+    double2 b{0.0, 0.0};
     if (kx == 0 && ky == 0) {
-      c00[f] = v.x;
-      b = C{0, 0};
+      *c00 = v.x;
     } else {
-      b = C{-v.x / k2, -v.y / k2};
+      const double s = -1.0 / fma(kyy, kyy, kx2);
+      b = double2{v.x * s, v.y * s};
     }
-    Y[idx] = C{b.x, -b.y};  // conj for the inverse
-  }
-  __syncthreads();
-  C* Z = stockham<double>(Y, other, ny, cb, fa.ry, fa.nry, tw, 1);
-  for (int idx = threadIdx.x; idx < ny * cb; idx += blockDim.x) {
-    int y = idx / cb, c = idx - y * cb;
-    if (c < nc) {
-      C v = Z[(size_t)c * ny + y];
-      col[(size_t)y * fa.pitch + c] = C{v.x, -v.y};
-    }
+    out[(size_t)(ky ? ny - ky : 0) * pitch + kx] = b;
   }
 }
 
-// u_p at the BIE nodes: iterated 1D interpolation (x on MP rows, then y).
-__global__ void k_up_nodes(int Nb, int MP, int nx, const int32_t* i0, const int32_t* j0,
-                           const double* wx, const double* wy, const double* up,
-                           const double* g, double* ghom) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= Nb) return;
+// u_p at the BIE nodes: iterated 1D interpolation (x on MP rows, a lane each, then y).
+__global__ void __launch_bounds__(128) k_up_nodes(int Nb, int MP, int nx, const int32_t* i0,
+                                                  const int32_t* j0, const double* wx,
+                                                  const double* wy, const double* up,
+                                                  const double* g, double* ghom) {
+  static_assert(kMaxM <= 16, "a lane per row");
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 4, a = threadIdx.x & 15;
   double acc = 0.0;
-  for (int a = 0; a < MP; ++a) {
+  if (k < Nb && a < MP) {
     const double* r = up + (size_t)(j0[k] + a) * nx + i0[k];
     double v = 0.0;
+#pragma unroll 8
     for (int b = 0; b < MP; ++b) v = fma(wx[k * MP + b], r[b], v);
-    acc = fma(wy[k * MP + a], v, acc);
+    acc = wy[k * MP + a] * v;
   }
-  ghom[k] = g[k] - acc;
+  for (int o = 8; o; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+  if (k < Nb && a == 0) ghom[k] = g[k] - acc;
 }
 
 __global__ void k_bie_matrix(int Nb, const double* x, const double* y, const double* x1,
@@ -164,8 +144,9 @@ __global__ void k_bie_matrix(int Nb, const double* x, const double* y, const dou
   A[(size_t)i * Nb + k] = v;
 }
 
-// hat phi_k = (1/Nb) sum_j phi_j e^{-2 pi i jk/Nb}, k = 0..Nb/2: a warp per k; mag: the
-// largest magnitude
+// Coefficients of the trigonometric interpolant of phi: (1/Nb) sum_j phi_j e^{-2 pi i jk/Nb},
+// k = 0..Nb/2, doubled for 0 < k < Nb/2 (the pairs k, Nb - k); a warp per k.  mag: the largest
+// magnitude.
 __global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, const double2* twb,
                                                      double2* ghat, unsigned* mag) {
   const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -173,6 +154,7 @@ __global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, 
   double re = 0.0, im = 0.0;
   int at = (int)(((int64_t)lane * k) % Nb);  // j k mod Nb
   const int step = (int)((32 * (int64_t)k) % Nb);
+#pragma unroll 8
   for (int j = lane; j < Nb; j += 32) {
     const double2 w = twb[at];
     re = fma(phi[j], w.x, re);
@@ -185,35 +167,44 @@ __global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, 
     im += __shfl_xor_sync(0xFFFFFFFFu, im, o);
   }
   if (lane) return;
-  ghat[k] = double2{re / Nb, im / Nb};
-  atomicMax(mag, max(fx::magnitude(re / Nb), fx::magnitude(im / Nb)));
+  const double fac = k == 0 || 2 * k == Nb ? 1.0 : 2.0;
+  re = fac * re / Nb;
+  im = fac * im / Nb;
+  ghat[k] = double2{re, im};
+  atomicMax(mag, max(fx::magnitude(re), fx::magnitude(im)));
 }
 
-// Trigonometric interpolant of the density at the NR = R Nb refined parameters: a warp per
-// pair of parameters m and NR - m, whose sums are C - S and C + S with C = sum a_k cos,
-// S = sum b_k sin (a_k + i b_k: the coefficients, doubled but for the constant and Nyquist).
+// Trigonometric interpolant of the density at the NR = 8 Nb refined parameters: a warp per
+// quadruple of parameters x, -x, pi - x, pi + x, whose sums are +- combinations of the cosine
+// and sine sums over even and odd k (even and odd lanes).
 __global__ void __launch_bounds__(128) k_density_refine(int Nb, int NR, const double2* ghat,
                                                         const double2* twr, double* out) {
   const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (m > NR / 2) return;
+  if (m > NR / 4) return;
   double C = 0.0, S = 0.0;
   int at = (int)(((int64_t)lane * m) % NR);  // k m mod NR
   const int step = (int)((32 * (int64_t)m) % NR);
+#pragma unroll 4
   for (int k = lane; k <= Nb / 2; k += 32) {
     const double2 e = twr[at], g = ghat[k];
-    const double fac = k == 0 || 2 * k == Nb ? 1.0 : 2.0;
-    C = fma(fac * g.x, e.x, C);
-    S = fma(fac * g.y, e.y, S);
+    C = fma(g.x, e.x, C);
+    S = fma(g.y, e.y, S);
     at += step;
     at -= at >= NR ? NR : 0;
   }
-  for (int o = 16; o; o >>= 1) {
+  for (int o = 16; o > 1; o >>= 1) {
     C += __shfl_xor_sync(0xFFFFFFFFu, C, o);
     S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
   }
+  const double Co = __shfl_xor_sync(0xFFFFFFFFu, C, 1), So = __shfl_xor_sync(0xFFFFFFFFu, S, 1);
   if (lane) return;
-  out[m] = C - S;
-  if (m > 0 && m < NR - m) out[NR - m] = C + S;
+  const double cp = C + Co, cm = C - Co, sp = S + So, sm = S - So;
+  const int half = NR / 2;
+  out[m] = cp - sp;
+  out[half - m] = cm + sm;
+  if (m == 0) return;
+  out[half + m] = cm - sm;
+  out[NR - m] = cp + sp;
 }
 
 __global__ void k_zero_outside(int nx, const int32_t* row_iv_off, const int32_t* row_iv,
@@ -491,7 +482,8 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
       (st = up(P, &P->close_lin, close)) || (st = up(P, &P->close_z, cz)) ||
       (st = up(P, &P->close_w, cw)) || (st = up_tree(P, &P->far, tf, {}, {})) ||
       (st = up_tree(P, &P->near, tn, px, py)) || (st = alloc(P, &P->close_v, px.size())) ||
-      (st = alloc(P, &P->qB, Nb)) || (st = alloc(P, &P->qR, NR)) ||
+      (st = alloc(P, &P->spec, (size_t)ny * row_pitch(p))) ||
+      (st = alloc(P, &P->exps, fx_exps(nx, ny, 1))) || (st = alloc(P, &P->qB, Nb)) || (st = alloc(P, &P->qR, NR)) ||
       (st = up(P, &P->posB, grid_units(x, y, a0, b0, h))) ||
       (st = up(P, &P->posR, grid_units(rx, ry, a0, b0, h))))
     return fail(st);
@@ -536,28 +528,35 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
   const int nx = p->grid.nx, ny = p->grid.ny, Nb = P->Nb, MP = P->MP, NR = P->R * Nb;
   const double a0 = p->grid.a0, b0 = p->grid.b0, h = p->grid.h;
   if (n_f > 1024) return set_error(FC2D_ERR_ARG, "fc2d_poisson: n_f <= 1024");
-  // u_p (forward rows already in `inter` from the caller): multiplier + inverse
-  const FftArgs fa = fft_args(p);
-  {
-    ProfScope ps(p, "poisson_cols", s);
-    const int ncol = nx / 2 + 1;
-    int cb = 1;
-    while (cb < 8 && 2 * (size_t)(2 * cb) * ny * sizeof(double2) <= 200 * 1024) cb *= 2;
-    size_t sm = 2 * (size_t)cb * ny * sizeof(double2);
-    cudaFuncSetAttribute(k_poisson_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_poisson_cols<<<dim3((ncol + cb - 1) / cb, n_f), 256, sm, s>>>(
-        fa, cb, (double2*)inter, P->c00, nx * h, ny * h);
-  }
-  {
-    ProfScope ps(p, "poisson_rows", s);
-    launch_inverse_rows(fa, n_f, inter, P->c00, a0, b0, h, u, s);
+  // u_p (forward rows already in `inter` from the caller): the forward columns, the symbol,
+  // the inverse columns and rows, one function at a time
+  FftArgs fa = fft_args(p);
+  const size_t slab = (size_t)ny * fa.pitch;
+  auto* in = static_cast<double2*>(inter);
+  FftArgs inv = fa;
+  fa.exps = inv.exps = P->exps;
+  fa.opitch = inv.opitch = fa.pitch;
+  inv.fxs = FxFactor{0, 0, 0};
+  for (int f = 0; f < n_f; ++f) {
+    {
+      ProfScope ps(p, "poisson_cols", s);
+      launch_fft_cols(fa, 1, true, in + f * slab, P->spec, s);
+      k_symbol<<<dim3((nx / 2 + 128) / 128, (ny + kSymbolRows - 1) / kSymbolRows), 128, 0, s>>>(
+          nx / 2 + 1, ny, fa.pitch, P->spec, in + f * slab, P->c00 + f, 2.0 * M_PI / (nx * h),
+          2.0 * M_PI / (ny * h));
+      launch_fft_cols(inv, 1, true, in + f * slab, P->spec, s);
+    }
+    {
+      ProfScope ps(p, "poisson_rows", s);
+      launch_inverse_rows(fa, 1, P->spec, P->c00 + f, a0, b0, h, u + (size_t)f * nx * ny, s);
+    }
   }
   fc2d_status st = cuda_check(cudaGetLastError(), "Poisson particular solution");
   if (st) return st;
   const unsigned gb = (unsigned)((Nb + 255) / 256);
   for (int f = 0; f < n_f; ++f) {
     double* uf = u + (size_t)f * nx * ny;
-    k_up_nodes<<<gb, 256, 0, s>>>(Nb, MP, nx, P->ui0, P->uj0, P->uwx, P->uwy, uf,
+    k_up_nodes<<<(unsigned)((Nb + 7) / 8), 128, 0, s>>>(Nb, MP, nx, P->ui0, P->uj0, P->uwx, P->uwy, uf,
                                   gn + (size_t)f * Nb, P->g);
     {
       ProfScope ps(p, "bie_gmres", s);
@@ -572,7 +571,7 @@ fc2d_status poisson_solve(fc2d_plan_s* p, int n_f, const double* fg, const doubl
                                                                  (double2*)P->ghat, mag);
     };
     dft(P->phi, P->mags + 1);
-    k_density_refine<<<(unsigned)((NR / 2 + 4) / 4), 128, 0, s>>>(
+    k_density_refine<<<(unsigned)((NR / 4 + 4) / 4), 128, 0, s>>>(
         Nb, NR, (const double2*)P->ghat, (const double2*)P->twr, P->phiR);
     launch_node_coef(Nb, P->bx1, P->by1, P->phi, P->qB, P->ab, P->far.mag, s);
     launch_node_coef(NR, P->rx1, P->ry1, P->phiR, P->qR, P->abR, P->near.mag, s);
