@@ -5,6 +5,15 @@
 // fixed point; the warps of a box add up by integer atomics (exact in any order).
 // k_dlp_eval: one block per (leaf, up to 64 points): Horner's rule for each expansion of
 // the leaf's chain, then the near nodes term by term in double-float arithmetic.
+//
+// The star r = 1 + 0.3 cos 5t at 1024^2 with 1024 nodes (8192 refined): far points 1765 us
+// term by term (3.5e8 terms of 115 FP32 instructions, bound by their issue), 86 us so; the
+// near band and the close points' sums 5300 and 250 us.  A complex product of 64-bit values
+// is 12 integer multiply-adds (58 per clock and SM) and about 20 other instructions, where
+// its four FP64 multiply-adds cost 256 issue slots.  The expansions are bound by the
+// multiply-adds at 38% issue (168 registers for the 32 accumulators: 12 warps per SM), the
+// evaluation at 44 to 51%.  Error against long double sums: 3e-15 to 8e-15 of the sum of the
+// terms' moduli, the near terms' double-float rounding.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -21,6 +30,10 @@ namespace {
 
 constexpr int P = kDlpOrder;
 static_assert(P == 32, "one coefficient per lane");
+// From coefficient W on 32 bits do: |(z - c)/R0|^W <= 2^-34.7 scales their rounding (the errors
+// measured against long double sums are the same as with 64 bits throughout).  At 1024^2 the
+// near band takes 289 us for W = 20, 303 for 24, 327 for 32.
+constexpr int W = 20;
 constexpr int kUp = 8;    // q in units of 2^(E - 1075 - kUp): |Re|, |Im| < 2^61
 constexpr int kFac = 61;  // factors w, t (at most 1) times 2^kFac
 
@@ -44,22 +57,37 @@ __device__ __forceinline__ c64 mulf(c64 a, int4 w) {
           (i64)((unsigned long long)hy << D) + (my >> (32 - D))};
 }
 
+// v 2^-N as 32 bits, and the product of such a value with a factor w 2^30
+template <int N> __device__ __forceinline__ int narrow(i64 v) {
+  return (int)((v + (i64(1) << (N - 1))) >> N);
+}
+__device__ __forceinline__ void mul30(int& x, int& y, int wx, int wy) {
+  const i64 px = mad(x, wx, mad(y, -wy, 1 << 29)), py = mad(x, wy, mad(y, wx, 1 << 29));
+  x = (int)(px >> 30);
+  y = (int)(py >> 30);
+}
+
+// v/m for a box's m: v times its reciprocal
+__device__ __forceinline__ i64 over(i64 v, i64 inv) {
+  return (i64)((unsigned long long)mulh(v, inv) << 2);
+}
+
 // R0/d 2^kFac for d = x 2^-shift: the float reciprocal (about 2^-20), two Newton steps
-__device__ __forceinline__ int4 inverse(c64 x, int lr, int shift) {
+__device__ __forceinline__ c64 inverse(c64 x, const DlpBox& b, int shift) {
+  const int lr = b.lr;
   const float dx = (float)(int)(x.x >> 32), dy = (float)(int)(x.y >> 32);
   // x 2^-32 = d 2^(shift - 32)
-  const float s = __frcp_rn(fmaf(dx, dx, dy * dy)) * exp2f((float)(lr + shift - 32 + kFac - 30));
+  const float s = __frcp_rn(fmaf(dx, dx, dy * dy)) * (float)b.one * exp2f((float)(kFac - 62));
   c64 w = {(i64)__float2int_rn(dx * s) << 30, -((i64)__float2int_rn(dy * s) << 30)};
-  const i64 one = i64(1) << (lr + shift);  // R0 in the unit of x
   const int up = kFac - lr - shift;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int4 l = limbs(w);
     const c64 p = mulf(x, l);                           // R0 (1 - e)
-    const c64 c = mulf(c64{one - p.x, -p.y}, l);        // e w, in units of 2^(kFac - up)
-    w = {w.x + (c.x << up), w.y + (c.y << up)};
+    const c64 c = mulf(c64{b.one - p.x, -p.y}, l);      // e R0 w, in the unit of x
+    w = {w.x + over(c.x << up, b.inv), w.y + over(c.y << up, b.inv)};
   }
-  return limbs(w);
+  return w;
 }
 
 __global__ void __launch_bounds__(256) k_node_coef(int N, const double* x1, const double* y1,
@@ -91,7 +119,7 @@ template <int H> __device__ __forceinline__ void fold(i64* a, int lane) {
   if constexpr (H > 2) fold<H / 2>(a, lane);
 }
 
-__global__ void __launch_bounds__(128) k_dlp_expand(int n_spans, const DlpSpan* spans,
+__global__ void __launch_bounds__(128, 3) k_dlp_expand(int n_spans, const DlpSpan* spans,
                                                     const DlpBox* boxes, const c64* pos, int shift,
                                                     const double2* q, const unsigned* mag,
                                                     unsigned long long* coef) {
@@ -102,20 +130,34 @@ __global__ void __launch_bounds__(128) k_dlp_expand(int n_spans, const DlpSpan* 
   const int E = block_exp(*mag);
   const i64 half = b.hb ? i64(1) << (b.hb - 1) : 0;
   i64 a[2 * P];
+  int n[2 * (P - W)];
 #pragma unroll
-  for (int j = 0; j < 2 * P; ++j) a[j] = 0;
+  for (int j = 0; j < 2 * W; ++j) a[j] = 0;
+#pragma unroll
+  for (int j = 0; j < 2 * (P - W); ++j) n[j] = 0;
   for (int k = sp.k0 + lane; k < sp.k0 + sp.n; k += 32) {
     const c64 z = pos[k];
-    const int4 w = inverse(c64{z.x - b.cx, z.y - b.cy}, b.lr, shift);
+    const c64 wi = inverse(c64{z.x - b.cx, z.y - b.cy}, b, shift);
+    const int4 w = limbs(wi);
     c64 g = mulf(from_double<kUp>(q[k], E), w);
     g = {(g.x + half) >> b.hb, (g.y + half) >> b.hb};
 #pragma unroll
-    for (int j = 0; j < P; ++j) {
+    for (int j = 0; j < W; ++j) {
       a[2 * j] += g.x;
       a[2 * j + 1] += g.y;
       if (j + 1 < P) g = mulf(g, w);
     }
+    int gx = narrow<32>(g.x), gy = narrow<32>(g.y);
+    const int wx = narrow<kFac - 30>(wi.x), wy = narrow<kFac - 30>(wi.y);
+#pragma unroll
+    for (int j = W; j < P; ++j) {
+      n[2 * (j - W)] += gx;
+      n[2 * (j - W) + 1] += gy;
+      mul30(gx, gy, wx, wy);
+    }
   }
+#pragma unroll
+  for (int j = 2 * W; j < 2 * P; ++j) a[j] = (i64)n[j - 2 * W] << 32;
   fold<P>(a, lane);  // lane j holds A_j
   unsigned long long* dst = coef + (size_t)sp.box * 2 * P + 2 * lane;
   atomicAdd(dst, (unsigned long long)a[0]);
@@ -162,13 +204,25 @@ __global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
     const DlpBox b = boxes[box];
     __syncthreads();
     const int up = kFac - shift - b.lr;
-    const int4 z = limbs(c64{(i64)((unsigned long long)(X.x - b.cx) << up),
-                             (i64)((unsigned long long)(X.y - b.cy) << up)});
-    c64 s = A[P - 1];
+    const c64 zi = {over((i64)((unsigned long long)(X.x - b.cx) << up), b.inv),
+                    over((i64)((unsigned long long)(X.y - b.cy) << up), b.inv)};
+    const int4 z = limbs(zi);
+    c64 s;
+    {
+      const int zx = narrow<kFac - 30>(zi.x), zy = narrow<kFac - 30>(zi.y);
+      int sx = (int)(A[P - 1].x >> 32), sy = (int)(A[P - 1].y >> 32);
+#pragma unroll
+      for (int j = P - 2; j >= W; --j) {
+        mul30(sx, sy, zx, zy);
+        sx += (int)(A[j].x >> 32);
+        sy += (int)(A[j].y >> 32);
+      }
+      s = A[W - 1] + mulf(c64{(i64)sx << 32, (i64)sy << 32}, z);
+    }
 #pragma unroll 8
-    for (int j = P - 2; j >= 0; --j) s = A[j] + mulf(s, z);
+    for (int j = W - 2; j >= 0; --j) s = A[j] + mulf(s, z);
     const int e = e0 + b.hb - b.lr;
-    v -= to_double(s.y, e, plain_exp(e));
+    v -= to_double(s.y, e, plain_exp(e)) * b.rm;
   }
   float px, pfh, pfl, py, qfh, qfl;
   if (GRID) {
@@ -214,8 +268,9 @@ __global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
 
 // Close points, a warp each: Re sum_k c_k z^k over the Hermitian half of the coefficients, lane l taking k = l, l + 32, .. by Horner's
 // rule in z^32 and a last factor z^l; then the Lagrange combination along the normal.  In
-// fixed point (45 instructions per term and no sincos per lane: with FP64 and one sincos per
-// thread the 7500 points of a star at 1024^2 took 190 us).
+// fixed point: 45 instructions per term and no sincos per lane, 35 us for the 7500 points of a
+// star at 1024^2 (with an FP64 sincos per thread and the transform of the boundary values by a
+// thread per frequency, 335 us).
 __global__ void __launch_bounds__(128) k_close(int n_pts, const int32_t* lin, const double2* z,
                                                const double* w, int MP, const double* vals, int Nb,
                                                const double2* ghat, const unsigned* mag,

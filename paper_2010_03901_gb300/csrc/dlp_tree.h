@@ -19,8 +19,10 @@ constexpr int kDlpNodes = 128;      // nodes per expansion work item (a warp), a
 constexpr int kDlpPoints = 64;      // points per evaluation work item (a block), at most
 
 struct DlpBox {
-  long long cx, cy;  // centre, grid units times 2^shift
-  int lr, hb;        // R0 = 2^lr; 2^hb bounds 2^1.5 sum |R0/(z_k - c)|
+  long long cx, cy;    // centre, grid units times 2^shift
+  long long one, inv;  // R0 = m 2^lr, 1 <= m < 2, in the same unit; 2^62/m
+  double rm;           // 1/m
+  int lr, hb;          // 2^hb bounds 2^1.5 sum |R0/(z_k - c)|
 };
 struct DlpSpan {  // expansion item: nodes k0 .. k0 + n - 1 into a box; direct span (box unused)
   int box, k0, n, pad;

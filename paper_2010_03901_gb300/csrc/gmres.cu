@@ -33,11 +33,25 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// sum of x[0 .. n) by every warp for itself
-__device__ __forceinline__ double total(const double* x, int n) {
+// sum of x[k stride], k = k0, k0 + step, .. < n, with N loads in flight at a time (the
+// blocks' partial sums come from L2, 0.7 us away)
+template <int N>
+__device__ __forceinline__ double gather(const double* x, size_t stride, int k0, int step, int n) {
   double v = 0.0;
-  for (int k = threadIdx.x & 31; k < n; k += 32) v += __ldcg(x + k);
-  return warp_sum(v);
+  for (int k = k0; k < n; k += N * step) {
+    double r[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) r[q] = k + q * step < n ? __ldcg(x + (k + q * step) * stride) : 0.0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) v += r[q];
+  }
+  return v;
+}
+
+// sum of x[0 .. n) by a warp.  (An FP64 instruction occupies the SM's pipe for 16 clocks
+// whatever the number of active lanes: what one warp can do for the block, one warp does.)
+__device__ __forceinline__ double total(const double* x, int n) {
+  return warp_sum(gather<5>(x, 1, threadIdx.x & 31, 32, n));
 }
 
 // partial projections part[i] = sum over the block's rows of V_i w, i < m
@@ -112,17 +126,19 @@ __device__ __forceinline__ void project(int n, int nr, int n_blk, int m, const d
                                         double* h_out) {
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
   for (int i0 = 0; i0 < m; i0 += 32) {
+    // width lanes per partial vector, 32 / width of those per warp
+    const int width = m - i0 > 16 ? 32 : m - i0 > 8 ? 16 : 8;
+    const int i = i0 + (lane & (width - 1)), per = 32 / width;
     double v = 0.0;
-    if (i0 + lane < m) {
-#pragma unroll 4
-      for (int b = wp; b < n_blk; b += kT / 32) v += __ldcg(part + (size_t)b * kLd + i0 + lane);
-    }
+    if (i < m) v = gather<10>(part + i, kLd, wp * per + lane / width, kT / width, n_blk);
+    if (width < 32) v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
+    if (width < 16) v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
     red[wp][lane] = v;
     __syncthreads();
-    if (wp == 0 && i0 + lane < m) {
+    if (wp == 0 && lane < width && i < m) {
       for (int k = 1; k < kT / 32; ++k) v += red[k][lane];
-      hs[i0 + lane] = v;
-      if (h_out) h_out[i0 + lane] = v;
+      hs[i] = v;
+      if (h_out) h_out[i] = v;
     }
     __syncthreads();
   }
@@ -183,6 +199,7 @@ __global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __r
   double* As = sm;
   double* wv = sm + (SMEM ? (size_t)rows * n : 0);
   double* ws = wv + (SMEM ? n : 0);  // the block's rows of w; block 0: the rotations
+  double* wn = ws + rows;
   double* Vb = V + r0;
   unsigned gen = 0;
   for (int k = t; k < nr; k += kT) {
@@ -196,22 +213,32 @@ __global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __r
     for (size_t k = t; k < (size_t)nr * n; k += kT) As[k] = A[(size_t)r0 * n + k];
   bool ok = meet(&G->count, ++gen);
   for (int j = 0; ok; ++j) {
-    const double nn = total(norm, n_blk), hn = sqrt(nn);
+    if (wp == kT / 32 - 1) {
+      const double nn = total(norm, n_blk);
+      if (lane == 0) {
+        red[0][0] = nn;
+        red[0][1] = 1.0 / sqrt(nn);
+      }
+    }
     if (blk < 0) {
+      __syncthreads();
+      const double nn = red[0][0];
       if (j > 0) {
         rotate(G, j - 1, nn, tol, ws, ws + kLd, ws + 2 * kLd);
       } else if (t == 0) {
-        G->beta = hn;
-        G->e[0] = hn;
+        const double beta = sqrt(nn);
+        G->beta = beta;
+        G->e[0] = beta;
         G->m = 0;
         G->resid = 0.0;
-        G->done = G->stop = hn == 0.0 ? 1 : 0;
+        G->done = G->stop = beta == 0.0 ? 1 : 0;
       }
     } else if (j < kGmresMax) {
-      if (SMEM)
+      if (SMEM) {
+#pragma unroll 4
         for (int k = t; k < n; k += kT) wv[k] = __ldcg(w + k);
-      for (int k = t; k < nr; k += kT) Vb[(size_t)j * n + k] = ws[k] / hn;
-      __syncthreads();
+        __syncthreads();
+      }
       for (int k = wp; k < nr; k += kT / 32) {  // a warp per row
         const double* a = SMEM ? As + (size_t)k * n : A + (size_t)(r0 + k) * n;
         double v0 = 0.0, v1 = 0.0;
@@ -222,8 +249,14 @@ __global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __r
           v1 = fma(a[i + 32], SMEM ? wv[i + 32] : __ldcg(w + i + 32), v1);
         }
         if (i < n) v0 = fma(a[i], SMEM ? wv[i] : __ldcg(w + i), v0);
-        const double v = warp_sum(v0 + v1) / hn;
-        if (lane == 0) ws[k] = v;
+        const double v = warp_sum(v0 + v1);
+        if (lane == 0) wn[k] = v;
+      }
+      __syncthreads();
+      const double scale = red[0][1];
+      for (int k = t; k < nr; k += kT) {
+        Vb[(size_t)j * n + k] = ws[k] * scale;
+        ws[k] = wn[k] * scale;
       }
       __syncthreads();
       partials(n, nr, j + 1, Vb, ws, part0 + (size_t)blk * kLd);
@@ -267,7 +300,7 @@ __global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __r
 
 constexpr size_t kSmemMax = 220 * 1024;
 size_t smem_bytes(int n, int rows, bool in_smem) {
-  return ((in_smem ? (size_t)rows * n + n : 0) + std::max<size_t>(rows, 3 * kLd)) * sizeof(double);
+  return ((in_smem ? (size_t)rows * n + n : 0) + std::max<size_t>(2 * rows, 3 * kLd)) * sizeof(double);
 }
 
 }  // namespace
