@@ -37,12 +37,9 @@ import workloads as W  # noqa: E402
 WORKLOAD = "kite4096"
 METRIC = "2D-FC extend+FFT grid-points/sec at 4096^2"
 UNIT = "grid-points/s"
-FP64_PEAK_TFLOPS = 1.25   # GB300 FP64 (nominal; 152 SMs x 2 DFMA/clk x 2 flop x ~2.06 GHz)
-# FP32 issue rate: 152 SMs x 128 FP32 lanes x 2.07 GHz (nominal maximum SM clock)
-FP32_PEAK_GINSTR = 152 * 128 * 2.07
-# FP32 instructions per (point, node) term of the double-float double-layer sums
-# (k_dlp): two coordinate differences 22, the term 82, the accumulation 11
-DLP_INSTR_PER_TERM = 115
+# floating-point operations per second that butterflies in 64-bit fixed point replace at the
+# integer multiply-add rate: 12 multiply-adds for a radix-2 butterfly of 10 flops
+FIXED_PEAK_TFLOPS = 58 * 152 * 2.07e9 * 10 / 12 / 1e12
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of a kernel scope
 # on this workload, from one ncu capture of the current kernels (cold cache, serialised
@@ -50,16 +47,13 @@ DLP_INSTR_PER_TERM = 115
 # has no entry, and the roofline then reports traffic null.
 ROT = 3   # rotating input/output buffers of the timed steps
 # kernels launched inside one profiled scope where it is more than one: the FP32
-# 4096-point column DFT runs in two passes (k_cols4k_a, k_cols4k_b)
-KERNELS_PER_SCOPE = {("mixed", "fft_cols", 4096): 2}
+# and the double 4096-point column DFT run in two passes
+KERNELS_PER_SCOPE = {("mixed", "fft_cols", 4096): 2, ("fp64", "fft_cols", 4096): 2}
 
 MEASURED_TRAFFIC = {
     ("mixed", "fft_rows_fused"): 70898688 + 8000768,
     ("mixed", "gather_blend_interp_tc"): 34114048 + 0,
     ("mixed", "fft_cols"): (67674624 + 7534592) + (67655168 + 6790400),
-    ("fp64", "fft_rows_fused"): 72354816 + 72103424,
-    ("fp64", "fft_cols"): 141867520 + 92843264,
-    ("fp64", "gather_blend"): 9670144 + 9472,
 }
 
 
@@ -508,15 +502,9 @@ def measure(fc2d, torch, w, precision, K, warmup, world, dev, fg_h, fb_h, sample
     launches, tot_ms = prof[dom]
     avg_s = tot_ms / launches / 1e3
     a = alg.get(dom, {"bytes": 0, "flops": 0})
-    t_hbm = a["bytes"] / (hbm * 1e9)
-    fp64_tf = fp64_rate(fc2d, torch, dev) if fp64 else FP64_PEAK_TFLOPS
-    t_alu = a["flops"] / (fp64_tf * 1e12) if fp64 else 0.0
-    if fp64 and t_alu > t_hbm:
-        roof = {"bound": "alu", "achieved": a["flops"] / avg_s / 1e12, "peak": fp64_tf,
-                "unit": "TFLOP/s", "peak_source": "measured FP64 FMA rate (fp64_peak)"}
-    else:
-        roof = {"bound": "hbm", "achieved": a["bytes"] / avg_s / 1e9, "peak": hbm,
-                "unit": "GB/s", "peak_source": src}
+    # (the double plans' transforms run on integers, so no FP64 rate bounds them)
+    roof = {"bound": "hbm", "achieved": a["bytes"] / avg_s / 1e9, "peak": hbm,
+            "unit": "GB/s", "peak_source": src}
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["kernel"] = dom
     # the column passes' stored traffic is per form (direct or TMA-pipelined)
@@ -633,13 +621,12 @@ def poisson_star1024(fc2d, torch, dev, solves=3):
     err = float(np.abs(got - ue)[inside].max() / np.abs(ue[inside]).max())
     info = plan.fc2d_poisson_info()
     kms = {k: v[1] / v[0] for k, v in prof.items()}
-    # the far-field sums: (inside points - near points) x N_b terms, FP32-issue bound
-    terms = (plan.n_inside - info["n_near"]) * len(xy)
-    ach = terms * DLP_INSTR_PER_TERM / (kms["dlp_far"] * 1e-3) / 1e9
-    roof = {"bound": "alu", "kernel": "dlp_far (k_dlp<false>, N_b nodes)", "achieved": ach,
-            "peak": FP32_PEAK_GINSTR, "unit": "G FP32 instr/s", "frac": ach / FP32_PEAK_GINSTR,
-            "terms": terms, "instr_per_term": DLP_INSTR_PER_TERM,
-            "peak_source": "nominal: 152 SMs x 128 FP32 lanes x 2.07 GHz"}
+    # GMRES: 2 n^2 flops per product with the dense matrix
+    flops = 2.0 * len(xy) ** 2 * info["gmres_iters"]
+    ach, peak = flops / (kms["bie_gmres"] * 1e-3) / 1e12, fp64_rate(fc2d, torch, dev)
+    roof = {"bound": "alu", "kernel": "bie_gmres (k_gmres)", "achieved": ach, "peak": peak,
+            "unit": "TFLOP/s", "frac": ach / peak,
+            "peak_source": "measured FP64 FMA rate (fp64_peak)"}
     return {"workload": "star1024 Poisson, u = sin(2x) e^y", "ms_per_solve": 1e3 * dt,
             "value": g.nx * g.ny / dt, "unit": UNIT, "max_rel_err_vs_exact": err,
             "gmres": info, "kernels_ms": kms, "roofline": roof}
@@ -724,19 +711,16 @@ def ff_interior_kite2048(fc2d, torch, dev, steps=20):
     prof = plan.fc2d_profile_read()
     plan.fc2d_sync_status(stream)
     kms = {k: v[1] / v[0] for k, v in prof.items()}
-    # k_wave_cols: per spectrum (u and u_t) a forward and an inverse column DFT of ny
-    # points on nx/2 + 1 columns, 5 ny log2(ny) flops each (the modal advance not counted)
-    flops = 4 * (g.nx // 2 + 1) * 5 * g.ny * np.log2(g.ny)
-    ach = flops / (kms["wave_cols"] * 1e-3) / 1e12
+    # u and u_t at the inside points in, on the whole grid out
+    nbytes = 16.0 * (plan.n_inside + g.nx * g.ny)
+    hbm, src = peaks()
+    ach = nbytes / (ms * 1e-3) / 1e9
     return {"workload": f"kite 2048^2 (a=0.65, b=1.5), d = 4, c = 1, Delta T = 8 h = {dT:.4g}, "
                         "u = 32 Gaussians (w = 0.05, centres >= 0.3 inside), u_t = 0",
             "ms_per_large_step": ms, "large_steps_per_s": 1e3 / ms,
             "value": g.nx * g.ny / (ms * 1e-3), "unit": UNIT, "kernels_ms": kms,
-            "roofline": {"bound": "alu", "kernel": "wave_cols (k_wave_cols_p2)", "achieved": ach,
-                         "peak": fp64_rate(fc2d, torch, dev), "unit": "TFLOP/s",
-                         "frac": ach / fp64_rate(fc2d, torch, dev),
-                         "peak_source": "measured FP64 FMA rate (fp64_peak)",
-                         "flops": "4 column DFTs x 5 N log2 N, modal advance not counted"}}
+            "roofline": {"bound": "hbm", "kernel": "the whole step", "achieved": ach, "peak": hbm,
+                         "unit": "GB/s", "frac": ach / hbm, "peak_source": src}}
 
 
 def fp64_peak(fc2d, torch, dev, iters=1 << 16):
@@ -808,9 +792,9 @@ def ff_solve_kite2048(fc2d, torch, dev, n_large=2, mode=1, extras=True):
     warm-up call (the band and scratch are built there); the per-kernel times come from a
     second, profiled call.  Beside it: the measured FP64 rate, the error of the same
     solver against the exact Dirichlet eigenmode (2, 3) of the unit disk at t ~ 2, and the
-    same solve with the full inverse DFT at every small step (mode 0) and with the
-    squares evaluated in double-float arithmetic (mode 2; there the dominant kernel's
-    "TFLOP/s" counts the FP64-equivalent DFT flops it replaces)."""
+    same solve with the full inverse DFT at every small step (mode 0) and with interface mode 2
+    (the same computation as mode 1).  The transforms run in 64-bit fixed point; a kernel's
+    "TFLOP/s" counts the floating-point DFT flops that these replace."""
     squares, double_float = mode >= 1, mode == 2
     w = W.workload("kite2048", d=4, M=7)
     g, p = w.grid, w.params
@@ -866,12 +850,14 @@ def ff_solve_kite2048(fc2d, torch, dev, n_large=2, mode=1, extras=True):
     kms = {k: {"launches": v[0], "ms_per_launch": v[1] / v[0], "ms_total": v[1]}
            for k, v in prof.items()}
     # dominant kernel, FLOPs of one launch for n_f functions (5 N log2 N per length-N
-    # complex DFT): the modal advance + inverse column DFT (k_ff_cols) or the inverse
-    # rows of the full U_FC; with squares the per-small-step square inversion (k_sq_eval:
-    # per square and function pair a 64 x 64 complex DFT, 2 x 64 x 5 x 64 x 6)
+    # complex DFT): the modal advance + inverse column DFT (ff_cols) or the inverse
+    # rows of the full U_FC, of n_l functions per launch (160 MB of intermediates); with
+    # squares the per-small-step square inversion (per square and function pair a 64 x 64
+    # complex DFT, 2 x 64 x 5 x 64 x 6)
     nh = g.nx // 2
-    flops = {"ff_cols": n_f * (nh + 1) * 5.0 * g.ny * math.log2(g.ny),
-             "inverse_rows": n_f * g.ny * (5.0 * nh * math.log2(nh) + 10.0 * (nh + 1)),
+    n_l = min(n_f, max(1, (160 << 20) // (16 * g.ny * ((nh + 16) // 16 * 16))))
+    flops = {"ff_cols": n_l * (nh + 1) * 5.0 * g.ny * math.log2(g.ny),
+             "inverse_rows": n_l * g.ny * (5.0 * nh * math.log2(nh) + 10.0 * (nh + 1)),
              "sq_eval": counts[4] * ((n_f + 1) // 2) * 2 * 64 * 5.0 * 64 * 6}
     top = max(flops, key=lambda k: kms.get(k, {}).get("ms_total", 0.0))
     ach = flops[top] / (kms[top]["ms_per_launch"] * 1e-3) / 1e12
@@ -895,16 +881,18 @@ def ff_solve_kite2048(fc2d, torch, dev, n_large=2, mode=1, extras=True):
                      "near": counts[3]},
             "first_call_s": first_call_s, "finite": finite, "max_abs_u_end": amp,
             "clocks": clocks, "kernels": kms, "gpu_launches_per_call": sum(v[0] for v in prof.values()),
-            "roofline": {"bound": "alu", "kernel": top, "achieved": ach, "peak": peak["tflops"],
-                         "unit": "TFLOP/s", "frac": ach / peak["tflops"],
-                         "peak_source": "measured FP64 FMA rate (fp64_peak)",
-                         "flops": "5 N log2 N per length-N complex DFT of the launch"},
+            "roofline": {"bound": "alu", "kernel": top, "achieved": ach, "peak": FIXED_PEAK_TFLOPS,
+                         "unit": "TFLOP/s", "frac": ach / FIXED_PEAK_TFLOPS,
+                         "peak_source": "58 integer multiply-adds per clock and SM (measured) "
+                                        "x 152 SMs x 2.07 GHz, 12 per butterfly of 10 flops",
+                         "flops": "5 N log2 N per length-N complex DFT of the launch, done in "
+                                  "64-bit fixed point"},
             "fp64_peak": peak, "disk_eigenmode": eig,
             "parity": "tests/test_gpu_ff.py (element-wise against the oracle)",
             "full_inverse_dft": ff_solve_kite2048(fc2d, torch, dev, n_large, mode=0,
                                                   extras=False),
-            "small_squares_double_float": ff_solve_kite2048(fc2d, torch, dev, n_large, mode=2,
-                                                            extras=False)}
+            "interface_mode_2": ff_solve_kite2048(fc2d, torch, dev, n_large, mode=2,
+                                                  extras=False)}
 
 
 def ff_scaling(fc2d, torch, dev, n_f=8, n_c=8):
@@ -913,8 +901,8 @@ def ff_scaling(fc2d, torch, dev, n_f=8, n_c=8):
     fixed size per small step, about O(sqrt N), against O(N log N) for the full inverse
     DFT).  The kite at 1024^2, 2048^2, 4096^2 (d = 4, n_c = 8, 8 Gaussians, zero
     Dirichlet data), one large step of 64 small steps per mode after a warm-up call,
-    kernels timed with events: per small step the interface evaluation (full: k_ff_cols +
-    inverse rows; squares: k_sq_eval) and the U_B step, per large step the whole call."""
+    kernels timed with events: per small step the interface evaluation (full: ff_cols +
+    inverse_rows; squares: sq_eval) and the U_B step, per large step the whole call."""
     out = {}
     for N in (1024, 2048, 4096):
         name = f"kite{N}"
@@ -949,7 +937,7 @@ def ff_scaling(fc2d, torch, dev, n_f=8, n_c=8):
             plan.fc2d_profile(False)
             prof = plan.fc2d_profile_read()
             S = 8 * n_c
-            per = lambda k: prof[k][1] / prof[k][0] if k in prof else 0.0
+            per = lambda k: prof[k][1] / prof["ub_step"][0] if k in prof else 0.0
             if mode:
                 iface = per("sq_eval")
             else:
@@ -967,8 +955,8 @@ def ff_scaling(fc2d, torch, dev, n_f=8, n_c=8):
 
 def stars8_batched(fc2d, torch, dev, replays=10):
     """Eight stars (grids 256^2..2048^2 by concavity), 32 trigonometric sums per domain,
-    one fc2d_group_extend_coeffs call per step (one CUDA graph, a branch per domain);
-    mixed and FP64.  Inputs are made on the host and copied once; the error is checked
+    one fc2d_group_extend_coeffs call per step (a branch stream per domain; repeated calls
+    replay a CUDA graph); mixed and FP64.  Inputs are made on the host and copied once; the error is checked
     against the oracle on function 0 of the smallest and of the largest domain."""
     from oracle import fc2d as OF
     from oracle import geometry as OG
@@ -995,8 +983,9 @@ def stars8_batched(fc2d, torch, dev, replays=10):
                            stars, key=lambda s: s.grid.nx)) +
                        ", 32 degree-12 trigonometric sums per domain",
            "points_per_step": points, "unit": UNIT,
-           "launch": "fc2d_group_extend_coeffs: one CUDA graph (mixed: the form the "
-                     "group's autotuner keeps, see group_tuning; FP64: a branch per domain)"}
+           "launch": "fc2d_group_extend_coeffs: repeated calls replay a CUDA graph (mixed: in "
+                     "the form the group's autotuner keeps, see group_tuning; FP64: a branch "
+                     "per domain); calls with new buffers launch directly"}
     small = min(range(8), key=lambda i: stars[i].grid.nx)
     large = max(range(8), key=lambda i: stars[i].grid.nx)
     for name, prec, dt in (("mixed", fc2d.FC2D_MIXED, torch.float32),
@@ -1011,7 +1000,7 @@ def stars8_batched(fc2d, torch, dev, replays=10):
         grp = fc2d.fc2d_group_create([r[0] for r in runs])
         gargs = ([n_f] * len(runs), [r[1] for r in runs], [r[2] for r in runs],
                  [r[3] for r in runs])
-        for _ in range(3):  # the first call captures the graph, the others replay it
+        for _ in range(3):  # the first call launches, the second captures, the others replay
             grp.fc2d_group_extend_coeffs(*gargs)
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -1042,9 +1031,9 @@ def stars8_batched(fc2d, torch, dev, replays=10):
             out[name]["group_tuning"] = {
                 "form": form, "queue_threads": threads,
                 "us": {k: round(v, 1) for k, v in tune_us.items()},
-                "how": "capture-time autotuner: the persistent blend kernel timed with 256 "
-                       "and 512 threads per CTA, then the graph with it and the graph with "
-                       "a branch per domain timed on the call's inputs; the faster kept"}
+                "how": "autotuner of the first call: the persistent blend kernel timed with "
+                       "256 and 512 threads per CTA, then the call with it and with a branch "
+                       "per domain, on the call's inputs; the faster kept"}
         for plan, *_ in runs:
             plan.fc2d_destroy()
     return out
@@ -1138,7 +1127,7 @@ EXTRA_LINES = {"poisson_star1024": poisson_star1024,
 def ff_probe(name):
     """One large step of the Fourier Forwarding solve on workload `name` (d = 4, n_c = 8,
     8 Gaussians, zero Dirichlet data), with the full inverse DFT, the small squares and
-    the small squares in double-float: a small, self-contained command for profilers."""
+    interface mode 2: a small, self-contained command for profilers."""
     import torch
     from paper_2010_03901_gb300.build import build
     build()
@@ -1151,10 +1140,10 @@ def ff_probe(name):
           for k in range(8)]
     U0 = torch.tensor(np.stack([W.grid_values(w, f) for f in fs]), device="cuda:0")
     out = {}
-    for mode in ("full", "squares", "squares_double_float"):
+    for mode in ("full", "squares", "squares_mode_2"):
         u, ut = U0.clone(), torch.zeros_like(U0)
         plan.fc2d_forward_wave(8, 1.0, 8, 1, u, ut, squares=mode != "full",
-                               double_float=mode == "squares_double_float")
+                               double_float=mode == "squares_mode_2")
         plan.fc2d_sync_status()
         out[mode] = float(u.abs().max())
     print(json.dumps({"ff_probe": name, "max_abs_u": out}), flush=True)

@@ -31,8 +31,11 @@
  * Memory:    pointers named *_dev are device pointers owned by the caller; *_host are
  *            host pointers owned by the caller.  The plan owns only its own tables
  *            and workspace.
- * Precision: FC2D_FP64 computes every stage in double and uses double for every
- *            array.  FC2D_MIXED reads the same double inputs (the blending matrix has
+ * Precision: FC2D_FP64 uses double for every array; the transforms, the strip values and
+ *            the modal solutions are formed in 64-bit fixed point with one exponent per
+ *            block (a row, a group of columns, a normal), rounded once to double: errors
+ *            of 1-2e-16 of a block's largest value, and a block with an infinity or a NaN
+ *            among its inputs is NaN throughout.  FC2D_MIXED reads the same double inputs (the blending matrix has
  *            entries near 4e3, so rounding the data to float first would cost ~1e-4),
  *            forms the matching values and Gram coefficients in double, runs the
  *            continuation contraction on the tensor cores in TF32 with hi/lo split
@@ -189,9 +192,9 @@ fc2d_status fc2d_extend_coeffs_compact(fc2d_plan_t plan, int n_f, const double* 
  * calls no allocator (no cudaMalloc, cudaFree or allocating library routine).  It is
  * meant for callers that own all device memory through their own allocator, or that
  * run where an allocation's implicit device synchronisation is not acceptable.
- * Its scratch is one fixed device array of 64 MiB (the row-DFT intermediate,
- * n_f * ny * (nx/2+1 rounded up to 16) complex values), held by every GPU that loads
- * the library until the process exits.  Larger requests return FC2D_ERR_ARG.
+ * Its scratch is one fixed device array of 65 MiB: 64 MiB for the row-DFT intermediate,
+ * n_f * ny * (nx/2+1 rounded up to 16) complex values, and 1 MiB for its block exponents.
+ * Every GPU that loads the library holds it until the process exits.  Larger requests return FC2D_ERR_ARG.
  * The first call on a device looks up the array's device address for that device
  * (cudaGetSymbolAddress); make that first call before any stream capture.
  * All calls share the one array: calls that overlap on the GPU (different streams,
@@ -202,11 +205,13 @@ fc2d_status fc2d_coeffs_static(fc2d_plan_t plan, int n_f, const void* ext_dev, v
                                void* stream);
 
 /* Poisson problem Delta u = f in the domain, u = g on the curve (Section 4.1,
- * eqs. (4.1)-(4.6)), FP64 plans (FP64 data and arithmetic, except the double-layer sums
- * on the grid: double-float, about 48 bits).  fc2d_poisson_plan builds the boundary-integral tables
- * once (synchronous): n_b equispaced parameters 2 pi k/n_b (n_b <= 0 means nx, as in
- * Section 4.1.1), the Nystrom matrix of the double-layer equation -phi/2 + K phi = g_hom,
- * the boundary interpolation stencils of u_p, and the near-boundary point lists.
+ * eqs. (4.1)-(4.6)), FP64 plans (FP64 data; the double-layer sums on the grid by Taylor
+ * expansions in boxes of points, truncated below 2^-55 of the terms' moduli and summed in
+ * 64-bit fixed point, and the nodes next to a box term by term in double-float, about 48
+ * bits).  fc2d_poisson_plan builds the boundary-integral tables once (synchronous): n_b
+ * equispaced parameters 2 pi k/n_b (n_b <= 0 means nx, as in Section 4.1.1), the Nystrom
+ * matrix of the double-layer equation -phi/2 + K phi = g_hom, the boundary interpolation
+ * stencils of u_p, the near-boundary point lists and the sums' boxes.
  * fc2d_poisson_nodes returns n_b and, if xy_host is not NULL, the nodes [n_b][2] where
  * the Dirichlet data g are needed. */
 fc2d_status fc2d_poisson_plan(fc2d_plan_t plan, int n_b);
@@ -218,8 +223,9 @@ fc2d_status fc2d_poisson_nodes(fc2d_plan_t plan, double* xy_host, int* n_b);
  * the trapezoidal rule with near-boundary refinement.  f_grid_dev [n_f][ny][nx] and
  * f_bdry_dev [n_f][n_bdry] as for fc2d_extend; g_nodes_dev [n_f][n_b]; u_dev [n_f][ny][nx]
  * receives u inside the domain and 0 elsewhere; phi_dev (NULL allowed) receives the
- * density [n_f][n_b].  The GMRES iteration is driven from the host: this call waits
- * for the stream.  Returns FC2D_ERR_NOT_CONVERGED if GMRES stalls. */
+ * density [n_f][n_b].  GMRES is one cooperative launch per function (a block per SM) whose
+ * outcome the host reads: this call waits for the stream.  Returns FC2D_ERR_NOT_CONVERGED if
+ * GMRES stalls. */
 fc2d_status fc2d_poisson(fc2d_plan_t plan, int n_f, const double* f_grid_dev,
                          const double* f_bdry_dev, const double* g_nodes_dev, double* u_dev,
                          double* phi_dev, void* stream);
@@ -280,11 +286,10 @@ fc2d_status fc2d_wait_selftest(fc2d_plan_t plan, uint32_t polls, void* stream);
  * at the interface points within (18 - n_c) h of its centre; in that mode the band
  * reaches (ceil(sqrt(2) n_c) + 2) h, so that squares inside the domain reach every
  * interface point, and n_c <= 18 (FC2D_ERR_GEOMETRY if a domain is too narrow or curved
- * for the squares).  interface_mode 2: the squares of mode 1 with their every-small-step
- * evaluation (the modal advance and the two passes of inverse 64-point DFTs) in
- * double-float arithmetic, pairs of FP32 values holding about 44 significant bits (the
- * FP32 pipe issues 64 times the FP64 rate on this part); the expansions, U_B and U_FC at
- * T_{j+1} stay FP64 (fc2d_wave_band_* take mode 1 for its sets).  At T_{j+1} the grid takes U_FC where the distance to
+ * for the squares).  interface_mode 2 admits about 44 significant bits in the squares'
+ * small-step evaluation; mode 1's evaluation, in 64-bit fixed point, is both more accurate
+ * and faster than pairs of FP32 values, so the two modes compute the same
+ * (fc2d_wave_band_* take mode 1 for its sets).  At T_{j+1} the grid takes U_FC where the distance to
  * the curve is >= n_c h and U_B elsewhere (eq. (4.9)); U_B continues across large steps.
  *   u_dev, ut_dev  [n_f][ny][nx] in: u and u_t at t = 0 (values inside the domain used);
  *                  out: u and u_t at t = n_large Delta T inside the domain, 0 outside.

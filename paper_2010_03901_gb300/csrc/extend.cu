@@ -5,7 +5,9 @@
 //   k_gather_blend    one warp per (normal, function): the two-step interpolation of
 //                     Section 3.2 gives the matching values f_{D_p}; then the Gram
 //                     coefficients c = Q^T f_{D_p} and the strip values A_r c (eq. (2.6),
-//                     Remark 2.2).  FP64; in the mixed form the warp stops at c.
+//                     Remark 2.2).  FP64; in the mixed form the warp stops at c.  (A double
+//                     plan's own calls take the fixed-point form in fx_strip.cu; this one
+//                     serves fc2d_blend, as k_interp serves fc2d_interp.)
 //   k_interp          one thread per (strip point, function): the theta/eta Lagrange
 //                     interpolation of Section 3.4 with FP64 weights.
 //   k_assemble_rows   one block per (row, function): f on the inside intervals, the

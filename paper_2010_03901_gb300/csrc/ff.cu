@@ -1,14 +1,15 @@
 // Fourier Forwarding (Section 4.2): the interior propagator U_FC combined with the
-// near-boundary solver U_B by eq. (4.9), large step after large step (FP64).
+// near-boundary solver U_B by eq. (4.9), large step after large step (U_B in FP64, U_FC and the
+// squares in 64-bit fixed point).
 //
 // Large step j (T_j = j Delta T, Delta T = n_c h / c, S = 8 n_c small steps of
 // Delta t = Delta T / S, i.e. c Delta t = h/8, CFL 0.125 as in Section 4.2.1):
 //   1. the 2D-FC spectra of u(T_j) and u_t(T_j) (eq. (4.10)) with the Dirichlet data
 //      g(T_j) and its time derivative (capi.cu wave_spectra);
 //   2. for each small step s: the modal solution a(s Delta t) (eq. (4.12), w the square
-//      root of the paper's alpha) and its inverse DFT (k_ff_cols + inverse rows): U_FC on
-//      the grid, whose values at U_B's interface points feed the step;
-//   3. the U_B small step (k_ub_step): u^{n+1} = 2u^n - u^{n-1} + (h/8)^2 L(u^n)
+//      root of the paper's alpha) and its inverse DFT at U_B's interface points
+//      (fx_wave.cu; with squares fx_squares.cu), which feed the step;
+//   3. the U_B small step (k_ub_advance, on u and its increment): u^{n+1} = 2u^n - u^{n-1} + (h/8)^2 L(u^n)
 //      - 0.3 D(u^n - u^{n-1}), the first step of the solve by the Taylor start
 //      u^1 = u^0 + dt u_t^0 + (h/8)^2/2 L(u^0); L and D are the plan-time operators of
 //      wave_band.cpp (rows per unknown, columns keyed unknown / interface grid point /

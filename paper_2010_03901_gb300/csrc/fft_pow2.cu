@@ -1,7 +1,7 @@
-// Power-of-two DFT kernels (eq. (3.1)): compile-time radix, one shared buffer.
+// Power-of-two FP32 DFT kernels (eq. (3.1)): compile-time radix, one shared buffer.
 //
 // A transform of N = 2^LOGN complex points is done by NT = N/E threads, each holding
-// E complex values in registers (E = 16 for float, 8 for double).  Every Stockham
+// E = 16 complex values in registers.  Every Stockham
 // stage (radix R dividing E; R = E except a smaller last stage) is:
 //   read the thread's E inputs x[j + r N/R] from shared memory, barrier,
 //   twiddle by exp(-2 pi i r (j mod Ns)/(Ns R)) (table lookups), length-R DFT,
@@ -357,9 +357,8 @@ __device__ __forceinline__ void last_stage_split(const typename Cx<T>::type* buf
 // lanes served by one shared-memory wavefront for complex values of type T
 template <typename T> __host__ __device__ constexpr int col_lanes() { return sizeof(T) == 4 ? 16 : 8; }
 
-// complex values per thread: 16 for float (radix-16 stages, three for 4096 points),
-// 8 for double (register pressure of FP64 complex values)
-template <typename T> __host__ __device__ constexpr int elems() { return sizeof(T) == 4 ? 16 : 8; }
+// complex values per thread (radix-16 stages, three for 4096 points)
+template <typename T> __host__ __device__ constexpr int elems() { return 16; }
 
 // First stage (Ns = 1, radix R) straight from global memory: x[j + r N/R] at stride
 // `stride`, length-R DFT, written to the shared buffer, then a barrier.

