@@ -186,9 +186,51 @@ __device__ void triangle(GmresDev* G, int m, double* yi) {
   }
 }
 
+// out = the block's rows of A times w, both from L2 or HBM: four rows per warp share the
+// vector and keep 32 loads per lane in flight (64 KB per SM, about the latency times the
+// bandwidth)
+__device__ __forceinline__ void rows_times(int n, int nr, const double* __restrict__ A,
+                                           const double* w, double* out) {
+  constexpr int R = 4, U = 8;
+  const int lane = threadIdx.x & 31;
+  for (int k0 = (threadIdx.x >> 5) * R; k0 < nr; k0 += kT / 32 * R) {
+    const double* a[R];
+    double v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      a[r] = A + (size_t)min(k0 + r, nr - 1) * n;
+      v[r] = 0.0;
+    }
+    int i = lane;
+    for (; i + 32 * (U - 1) < n; i += 32 * U) {
+      double x[U], y[R][U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        x[u] = __ldcg(w + i + 32 * u);
+#pragma unroll
+        for (int r = 0; r < R; ++r) y[r][u] = __ldcg(a[r] + i + 32 * u);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = fma(y[r][u], x[u], v[r]);
+    }
+    for (; i < n; i += 32) {
+      const double x = __ldcg(w + i);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = fma(__ldcg(a[r] + i), x, v[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      v[r] = warp_sum(v[r]);
+      if (lane == 0 && k0 + r < nr) out[k0 + r] = v[r];
+    }
+  }
+}
+
 // SMEM: the block's rows of A and the vector in shared memory
 template <bool SMEM>
-__global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __restrict__ A,
+__global__ void __launch_bounds__(kT, 1) k_gmres(int n, int rows, const double* __restrict__ A,
                                               const double* __restrict__ g, double* V, double* w,
                                               double* part0, double* part1, double* norm,
                                               GmresDev* G, double* x, double tol) {
@@ -240,18 +282,22 @@ __global__ void __launch_bounds__(kT) k_gmres(int n, int rows, const double* __r
         for (int k = t; k < n; k += kT) wv[k] = __ldcg(w + k);
         __syncthreads();
       }
-      for (int k = wp; k < nr; k += kT / 32) {  // a warp per row
-        const double* a = SMEM ? As + (size_t)k * n : A + (size_t)(r0 + k) * n;
-        double v0 = 0.0, v1 = 0.0;
-        int i = lane;
+      if (SMEM) {
+        for (int k = wp; k < nr; k += kT / 32) {  // a warp per row
+          const double* a = As + (size_t)k * n;
+          double v0 = 0.0, v1 = 0.0;
+          int i = lane;
 #pragma unroll 4
-        for (; i + 32 < n; i += 64) {
-          v0 = fma(a[i], SMEM ? wv[i] : __ldcg(w + i), v0);
-          v1 = fma(a[i + 32], SMEM ? wv[i + 32] : __ldcg(w + i + 32), v1);
+          for (; i + 32 < n; i += 64) {
+            v0 = fma(a[i], wv[i], v0);
+            v1 = fma(a[i + 32], wv[i + 32], v1);
+          }
+          if (i < n) v0 = fma(a[i], wv[i], v0);
+          const double v = warp_sum(v0 + v1);
+          if (lane == 0) wn[k] = v;
         }
-        if (i < n) v0 = fma(a[i], SMEM ? wv[i] : __ldcg(w + i), v0);
-        const double v = warp_sum(v0 + v1);
-        if (lane == 0) wn[k] = v;
+      } else {
+        rows_times(n, nr, A + (size_t)r0 * n, w, wn);
       }
       __syncthreads();
       const double scale = red[0][1];
