@@ -12,8 +12,8 @@
 // is 12 integer multiply-adds (58 per clock and SM) and about 20 other instructions, where
 // its four FP64 multiply-adds cost 256 issue slots.  The expansions are bound by the
 // multiply-adds at 38% issue (168 registers for the 32 accumulators: 12 warps per SM), the
-// evaluation at 44 to 51%.  Error against long double sums: 3e-15 to 8e-15 of the sum of the
-// terms' moduli, the near terms' double-float rounding.
+// evaluation at 44 to 51%.  Error against long double sums: 6e-16 to 1.2e-15 of the sum of the
+// terms' moduli.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -232,7 +232,9 @@ __global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
     cell(X.x, shift, px, pfh, pfl);
     cell(X.y, shift, py, qfh, qfl);
   }
-  dfl acc = {0.f, 0.f};
+  // three floats: a pair would round at 2^-48 of the sum so far with every term, and the close
+  // points' Lagrange weights multiply that by several hundred
+  float sh = 0.f, sl = 0.f, sr = 0.f;
   for (int d = 0; d < lf.nd; ++d) {
     const DlpSpan sp = near[lf.d0 + d];
     for (int k0 = sp.k0; k0 < sp.k0 + sp.n; k0 += T) {
@@ -255,13 +257,15 @@ __global__ void __launch_bounds__(kDlpPoints) k_dlp_eval(
           dy = df_add(dy, {qfh, qfl});
         }
         const dfl term = dl_term(dx, dy, c.x, c.y, c.z, c.w);
-        const dfl s = two_sum(acc.hi, term.hi);
-        acc = fast_two_sum(s.hi, s.lo + (acc.lo + term.lo));
+        const dfl s = two_sum(sh, term.hi), a1 = two_sum(sl, s.lo), a2 = two_sum(a1.hi, term.lo);
+        sh = s.hi;
+        sl = a2.hi;
+        sr += a1.lo + a2.lo;
       }
     }
   }
   if (t >= it.n) return;
-  v += (double)acc.hi + (double)acc.lo;
+  v += (double)sh + ((double)sl + (double)sr);
   if (GRID) out[l] += v * inv_h;
   else out[l] = v * inv_h;
 }
