@@ -78,6 +78,8 @@ static void drop_graph(fc2d_group_s* g) {
   if (g->graph) cudaGraphDestroy(g->graph);
   g->exec = nullptr;
   g->graph = nullptr;
+  g->graph_nf.clear();
+  g->graph_ptr.clear();
 }
 
 static void group_free(fc2d_group_s* g) {
@@ -244,6 +246,9 @@ static fc2d_status tune(fc2d_group_s* g, const Call& c) {
   // write the plans' workspaces and outputs: let earlier work finish
   fc2d_status st = cuda_check(cudaDeviceSynchronize(), "fc2d_group: synchronise");
   if (st) return st;
+  // the captured graph holds the addresses of the items and records, and the number of items,
+  // that are replaced here
+  drop_graph(g);
   g->n_items = (int)items.size();
   g->nt = 0;
   g->persistent = 0;

@@ -47,3 +47,55 @@ def test_calls_in_any_order(form, precision):
             p.fc2d_extend_coeffs(n_f[i], f[i], b[i] if bdry else None, ref)
             assert torch.equal(ref, outs[k][i]), (k, bdry, i)
     grp.fc2d_group_destroy()
+
+
+def mixed_plans(fc2d):
+    plans = []
+    for name in ["disk64", "star200", "kite160x144"]:
+        w = W.workload(name)
+        g, p = w.grid, w.params
+        plans.append(fc2d.fc2d_plan(w.boundary.arrays(), (g.a0, g.b0, g.h, g.nx, g.ny),
+                                    dict(B=p.B, k1=p.k1), precision=fc2d.FC2D_MIXED))
+    return plans
+
+
+def call_set(torch, plans, n_f, gen):
+    rnd = lambda *s: torch.randn(s, dtype=torch.float64, device="cuda", generator=gen)  # noqa: E731
+    f = [rnd(n, p.ny, p.nx) for n, p in zip(n_f, plans)]
+    b = [rnd(n, p.n_bdry) for n, p in zip(n_f, plans)]
+    out = [torch.zeros((n, p.ny, p.nx // 2 + 1, 2), dtype=torch.float32, device="cuda")
+           for n, p in zip(n_f, plans)]
+    return list(n_f), f, b, out
+
+
+@pytest.mark.parametrize("form", ["branches", "persistent"])
+@pytest.mark.parametrize("counts,grown", [(([3, 2, 3], [1, 1, 1]), False),
+                                          (([1, 1, 1], [3, 2, 3]), True),
+                                          (([2, 1, 3], [3, 1, 2]), True)])
+def test_return_to_captured_arguments(form, counts, grown):
+    """A call is repeated until it runs as a graph, calls with other function counts (fewer;
+    more, with the workspaces already large enough; exchanged) replace the work items, then
+    the first call's arguments come back: equal to separate calls bit for bit every time."""
+    torch = pytest.importorskip("torch")
+    from paper_2010_03901_gb300 import fc2d
+    plans = mixed_plans(fc2d)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    sets = [call_set(torch, plans, n_f, gen) for n_f in counts]
+    refs = []
+    for n_f, f, b, out in sets if grown else sets[:1]:
+        for i, p in enumerate(plans):  # the workspaces take their final size
+            p.fc2d_extend_coeffs(n_f[i], f[i], b[i], out[i])
+    for n_f, f, b, out in sets:
+        refs.append([torch.zeros_like(o) for o in out])
+        for i, p in enumerate(plans):
+            p.fc2d_extend_coeffs(n_f[i], f[i], b[i], refs[-1][i])
+    grp = fc2d.fc2d_group_create(plans)
+    grp.fc2d_group_tuning_set(form, 256)
+    for k in (0, 0, 0, 1, 0, 0, 0, 1, 1, 1, 0, 1):
+        n_f, f, b, out = sets[k]
+        for o in out:
+            o.fill_(7.0)
+        grp.fc2d_group_extend_coeffs(n_f, f, b, out)
+        for i in range(len(plans)):
+            assert torch.equal(refs[k][i], out[i]), (k, i)
+    grp.fc2d_group_destroy()
