@@ -338,15 +338,15 @@ extern "C" fc2d_status fc2d_group_extend_coeffs(fc2d_group_t g, const int* n_f,
       cudaGetLastError();
       again = false;  // the caller is capturing: its graph takes the kernels themselves
     }
-    if (!again) {
-      g->key_nf = knf;
-      g->key_ptr = kptr;
-      return launch(g, c, g->persistent != 0, (cudaStream_t)stream);
-    }
+    g->key_nf = knf;
+    g->key_ptr = kptr;
+    if (!again) return launch(g, c, g->persistent != 0, (cudaStream_t)stream);
     if ((st = capture(g, c))) return st;
     g->graph_nf = knf;
     g->graph_ptr = kptr;
   }
+  g->key_nf = knf;  // a replayed call is the next one's last call too
+  g->key_ptr = kptr;
   if (cudaGraphLaunch(g->exec, (cudaStream_t)stream) != cudaSuccess)
     return set_error(FC2D_ERR_CUDA, "fc2d_group: graph launch failed");
   return FC2D_OK;

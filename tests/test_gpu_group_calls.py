@@ -99,3 +99,43 @@ def test_return_to_captured_arguments(form, counts, grown):
         for i in range(len(plans)):
             assert torch.equal(refs[k][i], out[i]), (k, i)
     grp.fc2d_group_destroy()
+
+
+@pytest.mark.parametrize("form", ["branches", "persistent"])
+def test_alternating_calls_do_not_wait_for_the_device(form):
+    """Only a call with the arguments of the call just before it is captured, which waits for
+    the device: after A has been captured, calls that alternate between two sets of buffers
+    return while an unrelated stream is still busy."""
+    torch = pytest.importorskip("torch")
+    from paper_2010_03901_gb300 import fc2d
+    plans = mixed_plans(fc2d)
+    gen = torch.Generator(device="cuda").manual_seed(10)
+    sets = [call_set(torch, plans, [1, 2, 1], gen) for _ in range(2)]
+    refs = []
+    for n_f, f, b, out in sets:
+        refs.append([torch.zeros_like(o) for o in out])
+        for i, p in enumerate(plans):
+            p.fc2d_extend_coeffs(n_f[i], f[i], b[i], refs[-1][i])
+    grp = fc2d.fc2d_group_create(plans)
+    grp.fc2d_group_tuning_set(form, 256)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    call = lambda k: grp.fc2d_group_extend_coeffs(*sets[k], stream=mine.cuda_stream)  # noqa: E731
+    call(0)
+    call(0)  # captured
+    waited = []
+    for k in (1, 0, 1, 0, 1, 0):
+        torch.cuda.synchronize()
+        for o in sets[k][3]:
+            o.fill_(7.0)
+        torch.cuda.synchronize()
+        busy = torch.cuda.Event()
+        with torch.cuda.stream(other):
+            torch.cuda._sleep(200_000_000)  # about 0.1 s
+            busy.record()
+        call(k)
+        waited.append(busy.query())
+        torch.cuda.synchronize()
+        for i in range(len(plans)):
+            assert torch.equal(refs[k][i], sets[k][3][i]), (k, i)
+    assert not any(waited), waited
+    grp.fc2d_group_destroy()
