@@ -371,7 +371,10 @@ fc2d_status fc2d_probe_fp64(double* out_dev, int blocks, int64_t iters, double* 
  * CTA shape, 256 threads two per SM or 512 one per SM, timed first) and keeps the faster.
  * A call that repeats the previous call's arguments is captured as a CUDA graph, which is
  * replayed while n_f, every pointer and every plan's workspace stay the same; any other
- * call launches its kernels directly.  A plan may appear once in a group (FC2D_ERR_ARG
+ * call launches its kernels directly.  Inside a capture of the caller's own, the function
+ * counts must be those of the last call (FC2D_ERR_CUDA otherwise); the caller's graph stays
+ * valid, whatever later calls pass, until the group is destroyed or a call on a member plan
+ * needs a larger workspace.  A plan may appear once in a group (FC2D_ERR_ARG
  * otherwise).  Calls on one group must not overlap in time on different streams (the
  * plans' workspaces are shared).  The result equals the separate calls bit for bit.
  * fc2d_group_tuning: choice[0] the kept form (0 branches, 1 persistent), choice[1] the

@@ -63,6 +63,10 @@ struct fc2d_group_s {
   size_t items_cap = 0;
   int* counter = nullptr;
   int n_items = 0;
+  // a caller's own capture holds the records' and items' addresses: the next set of function
+  // counts takes other buffers, these stay until the group goes
+  bool lent = false;
+  std::vector<void*> retired;
   int nt = 0;                             // its threads per CTA (tuned)
   int persistent = 0;                     // the kept form (tuned)
   int forced_form = -1, forced_nt = 0;    // fc2d_group_tuning_set (-1: tune)
@@ -91,6 +95,7 @@ static void group_free(fc2d_group_s* g) {
   if (g->fork_dft) cudaEventDestroy(g->fork_dft);
   if (g->work) cudaFree(g->work);
   if (g->items) cudaFree(g->items);
+  for (void* q : g->retired) cudaFree(q);
   if (g->counter) cudaFree(g->counter);
   for (cudaStream_t s : g->branch)
     if (s) cudaStreamDestroy(s);
@@ -249,6 +254,14 @@ static fc2d_status tune(fc2d_group_s* g, const Call& c) {
   // the captured graph holds the addresses of the items and records, and the number of items,
   // that are replaced here
   drop_graph(g);
+  if (g->lent) {
+    for (void* q : {g->work, (void*)g->items})
+      if (q) g->retired.push_back(q);
+    g->work = nullptr;
+    g->items = nullptr;
+    g->work_cap = g->items_cap = 0;
+    g->lent = false;
+  }
   g->n_items = (int)items.size();
   g->nt = 0;
   g->persistent = 0;
@@ -311,6 +324,16 @@ extern "C" fc2d_status fc2d_group_extend_coeffs(fc2d_group_t g, const int* n_f,
   const int n = (int)g->plans.size();
   std::vector<int> knf(n_f, n_f + n);
   std::vector<const void*> kptr;
+  // inside a caller's capture its graph takes the kernels themselves
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing((cudaStream_t)stream, &cs) != cudaSuccess ||
+                         cs != cudaStreamCaptureStatusNone;
+  if (capturing) {
+    cudaGetLastError();
+    if (knf != g->tuned_nf)
+      return set_error(FC2D_ERR_CUDA, "fc2d_group_extend_coeffs: the first call for these function "
+                                      "counts cannot be made inside a stream capture");
+  }
   for (int i = 0; i < n; ++i) {
     if (n_f[i] < 1 || !f_grid_dev[i] || !fhat_dev[i])
       return set_error(FC2D_ERR_ARG, "fc2d_group_extend_coeffs: bad entry");
@@ -326,21 +349,18 @@ extern "C" fc2d_status fc2d_group_extend_coeffs(fc2d_group_t g, const int* n_f,
     kptr.push_back(g->plans[i]->ws.base);
     kptr.push_back(reinterpret_cast<const void*>(g->plans[i]->ws.bytes));
   }
-  if (!g->exec || knf != g->graph_nf || kptr != g->graph_ptr) {
+  if (capturing || !g->exec || knf != g->graph_nf || kptr != g->graph_ptr) {
     Call c{n_f, f_grid_dev, f_bdry_dev, fhat_dev};
     fc2d_status st = describe(g, c);
     if (!st && knf != g->tuned_nf) st = tune(g, c);
     if (st) return st;
-    bool again = knf == g->key_nf && kptr == g->key_ptr;
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (again && (cudaStreamIsCapturing((cudaStream_t)stream, &capturing) != cudaSuccess ||
-                  capturing != cudaStreamCaptureStatusNone)) {
-      cudaGetLastError();
-      again = false;  // the caller is capturing: its graph takes the kernels themselves
+    const bool again = knf == g->key_nf && kptr == g->key_ptr;
+    if (capturing) g->lent = true;
+    if (capturing || !again) {
+      g->key_nf = knf;
+      g->key_ptr = kptr;
+      return launch(g, c, g->persistent != 0, (cudaStream_t)stream);
     }
-    g->key_nf = knf;
-    g->key_ptr = kptr;
-    if (!again) return launch(g, c, g->persistent != 0, (cudaStream_t)stream);
     if ((st = capture(g, c))) return st;
     g->graph_nf = knf;
     g->graph_ptr = kptr;

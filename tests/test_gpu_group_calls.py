@@ -139,3 +139,50 @@ def test_alternating_calls_do_not_wait_for_the_device(form):
             assert torch.equal(refs[k][i], sets[k][3][i]), (k, i)
     assert not any(waited), waited
     grp.fc2d_group_destroy()
+
+
+@pytest.mark.parametrize("form", ["branches", "persistent"])
+@pytest.mark.parametrize("seen", [0, 1, 3])
+def test_inside_a_capture_of_the_caller(form, seen):
+    """A caller's graph that holds a group call (whose arguments were never passed before, once,
+    or run as the group's own graph) keeps its work items when calls with fewer and with more
+    functions follow; function counts that were not called before are refused, and the capture
+    goes on."""
+    torch = pytest.importorskip("torch")
+    from paper_2010_03901_gb300 import fc2d
+    plans = mixed_plans(fc2d)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    sets = [call_set(torch, plans, n_f, gen) for n_f in ([2, 1, 2], [2, 1, 2], [1, 1, 1], [3, 2, 3])]
+    refs = []
+    for n_f, f, b, out in reversed(sets):  # the largest counts first: no workspace grows later
+        refs.insert(0, [torch.zeros_like(o) for o in out])
+        for i, p in enumerate(plans):
+            p.fc2d_extend_coeffs(n_f[i], f[i], b[i], refs[0][i])
+    grp = fc2d.fc2d_group_create(plans)
+    grp.fc2d_group_tuning_set(form, 256)
+
+    def check(k, run):
+        for o in sets[k][3]:
+            o.fill_(7.0)
+        run()
+        torch.cuda.synchronize()
+        for i in range(len(plans)):
+            assert torch.equal(refs[k][i], sets[k][3][i]), (k, i)
+
+    call = lambda k: grp.fc2d_group_extend_coeffs(*sets[k])  # noqa: E731
+    call(1)
+    for _ in range(seen):
+        call(0)
+    torch.cuda.synchronize()
+    graph, mark = torch.cuda.CUDAGraph(), torch.zeros(1, device="cuda")
+    with torch.cuda.graph(graph):
+        call(0)
+        with pytest.raises(fc2d.Fc2dError, match="stream capture"):
+            call(2)
+        mark.add_(1.0)
+    check(0, graph.replay)
+    for k in (2, 2, 2, 3, 0, 0, 0, 1):
+        check(k, lambda: call(k))  # noqa: B023
+        check(0, graph.replay)
+    assert float(mark) == 9.0
+    grp.fc2d_group_destroy()
