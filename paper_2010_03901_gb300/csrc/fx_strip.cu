@@ -36,9 +36,9 @@ struct Sum {
   }
 };
 
-// shift left by n (n < 0: right, rounded)
+// shift left by n (n < 0: right, rounded; -63 <= n)
 __device__ __forceinline__ i64 shift(i64 v, int n) {
-  return n >= 0 ? v << n : (v + ((1ll << -n) >> 1)) >> -n;
+  return n >= 0 ? v << n : (v + (i64)((1ull << -n) >> 1)) >> -n;
 }
 
 // As k_gather_blend (extend.cu), a group of GS lanes per normal, up to the Gram coefficients;

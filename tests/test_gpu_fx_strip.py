@@ -71,3 +71,21 @@ def test_scaling_and_non_finite_values():
     theta = plan.fc2d_strip_points()[1]
     touched = np.abs((theta / (2 * np.pi) * 250 - 3 + 125) % 250 - 125) < 3  # within the 8 normals
     assert bool(torch.isnan(got[0][torch.tensor(touched, device="cuda")]).all())
+
+
+@pytest.mark.parametrize("M", [7, 8, 13])
+@pytest.mark.parametrize("tiny", [0.0, 2.0 ** -300])
+def test_normals_that_vanish_beside_others(M, tiny):
+    """Ten boundary data, 25 normals apart, all other data zero (or far below it): the normals without data add
+    nothing, so strip values of the opposite datum are the opposite ones.  Every rounding is to
+    nearest, symmetric but for ties; a unit lost per vanishing normal shows where the weight of
+    the datum's normals is below 2^-8 and the value keeps its last bits."""
+    import torch
+    plan = make(5, M, 6, 27)
+    f, b = (tiny * x for x in fields(plan, 1))
+    b[0, ::25] = 1.2345678901234567
+    got, opp = extend(plan, f, b)[0], extend(plan, -f, -b)[0]
+    top = float(got.abs().max())
+    small = (got != 0) & (got.abs() < 2.0 ** -9 * top) & (got.abs() > 2.0 ** -60 * top)
+    assert int(small.sum()) > 20
+    assert float((got + opp)[small].ne(0).double().mean()) < 0.05
