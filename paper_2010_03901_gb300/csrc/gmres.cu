@@ -361,16 +361,23 @@ int gmres_rows(int n, int n_sm) {
 fc2d_status gmres_solve(Gmres& q, const double* g, double* x, double tol, int* iters,
                         double* resid, cudaStream_t s) {
   static_assert(kT >= kGmresMax, "triangle: a thread per column");
-  const bool in_smem = smem_bytes(q.n, q.rows, true) <= kSmemMax;
-  const size_t sm = smem_bytes(q.n, q.rows, in_smem);
-  auto kernel = in_smem ? k_gmres<true> : k_gmres<false>;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  cudaMemsetAsync(&q.dev->count, 0, sizeof(unsigned), s);
   int n = q.n, rows = q.rows;
   void* args[] = {&n, &rows, &q.A, &g, &q.V, &q.w, &q.part[0], &q.part[1], &q.norm, &q.dev, &x, &tol};
-  if (cudaLaunchCooperativeKernel((const void*)kernel, dim3(q.n_blk + 1), dim3(kT), args, sm, s) !=
-      cudaSuccess)
-    return cuda_check(cudaGetLastError(), "GMRES");
+  for (int n_blk = q.n_blk;; n_blk = (n_blk + 1) / 2) {
+    rows = (n + n_blk - 1) / n_blk;
+    const bool in_smem = smem_bytes(n, rows, true) <= kSmemMax;
+    const size_t sm = smem_bytes(n, rows, in_smem);
+    auto kernel = in_smem ? k_gmres<true> : k_gmres<false>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaMemsetAsync(&q.dev->count, 0, sizeof(unsigned), s);
+    const unsigned blocks = (unsigned)((n + rows - 1) / rows) + 1;
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel((const void*)kernel, dim3(blocks), dim3(kT), args, sm, s);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    // a stream whose context has a part of the SMs only: fewer blocks, of more rows each
+    if (e != cudaErrorCooperativeLaunchTooLarge || n_blk == 1) return cuda_check(e, "GMRES");
+  }
   GmresDev::State st;
   cudaMemcpyAsync(&st, static_cast<GmresDev::State*>(q.dev), sizeof(st), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "GMRES");
