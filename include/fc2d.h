@@ -262,12 +262,14 @@ fc2d_status fc2d_profile_read(fc2d_plan_t plan, int max_kernels, char* names_hos
  * a new one). */
 fc2d_status fc2d_sync_status(fc2d_plan_t plan, void* stream);
 
-/* Failure detection check (no operation of the paper).  Runs the bounded device wait
- * of the tensor-core blend kernels on an mbarrier that nothing arrives on: after
- * 2 x polls polls the kernel latches FC2D_ERR_TIMEOUT in the plan's status word and
- * returns, so that fc2d_sync_status then returns FC2D_ERR_TIMEOUT; nothing hangs or
- * traps and the plan stays usable.  polls in 1 .. 2^22 (FC2D_ERR_ARG otherwise); one
- * block of 32 threads on `stream`, asynchronous. */
+/* Failure detection check (no operation of the paper).  Runs the bounded device wait of
+ * the plan's kernels where nothing ends it: on a mixed plan the tensor-core blend kernels'
+ * wait on an mbarrier that nothing arrives on (2 x polls polls), on an FP64 plan the
+ * meeting of the GMRES launch's blocks with a block missing (polls polls).  Then the
+ * kernel latches FC2D_ERR_TIMEOUT in the plan's status word and returns, so that
+ * fc2d_sync_status returns FC2D_ERR_TIMEOUT; nothing hangs or traps and the plan stays
+ * usable.  polls in 1 .. 2^22 (FC2D_ERR_ARG otherwise); one block of 32 threads on
+ * `stream`, asynchronous. */
 fc2d_status fc2d_wait_selftest(fc2d_plan_t plan, uint32_t polls, void* stream);
 
 /* Fourier Forwarding solve (Section 4.2, eq. (4.9)), FP64 plans: the wave equation

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "fc2d_kernels.cuh"
+#include "gmres.h"
 #include "plan_internal.h"
 
 using namespace fc2d;
@@ -530,7 +531,8 @@ extern "C" fc2d_status fc2d_wait_selftest(fc2d_plan_t p, uint32_t polls, void* s
   if (!p) return set_error(FC2D_ERR_ARG, "null plan");
   if (polls < 1 || polls > (1u << 22)) return set_error(FC2D_ERR_ARG, "polls must be in 1 .. 2^22");
   cudaSetDevice(p->device);
-  return fc2d::launch_wait_probe(p->dev.status, polls, (cudaStream_t)stream);
+  auto probe = p->prm.precision == FC2D_FP64 ? fc2d::launch_meet_probe : fc2d::launch_wait_probe;
+  return probe(p->dev.status, polls, (cudaStream_t)stream);
 }
 
 // ------------------------------------------------------------------------- //

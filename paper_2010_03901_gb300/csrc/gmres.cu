@@ -107,15 +107,16 @@ __device__ void rotate(GmresDev* G, int j, double nn, double tol, double* col, d
 
 // Waits until all blocks of the launch have come here `gen` times; false when a block does
 // not come within a second or so (every block then leaves).
-__device__ bool meet(unsigned* count, unsigned gen) {
+constexpr unsigned kMeetPolls = 1u << 21;
+__device__ bool meet(unsigned* count, unsigned gen, unsigned limit = kMeetPolls) {
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(count, 1u);
     const unsigned all = gen * gridDim.x;
-    int polls = 0;
-    while (*(volatile unsigned*)count < all && ok) ok = ++polls < (1 << 21);
+    unsigned polls = 0;
+    while (*(volatile unsigned*)count < all && ok) ok = ++polls < limit;
     __threadfence();
   }
   return !__syncthreads_or(!ok);
@@ -345,12 +346,25 @@ __global__ void __launch_bounds__(kT, 1) k_gmres(int n, int rows, const double* 
   }
 }
 
+// A meeting whose other block never comes: meet(), as k_gmres calls it, with a given number
+// of polls, so that the way out can be taken on purpose.  One warp.
+__global__ void __launch_bounds__(32) k_meet_probe(int* status, unsigned limit) {
+  __shared__ unsigned count;
+  if (threadIdx.x == 0) count = 0;
+  if (!meet(&count, 2, limit) && threadIdx.x == 0) atomicExch(status, (int)FC2D_ERR_TIMEOUT);
+}
+
 constexpr size_t kSmemMax = 220 * 1024;
 size_t smem_bytes(int n, int rows, bool in_smem) {
   return ((in_smem ? (size_t)rows * n + n : 0) + std::max<size_t>(2 * rows, 3 * kLd)) * sizeof(double);
 }
 
 }  // namespace
+
+fc2d_status launch_meet_probe(int* status, unsigned limit, cudaStream_t s) {
+  k_meet_probe<<<1, 32, 0, s>>>(status, limit);
+  return cuda_check(cudaGetLastError(), "meeting probe launch");
+}
 
 // One block per SM, one of them for the rotations
 int gmres_rows(int n, int n_sm) {

@@ -37,5 +37,7 @@ int gmres_rows(int n, int n_sm);
 // A x = g to |residual| <= tol |g|; iterations and the relative residual estimate
 fc2d_status gmres_solve(Gmres& q, const double* g, double* x, double tol, int* iters,
                         double* resid, cudaStream_t s);
+// the blocks' bounded meeting with a block missing: FC2D_ERR_TIMEOUT in *status after `limit` polls
+fc2d_status launch_meet_probe(int* status, unsigned limit, cudaStream_t s);
 
 }  // namespace fc2d

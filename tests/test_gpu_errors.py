@@ -107,3 +107,26 @@ def test_a_stalled_device_wait_times_out_and_the_plan_stays_usable(env):
         with pytest.raises(fc2d.Fc2dError, match="polls must be") as e:
             mixed.fc2d_wait_selftest(polls)
         assert _status(e) == 1
+
+
+@pytest.mark.parametrize("polls", [1, 1 << 12])
+def test_a_missed_meeting_of_the_gmres_blocks_times_out(env, polls):
+    """The wait of the cooperative GMRES launch (FP64 plans), run with a block that never comes,
+    gives up after its polls and latches FC2D_ERR_TIMEOUT (4); the plan then solves the same
+    Poisson problem, bit for bit, as before."""
+    torch, fc2d, w, plan, _, fg, fb = env
+    plan.fc2d_poisson_plan(0)
+    n = len(plan.fc2d_poisson_nodes())
+    gn = torch.linspace(-1.0, 1.0, n, dtype=torch.float64, device=fg.device)[None]
+    outs = [(torch.zeros_like(fg), torch.zeros_like(gn)) for _ in range(2)]
+    plan.fc2d_poisson(1, fg, fb, gn, *outs[0])
+    plan.fc2d_sync_status()
+    plan.fc2d_wait_selftest(polls)
+    with pytest.raises(fc2d.Fc2dError, match="device status latched") as e:
+        plan.fc2d_sync_status()
+    assert _status(e) == 4
+    plan.fc2d_sync_status()  # reported once
+    plan.fc2d_poisson(1, fg, fb, gn, *outs[1])
+    plan.fc2d_sync_status()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
