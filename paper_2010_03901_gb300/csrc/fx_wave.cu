@@ -463,7 +463,34 @@ int wave_fx_time(double t, double h, double c) {
   return e;
 }
 
-// The plan's mode table, built on first use
+// The plan's mode table, built on first use: on a stream of its own and in the relaxed capture
+// mode, so that the first call may come while streams are captured and waits for nothing else
+static fc2d_status build_modes(fc2d_plan_s* p, fx::Modes* m) {
+  const int nx = p->grid.nx, ny = p->grid.ny;
+  const std::vector<int64_t> turn = fx_turn_table(fx::kTurn);
+  const size_t modes = (size_t)(ny / 2 + 1) * (nx / 2 + 1);
+  fx::Mode* tab = nullptr;
+  if ((!m->turn && cudaMalloc(&m->turn, turn.size() * 8) != cudaSuccess) ||
+      (!m->fac && cudaMalloc(&m->fac, modes * sizeof(int4)) != cudaSuccess) ||
+      cudaMalloc(&tab, modes * sizeof(fx::Mode)) != cudaSuccess) {
+    cudaGetLastError();
+    return set_error(FC2D_ERR_NOMEM, "wave modes: device allocation failed");
+  }
+  cudaStream_t s = nullptr;
+  fc2d_status st = cuda_check(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "wave modes");
+  if (!st) {
+    st = cuda_check(cudaMemcpyAsync(m->turn, turn.data(), turn.size() * 8, cudaMemcpyHostToDevice, s),
+                    "wave modes");
+    fx::k_modes<<<dim3((nx / 2 + 256) / 256, ny / 2 + 1), 256, 0, s>>>(nx, ny, tab);
+    const fc2d_status done = cuda_check(cudaStreamSynchronize(s), "wave modes");
+    if (!st) st = done;
+    cudaStreamDestroy(s);
+  }
+  if (st) cudaFree(tab);
+  else m->tab = tab;
+  return st;
+}
+
 static fc2d_status wave_modes(fc2d_plan_s* p, fx::Modes** out) {
   auto* m = static_cast<fx::Modes*>(p->modes);
   if (!m) {
@@ -471,23 +498,11 @@ static fc2d_status wave_modes(fc2d_plan_s* p, fx::Modes** out) {
     p->modes = m;  // freed with the plan, whatever happens below
   }
   if (!m->tab) {
-    const int nx = p->grid.nx, ny = p->grid.ny;
-    const std::vector<int64_t> turn = fx_turn_table(fx::kTurn);
-    fx::Mode* tab = nullptr;
-    if (!m->turn && (cudaMalloc(&m->turn, turn.size() * 8) != cudaSuccess ||
-                     cudaMemcpy(m->turn, turn.data(), turn.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess))
-      return set_error(FC2D_ERR_NOMEM, "wave modes: device allocation failed");
-    const size_t modes = (size_t)(ny / 2 + 1) * (nx / 2 + 1);
-    if ((!m->fac && cudaMalloc(&m->fac, modes * sizeof(int4)) != cudaSuccess) ||
-        cudaMalloc(&tab, modes * sizeof(fx::Mode)) != cudaSuccess)
-      return set_error(FC2D_ERR_NOMEM, "wave modes: device allocation failed");
-    fx::k_modes<<<dim3((nx / 2 + 256) / 256, ny / 2 + 1), 256>>>(nx, ny, tab);
-    const fc2d_status st = cuda_check(cudaDeviceSynchronize(), "wave modes");
-    if (st) {
-      cudaFree(tab);
-      return st;
-    }
-    m->tab = tab;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const fc2d_status st = build_modes(p, m);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (st) return st;
   }
   *out = m;
   return FC2D_OK;

@@ -60,3 +60,40 @@ def test_modal_solutions(nx, ny, cells):
     eps = 10 * 2.0 ** -53 + slack
     assert norm(got.cpu().numpy()[0] - ref) < eps * (f + t * g)
     assert norm(got_t.cpu().numpy()[0] - ref_t) < eps * (float(w.max()) * f + g)
+
+
+def test_first_call_inside_a_capture():
+    """A plan whose workspace an earlier call has grown takes its first wave call inside a stream
+    capture, and without waiting for other streams: equal to another plan's call bit for bit."""
+    torch = pytest.importorskip("torch")
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    plans = [plan_of(256, 192) for _ in range(3)]
+    rnd = lambda *s: torch.randn(s, dtype=torch.float64, device="cuda", generator=gen)  # noqa: E731
+    fields = [rnd(16, p, q) for p, q in [(192, 256)] * 2]
+    bdry = [rnd(16, plans[0].n_bdry) for _ in range(2)]
+    spec = torch.zeros((16, 192, 129, 2), dtype=torch.float64, device="cuda")
+    for p in plans:
+        p.fc2d_extend_coeffs(16, fields[0], bdry[0], spec)
+    outs = [(torch.zeros_like(fields[0][:1]), torch.zeros_like(fields[0][:1])) for _ in plans]
+
+    def call(k, **kw):
+        plans[k].fc2d_wave_interior(1, 1.3, 0.02, fields[0][:1], bdry[0][:1], fields[1][:1], bdry[1][:1],
+                                    *outs[k], **kw)
+
+    call(0)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(1)
+    graph.replay()
+    mine, other, busy = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Event()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(400_000_000)  # about 0.2 s
+        busy.record()
+    call(2, stream=mine)
+    waited = busy.query()
+    torch.cuda.synchronize()
+    assert not waited
+    for got in outs[1:]:
+        assert torch.equal(outs[0][0], got[0]) and torch.equal(outs[0][1], got[1])
