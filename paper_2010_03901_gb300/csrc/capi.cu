@@ -811,16 +811,30 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
   cudaStream_t s = (cudaStream_t)stream;
   const size_t spec = al((size_t)2 * n_f * p->grid.ny * (p->grid.nx / 2 + 1) * 16);
   const size_t nexp = al(wave_fx_exps(p->grid.nx, p->grid.ny, n_f) * sizeof(int));
-  if ((st = ensure_workspace(p, L.total + spec + nexp)) || (st = wave_fx_prepare(p))) return st;
+  // cells crossed in time t.  From an eighth of a cell on (up to 2^53, past which the phase is
+  // lost in any case, and for factors that doubles hold) the factors are formed in fixed point;
+  // otherwise in FP64.  Where the line lies: the relative error of u from u_t alone is 5e-17/cells
+  // in fixed point below it (5e-12 at 1e-5 cells), 4e-16 in FP64.
+  const double h = p->grid.h, cells = c * t / h;
+  const bool fixed = cells >= 0.125 && cells < 9007199254740992.0 && std::isfinite(8 * c / h);
+  if ((st = ensure_workspace(p, L.total + spec + nexp + (fixed ? 0 : spec))) || (st = wave_fx_prepare(p)))
+    return st;
   void* S = ws(p, L.total);
   int* exps = reinterpret_cast<int*>(ws(p, L.total + spec));
+  void* S2 = ws(p, L.total + spec + nexp);
   if ((st = wave_spectra(p, n_f, u0, u0_bdry, ut0, ut0_bdry, S, s))) return st;
   const FftArgs fa = fft_args(p);
-  const int eT = wave_fx_time(t, p->grid.h, c);
-  wave_fx_spectra(fa, n_f, eT, S, exps, s);
-  for (int k = 0; k < 2; ++k)
-    if ((st = wave_fx_eval(p, fa, n_f, k == 1, c, t, c * t / p->grid.h, eT, S, exps,
-                           ws(p, L.ointer), k ? ut_out : u_out, nullptr, nullptr, s)))
-      return st;
+  if (!fixed) wave_modal_double(fa, n_f, c, t, h, S, S2, s);
+  const int eT = fixed ? wave_fx_time(t, h, c) : 0;
+  for (int k = 0; k < 2; ++k) {
+    void* z = k && !fixed ? S2 : S;
+    if (k == 0 || !fixed) wave_fx_spectra(fa, n_f, eT, z, exps, s);
+    double* out = k ? ut_out : u_out;
+    st = fixed ? wave_fx_eval(p, fa, n_f, k == 1, c, t, cells, eT, z, exps, ws(p, L.ointer), out,
+                              nullptr, nullptr, s)
+               : wave_fx_eval(p, fa, n_f, false, 1.0, 0.0, 0.0, 0, z, exps, ws(p, L.ointer), out,
+                              nullptr, nullptr, s);
+    if (st) return st;
+  }
   return launched("fc2d_wave_interior");
 }

@@ -222,6 +222,10 @@ void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, 
 fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
                          double cells, int eT, const void* spec, int* exps, void* inter, double* out,
                          const int32_t* off, const int32_t* points, cudaStream_t s);
+// the same solutions at time t in FP64: [2 n_f] spectra to u's (in place) and u_t's (deriv), each
+// for wave_fx_spectra with eT = 0 and wave_fx_eval at time 0
+void wave_modal_double(const FftArgs& fa, int n_f, double c, double t, double h, void* spec, void* deriv,
+                       cudaStream_t s);
 // Inverse real row DFT of an [n_f][ny][pitch] half spectrum (double) already inverted along
 // the columns; c00 (NULL allowed) adds c00[f] (x^2 + y^2)/4.
 void launch_inverse_rows(const FftArgs& fa, int n_f, const void* inter, const double* c00,

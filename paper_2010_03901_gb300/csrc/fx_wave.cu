@@ -180,6 +180,35 @@ k_factors(int nxh, bool deriv, When w, const Mode* __restrict__ modes,
   if (l < nxh) fac[at] = v;
 }
 
+// The modal solutions in FP64: a into F and a' into the first half of `deriv`, whose other half
+// and G become zero.  For times in which a wave crosses less than kSmallCells of a cell (or
+// times that no fixed-point phase holds): F and G t, or F w^2 t and G, then differ by
+// more orders of magnitude than their common exponent leaves bits for.  A thread per mode for all
+// functions, bound by the FP64 pipe.
+__global__ void __launch_bounds__(128)
+k_modal_double(int nxh, int ny, int n_f, double c, double t, double Lx, double Ly,
+               double2* __restrict__ spec, double2* __restrict__ deriv) {
+  const int kx = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y;
+  pdl_wait();
+  pdl_trigger();
+  if (kx >= nxh) return;
+  const double fl = kx / Lx, fm = (ky <= ny / 2 ? ky : ky - ny) / Ly;
+  const double w = 6.283185307179586476925286766559 * c * sqrt(fl * fl + fm * fm);
+  double si = 0.0, co = 1.0, sw = t;
+  if (w != 0.0) {
+    sincos(w * t, &si, &co);
+    sw = si / w;
+  }
+  const size_t slab = (size_t)ny * nxh;
+  for (int f = 0; f < n_f; ++f) {
+    const size_t o = f * slab + (size_t)ky * nxh + kx, g = o + n_f * slab;
+    const double2 F = spec[o], G = spec[g];
+    spec[o] = {F.x * co + G.x * sw, F.y * co + G.y * sw};
+    deriv[o] = {G.x * co - F.x * w * si, G.y * co - F.y * w * si};
+    spec[g] = deriv[g] = {0.0, 0.0};
+  }
+}
+
 // Modal advance and pass A of the inverse column transform (a forward transform of the
 // conjugate) for the functions f0 <= f < f0 + gridDim.z: spec, exps as k_spec_fix leaves
 // them; mid [nf][ny][pitch] integers with exponents mexps[nf][N2][column group].
@@ -458,8 +487,9 @@ static bool wave_cols64(int ny) { return ny == 512 || ny == 1024 || ny == 2048 |
 // The exponent eT of the times up to t: 2^eT >= t, and at least the time h/(8 c) in which a
 // wave crosses an eighth of a cell (u_t is of the size of w u, w up to 4.4 c/h)
 int wave_fx_time(double t, double h, double c) {
-  int e;
-  std::frexp(std::max(t, h / (8 * c)), &e);
+  const double x = std::max(t, h / (8 * c));
+  int e = 0;
+  if (std::isfinite(x)) std::frexp(x, &e);
   return e;
 }
 
@@ -551,6 +581,15 @@ void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, 
 #undef CALL
 }
 
+// Modal solutions at time t in FP64, in place of the spectra; their time derivatives to `deriv`
+// (as large).  wave_fx_eval at time 0 then gives either.
+void wave_modal_double(const FftArgs& fa, int n_f, double c, double t, double h, void* spec, void* deriv,
+                       cudaStream_t s) {
+  const int nxh = fa.nx / 2 + 1;
+  launch_pdl(fx::k_modal_double, dim3((nxh + 127) / 128, fa.ny), dim3(128), 0, s, nxh, fa.ny, n_f, c, t,
+             fa.nx * h, fa.ny * h, (double2*)spec, (double2*)deriv);
+}
+
 // u (or, deriv, u_t) at time t = cells h / c of the modal solutions, on the grid or, with
 // off, at the listed points (out[point][n_f]).  spec, exps: from wave_fx_spectra (exps has wave_fx_exps ints); inter:
 // 2 n_f ny pitch complex values of scratch.
@@ -562,7 +601,10 @@ fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv,
   if (st) return st;
   const int nxh = fa.nx / 2 + 1, groups = fa.nx / 32 + 1, N2 = fa.ny / 64;
   const unsigned pitch = (unsigned)fa.pitch;
-  const fx::When w = fx::when(t, cells, c, p->grid.h, eT);
+  // a speed or time without finite factors: NaN everywhere
+  const bool lost = !std::isfinite(8 * c / p->grid.h) || !std::isfinite(t);
+  const fx::When w = lost ? fx::when(0.0, 0.0, 1.0, p->grid.h, 0) : fx::when(t, cells, c, p->grid.h, eT);
+  const int eS = lost ? fx::kNaN : deriv ? w.eS : 0;
   const int chunk = wave_chunk(fa, n_f);
   const size_t slab = (size_t)fa.ny * fa.pitch;
   auto* mid = static_cast<fx::c64*>(inter);
@@ -578,11 +620,11 @@ fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv,
     {
       ProfScope ps(p, "ff_cols", s);
       if (!wave_cols64(fa.ny)) {
-        launch_adv_mixed(fa, n_f, f0, nf, deriv, deriv ? w.eS : 0, m->fac, spec, exps, mid, mexps, res, s);
+        launch_adv_mixed(fa, n_f, f0, nf, deriv, eS, m->fac, spec, exps, mid, mexps, res, s);
       } else {
 #define CALL(N)                                                                                   \
   launch_pdl(deriv ? fx::k_adv_a<N, true> : fx::k_adv_a<N, false>, dim3(groups, N2, nf),           \
-             dim3(fx::kColThreads), 0, s, nxh, pitch, n_f, f0, deriv ? w.eS : 0, m->fac,             \
+             dim3(fx::kColThreads), 0, s, nxh, pitch, n_f, f0, eS, m->fac,             \
              (const fx::c64*)spec, exps, fa.fxwy, mid, mexps);                                       \
   launch_pdl(fx::k_adv_b<N>, dim3(groups, N2, nf), dim3(fx::kColThreads), 0, s, nxh, pitch,          \
              (const fx::c64*)mid, (const int*)mexps, fa.fxwy, res)

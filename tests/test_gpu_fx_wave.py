@@ -97,3 +97,64 @@ def test_first_call_inside_a_capture():
     assert not waited
     for got in outs[1:]:
         assert torch.equal(outs[0][0], got[0]) and torch.equal(outs[0][1], got[1])
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 512), (90, 100), (1200, 512)])
+@pytest.mark.parametrize("cells", [1e-9, 1e-5, 1e-3, 0.05, 0.2])
+@pytest.mark.parametrize("amp", [(1, 0), (0, 1), (1, 1)])
+def test_times_below_a_cell(nx, ny, cells, amp):
+    """u and t u_t of the same size (or one of them zero) at times in which a wave crosses a small
+    part of a cell.  The bars of test_modal_solutions with u_t's factor at that time: w sin(w t)
+    is at most w min(1, w t)."""
+    torch = pytest.importorskip("torch")
+    fft = pytest.importorskip("scipy.fft")
+    plan = plan_of(nx, ny)
+    h, c = 2.0 / (0.45 * min(nx, ny)), 1.7
+    t = cells * h / c
+    x, y = (np.arange(nx) - 0.5 * nx) * h, (np.arange(ny) - 0.5 * ny) * h
+    xy = plan.fc2d_boundary_points().T
+    fn = lambda X, Y: np.cos(2.1 * X + 0.3) * np.cos(1.7 * Y - 0.2)  # noqa: E731
+    T = lambda a: torch.tensor(a[None], dtype=torch.float64, device="cuda")  # noqa: E731
+    data, ext = [], []
+    for a in (amp[0], amp[1] / t):
+        data += [T(a * fn(x[None, :], y[:, None])), T(a * fn(xy[0], xy[1]))]
+        e = torch.zeros_like(data[0])
+        plan.fc2d_extend(1, data[-2], data[-1], e)
+        ext.append(e.cpu().numpy()[0].astype(np.longdouble))
+    got, got_t = data[0], data[2]  # in place
+    plan.fc2d_wave_interior(1, c, t, *data, got, got_t)
+    plan.fc2d_sync_status()
+    F, G = fft.rfft2(ext[0]), fft.rfft2(ext[1])
+    L = np.longdouble
+    l, m = np.arange(nx // 2 + 1, dtype=L) / nx, np.abs(np.fft.fftfreq(ny) * ny).astype(L) / ny
+    w = 2 * L("3.14159265358979323846264338327950288") * L(c) * np.sqrt(l[None, :] ** 2 + m[:, None] ** 2) / L(h)
+    sw = np.where(w > 0, np.sin(w * L(t)) / np.where(w > 0, w, 1), L(t))
+    ref = fft.irfft2(F * np.cos(w * L(t)) + G * sw, s=(ny, nx))
+    ref_t = fft.irfft2(G * np.cos(w * L(t)) - F * w * np.sin(w * L(t)), s=(ny, nx))
+    norm = lambda a: float(np.sqrt((np.abs(a) ** 2).sum()))  # noqa: E731
+    f, g, top = norm(ext[0]), norm(ext[1]), float(w.max())
+    eps = 10 * 2.0 ** -53 + top * t * 2.0 ** -52
+    e = norm(got.cpu().numpy()[0] - ref), norm(got_t.cpu().numpy()[0] - ref_t)
+    bar = eps * (f + t * g), eps * (top * min(1.0, top * t) * f + g)
+    print(nx, ny, cells, amp, e[0] / bar[0], e[1] / bar[1])
+    assert e[0] < bar[0] and e[1] < bar[1]
+
+
+def test_times_without_a_phase():
+    """Time zero gives the data's extensions, times and speeds whose phase is not finite NaN."""
+    import torch
+    plan = plan_of(128, 96)
+    gen = torch.Generator(device="cuda").manual_seed(13)
+    rnd = lambda *s: torch.randn(s, dtype=torch.float64, device="cuda", generator=gen)  # noqa: E731
+    u, v, ub, vb = rnd(2, 96, 128), rnd(2, 96, 128), rnd(2, plan.n_bdry), rnd(2, plan.n_bdry)
+    a, b, e = torch.zeros_like(u), torch.zeros_like(u), torch.zeros_like(u)
+    for c, t in ((1.0, float("inf")), (float("inf"), 1.0), (1e200, 1e200)):
+        plan.fc2d_wave_interior(2, c, t, u, ub, v, vb, a, b)
+        assert bool(torch.isnan(a).all()) and bool(torch.isnan(b).all()), (c, t)
+    plan.fc2d_wave_interior(2, 1.0, 1e25, u, ub, v, vb, a, b)
+    assert bool(torch.isfinite(a).all()) and bool(torch.isfinite(b).all())
+    plan.fc2d_wave_interior(2, 1.0, 0.0, u, ub, v, vb, a, b)
+    for got, f, fb in ((a, u, ub), (b, v, vb)):
+        plan.fc2d_extend(2, f, fb, e)
+        # each transform within 3 2^-53 in the 2-norm
+        assert float((got - e).norm() / e.norm()) < 6 * 2.0 ** -53
