@@ -418,3 +418,29 @@ def test_double_float_mode_against_fp64_squares(torch_cuda):
         assert np.abs(u2[ins] - u1[ins]).max() < du, k
         assert np.abs(t2[ins] - t1[ins]).max() < dut, k
         assert np.array_equal(u2[~ins], u1[~ins])
+
+
+@pytest.mark.parametrize("size,n_c,n_f,n_large", [(256, 6, 3, 2), (1024, 8, 5, 1)])
+def test_interface_mode_2_computes_mode_1(torch_cuda, size, n_c, n_f, n_large):
+    """Interface modes 1 and 2 run the same kernels: u and u_t equal bit for bit, so that the bars
+    against the oracle without df_bars hold for both."""
+    torch = torch_cuda
+    from paper_2010_03901_gb300 import fc2d
+    w = _disk_offset(2.56 / size) if size < 1024 else W.workload(f"kite{size}", d=4, M=7)
+    g, p = w.grid, w.params
+    plan = fc2d.fc2d_plan(w.boundary.arrays(), (g.a0, g.b0, g.h, g.nx, g.ny),
+                          dict(d=4, M=7, B=p.B, k1=p.k1))
+    gen = torch.Generator(device="cuda").manual_seed(14)
+    k = torch.rand((2, n_f, 2), dtype=torch.float64, device="cuda", generator=gen) * 6 + 1
+    xs = torch.arange(g.nx, device="cuda", dtype=torch.float64) * g.h
+    ys = torch.arange(g.ny, device="cuda", dtype=torch.float64) * g.h
+    field = lambda q: torch.sin(q[:, 0, None, None] * xs + q[:, 1, None, None] * ys[:, None])  # noqa: E731
+    out = []
+    for df in (False, True):
+        u, ut = field(k[0]), field(k[1])
+        plan.fc2d_forward_wave(n_f, 1.0, n_c, n_large, u, ut, squares=True, double_float=df)
+        plan.fc2d_sync_status()
+        out.append((u, ut))
+    assert bool(out[0][0].isfinite().all()) and float(out[0][0].abs().max()) > 0
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
