@@ -76,8 +76,8 @@ struct DevOp {
 
 struct DevBand {
   WaveBand host;
-  DevCsr L, D, S;                   // with keys (one step with caller data, the merge)
-  DevOp Ls, Ds;                     // with state rows (the solve)
+  DevCsr S;                         // with keys (the merge)
+  DevOp L, D;                       // with state rows (the small step)
   int32_t* unknown_lin = nullptr;
   int32_t* near_lin = nullptr;
   int32_t* near_src = nullptr;
@@ -207,8 +207,7 @@ fc2d_status get_band(fc2d_plan_s* p, int n_c, int mode, DevBand** out) {
   // operator entries of a grid kind must index the grid (30 bits), boundary data too
   if ((int64_t)p->grid.nx * p->grid.ny > (int64_t)kKeyIndex || p->n_bdry > (int64_t)kKeyIndex)
     return set_error(FC2D_ERR_UNSUPPORTED, "wave band: grid too large for the operator keys");
-  if ((st = upload_csr(b->L, b->host.L)) || (st = upload_csr(b->D, b->host.D)) ||
-      (st = upload_csr(b->S, b->host.S)) || (st = upload(&b->unknown_lin, b->host.unknown_lin)) ||
+  if ((st = upload_csr(b->S, b->host.S)) || (st = upload(&b->unknown_lin, b->host.unknown_lin)) ||
       (st = upload(&b->near_lin, b->host.near_lin)) || (st = upload(&b->near_src, b->host.near_src)))
     return st;
   const std::vector<int32_t>& q = b->host.iface_lin;
@@ -216,8 +215,8 @@ fc2d_status get_band(fc2d_plan_s* p, int n_c, int mode, DevBand** out) {
   for (int j = 0; j <= p->grid.ny; ++j)
     off[j] = (int32_t)(std::lower_bound(q.begin(), q.end(), (int64_t)j * p->grid.nx) - q.begin());
   if ((st = upload(&b->iface_off, off)) || (st = upload(&b->iface_lin, q)) ||
-      (st = upload_op(b->Ls, b->host.L, b->host, (int32_t)(b->host.unknown_lin.size() + q.size()))) ||
-      (st = upload_op(b->Ds, b->host.D, b->host, (int32_t)b->host.unknown_lin.size())))
+      (st = upload_op(b->L, b->host.L, b->host, (int32_t)(b->host.unknown_lin.size() + q.size()))) ||
+      (st = upload_op(b->D, b->host.D, b->host, (int32_t)b->host.unknown_lin.size())))
     return st;
   *out = b.get();
   W->bands[{n_c, mode}] = std::move(b);
@@ -249,80 +248,40 @@ __device__ __forceinline__ double ub_value(uint32_t key, int f, int n_f, int64_t
   return g ? g[(size_t)f * n_b + idx] : 0.0;
 }
 
-// One U_B small step for every (unknown r, function f), thread t = r n_f + f.
-//   mode 0: out = u + dt ut + cdt2/2 L(u)                (Taylor start; ut: [N][n_f])
-//   mode 1: out = 2u - up + cdt2 L(u) - sigma D(u - up)
-//   mode 2: the mode-1 value v, stored as (v - up)/(2 dt)  (the time derivative at u's time)
-// L's interface columns read `grid` (U_FC at u's time), D's the difference grid - grid_prev;
-// g: Dirichlet data [n_f][n_b] at u's time (NULL: zero).
-__global__ void __launch_bounds__(256) k_ub_step(int mode, int64_t n, int n_f, int64_t grid_stride,
-                                                 int64_t n_b, const int32_t* __restrict__ Loff,
-                                                 const uint32_t* __restrict__ Lcol,
-                                                 const double* __restrict__ Lw,
-                                                 const int32_t* __restrict__ Doff,
-                                                 const uint32_t* __restrict__ Dcol,
-                                                 const double* __restrict__ Dw,
-                                                 const double* __restrict__ u,
-                                                 const double* __restrict__ up,
-                                                 const double* __restrict__ ut,
-                                                 const double* __restrict__ grid,
-                                                 const double* __restrict__ grid_prev,
-                                                 const double* __restrict__ g, double cdt2,
-                                                 double dt, double sigma, double* __restrict__ out) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * n_f) return;
-  const int64_t r = t / n_f;
-  const int f = (int)(t - r * n_f);
-  double lap = 0.0;
-  for (int k = Loff[r]; k < Loff[r + 1]; ++k)
-    lap += Lw[k] * ub_value(Lcol[k], f, n_f, grid_stride, n_b, u, grid, g);
-  const double u0 = u[t];
-  if (mode == 0) {
-    out[t] = u0 + dt * ut[t] + 0.5 * cdt2 * lap;
-    return;
-  }
-  double dis = 0.0;
-  for (int k = Doff[r]; k < Doff[r + 1]; ++k) {
-    const uint32_t key = Dcol[k], idx = key & kKeyIndex;
-    double d;
-    if ((key & kKeyKind) == kKeyUnknown) {
-      d = u[(size_t)idx * n_f + f] - up[(size_t)idx * n_f + f];
-    } else {
-      const size_t o = (size_t)f * grid_stride + idx;
-      d = grid[o] - grid_prev[o];
-    }
-    dis += Dw[k] * d;
-  }
-  const double v = 2.0 * u0 - up[t] + cdt2 * lap - sigma * dis;
-  out[t] = mode == 1 ? v : (v - up[t]) / (2.0 * dt);
-}
-
-// The small step of the solve, on u and w = u^n - u^{n-1}, function-minor: rows of U are the N
-// unknowns, then the n_i interface points (U_FC at u's time), and boundary columns come after
-// those; Uold holds the interface points of the step before in the same rows.
+// One U_B small step for every (unknown r, function f), thread t = r n_f + f, on u and
+// w = u^n - u^{n-1}.  The columns of the operators are rows of the state: the N unknowns, the n_i
+// interface points (U_FC at u's time), then boundary points (g: Dirichlet data [n_f][n_b] at u's
+// time, NULL: zero).
 //   mode 0: w' = dt u_t + cdt2/2 L(u)     (Taylor start; W holds u_t)
 //   mode 1: w' = w + cdt2 L(u) - sigma D(w)
 //   mode 2: (w' + w)/(2 dt), w' of mode 1, to Uout (the time derivative at u's time)
 // and u' = u + w'.  The FP64 pipe bounds it: w saves the difference u - u_prev of every
 // D entry (38 multiply-adds and 33 additions per value before), and does not cancel.
+// GRIDS false (the solve): function-minor rows, U [N + n_i][n_f] and Uold the step before (only its
+// interface rows are read), W [N][n_f]; Wout receives w'.  GRIDS true (a caller's own arrays): U and
+// Uold are u^n and u^{n-1} of the unknowns, the interface points iface[n_i] lie in grid and
+// grid_prev [n_f][stride], W is u_t (mode 0 only).
+template <bool GRIDS>
 __global__ void __launch_bounds__(256) k_ub_advance(
     int mode, int n, int n_i, int n_f, int64_t n_b, const int2* __restrict__ Lrow,
     const UbEntry* __restrict__ Le, const int2* __restrict__ Drow, const UbEntry* __restrict__ De,
     const double* __restrict__ U, const double* __restrict__ Uold, const double* __restrict__ W,
-    const double* __restrict__ g, double cdt2, double dt, double sigma, double* __restrict__ Uout,
-    double* __restrict__ Wout) {
+    const double* __restrict__ g, const double* __restrict__ grid, const double* __restrict__ grid_prev,
+    int64_t stride, const int32_t* __restrict__ iface, double cdt2, double dt, double sigma,
+    double* __restrict__ Uout, double* __restrict__ Wout) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n_f) return;
   const int r = (int)(t / n_f), f = (int)(t - (int64_t)r * n_f);
-  const double u = U[t], w = W[t];
+  const double u = U[t], w = GRIDS && mode ? u - Uold[t] : W[t];
   double lap = 0.0, dis = 0.0;
   const double *Uf = U + f, *Wf = W + f;
+  auto face = [&](int col) { return (size_t)f * stride + __ldg(iface + (col - n)); };  // GRIDS
   const int2 l0 = __ldg(Lrow + r);
   const int l1 = __ldg(&Lrow[r + 1].x);
 #pragma unroll 4
   for (int k = l0.x; k < l0.y; ++k) {
     const UbEntry e = Le[k];
-    lap += e.w * Uf[(size_t)e.col * n_f];
+    lap += e.w * (GRIDS && e.col >= n ? grid[face(e.col)] : Uf[(size_t)e.col * n_f]);
   }
   if (g)  // boundary points
     for (int k = l0.y; k < l1; ++k) {
@@ -338,12 +297,13 @@ __global__ void __launch_bounds__(256) k_ub_advance(
 #pragma unroll 4
     for (int k = d0.x; k < d0.y; ++k) {
       const UbEntry e = De[k];
-      dis += e.w * Wf[(size_t)e.col * n_f];
+      const size_t o = (size_t)e.col * n_f;
+      dis += e.w * (GRIDS ? Uf[o] - Uold[o + f] : Wf[o]);
     }
     for (int k = d0.y; k < d1; ++k) {  // interface points
       const UbEntry e = De[k];
-      const size_t o = (size_t)e.col * n_f + f;
-      dis += e.w * (U[o] - Uold[o]);
+      const size_t o = GRIDS ? face(e.col) : (size_t)e.col * n_f + f;
+      dis += e.w * (GRIDS ? grid[o] - grid_prev[o] : U[o] - Uold[o]);
     }
     wn = w + cdt2 * lap - sigma * dis;
     if (mode == 2) {
@@ -351,7 +311,7 @@ __global__ void __launch_bounds__(256) k_ub_advance(
       return;
     }
   }
-  Wout[t] = wn;
+  if (!GRIDS) Wout[t] = wn;
   Uout[t] = u + wn;
 }
 
@@ -416,10 +376,8 @@ void wave_destroy(fc2d_plan_s* p) {
   auto* W = static_cast<WaveState*>(p->wave);
   for (auto& kv : W->bands) {
     DevBand& b = *kv.second;
-    free_csr(b.L);
-    free_csr(b.D);
     free_csr(b.S);
-    for (DevOp* o : {&b.Ls, &b.Ds}) {
+    for (DevOp* o : {&b.L, &b.D}) {
       cudaFree(o->row);
       cudaFree(o->e);
     }
@@ -511,11 +469,12 @@ extern "C" fc2d_status fc2d_wave_ub_step(fc2d_plan_t p, int n_c, int n_f, int mo
   if ((st = get_band(p, n_c, 0, &b))) return st;
   const double h = p->grid.h, cdt2 = (kUbCfl * h) * (kUbCfl * h);
   const double dt = kUbCfl * h / c;
-  const int64_t n = b->L.rows;
+  const int64_t n = (int64_t)b->host.unknown_lin.size();
   if (n > 0)
-    k_ub_step<<<blocks(n * n_f, 256), 256, 0, (cudaStream_t)stream>>>(
-        mode, n, n_f, (int64_t)p->grid.nx * p->grid.ny, p->n_bdry, b->L.off, b->L.col, b->L.w,
-        b->D.off, b->D.col, b->D.w, u, u_prev, ut, grid, grid_prev, g, cdt2, dt, kUbSigma, out);
+    k_ub_advance<true><<<blocks(n * n_f, 256), 256, 0, (cudaStream_t)stream>>>(
+        mode, (int)n, (int)b->host.iface_lin.size(), n_f, p->n_bdry, b->L.row, b->L.e, b->D.row, b->D.e,
+        u, u_prev, ut, g, grid, grid_prev, (int64_t)p->grid.nx * p->grid.ny, b->iface_lin, cdt2, dt,
+        kUbSigma, out, nullptr);
   return cuda_check(cudaGetLastError(), "fc2d_wave_ub_step");
 }
 
@@ -541,7 +500,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   // mode 1, which are both faster and more accurate
   if ((st = get_band(p, n_c, interface_mode ? 1 : 0, &b))) return st;
   const int nx = p->grid.nx, ny = p->grid.ny, nxh = nx / 2 + 1;
-  const int64_t NN = (int64_t)nx * ny, nb = p->n_bdry, Nu = b->L.rows;
+  const int64_t NN = (int64_t)nx * ny, nb = p->n_bdry, Nu = b->host.unknown_lin.size();
   const int64_t Ni = (int64_t)b->host.iface_lin.size();
   const size_t pitch = row_pitch(p);
   const int S = 8 * n_c;
@@ -602,9 +561,9 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   auto ub_step = [&](int mode, const double* g, double* uo, double* wo) {
     if (Nu == 0) return;
     ProfScope ps(p, "ub_step", s);
-    k_ub_advance<<<blocks(Nu * n_f, 256), 256, 0, s>>>(
-        mode, (int)Nu, (int)Ni, n_f, nb, b->Ls.row, b->Ls.e, b->Ds.row, b->Ds.e, U[a], U[1 - a], V[a],
-        g, cdt2, dt, kUbSigma, uo, wo);
+    k_ub_advance<false><<<blocks(Nu * n_f, 256), 256, 0, s>>>(
+        mode, (int)Nu, (int)Ni, n_f, nb, b->L.row, b->L.e, b->D.row, b->D.e, U[a], U[1 - a], V[a],
+        g, nullptr, nullptr, 0, nullptr, cdt2, dt, kUbSigma, uo, wo);
   };
   // U_B at t = 0: u^0, and u_t^0 in the place of w
   gather(Nu, b->unknown_lin, u, U[a]);

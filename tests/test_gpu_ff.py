@@ -444,3 +444,34 @@ def test_interface_mode_2_computes_mode_1(torch_cuda, size, n_c, n_f, n_large):
     assert bool(out[0][0].isfinite().all()) and float(out[0][0].abs().max()) > 0
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_f", [1, 33])
+def test_one_small_step_without_dirichlet_data(torch_cuda, n_f):
+    """fc2d_wave_ub_step, which runs the solve's kernel and operators on a caller's arrays, with
+    zero Dirichlet data (NULL) and one and 33 functions, against the oracle."""
+    torch = torch_cuda
+    name, n_c = CASES[1]
+    w, plan, geo = _setup(name)
+    band = OWB.build_band(geo, n_c)
+    g, c = w.grid, 0.7
+    Nu, nb = len(band.unknown_lin), len(geo.bdry_x)
+    rnd = lambda seed, *shape: W.normal(seed, int(np.prod(shape))).reshape(shape)  # noqa: E731
+    u, up, ut = rnd(41, n_f, Nu), rnd(42, n_f, Nu), rnd(43, n_f, Nu)
+    grid, grid_p = rnd(44, n_f, g.ny, g.nx), rnd(45, n_f, g.ny, g.nx)
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")  # noqa: E731
+    dt = OWB.CFL * g.h / c
+    out = torch.zeros((Nu, n_f), dtype=torch.float64, device="cuda")
+    for mode in range(3):
+        old = (None, None) if mode == 0 else (T(up.T), T(grid_p))
+        plan.fc2d_wave_ub_step(n_c, n_f, mode, c, T(u.T), old[0], T(ut.T), T(grid), old[1], None, out)
+        got = out.cpu().numpy().T
+        for f in (0, n_f - 1):
+            fi, fpi = grid[f].ravel()[band.iface_lin], grid_p[f].ravel()[band.iface_lin]
+            if mode == 0:
+                ref = OWB.first_step(band, g.h, u[f], ut[f], fi, np.zeros(nb), dt)
+            else:
+                ref = OWB.step(band, g.h, u[f], up[f], fi, fpi, np.zeros(nb))
+                if mode == 2:
+                    ref = (ref - up[f]) / (2 * dt)
+            assert np.abs(got[f] - ref).max() < 1e-12 * np.abs(ref).max(), (mode, f)
