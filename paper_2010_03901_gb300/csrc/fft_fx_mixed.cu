@@ -45,11 +45,7 @@ k_rows_mixed(FftArgs fa, RowArgs ra, int mode, const double* __restrict__ ext,
             [&](int b, int i) { return b ? buf[i] : b0[i]; },
             [&](int b, int i, c64 v) { (b ? buf : b0)[i] = v; }, fa.fxwx, 1, st, e);
   const c64* z = (fa.mix.row.n - 1) & 1 ? buf : b0;
-  if (fa.mix.row.n == 0) {  // NH = 1
-    if (t == 0) b0[0] = from_double(row[0], E);
-    __syncthreads();
-  }
-  const int L = fa.mix.row.n ? max(headroom(st[fa.mix.row.n]) - 1, 0) : 0;  // |z| <= 2^61
+  const int L = max(headroom(st[fa.mix.row.n]) - 1, 0);  // |z| <= 2^61
   e += kDrop - 1 - L;
   if (E >= 0x7FF) e = kNaN;
   const bool plain = plain_exp(e);
@@ -100,7 +96,7 @@ k_inverse_rows_mixed(FftArgs fa, const double2* __restrict__ inter, const double
   mixed_dft(fa.mix.row, NH, t, nt, [&](int i) { return b1[i]; },
             [&](int b, int i) { return b ? b1[i] : bz[i]; },
             [&](int b, int i, c64 v) { (b ? b1 : bz)[i] = v; }, fa.fxwx, 1, st, e);
-  const c64* z = fa.mix.row.n && !((fa.mix.row.n - 1) & 1) ? bz : b1;
+  const c64* z = (fa.mix.row.n - 1) & 1 ? b1 : bz;
   if (E >= 0x7FF) e = kNaN;
   const bool plain = plain_exp(e);
   if (point_off) {
@@ -158,7 +154,7 @@ __device__ __forceinline__ void mixed_pass_a(const FxMixed& mx, unsigned char* s
             [&](int b, int i, c64 v) { (b ? b1 : b0)[i * kCols] = v; }, w, n2, st, e);
   const c64* z = (mx.a.n - 1) & 1 ? b1 : b0;
   if (live)
-    for (int i = t; i < n1; i += ct) mid[(unsigned)(n2 * i + j2) * pitch + kx] = mx.a.n ? z[i * kCols] : first(i);
+    for (int i = t; i < n1; i += ct) mid[(unsigned)(n2 * i + j2) * pitch + kx] = z[i * kCols];
   if (threadIdx.x == 0) *exp_out = E >= 0x7FF ? kNaN : e;
 }
 
@@ -193,7 +189,7 @@ __device__ __forceinline__ void mixed_pass_b(const FxMixed& mx, unsigned char* s
   e += eadd;
   const bool plain = plain_exp(e);
   if (live)
-    for (int i = t; i < n2; i += ct) out(m1 + n1 * i, mx.b.n ? z[i * kCols] : first(i), e, plain);
+    for (int i = t; i < n2; i += ct) out(m1 + n1 * i, z[i * kCols], e, plain);
 }
 
 __global__ void __launch_bounds__(160, 4)

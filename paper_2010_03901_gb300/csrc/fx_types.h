@@ -16,7 +16,7 @@ struct FxRadices {
   signed char r[kFxMaxRadices];
 };
 struct FxMixed {
-  FxRadices row, a, b;  // nx/2, n1, n2
+  FxRadices row, a, b;  // nx/2, n1, n2: at least one stage each (nx, ny >= 8)
   int n1, n2;           // ny = n1 n2, n2 the largest divisor up to sqrt(ny)
   int ta, tb;           // threads per column of both passes
 };
