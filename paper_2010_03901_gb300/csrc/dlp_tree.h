@@ -42,14 +42,14 @@ struct DlpTree {
   std::vector<int32_t> chain;
   std::vector<DlpLeaf> leaf;
   std::vector<DlpItem> grid_items, free_items;
-  std::vector<int32_t> grid_order;    // point lists in leaf order: indices into the given lists
-  std::vector<int32_t> free_order;
+  // the points in leaf order: linear indices of grid points, indices of free points
+  std::vector<int32_t> grid_order, free_order;
 };
 
-// nodes, grid points (integers) and free points, all in grid units; extent: bound of all
-// coordinates
+// nodes and free points in grid units, grid points as linear indices j stride + i; extent: bound
+// of all coordinates.  The partition is the same with threads and without.
 DlpTree dlp_tree(const std::vector<double>& nx, const std::vector<double>& ny,
-                 const std::vector<int32_t>& gi, const std::vector<int32_t>& gj,
-                 const std::vector<double>& px, const std::vector<double>& py, int extent);
+                 const std::vector<int32_t>& lin, int stride, const std::vector<double>& px,
+                 const std::vector<double>& py, int extent, bool threads = true);
 
 }  // namespace fc2d

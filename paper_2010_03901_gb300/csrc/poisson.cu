@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <future>
 #include <string>
 #include <vector>
 
@@ -466,15 +467,15 @@ fc2d_status poisson_setup(fc2d_plan_s* p, int Nb) {
   auto partition = [&](std::vector<int32_t>& lin, const std::vector<double>& X,
                        const std::vector<double>& Y, const std::vector<double>& fx,
                        const std::vector<double>& fy) {
-    std::vector<int32_t> gi(lin.size()), gj(lin.size()), ord(lin.size());
-    for (size_t k = 0; k < lin.size(); ++k) gi[k] = lin[k] % nx, gj[k] = lin[k] / nx;
-    DlpTree t = dlp_tree(grid(X, a0), grid(Y, b0), gi, gj, fx, fy, std::max(nx, ny));
-    for (size_t k = 0; k < lin.size(); ++k) ord[k] = lin[t.grid_order[k]];
-    lin.swap(ord);
+    DlpTree t = dlp_tree(grid(X, a0), grid(Y, b0), lin, nx, fx, fy, std::max(nx, ny));
+    lin.swap(t.grid_order);
     return t;
   };
-  const DlpTree tf = partition(far, x, y, {}, {});
+  // the two side by side
+  auto far_tree = std::async(std::launch::async | std::launch::deferred,
+                             [&] { return partition(far, x, y, {}, {}); });
   const DlpTree tn = partition(mid, rx, ry, px, py);
+  const DlpTree tf = far_tree.get();
   P->n_far = (int64_t)far.size();
   P->n_mid = (int64_t)mid.size();
   P->n_close = (int64_t)close.size();
