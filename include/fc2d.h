@@ -241,7 +241,7 @@ fc2d_status fc2d_poisson_info(fc2d_plan_t plan, int* gmres_iters, double* gmres_
  * w = 2 pi c sqrt((l/L_x)^2 + (m/L_y)^2), and their inverse DFTs.  u_out and ut_out
  * [n_f][ny][nx] receive U_FC(., t) and its time derivative on the whole grid; they are
  * the wave solution at the grid points farther than c t from the curve (domain of
- * dependence).  ny <= 4736.  The first wave call on a plan (this one or
+ * dependence).  ny <= 4842.  The first wave call on a plan (this one or
  * fc2d_forward_wave) makes the plan's table of modes, 32 bytes for each of the
  * (nx/2 + 1)(ny/2 + 1) modes, without waiting for other streams; the workspace holds
  * both spectra beside the row transforms. */

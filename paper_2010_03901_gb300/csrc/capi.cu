@@ -804,8 +804,8 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
   if (!(c > 0) || !(t >= 0)) return set_error(FC2D_ERR_ARG, "fc2d_wave_interior: c > 0, t >= 0");
   if (p->prm.precision != FC2D_FP64)
     return set_error(FC2D_ERR_UNSUPPORTED, "fc2d_wave_interior: FP64 plans only");
-  if (3 * (size_t)p->grid.ny * sizeof(double2) > 227 * 1024)
-    return set_error(FC2D_ERR_UNSUPPORTED, "fc2d_wave_interior: ny <= 4736");
+  if (p->grid.ny > kWaveMaxRows)
+    return set_error(FC2D_ERR_UNSUPPORTED, "fc2d_wave_interior: ny <= 4842");
   cudaSetDevice(p->device);
   Layout L = layout(p, 2 * n_f);
   cudaStream_t s = (cudaStream_t)stream;

@@ -490,7 +490,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
     return set_error(FC2D_ERR_ARG, "fc2d_forward_wave: c > 0 and n_large >= 0 required");
   if (interface_mode < 0 || interface_mode > 2)
     return set_error(FC2D_ERR_ARG, "fc2d_forward_wave: interface_mode 0, 1 or 2");
-  if (3 * (size_t)p->grid.ny * sizeof(double2) > 227 * 1024)
+  if (p->grid.ny > kWaveMaxRows)
     return set_error(FC2D_ERR_UNSUPPORTED, "fc2d_forward_wave: ny <= 4842");
   if (n_large == 0) return FC2D_OK;
   cudaSetDevice(p->device);

@@ -20,6 +20,10 @@ constexpr int kMaxM = 16;
 constexpr int kTcComputed = 64;
 constexpr int kTcOwned = 57;
 constexpr int kOwnerSets = 4;   // partitions of the normals over the CTAs (plan.cpp)
+// Tallest grid of the Fourier Forwarding calls: the range that they have been run and tested on
+// (three columns of a former kernel in a block's shared memory; the present ones need about
+// sqrt(ny) rows).
+constexpr int kWaveMaxRows = 4842;
 
 // One 1D FFT length: its radix sequence and twiddle tables exp(-2 pi i t/N), t < N.
 struct FftAxis {

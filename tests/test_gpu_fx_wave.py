@@ -158,3 +158,26 @@ def test_times_without_a_phase():
         plan.fc2d_extend(2, f, fb, e)
         # each transform within 3 2^-53 in the 2-norm
         assert float((got - e).norm() / e.norm()) < 6 * 2.0 ** -53
+
+
+def test_the_tallest_grid():
+    """ny up to 4842 in both wave calls (4800 = 2^6 3 5^2 is the largest such size), one message
+    above."""
+    import torch
+    from paper_2010_03901_gb300 import fc2d
+    z = lambda p: torch.zeros((1, p.ny, p.nx), dtype=torch.float64, device="cuda")  # noqa: E731
+    tall = plan_of(64, 4860)
+    u = z(tall)
+    b = torch.zeros((1, tall.n_bdry), dtype=torch.float64, device="cuda")
+    for call in (lambda: tall.fc2d_wave_interior(1, 1.0, 0.1, u, b, u, b, z(tall), z(tall)),
+                 lambda: tall.fc2d_forward_wave(1, 1.0, 4, 1, u, u.clone())):
+        with pytest.raises(fc2d.Fc2dError, match="ny <= 4842") as e:
+            call()
+        assert e.value.status == 7
+    plan = plan_of(64, 4800)
+    u, ut = torch.ones_like(z(plan)), z(plan)
+    b = torch.ones((1, plan.n_bdry), dtype=torch.float64, device="cuda")
+    out, ext = [z(plan), z(plan)], z(plan)
+    plan.fc2d_wave_interior(1, 1.0, 0.0, u, b, ut, 0 * b, *out)
+    plan.fc2d_extend(1, u, b, ext)
+    assert float((out[0] - ext).norm() / ext.norm()) < 6 * 2.0 ** -53
