@@ -41,7 +41,7 @@ k_rows_mixed(FftArgs fa, RowArgs ra, int mode, const double* __restrict__ ext,
   int e = E - 1080;
   // the doubles lie in buffer 1, which the second stage overwrites
   c64* b0 = buf + NH;
-  mixed_dft(fa.mix.row, NH, t, nt, [&](int i) { return from_double(row[i], E); },
+  mixed_dft<FORWARD>(fa.mix.row, NH, t, nt, [&](int i) { return from_double(row[i], E); },
             [&](int b, int i) { return b ? buf[i] : b0[i]; },
             [&](int b, int i, c64 v) { (b ? buf : b0)[i] = v; }, fa.fxwx, 1, st, e);
   const c64* z = (fa.mix.row.n - 1) & 1 ? buf : b0;
@@ -93,7 +93,7 @@ k_inverse_rows_mixed(FftArgs fa, const double2* __restrict__ inter, const double
     if (k && k != NH - k) b1[NH - k] = {s.x + q.y, s.y - q.x};
   }
   __syncthreads();
-  mixed_dft(fa.mix.row, NH, t, nt, [&](int i) { return b1[i]; },
+  mixed_dft<INVERSE>(fa.mix.row, NH, t, nt, [&](int i) { return b1[i]; },
             [&](int b, int i) { return b ? b1[i] : bz[i]; },
             [&](int b, int i, c64 v) { (b ? b1 : bz)[i] = v; }, fa.fxwx, 1, st, e);
   const c64* z = (fa.mix.row.n - 1) & 1 ? b1 : bz;
@@ -150,7 +150,7 @@ __device__ __forceinline__ void mixed_pass_a(const FxMixed& mx, unsigned char* s
     if constexpr (ADV) return live ? in(n2 * i + j2, kx) : c64{0, 0};
     else return from_double(raw[i * kCols], E);
   };
-  mixed_dft(mx.a, n1, t, ct, first, [&](int b, int i) { return (b ? b1 : b0)[i * kCols]; },
+  mixed_dft<ADV ? INVERSE : FORWARD>(mx.a, n1, t, ct, first, [&](int b, int i) { return (b ? b1 : b0)[i * kCols]; },
             [&](int b, int i, c64 v) { (b ? b1 : b0)[i * kCols] = v; }, w, n2, st, e);
   const c64* z = (mx.a.n - 1) & 1 ? b1 : b0;
   if (live)
@@ -159,7 +159,7 @@ __device__ __forceinline__ void mixed_pass_a(const FxMixed& mx, unsigned char* s
 }
 
 // Pass B for one m1: out(row, v, e, plain) for the rows m1 + n1 m2 of the transform
-template <typename Out>
+template <Order O, typename Out>
 __device__ __forceinline__ void mixed_pass_b(const FxMixed& mx, unsigned char* smem, unsigned* st,
                                              const c64* __restrict__ mid, unsigned pitch, int m1, int kx,
                                              bool live, const int4* __restrict__ w,
@@ -183,7 +183,7 @@ __device__ __forceinline__ void mixed_pass_b(const FxMixed& mx, unsigned char* s
     const c64 v = b1[i * kCols];
     return mulw(c64{((v.x << up) + rnd) >> dn, ((v.y << up) + rnd) >> dn}, __ldg(w + i * m1));
   };
-  mixed_dft(mx.b, n2, t, ct, first, [&](int b, int i) { return (b ? b1 : b0)[i * kCols]; },
+  mixed_dft<O>(mx.b, n2, t, ct, first, [&](int b, int i) { return (b ? b1 : b0)[i * kCols]; },
             [&](int b, int i, c64 v) { (b ? b1 : b0)[i * kCols] = v; }, w, n1, st, e);
   const c64* z = (mx.b.n - 1) & 1 ? b1 : b0;
   e += eadd;
@@ -220,7 +220,7 @@ k_cols_mixed_b(FftArgs fa, const double2* __restrict__ inter, const int* __restr
   __syncthreads();
   pdl_wait();
   pdl_trigger();
-  mixed_pass_b(fa.mix, smem_raw, st, slab, fa.pitch, blockIdx.y, kx, kx < ncol, fa.fxwy,
+  mixed_pass_b<FORWARD>(fa.mix, smem_raw, st, slab, fa.pitch, blockIdx.y, kx, kx < ncol, fa.fxwy,
                exps + (size_t)f * fa.mix.n2 * gridDim.x + blockIdx.x, gridDim.x, fa.fxs.exp,
                [&](int row, c64 v, int e, bool plain) {
                  dst[(unsigned)row * (unsigned)fa.opitch] = to_double(scaled(v, fa.fxs), e, plain);
@@ -321,7 +321,7 @@ k_adv_mixed_b(FxMixed mx, int ny, int nxh, unsigned pitch, const c64* __restrict
   __syncthreads();
   pdl_wait();
   pdl_trigger();
-  mixed_pass_b(mx, smem_raw, st, mid + (size_t)f * ny * pitch, pitch, blockIdx.y, kx, kx < nxh, tw,
+  mixed_pass_b<INVERSE>(mx, smem_raw, st, mid + (size_t)f * ny * pitch, pitch, blockIdx.y, kx, kx < nxh, tw,
                mexps + (size_t)f * mx.n2 * gridDim.x + blockIdx.x, gridDim.x, 0,
                [&](int row, c64 v, int e, bool plain) {
                  const double2 z = to_double(v, e, plain);

@@ -147,11 +147,11 @@ __device__ __forceinline__ unsigned mixed_stage(int N, int Ns, int first, int ev
 
 // All stages.  in(i): the inputs (|z| <= 2^58.5, in units of 2^e); stage s writes to
 // store(s & 1, i, v) and the next one reads load(s & 1, i).  The block is rescaled before
-// every other stage (st: kMixedSlots zeroed shared words).  Every thread of the block calls it;
+// every other stage, as shifts() says (st: kMixedSlots zeroed shared words).  Every thread of the block calls it;
 // on return (after a barrier) the result is in buffer (n - 1) & 1, its spread in *out_spread
 // if given.
 constexpr int kMixedSlots = 20;
-template <typename In, typename Load, typename Store>
+template <Order O, typename In, typename Load, typename Store>
 __device__ __forceinline__ void mixed_dft(const FxRadices& rad, int N, int first, int every, In in,
                                           Load load, Store store, const int4* __restrict__ tw, int ts,
                                           unsigned* st, int& e) {
@@ -160,7 +160,7 @@ __device__ __forceinline__ void mixed_dft(const FxRadices& rad, int N, int first
     const int R = rad.r[s];
     int L = 0;
     if (s > 0) {
-      if (s % 2 == 0) L = headroom(st[s]);
+      if (shifts(s, O)) L = headroom(st[s]);
       e += kDrop - L;
     }
     auto src = [&](int i) { return s ? load((s - 1) & 1, i) : in(i); };

@@ -221,11 +221,12 @@ k_adv_a(int nxh, unsigned pitch, int n_f, int f0, int eS, const int4* __restrict
         c64* __restrict__ mid, int* __restrict__ mexps) {
   constexpr int ny = 64 * N2;
   __shared__ c64 ex[64 * kCols];
-  __shared__ unsigned st[1];
-  if (threadIdx.x == 0) st[0] = 0;
+  __shared__ unsigned st[2];
+  if (threadIdx.x < 2) st[threadIdx.x] = 0;
   const int c = threadIdx.x & (kCols - 1), l = threadIdx.x / kCols, kx = blockIdx.x * kCols + c;
   const int j2 = blockIdx.y, f = blockIdx.z;
   const bool live = kx < nxh;
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
   const c64* F = spec + (size_t)(f0 + f) * ny * nxh + kx;
@@ -249,7 +250,6 @@ k_adv_a(int nxh, unsigned pitch, int n_f, int f0, int eS, const int4* __restrict
         h |= spread(x[i].hi + (x[i].mid >> 32)) | spread(y[i].hi + (y[i].mid >> 32));
       }
     }
-    __syncthreads();
     block_or(h, st);
     __syncthreads();
     up = min(max(headroom(st[0]) - 4, 0), 28);  // values below 2^58
@@ -269,7 +269,7 @@ k_adv_a(int nxh, unsigned pitch, int n_f, int f0, int eS, const int4* __restrict
       }
     }
   }
-  dft_group<8>(v, c, l, ex, tw, N2);
+  const int L = dft_group<8, true>(v, c, l, ex, tw, N2, st + 1);
   if (live) {
     c64* out = mid + (size_t)f * ny * pitch + kx;
 #pragma unroll
@@ -277,7 +277,7 @@ k_adv_a(int nxh, unsigned pitch, int n_f, int f0, int eS, const int4* __restrict
   }
   if (threadIdx.x == 0)
     mexps[((size_t)f * N2 + j2) * gridDim.x + blockIdx.x] =
-        exps[((size_t)(f0 + f) * N2 + j2) * gridDim.x + blockIdx.x] + 2 * kDrop + eS - up;
+        exps[((size_t)(f0 + f) * N2 + j2) * gridDim.x + blockIdx.x] + 2 * kDrop + eS - up - L;
 }
 
 // Pass B of the inverse column transform: its conjugate, as doubles, [nf][ny][pitch]
