@@ -815,7 +815,8 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
   // lost in any case, and for factors that doubles hold) the factors are formed in fixed point;
   // otherwise in FP64.  Where the line lies: the relative error of u from u_t alone is 5e-17/cells
   // in fixed point below it (5e-12 at 1e-5 cells), 4e-16 in FP64.
-  const double h = p->grid.h, cells = c * t / h;
+  const double h = p->grid.h, ct = c * t, cells = ct / h;
+  const double cells_lo = (std::fma(-cells, h, ct) + std::fma(c, t, -ct)) / h;
   const bool fixed = cells >= 0.125 && cells < 9007199254740992.0 && std::isfinite(8 * c / h);
   if ((st = ensure_workspace(p, L.total + spec + nexp + (fixed ? 0 : spec))) || (st = wave_fx_prepare(p)))
     return st;
@@ -830,9 +831,9 @@ extern "C" fc2d_status fc2d_wave_interior(fc2d_plan_t p, int n_f, double c, doub
     void* z = k && !fixed ? S2 : S;
     if (k == 0 || !fixed) wave_fx_spectra(fa, n_f, eT, z, exps, s);
     double* out = k ? ut_out : u_out;
-    st = fixed ? wave_fx_eval(p, fa, n_f, k == 1, c, t, cells, eT, z, exps, ws(p, L.ointer), out,
+    st = fixed ? wave_fx_eval(p, fa, n_f, k == 1, c, t, cells, cells_lo, eT, z, exps, ws(p, L.ointer), out,
                               nullptr, nullptr, s)
-               : wave_fx_eval(p, fa, n_f, false, 1.0, 0.0, 0.0, 0, z, exps, ws(p, L.ointer), out,
+               : wave_fx_eval(p, fa, n_f, false, 1.0, 0.0, 0.0, 0.0, 0, z, exps, ws(p, L.ointer), out,
                               nullptr, nullptr, s);
     if (st) return st;
   }

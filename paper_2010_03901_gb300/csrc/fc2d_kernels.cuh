@@ -213,15 +213,16 @@ void launch_fft_cols(const FftArgs& fa, int n_f, bool fp64, void* inter, void* f
 void launch_complex_spectrum(int nx, int ny, int n_f, bool fp64, const void* half, void* out,
                              cudaStream_t s);
 // Fourier Forwarding in fixed point (fx_wave.cu): the spectra [2 n_f][ny][nx/2+1] (u's, then u_t's) to integers in place for times up to
-// 2^eT (exps: wave_fx_exps ints), then u or (deriv) u_t at t = cells h / c, on the grid or at
+// 2^eT (exps: wave_fx_exps ints), then u or (deriv) u_t at t = (cells + cells_lo) h / c, on the grid or at
 // listed points (off[ny + 1], linear indices ascending; out [point][n_f]); inter: 2 n_f ny pitch complex values.
 int wave_fx_time(double t, double h, double c);  // eT for times up to t
 size_t wave_fx_exps(int nx, int ny, int n_f);
 fc2d_status wave_fx_prepare(fc2d_plan_s* p);
 void wave_fx_spectra(const FftArgs& fa, int n_f, int eT, void* spec, int* exps, cudaStream_t s);
 fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
-                         double cells, int eT, const void* spec, int* exps, void* inter, double* out,
-                         const int32_t* off, const int32_t* points, cudaStream_t s);
+                         double cells, double cells_lo, int eT, const void* spec, int* exps,
+                         void* inter, double* out, const int32_t* off, const int32_t* points,
+                         cudaStream_t s);
 // the same solutions at time t in FP64: [2 n_f] spectra to u's (in place) and u_t's (deriv), each
 // for wave_fx_spectra with eT = 0 and wave_fx_eval at time 0
 void wave_modal_double(const FftArgs& fa, int n_f, double c, double t, double h, void* spec, void* deriv,

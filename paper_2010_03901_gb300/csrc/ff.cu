@@ -548,7 +548,7 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   // U_FC at tau = cells h / c: u, or (deriv) its time derivative, on the grid or at the
   // interface points
   auto eval_ufc = [&](double tau, double cells, bool deriv, double* out, bool points) {
-    return wave_fx_eval(p, fa, n_f, deriv, c, tau, cells, eT, spec, exps, inter, out,
+    return wave_fx_eval(p, fa, n_f, deriv, c, tau, cells, 0.0, eT, spec, exps, inter, out,
                         points ? b->iface_off : nullptr, points ? b->iface_lin : nullptr, s);
   };
   // U_B: u and w in (U[a], V[a]), the next ones into the other pair

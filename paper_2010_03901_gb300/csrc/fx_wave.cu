@@ -51,10 +51,13 @@ __global__ void k_modes(int nx, int ny, Mode* __restrict__ tab) {
   Mode o;
   o.kappa = (unsigned long long)fl + (unsigned long long)__double2ll_rn((hi - fl) + dq * 18446744073709551616.0);
   o.inv = 0;
-  if (s > 0) {
+  if (s > 0) {  // 1/(2 pi (q + dq)) = r + dr
+    const double two_pi = 6.283185307179586476925286766559, two_pi_lo = 2.4492935982947064e-16;
+    const double p = two_pi * q, dp = fma(two_pi, q, -p) + fma(two_pi_lo, q, two_pi * dq);
+    const double r = 1.0 / p, dr = r * (fma(-r, p, 1.0) - r * dp);
     int e;
-    const double f = frexp(1.0 / (6.283185307179586476925286766559 * q), &e);  // [1/2, 1)
-    o.inv = ((i64)(f * 36028797018963968.0) << 8) | (i64)(e & 255);  // 2^55; 0 < 1/(2 pi kappa)
+    const double f = frexp(r, &e);  // [1/2, 1)
+    o.inv = (((i64)(f * 36028797018963968.0) + __double2ll_rn(ldexp(dr, 55 - e))) << 8) | (i64)(e & 255);  // 2^55
   }
   tab[(size_t)m * (nx / 2 + 1) + l] = o;
 }
@@ -439,20 +442,31 @@ static int ilog2_exact(int n) {
   return l;
 }
 
-// (t, eT): t <= 2^eT; cells = c t / h
-static When when(double t, double cells, double c, double h, int eT) {
+// v + lo times 2^k, rounded
+static i64 scaled_pair(double v, double lo, int k) {
+  return (i64)std::ldexp(v, k) + (i64)std::nearbyint(std::ldexp(lo, k));
+}
+
+// (t, eT): t <= 2^eT; cells + cells_lo = c t / h.  Quotients in two doubles each: a factor rounded to
+// 53 bits is off by the same relative amount at every mode.
+static When when(double t, double cells, double cells_lo, double c, double h, int eT) {
   When w{};
   const double x = std::min(cells, 9.0e18), fl = std::floor(x);
-  w.cells = (unsigned long long)fl;
-  w.frac = (unsigned long long)std::ldexp(x - fl, 64);
+  const __int128 n = ((__int128)(i64)fl << 64) + (__int128)std::ldexp(x - fl, 64) +
+                     (__int128)std::nearbyint(std::ldexp(cells_lo, 64));
+  w.cells = n < 0 ? 0 : (unsigned long long)(n >> 64);
+  w.frac = n < 0 ? 0 : (unsigned long long)n;
   w.tau = (i64)std::ldexp(t, 62 - eT);
-  w.hc = (i64)std::ldexp(std::frexp(h / c, &w.ehc), 62);
+  const double hc = h / c, hc_lo = std::fma(-hc, c, h) / c;
+  std::frexp(hc, &w.ehc);
+  w.hc = scaled_pair(hc, hc_lo, 62 - w.ehc);
   w.ehc -= eT;
+  const double nu = 8 * c / h, nu_lo = std::fma(-nu, h, 8 * c) / h;
   int k;
-  std::frexp(8 * c / h, &k);
+  std::frexp(nu, &k);
   w.eT = eT;
   w.eS = std::max(k, -eT);
-  w.nu = (i64)std::ldexp(8 * c / h, 62 - w.eS);
+  w.nu = scaled_pair(nu, nu_lo, 62 - w.eS);
   w.down = eT + w.eS;
   return w;
 }
@@ -590,12 +604,13 @@ void wave_modal_double(const FftArgs& fa, int n_f, double c, double t, double h,
              fa.nx * h, fa.ny * h, (double2*)spec, (double2*)deriv);
 }
 
-// u (or, deriv, u_t) at time t = cells h / c of the modal solutions, on the grid or, with
+// u (or, deriv, u_t) at time t = (cells + cells_lo) h / c of the modal solutions, on the grid or, with
 // off, at the listed points (out[point][n_f]).  spec, exps: from wave_fx_spectra (exps has wave_fx_exps ints); inter:
 // 2 n_f ny pitch complex values of scratch.
 fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv, double c, double t,
-                         double cells, int eT, const void* spec, int* exps, void* inter, double* out,
-                         const int32_t* off, const int32_t* points, cudaStream_t s) {
+                         double cells, double cells_lo, int eT, const void* spec, int* exps,
+                         void* inter, double* out, const int32_t* off, const int32_t* points,
+                         cudaStream_t s) {
   fx::Modes* m;
   fc2d_status st = wave_modes(p, &m);
   if (st) return st;
@@ -603,7 +618,8 @@ fc2d_status wave_fx_eval(fc2d_plan_s* p, const FftArgs& fa, int n_f, bool deriv,
   const unsigned pitch = (unsigned)fa.pitch;
   // a speed or time without finite factors: NaN everywhere
   const bool lost = !std::isfinite(8 * c / p->grid.h) || !std::isfinite(t);
-  const fx::When w = lost ? fx::when(0.0, 0.0, 1.0, p->grid.h, 0) : fx::when(t, cells, c, p->grid.h, eT);
+  const fx::When w = lost ? fx::when(0.0, 0.0, 0.0, 1.0, p->grid.h, 0)
+                           : fx::when(t, cells, cells_lo, c, p->grid.h, eT);
   const int eS = lost ? fx::kNaN : deriv ? w.eS : 0;
   const int chunk = wave_chunk(fa, n_f);
   const size_t slab = (size_t)fa.ny * fa.pitch;

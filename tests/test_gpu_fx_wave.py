@@ -203,3 +203,34 @@ def test_transforms_of_smooth_fields(nx, ny):
     err = float((out[0] - ext).norm() / ext.norm())
     print(nx, ny, err * 2.0 ** 53)
     assert err < 3 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 512), (64, 4096), (4096, 64)])
+@pytest.mark.parametrize("cells", [8.0, 200.25])
+def test_phases_after_many_cells(nx, ny, cells):
+    """u from u alone: c t/h and the modes' frequencies carry two doubles, so that the phases add
+    nothing to the error of the two transforms (the bar of test_transforms_of_smooth_fields, 3 2^-53 of the
+    2-norm) however many turns they make; rounded to one double they add w t 2^-53."""
+    torch = pytest.importorskip("torch")
+    fft = pytest.importorskip("scipy.fft")
+    plan = plan_of(nx, ny)
+    h, c = 2.0 / (0.45 * min(nx, ny)), 1.7
+    t = cells * h / c
+    x, y = (np.arange(nx) - 0.5 * nx) * h, (np.arange(ny) - 0.5 * ny) * h
+    xy = plan.fc2d_boundary_points().T
+    fn = lambda X, Y: np.cos(2.1 * X + 0.3) * np.cos(1.7 * Y - 0.2)  # noqa: E731
+    u, ub = (torch.tensor(a[None], dtype=torch.float64, device="cuda")
+             for a in (fn(x[None, :], y[:, None]), fn(xy[0], xy[1])))
+    got, got_t, ext = torch.zeros_like(u), torch.zeros_like(u), torch.zeros_like(u)
+    plan.fc2d_wave_interior(1, c, t, u, ub, 0 * u, 0 * ub, got, got_t)
+    plan.fc2d_extend(1, u, ub, ext)
+    L = np.longdouble
+    F = fft.rfft2(ext.cpu().numpy()[0].astype(L))
+    l = np.arange(nx // 2 + 1).astype(L) / nx
+    m = np.minimum(np.arange(ny), ny - np.arange(ny)).astype(L) / ny
+    w = 2 * L("3.14159265358979323846264338327950288") * L(c) * np.sqrt(l[None, :] ** 2 + m[:, None] ** 2) / L(h)
+    ref = fft.irfft2(F * np.cos(w * L(t)), s=(ny, nx))
+    norm = lambda a: float(np.sqrt((np.abs(a) ** 2).sum()))  # noqa: E731
+    err = norm(got.cpu().numpy()[0] - ref) / norm(ref)
+    print(nx, ny, cells, err * 2.0 ** 53)
+    assert err < 3 * 2.0 ** -53
