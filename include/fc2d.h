@@ -223,8 +223,8 @@ fc2d_status fc2d_poisson_nodes(fc2d_plan_t plan, double* xy_host, int* n_b);
  * the trapezoidal rule with near-boundary refinement.  f_grid_dev [n_f][ny][nx] and
  * f_bdry_dev [n_f][n_bdry] as for fc2d_extend; g_nodes_dev [n_f][n_b]; u_dev [n_f][ny][nx]
  * receives u inside the domain and 0 elsewhere; phi_dev (NULL allowed) receives the
- * density [n_f][n_b].  GMRES is one cooperative launch per function (a block per SM) whose
- * outcome the host reads: this call waits for the stream.  Returns FC2D_ERR_NOT_CONVERGED if
+ * density [n_f][n_b].  GMRES is one cooperative launch per function (at most a block per SM of
+ * the stream's context) whose outcome the host reads: this call waits for the stream.  Returns FC2D_ERR_NOT_CONVERGED if
  * GMRES stalls. */
 fc2d_status fc2d_poisson(fc2d_plan_t plan, int n_f, const double* f_grid_dev,
                          const double* f_bdry_dev, const double* g_nodes_dev, double* u_dev,

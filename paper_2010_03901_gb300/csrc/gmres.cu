@@ -3,7 +3,8 @@
 //
 // At the sizes of a boundary integral equation (n about 1000) an iteration is a few
 // microseconds of work with three points at which every block needs every other one's
-// result.  The whole solve is one cooperative launch of one block per SM: the blocks keep
+// result.  The whole solve is one cooperative launch of one block per SM (fewer where
+// they do not fit at once): the blocks keep
 // their rows of A in shared memory (from L2 where they do not fit) and their rows of the
 // basis in L1, and meet three times per iteration.  Each phase ends with the blocks' partial
 // sums (projections or squares), which every block adds up in the same order.  w is kept
