@@ -29,6 +29,7 @@
 #include <map>
 #include <memory>
 #include <string>
+#include <type_traits>
 
 #include "fc2d_kernels.cuh"
 #include "fx_squares.h"
@@ -257,31 +258,55 @@ __device__ __forceinline__ double ub_value(uint32_t key, int f, int n_f, int64_t
 //   mode 2: (w' + w)/(2 dt), w' of mode 1, to Uout (the time derivative at u's time)
 // and u' = u + w'.  The FP64 pipe bounds it: w saves the difference u - u_prev of every
 // D entry (38 multiply-adds and 33 additions per value before), and does not cancel.
-// GRIDS false (the solve): function-minor rows, U [N + n_i][n_f] and Uold the step before (only its
-// interface rows are read), W [N][n_f]; Wout receives w'.  GRIDS true (a caller's own arrays): U and
+// UbRows (the solve): function-minor rows, U [N + n_i][n_f] and Uold the step before (only its
+// interface rows are read), W [N][n_f]; Wout receives w'.  UbGrids (a caller's own arrays): U and
 // Uold are u^n and u^{n-1} of the unknowns, the interface points iface[n_i] lie in grid and
 // grid_prev [n_f][stride], W is u_t (mode 0 only).
-template <bool GRIDS>
+struct UbRows {};
+struct UbGrids {
+  const double *grid, *grid_prev;
+  int64_t stride;
+  const int32_t* iface;
+};
+template <typename State>
 __global__ void __launch_bounds__(256) k_ub_advance(
     int mode, int n, int n_i, int n_f, int64_t n_b, const int2* __restrict__ Lrow,
     const UbEntry* __restrict__ Le, const int2* __restrict__ Drow, const UbEntry* __restrict__ De,
     const double* __restrict__ U, const double* __restrict__ Uold, const double* __restrict__ W,
-    const double* __restrict__ g, const double* __restrict__ grid, const double* __restrict__ grid_prev,
-    int64_t stride, const int32_t* __restrict__ iface, double cdt2, double dt, double sigma,
-    double* __restrict__ Uout, double* __restrict__ Wout) {
+    const double* __restrict__ g, double cdt2, double dt, double sigma, double* __restrict__ Uout,
+    double* __restrict__ Wout, State state) {
+  constexpr bool GRIDS = std::is_same<State, UbGrids>::value;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n_f) return;
   const int r = (int)(t / n_f), f = (int)(t - (int64_t)r * n_f);
   const double u = U[t], w = GRIDS && mode ? u - Uold[t] : W[t];
   double lap = 0.0, dis = 0.0;
   const double *Uf = U + f, *Wf = W + f;
-  auto face = [&](int col) { return (size_t)f * stride + __ldg(iface + (col - n)); };  // GRIDS
+  // GRIDS: the interface point of a column in a grid
+  auto face = [&](int col) -> size_t {
+    if constexpr (GRIDS) return (size_t)f * state.stride + __ldg(state.iface + (col - n));
+    else return 0;
+  };
+  // u at a column, D's difference at a column of each kind
+  auto value = [&](int col) {
+    if constexpr (GRIDS) return col >= n ? state.grid[face(col)] : Uf[(size_t)col * n_f];
+    else return Uf[(size_t)col * n_f];
+  };
+  auto step = [&](int col) {
+    const size_t o = (size_t)col * n_f;
+    if constexpr (GRIDS) return Uf[o] - Uold[o + f];
+    else return Wf[o];
+  };
+  auto face_step = [&](int col) {
+    if constexpr (GRIDS) return state.grid[face(col)] - state.grid_prev[face(col)];
+    else return U[(size_t)col * n_f + f] - Uold[(size_t)col * n_f + f];
+  };
   const int2 l0 = __ldg(Lrow + r);
   const int l1 = __ldg(&Lrow[r + 1].x);
 #pragma unroll 4
   for (int k = l0.x; k < l0.y; ++k) {
     const UbEntry e = Le[k];
-    lap += e.w * (GRIDS && e.col >= n ? grid[face(e.col)] : Uf[(size_t)e.col * n_f]);
+    lap += e.w * value(e.col);
   }
   if (g)  // boundary points
     for (int k = l0.y; k < l1; ++k) {
@@ -297,13 +322,11 @@ __global__ void __launch_bounds__(256) k_ub_advance(
 #pragma unroll 4
     for (int k = d0.x; k < d0.y; ++k) {
       const UbEntry e = De[k];
-      const size_t o = (size_t)e.col * n_f;
-      dis += e.w * (GRIDS ? Uf[o] - Uold[o + f] : Wf[o]);
+      dis += e.w * step(e.col);
     }
     for (int k = d0.y; k < d1; ++k) {  // interface points
       const UbEntry e = De[k];
-      const size_t o = GRIDS ? face(e.col) : (size_t)e.col * n_f + f;
-      dis += e.w * (GRIDS ? grid[o] - grid_prev[o] : U[o] - Uold[o]);
+      dis += e.w * face_step(e.col);
     }
     wn = w + cdt2 * lap - sigma * dis;
     if (mode == 2) {
@@ -471,10 +494,10 @@ extern "C" fc2d_status fc2d_wave_ub_step(fc2d_plan_t p, int n_c, int n_f, int mo
   const double dt = kUbCfl * h / c;
   const int64_t n = (int64_t)b->host.unknown_lin.size();
   if (n > 0)
-    k_ub_advance<true><<<blocks(n * n_f, 256), 256, 0, (cudaStream_t)stream>>>(
+    k_ub_advance<<<blocks(n * n_f, 256), 256, 0, (cudaStream_t)stream>>>(
         mode, (int)n, (int)b->host.iface_lin.size(), n_f, p->n_bdry, b->L.row, b->L.e, b->D.row, b->D.e,
-        u, u_prev, ut, g, grid, grid_prev, (int64_t)p->grid.nx * p->grid.ny, b->iface_lin, cdt2, dt,
-        kUbSigma, out, nullptr);
+        u, u_prev, ut, g, cdt2, dt, kUbSigma, out, nullptr,
+        UbGrids{grid, grid_prev, (int64_t)p->grid.nx * p->grid.ny, b->iface_lin});
   return cuda_check(cudaGetLastError(), "fc2d_wave_ub_step");
 }
 
@@ -561,9 +584,9 @@ extern "C" fc2d_status fc2d_forward_wave(fc2d_plan_t p, int n_f, double c, int n
   auto ub_step = [&](int mode, const double* g, double* uo, double* wo) {
     if (Nu == 0) return;
     ProfScope ps(p, "ub_step", s);
-    k_ub_advance<false><<<blocks(Nu * n_f, 256), 256, 0, s>>>(
+    k_ub_advance<<<blocks(Nu * n_f, 256), 256, 0, s>>>(
         mode, (int)Nu, (int)Ni, n_f, nb, b->L.row, b->L.e, b->D.row, b->D.e, U[a], U[1 - a], V[a],
-        g, nullptr, nullptr, 0, nullptr, cdt2, dt, kUbSigma, uo, wo);
+        g, cdt2, dt, kUbSigma, uo, wo, UbRows{});
   };
   // U_B at t = 0: u^0, and u_t^0 in the place of w
   gather(Nu, b->unknown_lin, u, U[a]);
